@@ -19,7 +19,7 @@ HALF_W, HALF_H = 320.0, 240.0   # 640 x 480 images
 
 
 def _case(name, scene, cams, points, lmax=50, cap=100, clusters="joins", precision="mixed", entry="iterate", iters=5,
-          lambda0=3e-2, huber=0.0, solver="clusters"):
+          lambda0=0.05, huber=0.0, solver="clusters"):
     c = dict(scene=scene, cams=cams, points=points, lmax=lmax, cap=cap, clusters=clusters, precision=precision,
              entry=entry, iters=iters, lambda0=lambda0, huber=huber, solver=solver)
     return dict(c, name=name) if name else c
@@ -28,7 +28,7 @@ def _case(name, scene, cams, points, lmax=50, cap=100, clusters="joins", precisi
 def listed():
     return [
         # the smallest call: a local window of a tracker, refined in a few iterations
-        _case("window_10", "ring", 10, 200, cap=5, clusters="spatial", iters=5),
+        _case("window_10", "ring", 10, 200, cap=5, clusters="spatial", iters=3, lambda0=0.3),
         # the 30-camera ring in FP64, the library's default precision, with fixed clusters
         _case("ring_30_fp64", "ring", 30, 2000, cap=10, clusters="spatial", precision="fp64", iters=5),
         # FP64 at clusters of full size, with the heavy damping that turns the steepest-descent correction on
@@ -38,17 +38,17 @@ def listed():
         # the same with a fixed spatial partition and the Huber loss of the paper's experiments
         _case("photos_1000_huber", "hemisphere", 1000, 200_000, clusters="spatial", iters=5, huber=0.5),
         # sequential frames: uneven contiguous clusters of 20 to 300 cameras, re-used every iteration
-        _case("drive_2000_uneven", "drive", 2000, 200_000, lmax=20, cap=300, clusters="uneven", iters=3),
+        _case("drive_2000_uneven", "drive", 2000, 200_000, lmax=20, cap=300, clusters="uneven", iters=3, lambda0=0.09),
         # all cameras in one dense system: plain LM with the full reduced camera system
         _case("photos_400_dense", "hemisphere", 400, 40_000, cap=400, clusters="spatial", iters=2),
         # a large collection: more clusters than the GPU factors at once
         _case("photos_6000_draws", "hemisphere", 6000, 900_000, lmax=80, iters=2),
         # differentiable use: a recorded solve and its reverse pass
-        _case("adjoint_500", "hemisphere", 500, 50_000, clusters="spatial", entry="adjoint", iters=5, lambda0=0.1),
+        _case("adjoint_500", "hemisphere", 500, 50_000, clusters="spatial", entry="adjoint", iters=4, lambda0=0.3),
         # the conjugate-gradient solvers: the full system, and the clustered one
-        _case("photos_1000_pcg", "hemisphere", 1000, 200_000, iters=1, lambda0=1e-3, clusters="spatial",
+        _case("photos_1000_pcg", "hemisphere", 1000, 200_000, iters=1, lambda0=1e-2, clusters="spatial",
               solver="pcg_full"),
-        _case("photos_500_pcg_split", "hemisphere", 500, 50_000, iters=1, lambda0=1e-3, clusters="spatial",
+        _case("photos_500_pcg_split", "hemisphere", 500, 50_000, iters=1, lambda0=1e-2, clusters="spatial",
               solver="pcg_clusters"),
         # F(x) alone, without allocation, on arrays the caller holds
         _case("cost_1000", "hemisphere", 1000, 200_000, precision="fp64", entry="cost"),
@@ -63,9 +63,9 @@ def draw(rng):
     kind = rng.choice(["window", "ring64", "photos64", "photos", "photos", "photos", "huber", "drive", "drive", "dense",
                        "adjoint", "pcg", "split", "cost"])
     if kind == "window":
-        m = _log(rng, 8, 40)
+        m = _log(rng, 10, 40)
         return _case("", "ring", m, _log(rng, 20 * m, 100 * m), cap=max(3, m // rng.randint(1, 4)), clusters="spatial",
-                     iters=rng.randint(1, 5))
+                     iters=rng.randint(1, 3), lambda0=0.3)
     if kind == "ring64":
         m = _log(rng, 10, 60)
         return _case("", "ring", m, _log(rng, 25 * m, 100 * m), cap=rng.randint(5, 20), clusters="spatial",
@@ -73,7 +73,7 @@ def draw(rng):
     m = _log(rng, 150, 3000)
     n = _log(rng, 100 * m, 220 * m)
     cap = rng.choice([40, 70, 100, 100, 150])
-    lam = rng.choice([1e-2, 3e-2, 3e-2, 0.2])
+    lam = rng.choice([0.05, 0.09, 0.2])
     if kind == "photos64":
         m = _log(rng, 100, 400)
         return _case("", "hemisphere", m, _log(rng, 60 * m, 150 * m), cap=rng.choice([40, 70, 100]), precision="fp64",
@@ -94,10 +94,10 @@ def draw(rng):
     if kind == "adjoint":
         m = _log(rng, 100, 600)
         return _case("", "hemisphere", m, _log(rng, 60 * m, 120 * m), cap=rng.choice([40, 70, 100]), clusters="spatial",
-                     entry="adjoint", iters=rng.randint(2, 5), lambda0=rng.choice([0.05, 0.1, 0.3]))
+                     entry="adjoint", iters=rng.randint(2, 4), lambda0=rng.choice([0.2, 0.3, 1.0]))
     if kind in ("pcg", "split"):
         m = _log(rng, 150, 1000)
-        return _case("", "hemisphere", m, _log(rng, 100 * m, 200 * m), cap=cap, clusters="spatial", iters=1, lambda0=1e-3,
+        return _case("", "hemisphere", m, _log(rng, 100 * m, 200 * m), cap=cap, clusters="spatial", iters=1, lambda0=1e-2,
                      solver="pcg_full" if kind == "pcg" else "pcg_clusters")
     return _case("", "hemisphere", m, n, lmax=rng.randint(20, 80), precision="fp64", entry="cost")
 
