@@ -1540,8 +1540,8 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
       B.uvp = uv;
       B.split = true;
     }
-    if ((s = dalloc(c, &J, 24 * (size_t)q * rs)) != STBA_OK) return bail(s);
-    if ((s = dalloc(c, &pw, 9 * (size_t)m * rs)) != STBA_OK) return bail(s);
+    if ((s = dalloc(c, &J, 24 * (((size_t)q + 31) / 32 * 32) * rs)) != STBA_OK) return bail(s);
+    if ((s = dalloc(c, &pw, 12 * (size_t)m * rs)) != STBA_OK) return bail(s);
     if ((s = dalloc(c, &tpt, 3 * (size_t)n * rs)) != STBA_OK) return bail(s);
     if ((s = dalloc(c, &upt, 3 * (size_t)n * rs)) != STBA_OK) return bail(s);
     B.J = J;
@@ -1555,8 +1555,8 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
     if ((s = dalloc(c, &B.Bdiag, 9 * (size_t)m)) != STBA_OK) return bail(s);
     if ((s = dalloc(c, &B.Minv, 81 * (size_t)m)) != STBA_OK) return bail(s);
     if ((s = dalloc(c, &B.scal, 8)) != STBA_OK) return bail(s);
-    if ((s = dalloc(c, &B.partial, 3 * (size_t)RED_BLOCKS)) != STBA_OK) return bail(s);
-    if ((s = dalloc(c, &B.partial2, 3 * (size_t)RED_BLOCKS)) != STBA_OK) return bail(s);
+    if ((s = dalloc(c, &B.partial, 2 * (size_t)RED_BLOCKS)) != STBA_OK) return bail(s);
+    if ((s = dalloc(c, &B.pq, 64)) != STBA_OK) return bail(s);
   }
   {
     cudaError_t e1 = cudaMemcpyAsync(c->cams, h_cams.data(), h_cams.size() * 8, cudaMemcpyHostToDevice, c->stream);
@@ -1644,6 +1644,12 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
       for (int w = 0; w < nw; ++w) warp_cam.push_back((int)j);
     }
     const int nwarps = cam_warp_off[m];
+    if (c->use_pcg || c->use_spcg) {
+      char* js;
+      if ((s = dalloc(c, &js, 24 * 32 * (size_t)nwarps * (c->mixed ? sizeof(float) : sizeof(double)))) != STBA_OK)
+        return bail(s);
+      c->pcg.Jslot = js;
+    }
     ReorderArgs& A = c->reorder;
     A.q = (int)q;
     A.n = (int)n;

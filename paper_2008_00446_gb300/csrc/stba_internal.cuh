@@ -318,17 +318,19 @@ void launch_set_lambda(DevState* st, double lam, cudaStream_t stream);
 
 // Full-RCS comparator (stba_pcg.cu): block-Jacobi preconditioned CG on S dc = b over all cameras, matrix-free.
 struct PcgBuffers {
-  void* J;          // [q][24] J_c and J_p of every observation (working precision)
+  void* J;          // [q rounded up to 32][24] J_c and J_p of every observation (working precision), in groups of
+                    // 32 records interleaved by 16-byte pieces
+  void* Jslot;      // [32 * nwarps][24] the same in the order of the camera passes' slots
   double* Mblk;     // [m][45] diagonal blocks of S (lower, undamped B part)
   double* Bdiag;    // [m][9] diag(J_c^T J_c)
   double* Minv;     // [m][81] inverse damped diagonal blocks (the preconditioner)
   double *x, *r, *z, *p, *q;   // [m][9] CG vectors (q also carries the right-hand side at the start)
-  void* pw;         // [m][9] p in the working precision
+  void* pw;         // [m][12] p in the working precision (9 used)
   void* tpt;        // [n][3] E^T p
   void* upt;        // [n][3] C^-1 E^T p
   double* scal;     // b.b, r.z (two parity slots), r.r
-  double* partial;  // [3][RED_BLOCKS]
-  double* partial2; // [3][RED_BLOCKS]
+  double* partial;  // [2][RED_BLOCKS] partial sums of r.z and r.r
+  double* pq;       // [64] accumulators of p.q
   bool split;       // STBA_SOLVER_PCG_CLUSTERS: the method's clustered system S' over virtual points
   void* tvp;        // [q][3] (split) E'^T p per virtual point, working precision
   void* uvp;        // [q][3] (split) C'^-1 E'^T p
