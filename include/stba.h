@@ -104,15 +104,15 @@ typedef struct {
                                the SMs, else 4): more CTAs share a tile step's products, fewer make its
                                cluster barrier and distributed-shared-memory exchange cheaper. */
   int32_t pair_blocks;      /* off-diagonal camera blocks of S' (Eq. 10, 13), -sum over the observation pairs
-                               of a virtual point of G_a^T G_b with G_o = L_v^-1 Jp,o^T Jc,o:
-                               STBA_PAIR_BLOCKS_RECOMPUTE (default) = the pair pass recomputes each G_o from
-                               the point, the observation, its residual and the virtual point's L_v^-1 (no G
-                               buffer, fewer bytes moved);
-                               STBA_PAIR_BLOCKS_STORED = the camera pass stores every G_o (36 reals per
-                               observation of device memory) and the pair pass reads them.
-                               Both give the same S': in FP32 every pass evaluates the Jacobian rows with
-                               each operation rounded on its own, so stored and recomputed G_o are bitwise
-                               equal (up to the order of the FP64 atomic sums). */
+                               of a virtual point of Jc_a^T (P_a^T P_b) Jc_b with P_o = L_v^-1 Jp,o^T:
+                               STBA_PAIR_BLOCKS_RECOMPUTE = the pair pass recomputes P_o and Jc_o from the
+                               point, the camera and the virtual point's L_v^-1 (no buffer, fewer bytes moved);
+                               STBA_PAIR_BLOCKS_STORED = the camera pass stores them (24 reals per
+                               observation of device memory) and the pair pass reads them;
+                               0 (default) = RECOMPUTE in mixed precision; in FP64 STORED while that takes at
+                               most a quarter of the free device memory at create, else RECOMPUTE.
+                               Both give the same S': every pass evaluates the same rows (in FP32 with each
+                               operation rounded on its own), up to the order of the FP64 atomic sums. */
   int32_t factor_fp64;      /* STBA_MIXED only: 1 = factor the cluster systems in FP64 (tile 32, CUDA cores)
                                under the FP32 Jacobians and Schur terms instead of the default FP32 factor
                                with FP64 refinement -- the precision Eq. 13's solve has in the paper's

@@ -33,6 +33,7 @@
 #include <climits>
 
 #include "stba_camera.cuh"
+#include "stba_camtab.cuh"
 #include "stba_device.cuh"
 #include "stba_dual.cuh"
 #include "stba_internal.cuh"
@@ -43,14 +44,16 @@ namespace {
 
 constexpr int ADJ_THREADS = 128;
 
-// One observation's camera, point and measurement in the working precision: FP64 from the parameters, or
-// the per-iteration FP32 copies in mixed precision (the forward step's Jacobians are FP32 there too).
+// J_c and J_p of the observation at sorted position o: the forward step's rows (stba_camtab.cuh).
 template <typename real>
-__device__ __forceinline__ void load_obs_w(const DevProblem& P, int o, Cam<real>& C, real X[3], real& uo,
-                                           real& vo) {
-  C = load_cam_w<real>(P, P.obs_cam[o]);
+__device__ __forceinline__ void obs_rows(const DevProblem& P, int o, real (&Jc)[2][9], real (&Jp)[2][3]) {
+  const int cam = P.obs_cam[o];
+  const CamRow<real> C = gather_camrow<real>(P, cam);
+  real X[3], Jl[9];
   load_point_w<real>(P, P.obs_pt[o], X);
-  load_uv<real>(P, o, uo, vo);
+  proj_rows<real, true>(C, X, Jc, Jp);
+  load_jl(P, cam, Jl);
+  apply_jl<real>(Jl, Jc);
 }
 
 template <typename real>
@@ -96,10 +99,8 @@ __global__ void __launch_bounds__(ADJ_THREADS) k_adj_cam_rhs(DevProblem P, CamLi
   for (int i = 0; i < 9; ++i) acc[i] = 0.0;
   for (int e = CL.cam_obs_off[j] + threadIdx.x; e < CL.cam_obs_off[j + 1]; e += blockDim.x) {
     const int o = CL.cam_obs[e];
-    Cam<real> C;
-    real X[3], uo, vo, r[2], Jc[2][9], Jp[2][3];
-    load_obs_w<real>(P, o, C, X, uo, vo);
-    project_jacobian<real, true>(C, X, uo, vo, r, Jc, Jp);
+    real Jc[2][9], Jp[2][3];
+    obs_rows<real>(P, o, Jc, Jp);
     const double* up = u + 3 * (size_t)P.obs_pt[o];
     const real u0 = (real)up[0], u1 = (real)up[1], u2 = (real)up[2];
     const real t0 = Jp[0][0] * u0 + Jp[0][1] * u1 + Jp[0][2] * u2;
@@ -125,10 +126,8 @@ __global__ void __launch_bounds__(256) k_adj_vp(DevProblem P, const double* __re
   double val[6] = {0, 0, 0, 0, 0, 0};
   if (act) {
     v = P.obs_vp[o];
-    Cam<real> C;
-    real X[3], uo, vo, r[2], Jc[2][9], Jp[2][3];
-    load_obs_w<real>(P, o, C, X, uo, vo);
-    project_jacobian<real, true>(C, X, uo, vo, r, Jc, Jp);
+    real Jc[2][9], Jp[2][3];
+    obs_rows<real>(P, o, Jc, Jp);
     const double* z = zc + 9 * (size_t)P.obs_cam[o];
     const double* d = dc + 9 * (size_t)P.obs_cam[o];
     real jz0 = 0, jz1 = 0, jd0 = 0, jd1 = 0;
@@ -155,7 +154,7 @@ __global__ void __launch_bounds__(256) k_adj_vp(DevProblem P, const double* __re
 template <typename real>
 __global__ void k_adj_vp_final(int nv, const real* __restrict__ vp_info, double* __restrict__ vpz) {
   for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += gridDim.x * blockDim.x) {
-    const real* in = vp_info + 9 * (size_t)v;
+    const real* in = vp_info + VPI * (size_t)v;
     double Li[6];
 #pragma unroll
     for (int c = 0; c < 6; ++c) Li[c] = (double)in[c];
@@ -167,7 +166,7 @@ __global__ void k_adj_vp_final(int nv, const real* __restrict__ vp_info, double*
 #pragma unroll
     for (int s = 0; s < 3; ++s) {
       e[s] = -x1[s];
-      e[3 + s] = (double)in[6 + s] - x2[s];
+      e[3 + s] = (double)in[VPI_Y + s] - x2[s];
     }
   }
 }
@@ -205,8 +204,8 @@ __global__ void k_adj_zeta(DevProblem P, const real* __restrict__ vp_acc, const 
 // out += sum_s alpha_s d/de J_s(theta + e beta) (12 entries: camera 9, point 3) for one observation, on
 // dual numbers of the working precision.
 template <typename real>
-__device__ __forceinline__ void hess_vec(const Cam<real>& C0, const real X0[3], real uo, real vo, real al0, real al1,
-                                         const real beta[12], real out[12]) {
+__device__ __forceinline__ void hess_vec(const Cam<real>& C0, const real X0[3], real al0, real al1, const real beta[12],
+                                         real out[12]) {
   using D = DualT<real>;
   Cam<D> C;
 #pragma unroll
@@ -219,7 +218,7 @@ __device__ __forceinline__ void hess_vec(const Cam<real>& C0, const real X0[3], 
   C.k2 = D(C0.k2, beta[8]);
   const D X[3] = {D(X0[0], beta[9]), D(X0[1], beta[10]), D(X0[2], beta[11])};
   D r[2], Jc[2][9], Jp[2][3];
-  project_jacobian<D, true>(C, X, D(uo), D(vo), r, Jc, Jp);
+  project_jacobian<D, true>(C, X, D(real(0)), D(real(0)), r, Jc, Jp);   // the pixel enters r only
 #pragma unroll
   for (int c = 0; c < 9; ++c) out[c] += al0 * Jc[0][c].d + al1 * Jc[1][c].d;
 #pragma unroll
@@ -240,10 +239,10 @@ __global__ void __launch_bounds__(ADJ_THREADS) k_adj_obs(DevProblem P, const int
   const int o = blockIdx.x * blockDim.x + threadIdx.x;
   if (o >= P.q) return;
   const int cam = P.obs_cam[o], pt = P.obs_pt[o], v = P.obs_vp[o];
-  Cam<real> C;
-  real X[3], uo, vo, f[2], Jc[2][9], Jp[2][3];
-  load_obs_w<real>(P, o, C, X, uo, vo);
-  project_jacobian<real, true>(C, X, uo, vo, f, Jc, Jp);
+  const Cam<real> C = load_cam_w<real>(P, cam);   // for the dual-number products
+  real X[3], f[2], Jc[2][9], Jp[2][3];
+  load_point_w<real>(P, pt, X);
+  obs_rows<real>(P, o, Jc, Jp);
   f[0] = res_ptr<real>(P)[2 * (size_t)o];
   f[1] = res_ptr<real>(P)[2 * (size_t)o + 1];
   real z[12], dx[12], uu[3], dpp[3];
@@ -359,7 +358,7 @@ __global__ void __launch_bounds__(ADJ_THREADS) k_adj_obs(DevProblem P, const int
         for (int k = 0; k < 3; ++k) beta[9 + k] = (s == 0 ? Jp[0][k] : Jp[1][k]) * wdm[9 + k];
       }
     }
-    hess_vec<real>(C, X, uo, vo, al0, al1, beta, acc);
+    hess_vec<real>(C, X, al0, al1, beta, acc);
   }
   double* To = T + 12 * (size_t)o;
 #pragma unroll
@@ -419,7 +418,7 @@ void launch_adjoint_step(const DevProblem& P, Scratch<real> W, CamLists CL, cons
   int64_t v_total = fb.v_total;
   cudaMemsetAsync(W.b, 0, (size_t)v_total * sizeof(double), stream);
   k_adj_cam_rhs<real><<<P.m, ADJ_THREADS, 0, stream>>>(P, CL, A.u, A.a_c, W.b);
-  launch_solve<real>(P, W.S, W.b, fb, plan, refine_steps, A.zc, nullptr, stream);
+  launch_solve<real>(P, W.S, W.b, fb, plan, refine_steps, A.zc, stream);
   cudaMemsetAsync(A.vpz, 0, 6 * (size_t)P.nv * sizeof(double), stream);
   k_adj_vp<real><<<(P.q + 255) / 256, 256, 0, stream>>>(P, A.zc, W.dc, A.vpz);
   k_adj_vp_final<real><<<std::min((P.nv + 255) / 256, 4096), 256, 0, stream>>>(P.nv, W.vp_info, A.vpz);

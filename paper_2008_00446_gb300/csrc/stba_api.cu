@@ -86,7 +86,9 @@ struct stba_ctx {
   CamSlots cslots{};
   PairChunks pchunks{};
   CameraGraph cgraph;                   // camera graph with its observation pairs (host copy)
-  void* Gbuf = nullptr;
+  void* rowbuf = nullptr;               // stored rows of the pair pass (or a placeholder)
+  void* ctab = nullptr;                 // camera tables
+  bool pair_recompute = true;
   // re-ordering for new assignments: fixed arguments, the two inverse maps (previous / current), scratch
   ReorderArgs reorder{};
   int* inv[2] = {nullptr, nullptr};
@@ -115,7 +117,8 @@ struct stba_ctx {
        *t_acc = nullptr;
   double *dc = nullptr, *dp = nullptr, *partial = nullptr, *cam_rt = nullptr;
   float *cam_df = nullptr, *pt_df = nullptr;   // double-float tables of the mixed-mode cost
-  float *cams_f = nullptr, *pts_f = nullptr, *dcf = nullptr;   // FP32 copies (mixed precision)
+  float *cams_f = nullptr, *pts_f = nullptr;   // FP32 copies (mixed precision)
+  void* edc = nullptr;                         // E dc per camera (working precision)
   float4* obs_uvdf = nullptr;
   void *res_cur = nullptr, *res_cand = nullptr;   // residuals at x and at x + dx (working precision)
   DevState* st = nullptr;
@@ -277,8 +280,11 @@ DevProblem dev_problem(const stba_ctx* c) {
   P.huber_a = c->opt.huber_a;
   P.res_f = c->mixed ? (const float*)c->res_cur : nullptr;
   P.res_d = c->mixed ? nullptr : (const double*)c->res_cur;
+  P.ctab_f = c->mixed ? (const float*)c->ctab : nullptr;
+  P.ctab_d = c->mixed ? nullptr : (const double*)c->ctab;
+  P.base_vp = c->reorder.base_vp;
   P.base_pos = c->inv[c->inv_cur];
-  P.pair_recompute = c->opt.pair_blocks == STBA_PAIR_BLOCKS_STORED ? 0 : 1;   // recomputed by default
+  P.pair_recompute = c->pair_recompute ? 1 : 0;
   P.sharded = c->shard_world > 1 ? 1 : 0;
   P.cluster_owned = c->cl_owned;
   return P;
@@ -296,7 +302,7 @@ Scratch<real> scratch(const stba_ctx* c) {
   W.vgrad = (real*)c->vgrad;
   W.t_acc = (real*)c->t_acc;
   W.dc = c->dc;
-  W.dcf = c->dcf;
+  W.edc = (real*)c->edc;
   W.dp = c->dp;
   W.partial = c->partial;
   return W;
@@ -720,7 +726,7 @@ void enqueue_step(stba_ctx* c, bool stages) {
   mark(0);
   // stage 0: linearisation and virtual points
   launch_iter_begin<real>(c->st, c->set, s);
-  if (c->mixed) launch_params_to_float(P, c->cams_f, c->pts_f, s);
+  launch_params<real>(P, (real*)c->ctab, c->cams_f, c->pts_f, s);
   launch_zero_vp(c->vp_acc, c->counts, (int)rs, s);   // 9 nv reals, nv from the device counter
   cudaMemsetAsync(c->S, 0, (size_t)c->S_total * sizeof(double), s);
   cudaMemsetAsync(c->b, 0, (size_t)c->v_total * sizeof(double), s);
@@ -731,7 +737,7 @@ void enqueue_step(stba_ctx* c, bool stages) {
   launch_vp_finalize<real>(P, W, c->st, c->counts, s);
   mark(1);
   // stage 1: S' and b'
-  launch_rcs_build<real>(P, W, c->cslots, c->pchunks, (real*)c->Gbuf, c->st, s, c->side_stream, c->ev_sfork,
+  launch_rcs_build<real>(P, W, c->cslots, c->pchunks, (real*)c->rowbuf, c->st, s, c->side_stream, c->ev_sfork,
                          c->ev_sjoin);
   mark(2);
   // stage 2: factorisation (FP32 factor in mixed mode, FP64 factor in FP64 mode)
@@ -742,12 +748,13 @@ void enqueue_step(stba_ctx* c, bool stages) {
   mark(3);
   // stage 3: cluster solves with FP64 refinement
   if (c->f32f)
-    launch_solve<float>(P, W.S, W.b, c->fbuf, c->cplan, c->set.refine_steps, c->dc, c->dcf, s);
+    launch_solve<float>(P, W.S, W.b, c->fbuf, c->cplan, c->set.refine_steps, c->dc, s);
   else
-    launch_solve<double>(P, W.S, W.b, c->fbuf, c->cplan, c->set.refine_steps, c->dc, c->dcf, s);
+    launch_solve<double>(P, W.S, W.b, c->fbuf, c->cplan, c->set.refine_steps, c->dc, s);
   launch_count_failures(c->fail_flags, c->l, c->st, s);
   mark(4);
   // stage 4: points, cost, control
+  launch_step_rows<real>(P, c->dc, (real*)c->edc, s);
   launch_point_rhs<real>(P, W, s);
   launch_point_update<real>(P, W, s);
 }
@@ -773,7 +780,7 @@ int enqueue_pcg_iteration(stba_ctx* c) {
   cudaStream_t s = c->stream;
   record_stage(c, 0);
   launch_iter_begin<real>(c->st, c->set, s);
-  if (c->mixed) launch_params_to_float(P, c->cams_f, c->pts_f, s);
+  launch_params<real>(P, (real*)c->ctab, c->cams_f, c->pts_f, s);
   launch_zero_vp(c->vp_acc, c->counts, (int)sizeof(real), s);
   cudaMemsetAsync(c->t_acc, 0, 3 * (size_t)c->n * sizeof(real), s);
   if (c->use_spcg) {
@@ -787,7 +794,7 @@ int enqueue_pcg_iteration(stba_ctx* c) {
   if (c->use_spcg) {   // the camera pass alone: b', v and the diagonal blocks of S'
     PairChunks none = c->pchunks;
     none.nchunks = 0;
-    launch_rcs_build<real>(P, W, c->cslots, none, (real*)c->Gbuf, c->st, s);
+    launch_rcs_build<real>(P, W, c->cslots, none, (real*)c->rowbuf, c->st, s);
   }
   pcg_prepare<real>(P, W, c->cslots, c->pcg, c->st, s);
   record_stage(c, 2);
@@ -877,7 +884,7 @@ stba_status run_sharded_iteration(stba_ctx* c) {
   const size_t rs = sizeof(real);
   record_stage(c, 0);
   launch_iter_begin<real>(c->st, c->set, s);
-  if (c->mixed) launch_params_to_float(P, c->cams_f, c->pts_f, s);
+  launch_params<real>(P, (real*)c->ctab, c->cams_f, c->pts_f, s);
   launch_zero_vp(c->vp_acc, c->counts, (int)rs, s);
   cudaMemsetAsync(c->S, 0, (size_t)c->S_total * sizeof(double), s);
   cudaMemsetAsync(c->b, 0, (size_t)c->v_total * sizeof(double), s);
@@ -889,7 +896,7 @@ stba_status run_sharded_iteration(stba_ctx* c) {
   if ((st = shard_exchange(c, c->xch, 9 * (int64_t)c->n, 0)) != STBA_OK) return st;
   launch_vp_finalize<real>(P, W, c->st, c->counts, s, c->xch);
   record_stage(c, 1);
-  launch_rcs_build<real>(P, W, c->cslots, c->pchunks, (real*)c->Gbuf, c->st, s);
+  launch_rcs_build<real>(P, W, c->cslots, c->pchunks, (real*)c->rowbuf, c->st, s);
   record_stage(c, 2);
   if (c->f32f)
     launch_factor<float>(P, W.S, c->fbuf, c->cplan, s);
@@ -897,9 +904,9 @@ stba_status run_sharded_iteration(stba_ctx* c) {
     launch_factor<double>(P, W.S, c->fbuf, c->cplan, s);
   record_stage(c, 3);
   if (c->f32f)
-    launch_solve<float>(P, W.S, W.b, c->fbuf, c->cplan, c->set.refine_steps, c->dc, c->dcf, s);
+    launch_solve<float>(P, W.S, W.b, c->fbuf, c->cplan, c->set.refine_steps, c->dc, s);
   else
-    launch_solve<double>(P, W.S, W.b, c->fbuf, c->cplan, c->set.refine_steps, c->dc, c->dcf, s);
+    launch_solve<double>(P, W.S, W.b, c->fbuf, c->cplan, c->set.refine_steps, c->dc, s);
   launch_count_failures(c->fail_flags, c->l, c->st, s);
   double* nfail = c->xch + 9 * (size_t)c->n;
   launch_failed_io(c->st, nfail, 1, s);
@@ -907,7 +914,7 @@ stba_status run_sharded_iteration(stba_ctx* c) {
   if ((st = shard_exchange(c, c->vgrad, 9 * (int64_t)c->m, c->mixed ? 1 : 0)) != STBA_OK) return st;
   if ((st = shard_exchange(c, nfail, 1, 0)) != STBA_OK) return st;
   launch_failed_io(c->st, nfail, 0, s);
-  if (c->mixed) launch_dc_to_float(c->dc, c->dcf, 9 * (int64_t)c->m, s);
+  launch_step_rows<real>(P, c->dc, (real*)c->edc, s);
   record_stage(c, 4);
   launch_point_rhs<real>(P, W, s);
   launch_point_update<real>(P, W, s);
@@ -937,7 +944,7 @@ uint64_t graph_signature(const stba_ctx* c) {
   mix((uint64_t)c->set.refine_steps);
   mix((uint64_t)(c->mixed ? 1 : 0));
   mix((uint64_t)((c->pchunks.nchunks > 0 && c->l < c->m) ? 1 : 0));
-  mix((uint64_t)c->opt.pair_blocks);
+  mix((uint64_t)(c->pair_recompute ? 1 : 0));
   for (int kt = 0; kt < p.nsteps; ++kt) {
     const int npn = p.h_panel_off[kt + 1] - p.h_panel_off[kt];
     const int nu = p.h_update_off[kt + 1] - p.h_update_off[kt];
@@ -1512,12 +1519,19 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
   if ((s = dalloc(c, &c->dp, 3 * (size_t)n)) != STBA_OK) return bail(s);
   if ((s = dalloc(c, &c->partial, 6 * (size_t)RED_BLOCKS)) != STBA_OK) return bail(s);
   if ((s = dalloc(c, &c->cam_rt, 15 * (size_t)m)) != STBA_OK) return bail(s);
+  {
+    char* ct;
+    const size_t rs = c->mixed ? sizeof(float) : sizeof(double);
+    if ((s = dalloc(c, &ct, 40 * (size_t)m * rs)) != STBA_OK) return bail(s);
+    c->ctab = ct;
+    if ((s = dalloc(c, &ct, VPI * (size_t)m * rs)) != STBA_OK) return bail(s);
+    c->edc = ct;
+  }
   if ((s = dalloc(c, &c->cam_df, 28 * (size_t)m)) != STBA_OK) return bail(s);
   if ((s = dalloc(c, &c->pt_df, 6 * (size_t)n)) != STBA_OK) return bail(s);
   if (c->mixed) {
     if ((s = dalloc(c, &c->cams_f, 9 * (size_t)m)) != STBA_OK) return bail(s);
     if ((s = dalloc(c, &c->pts_f, 3 * (size_t)n)) != STBA_OK) return bail(s);
-    if ((s = dalloc(c, &c->dcf, 9 * (size_t)m)) != STBA_OK) return bail(s);
   }
   {
     char *r1, *r2;
@@ -1573,14 +1587,17 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
     for (int64_t o = 0; o < q; ++o) base_cam[o] = c->in_cam[c->base_order[o]];
     build_camera_graph((int)m, (int)n, c->h_pt_off, base_cam, c->cgraph, true);
     const CameraGraph& g = c->cgraph;
-    if ((int64_t)g.pairs.size() > INT32_MAX - PAIR_CHUNK)
+    if ((int64_t)g.pairs.size() > INT32_MAX - 64)
       return bail(fail(c, STBA_ERR_INVALID_ARG, "more than 2^31 co-visible observation pairs"));
     if (!c->use_pcg && !g.pairs.empty()) {
       std::vector<int4> chunks;
+      const int max_pairs = pair_chunk((int64_t)g.pairs.size());
       for (int x = 0; x < (int)m; ++x)
         for (int e = g.edge_off[x]; e < g.edge_off[x + 1]; ++e)
-          for (int64_t p0 = g.pair_off[e]; p0 < g.pair_off[e + 1]; p0 += PAIR_CHUNK)
-            chunks.push_back(make_int4(x, g.edge_y[e], (int)p0, (int)std::min<int64_t>(PAIR_CHUNK, g.pair_off[e + 1] - p0)));
+          for (int64_t p0 = g.pair_off[e]; p0 < g.pair_off[e + 1]; p0 += max_pairs)
+            chunks.push_back(make_int4(x, g.edge_y[e], (int)p0,
+                                       (int)std::min<int64_t>(max_pairs, g.pair_off[e + 1] - p0) |
+                                           (g.pair_off[e + 1] - g.pair_off[e] <= max_pairs ? PAIR_WHOLE_EDGE : 0)));
       int4* d_chunks = nullptr;
       int2* d_pairs = nullptr;
       int *d_active, *d_flag, *d_excl, *d_tiles;
@@ -1626,18 +1643,9 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
       for (int64_t j = 0; j < m; ++j)
         for (int e = cam_off[j]; e < cam_off[j + 1]; ++e) ecam[e] = (int)j;
     }
-    // point and observation of every camera-list entry, copied into the slots with each clustering
+    // point of every camera-list entry, copied into the slots with each clustering
     std::vector<int> ept(Q);
-    std::vector<float2> euvf(c->mixed ? Q : 0);
-    std::vector<double2> euvd(c->mixed ? 0 : Q);
-    for (size_t e = 0; e < Q; ++e) {
-      const int bo = cam_base[e];
-      ept[e] = base_pt[bo];
-      if (c->mixed)
-        euvf[e] = make_float2(base_uvf[2 * (size_t)bo], base_uvf[2 * (size_t)bo + 1]);
-      else
-        euvd[e] = make_double2(base_uv[2 * (size_t)bo], base_uv[2 * (size_t)bo + 1]);
-    }
+    for (size_t e = 0; e < Q; ++e) ept[e] = base_pt[cam_base[e]];
     for (int64_t j = 0; j < m; ++j) {
       const int nw = (cam_off[j + 1] - cam_off[j] + 31) / 32;
       cam_warp_off[j + 1] = cam_warp_off[j] + nw;
@@ -1667,20 +1675,9 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
     if ((s = upload(c, &d_cam_base, cam_base)) != STBA_OK) return bail(s);
     if ((s = upload(c, &d_ecam, ecam)) != STBA_OK) return bail(s);
     int* d_ept = nullptr;
-    float2* d_euvf = nullptr;
-    double2* d_euvd = nullptr;
     int2* d_slot_pv = nullptr;
-    float2* d_slot_uvf = nullptr;
-    double2* d_slot_uvd = nullptr;
     if ((s = upload(c, &d_ept, ept)) != STBA_OK) return bail(s);
     if ((s = dalloc(c, &d_slot_pv, 32 * (size_t)nwarps)) != STBA_OK) return bail(s);
-    if (c->mixed) {
-      if ((s = upload(c, &d_euvf, euvf)) != STBA_OK) return bail(s);
-      if ((s = dalloc(c, &d_slot_uvf, 32 * (size_t)nwarps)) != STBA_OK) return bail(s);
-    } else {
-      if ((s = upload(c, &d_euvd, euvd)) != STBA_OK) return bail(s);
-      if ((s = dalloc(c, &d_slot_uvd, 32 * (size_t)nwarps)) != STBA_OK) return bail(s);
-    }
     if ((s = dalloc(c, &d_eo, Q)) != STBA_OK) return bail(s);
     if ((s = dalloc(c, &d_nsing, Q)) != STBA_OK) return bail(s);
     if ((s = upload(c, &d_cam_warp_off, cam_warp_off)) != STBA_OK) return bail(s);
@@ -1722,21 +1719,35 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
     const size_t rs = c->mixed ? sizeof(float) : sizeof(double);
     char *vpa, *vpi, *pti, *pta, *vg, *ta, *gb;
     if ((s = dalloc(c, &vpa, 9 * Q * rs + 16)) != STBA_OK) return bail(s);   // zeroed in 16-byte pieces
-    if ((s = dalloc(c, &vpi, 9 * Q * rs)) != STBA_OK) return bail(s);
+    if ((s = dalloc(c, &vpi, VPI * Q * rs)) != STBA_OK) return bail(s);
     if ((s = dalloc(c, &pti, 9 * (size_t)n * rs)) != STBA_OK) return bail(s);
     if ((s = dalloc(c, &pta, 9 * (size_t)n * rs)) != STBA_OK) return bail(s);
     if ((s = dalloc(c, &vg, 9 * (size_t)m * rs)) != STBA_OK) return bail(s);
     if ((s = dalloc(c, &ta, 3 * (size_t)n * rs)) != STBA_OK) return bail(s);
-    // the stored G_o of the camera pass, only when the pair pass reads them (option pair_blocks)
-    const bool stored_g = !c->use_pcg && c->opt.pair_blocks == STBA_PAIR_BLOCKS_STORED;
-    if ((s = dalloc(c, &gb, (stored_g ? 36 * Q : 1) * rs)) != STBA_OK) return bail(s);
+    // the stored rows of the camera pass for the pair pass.  Default: recomputed in FP32 (cheaper than the reads,
+    // k_pair_build), stored in FP64, whose arithmetic runs at 1/64 of the FP32 rate -- unless they would take more
+    // than a quarter of the free device memory, where FP64 recomputes them too.
+    bool stored = c->opt.pair_blocks == STBA_PAIR_BLOCKS_STORED;
+    if (c->opt.pair_blocks == STBA_PAIR_BLOCKS_DEFAULT && !c->mixed) {
+      size_t free_b = 0, total_b = 0;
+      if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+        cudaGetLastError();
+        free_b = 0;
+      }
+      stored = 24 * Q * rs <= free_b / 4;
+    }
+    stored = stored && !c->use_pcg && !c->use_spcg;   // the PCG solvers form no off-diagonal blocks
+    c->pair_recompute = !stored;
+    if ((s = dalloc(c, &gb, (stored ? 24 * Q : 1) * rs)) != STBA_OK) return bail(s);
     c->vp_acc = vpa;
     c->vp_info = vpi;
     c->pt_info = pti;
     c->pt_acc = pta;
     c->vgrad = vg;
     c->t_acc = ta;
-    c->Gbuf = gb;
+    c->rowbuf = gb;
+    A.base_vp = nullptr;   // read by a pair pass that recomputes its rows
+    if (c->pair_recompute && !c->use_pcg && !c->use_spcg && (s = dalloc(c, &A.base_vp, Q)) != STBA_OK) return bail(s);
     A.obs_pt = c->obs_pt;
     A.pt_off = c->pt_off;
     A.base_cam = d_base_cam;
@@ -1757,11 +1768,7 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
     A.cam_base = d_cam_base;
     A.ecam = d_ecam;
     A.ept = d_ept;
-    A.euvf = d_euvf;
-    A.euvd = d_euvd;
     A.slot_pv = d_slot_pv;
-    A.slot_uvf = d_slot_uvf;
-    A.slot_uvd = d_slot_uvd;
     A.eo = d_eo;
     A.nsing = d_nsing;
     A.cam_warp_off = d_cam_warp_off;
@@ -1774,7 +1781,7 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
     c->pchunks.nactive = c->counts + 3;
     c->pcg.counts = c->counts;
     c->clist = CamLists{d_cam_off, d_cam_obs};
-    c->cslots = CamSlots{d_slots, d_warp_cam, nwarps, d_slot_pv, d_slot_uvf, d_slot_uvd};
+    c->cslots = CamSlots{d_slots, d_warp_cam, nwarps, d_slot_pv};
   }
   if ((s = set_clusters_host(c, h_cl)) != STBA_OK) return bail(s);
   double F;

@@ -1323,7 +1323,7 @@ __global__ void k_copy_vec(const Rreal* src, double* dst, int64_t n) {
 }
 
 // sharded: another process's clusters scatter zeros (their steps arrive by the exchange of dc)
-__global__ void k_scatter_dc(DevProblem P, const double* x, double* dc, float* dcf) {
+__global__ void k_scatter_dc(DevProblem P, const double* x, double* dc) {
   const int k = blockIdx.x;
   const int nk = P.cluster_n[k], cbase = P.cluster_cam_off[k];
   const bool own = !P.sharded || P.cluster_owned[k];
@@ -1332,7 +1332,6 @@ __global__ void k_scatter_dc(DevProblem P, const double* x, double* dc, float* d
     const int cam = P.cluster_cams[cbase + i / 9];
     const double v = own ? xk[i] : 0.0;
     dc[9 * (size_t)cam + i % 9] = v;
-    if (dcf) dcf[9 * (size_t)cam + i % 9] = (float)v;
   }
 }
 
@@ -1478,7 +1477,7 @@ void launch_factor_t(const DevProblem& P, const double* S, const FactorBuffers& 
 
 template <typename F, int T>
 void launch_solve_t(const DevProblem& P, const double* S, const double* b, const FactorBuffers& fb,
-                    const CholPlan& plan, int refine_steps, double* dc, float* dcf, cudaStream_t stream) {
+                    const CholPlan& plan, int refine_steps, double* dc, cudaStream_t stream) {
   using Sreal = double;
   const F* L = reinterpret_cast<const F*>(fb.L);
   const F* Dinv = reinterpret_cast<const F*>(fb.Dinv);
@@ -1491,7 +1490,7 @@ void launch_solve_t(const DevProblem& P, const double* S, const double* b, const
     launch_tri_solve<F, T, double>(P, L, Dinv, fb.scale, fb.r, fb.x, 1, plan.max_np, fb.v_total, plan.solve_cs,
                                    stream);
   }
-  k_scatter_dc<<<P.l, 256, 0, stream>>>(P, fb.x, dc, dcf);
+  k_scatter_dc<<<P.l, 256, 0, stream>>>(P, fb.x, dc);
 }
 
 // the tile size of the plan: FP32 factors 32 or 64 (chosen by stba_autotune), FP64 factors 32
@@ -1506,11 +1505,11 @@ void launch_factor(const DevProblem& P, const double* S, const FactorBuffers& fb
 
 template <typename F>
 void launch_solve(const DevProblem& P, const double* S, const double* b, const FactorBuffers& fb,
-                  const CholPlan& plan, int refine_steps, double* dc, float* dcf, cudaStream_t stream) {
+                  const CholPlan& plan, int refine_steps, double* dc, cudaStream_t stream) {
   if (sizeof(F) == 4 && plan.tile == 64)
-    launch_solve_t<F, 64>(P, S, b, fb, plan, refine_steps, dc, dcf, stream);
+    launch_solve_t<F, 64>(P, S, b, fb, plan, refine_steps, dc, stream);
   else
-    launch_solve_t<F, 32>(P, S, b, fb, plan, refine_steps, dc, dcf, stream);
+    launch_solve_t<F, 32>(P, S, b, fb, plan, refine_steps, dc, stream);
 }
 
 size_t solve_smem_bytes(bool mixed, int tile, int max_np) {   // with the smallest stage count
@@ -1586,8 +1585,8 @@ template void launch_factor<float>(const DevProblem&, const double*, const Facto
 template void launch_factor<double>(const DevProblem&, const double*, const FactorBuffers&, const CholPlan&,
                                     cudaStream_t);
 template void launch_solve<float>(const DevProblem&, const double*, const double*, const FactorBuffers&,
-                                  const CholPlan&, int, double*, float*, cudaStream_t);
+                                  const CholPlan&, int, double*, cudaStream_t);
 template void launch_solve<double>(const DevProblem&, const double*, const double*, const FactorBuffers&,
-                                   const CholPlan&, int, double*, float*, cudaStream_t);
+                                   const CholPlan&, int, double*, cudaStream_t);
 
 }  // namespace stba

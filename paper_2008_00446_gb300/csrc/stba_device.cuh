@@ -83,20 +83,21 @@ __device__ __forceinline__ void warp_load_rec9(const real* __restrict__ g, long 
   __syncwarp();
 }
 
-template <typename real>
-__device__ __forceinline__ void warp_store_rec9(real* __restrict__ g, long long r0, int cnt, real* sm, int lane,
-                                                const real (&x)[9]) {
+// the same for stores of records of NR reals (sm: 32 NR reals)
+template <int NR, typename real>
+__device__ __forceinline__ void warp_store_rec(real* __restrict__ g, long long r0, int cnt, real* sm, int lane,
+                                               const real (&x)[NR]) {
   if (lane < cnt) {
 #pragma unroll
-    for (int c = 0; c < 9; ++c) sm[9 * lane + c] = x[c];
+    for (int c = 0; c < NR; ++c) sm[NR * lane + c] = x[c];
   }
   __syncwarp();
-  real* blk = g + 9 * r0;
+  real* blk = g + NR * r0;
   if (cnt == 32 && ((reinterpret_cast<size_t>(blk) & 15) == 0)) {
-    constexpr int NQ = 9 * 32 * (int)sizeof(real) / 16;
+    constexpr int NQ = NR * 32 * (int)sizeof(real) / 16;
     for (int k = lane; k < NQ; k += 32) reinterpret_cast<float4*>(blk)[k] = reinterpret_cast<const float4*>(sm)[k];
   } else {
-    for (int k = lane; k < 9 * cnt; k += 32) blk[k] = sm[k];
+    for (int k = lane; k < NR * cnt; k += 32) blk[k] = sm[k];
   }
   __syncwarp();
 }

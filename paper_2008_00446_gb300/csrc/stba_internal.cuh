@@ -45,8 +45,11 @@ struct DevProblem {
   double huber_a;              // Huber scale a (0: plain least squares)
   const float* res_f;          // [q][2] residuals f_o at the current x, computed in FP64, stored in the
   const double* res_d;         //        working precision (res_f in mixed mode, res_d in FP64 mode)
+  const float* ctab_f;         // [m][40] per-camera tables of this linearisation (stba_camtab.cuh), in the working
+  const double* ctab_d;        //         precision (ctab_f in mixed mode, ctab_d in FP64 mode)
+  const int* base_vp;          // [q] virtual point of every base-order observation (null unless the pair pass reads it)
   const int* base_pos;         // [q] sorted position of every base-order observation (current assignment)
-  int pair_recompute;          // 1: the pair pass recomputes G_o instead of reading the camera pass's copy
+  int pair_recompute;          // 1: the pair pass recomputes its rows instead of reading the camera pass's copy
   int sharded;                 // 1: this process owns only some clusters (stba_set_shard)
   const int* cluster_owned;    // [l] 1 where this process builds, factors and solves cluster k (all 1 unless
                                //     sharded)
@@ -66,6 +69,7 @@ struct DevState {
   int failed;            // clusters whose factorisation failed this iteration
   int corrected;         // correction active this iteration
   int nonfinite;         // a non-positive depth was met in the cost at x + dx
+  unsigned pair_next;    // next chunk of the pair pass (zeroed by k_iter_begin)
   int boosted;           // FP32 pivots raised by static pivoting this iteration
   stba_iter_info info;   // record of the last finished iteration
 };
@@ -79,11 +83,14 @@ struct Settings {
 };
 
 constexpr int NSTAGES = 5;
+constexpr int VPI = 12;   // reals per virtual-point record (and per camera of E dc)
+constexpr int VPI_X = 6, VPI_Y = 9;
 
 // Kernel launchers (explicitly instantiated for float and double in stba_kernels.cu / stba_chol.cu).
 template <typename real> struct Scratch {
   real* vp_acc;    // [nv][9]: V = sum Jp^T Jp (6, packed xx xy xz yy yz zz) and w' = -sum Jp^T f (3)
-  real* vp_info;   // [nv][9]: L^-1 of V' (6, packed l00 l10 l11 l20 l21 l22) and y = V'^-1 w' (3)
+  real* vp_info;   // [nv][VPI]: L^-1 of V' (6, packed l00 l10 l11 l20 l21 l22), the point (3; written only for the
+                   // cluster and split solvers' passes) and y = V'^-1 w' (3): three 16-byte loads in FP32
   real* pt_info;   // [n][9]: C^-1 (6, packed symmetric) and w (3) of the physical points
   real* pt_acc;    // [n][9]: C (6, packed) and w (3) of the physical points, summed over their virtual points
   double* S;       // cluster-diagonal S' (dense lower triangles, per-cluster padded blocks); FP64 sums
@@ -91,7 +98,7 @@ template <typename real> struct Scratch {
   real* vgrad;     // [m][9] camera gradient v = -J_c^T f
   real* t_acc;     // [n][3] sum_o J_p^T J_c dc per point
   double* dc;      // [m][9] camera step
-  float* dcf;      // [m][9] FP32 copy of the camera step (mixed precision)
+  real* edc;       // [m][VPI] E dc per camera in the working precision (stba_camtab.cuh), for the point step
   double* dp;      // [n][3] point step
   double* partial; // reduction partials
 };
@@ -105,16 +112,15 @@ struct CamSlots {     // per-camera observation lists padded to whole warps, for
   const int* slots;         // [32 * nwarps] sorted observation position, or -1 (padding)
   const int* warp_cam;      // [nwarps] camera of each warp's 32 slots
   int nwarps;
-  // per slot, written with the lists (stba_order.cu), so that the camera pass reads them in its own order
-  // instead of gathering them by observation position: (point, virtual point | bit 31 when the virtual
-  // point has no other observation) and the observation in the working precision
+  // per slot, written with the lists (stba_order.cu), so that the camera passes read it in their own order
+  // instead of gathering it by observation position: (point, virtual point | bit 31 when the virtual
+  // point has no other observation)
   const int2* pv;           // [32 * nwarps]
-  const float2* uvf;        // [32 * nwarps] FP32 (mixed precision) or null
-  const double2* uvd;       // [32 * nwarps] FP64 or null
 };
 
 struct PairChunks {   // observation pairs of the camera graph, by edge, cut into chunks (built at create)
-  const int4* chunks;       // (camera x, camera y < x, first pair, number of pairs <= PAIR_CHUNK)
+  const int4* chunks;       // (camera x, camera y < x, first pair, number of pairs | PAIR_WHOLE_EDGE when the chunk
+                            // holds every pair of its edge)
   const int2* pairs;        // (base position of the observation by x, base position of the one by y)
   int nchunks;
   const int* active;        // [nchunks] the chunks whose two cameras share a cluster (set per assignment)
@@ -126,7 +132,15 @@ struct PairChunks {   // observation pairs of the camera graph, by edge, cut int
 // lists the chunks inside clusters for the current assignment (cam_cluster on the device)
 void launch_list_chunks(const PairChunks& B, const int* cam_cluster, const int* owned, long long* nactive,
                         cudaStream_t stream);
-constexpr int PAIR_CHUNK = 64;
+// Pairs per chunk: as many as leave eight chunks of the camera graph's pairs per resident warp of the pair pass
+// (24 warps on 152 SMs; chunks are handed out by a counter), between 64 and 128.  S' build stage with 64 / 128 /
+// 256 at most: 1000 cameras, 2.9M pairs inside clusters 183 / 177 / 185 us; 2000 sequential cameras, 10.5M pairs
+// 510 / 483 / 479; 6000 cameras, 12M pairs 868 / 774 / 774; 400 cameras in FP64, 0.5M pairs 574 / 625 / 605.
+constexpr int PAIR_CHUNK_MIN = 64, PAIR_CHUNK_MAX = 128;
+inline int pair_chunk(int64_t pairs) {
+  return (int)std::min<int64_t>(PAIR_CHUNK_MAX, std::max<int64_t>(PAIR_CHUNK_MIN, pairs / (8 * 24 * 152) / 16 * 16));
+}
+constexpr int PAIR_WHOLE_EDGE = 1 << 30, PAIR_COUNT_MASK = PAIR_WHOLE_EDGE - 1;
 
 // Camera graph (stba_graph.cu): edges (x, y), y < x, grouped by x with y ascending; weight = number of
 // common points; the observation pairs of each edge (base positions, observations sorted by (point,
@@ -168,15 +182,12 @@ struct ReorderArgs {
   float* obs_uvf;
   float4* obs_uvdf;
   int *obs_vp, *vp_off, *vp_point, *pt_vp_off;
+  int* base_vp;             // [q] virtual point of every base position, for the pair pass, or null
   const int* cam_off;       // [m+1] observations of every camera
   const int* cam_base;      // [q]   their base positions, ascending
   const int* ecam;          // [q]   the camera of every entry of cam_base
   const int* ept;           // [q]   the point of every entry of cam_base
-  const float2* euvf;       // [q]   its observation in FP32 (mixed precision) or null
-  const double2* euvd;      // [q]   its observation in FP64 (FP64 mode) or null
-  int2* slot_pv;            // CamSlots::pv, uvf, uvd (written by k_cam_place)
-  float2* slot_uvf;
-  double2* slot_uvd;
+  int2* slot_pv;            // CamSlots::pv (written by k_cam_place)
   int* eo;                  // [q]   the new position of every entry of cam_base (scratch of the assignment)
   int* nsing;               // [q]   per base position: its new position, bit 31 set when its virtual point
                             //       has no other observation (scratch of the assignment)
@@ -207,18 +218,20 @@ void launch_vp_finalize(const DevProblem& P, Scratch<real> W, DevState* st, cons
 // [n][9] (the other processes' virtual points are zero here); summed over the processes they are C_i, w_i.
 template <typename real>
 void launch_pt_sums(const DevProblem& P, Scratch<real> W, double* out, cudaStream_t stream);
-// dcf = (float) dc, n values
-void launch_dc_to_float(const double* dc, float* dcf, int64_t n, cudaStream_t stream);
+// E dc of every camera from dc and the camera tables
+template <typename real>
+void launch_step_rows(const DevProblem& P, const double* dc, real* edc, cudaStream_t stream);
 // to_double = 1: *x = st->failed; 0: st->failed = (int) *x
 void launch_failed_io(DevState* st, double* x, int to_double, cudaStream_t stream);
 template <typename real>
-void launch_rcs_build(const DevProblem& P, Scratch<real> W, CamSlots CS, PairChunks B, real* Gbuf, DevState* st,
+void launch_rcs_build(const DevProblem& P, Scratch<real> W, CamSlots CS, PairChunks B, real* rowbuf, DevState* st,
                       cudaStream_t stream, cudaStream_t side = nullptr, cudaEvent_t fork = nullptr,
                       cudaEvent_t join = nullptr);
 template <typename real>
 void launch_point_rhs(const DevProblem& P, Scratch<real> W, cudaStream_t stream);
-// FP32 copies of the cameras and points (mixed precision, once per iteration)
-void launch_params_to_float(const DevProblem& P, float* cams_f, float* pts_f, cudaStream_t stream);
+// camera tables, and FP32 copies of the cameras and points (mixed precision; else null): once per linearisation
+template <typename real>
+void launch_params(const DevProblem& P, real* ctab, float* cams_f, float* pts_f, cudaStream_t stream);
 template <typename real>
 void launch_point_update(const DevProblem& P, Scratch<real> W, cudaStream_t stream);
 // k_cam_rt + k_cost: rt is a [m][15] FP64 scratch (R, t, f, k1, k2 of x + dx); residuals go to rout.  In mixed
@@ -289,10 +302,10 @@ int factor_tile(bool mixed);
 template <typename F>
 void launch_factor(const DevProblem& P, const double* S, const FactorBuffers& fb, const CholPlan& plan,
                    cudaStream_t stream);
-// x = S'^-1 b per cluster, scattered to dc [m][9] (and to its FP32 copy dcf when not null)
+// x = S'^-1 b per cluster, scattered to dc [m][9]
 template <typename F>
 void launch_solve(const DevProblem& P, const double* S, const double* b, const FactorBuffers& fb,
-                  const CholPlan& plan, int refine_steps, double* dc, float* dcf, cudaStream_t stream);
+                  const CholPlan& plan, int refine_steps, double* dc, cudaStream_t stream);
 void launch_count_failures(const int* fail_flags, int l, DevState* st, cudaStream_t stream);
 
 // Adjoint of one accepted step (stba_adjoint.cu).  With the forward step at x_t recomputed in W and fb

@@ -23,6 +23,7 @@
 #include <climits>
 
 #include "stba_camera.cuh"
+#include "stba_camtab.cuh"
 #include "stba_device.cuh"
 #include "stba_strict.cuh"
 #include "stba_internal.cuh"
@@ -39,6 +40,7 @@ __global__ void k_iter_begin(DevState* st, Settings s) {
     st->failed = 0;
     st->nonfinite = 0;
     st->boosted = 0;
+    st->pair_next = 0;
   }
 }
 
@@ -63,17 +65,11 @@ __global__ void __launch_bounds__(256) k_vp_reduce(DevProblem P, real* vp_acc) {
     v = P.obs_vp[o];
     const int cam = P.obs_cam[o];
     const int pt = P.vp_point[v];
-    Cam<real> C = load_cam_w<real>(P, cam);
+    const CamRow<real> C = gather_camrow<real>(P, cam);
     real X[3];
     load_point_w(P, pt, X);
-    real uo, vo;
-    load_uv(P, o, uo, vo);
-    real r[2], Jc[2][9], Jp[2][3];
-    // FP32: the strict rows, bitwise those of the camera and pair passes
-    if constexpr (sizeof(real) == 4)
-      project_jacobian_strict<false>(C, X, uo, vo, Jc, Jp);
-    else
-      project_jacobian<real, false>(C, X, uo, vo, r, Jc, Jp);
+    real r[2], Jt[2][9], Jp[2][3];
+    proj_rows<real, false>(C, X, Jt, Jp);
     r[0] = res_ptr<real>(P)[2 * (size_t)o];
     r[1] = res_ptr<real>(P)[2 * (size_t)o + 1];
     real sw;   // 1 without a robust loss
@@ -157,7 +153,7 @@ __global__ void __launch_bounds__(256) k_pt_acc(DevProblem P, const real* __rest
         for (int c = 0; c < 9; ++c) acc[c] += sm[9 * (u - r) + c];
       __syncwarp();
     }
-    warp_store_rec9(pt_acc, i0, cnt, sm, lane, acc);
+    warp_store_rec(pt_acc, i0, cnt, sm, lane, acc);
   }
 }
 
@@ -171,7 +167,7 @@ template <typename real>
 __global__ void __launch_bounds__(256) k_vp_finalize(DevProblem P, Scratch<real> W, DevState* st,
                                                      const double* __restrict__ pt_sums,
                                                      const long long* __restrict__ counts) {
-  __shared__ __align__(16) real stage[8][288];
+  __shared__ __align__(16) real stage[8][32 * VPI];
   const real lam = (real)st->lambda_used;
   const bool corr = st->corrected != 0;
   const long long nv = counts[0];
@@ -202,6 +198,8 @@ __global__ void __launch_bounds__(256) k_vp_finalize(DevProblem P, Scratch<real>
       const int cnt = (int)(nv - v0 < 32 ? nv - v0 : 32);
       warp_load_rec9(W.vp_acc, v0, cnt, sm, lane, a);
       const bool other = pt_sums && a[0] == real(0) && a[3] == real(0) && a[5] == real(0);   // another process's
+      real X[3] = {0, 0, 0};
+      if (lane < cnt) load_point_w(P, P.vp_point[v], X);
       if (lane < cnt && !other) {
         real V[6] = {a[0], a[1], a[2], a[3], a[4], a[5]}, wv[3] = {a[6], a[7], a[8]};
         if (corr) {
@@ -222,7 +220,8 @@ __global__ void __launch_bounds__(256) k_vp_finalize(DevProblem P, Scratch<real>
 #pragma unroll
         for (int c = 0; c < 3; ++c) o[6 + c] = y[c];
       }
-      warp_store_rec9(W.vp_info, v0, cnt, sm, lane, o);
+      const real rec[VPI] = {o[0], o[1], o[2], o[3], o[4], o[5], X[0], X[1], X[2], o[6], o[7], o[8]};
+      warp_store_rec(W.vp_info, v0, cnt, sm, lane, rec);
     } else {
       // physical point: C + lambda diag(C), its inverse, uncorrected w
       const long long i0 = (ch - nvc) * 32;
@@ -253,7 +252,7 @@ __global__ void __launch_bounds__(256) k_vp_finalize(DevProblem P, Scratch<real>
         o[8] = a[8];
         gmax = fmax(gmax, fmax(fabs((double)a[6]), fmax(fabs((double)a[7]), fabs((double)a[8]))));
       }
-      warp_store_rec9(W.pt_info, i0, cnt, sm, lane, o);
+      warp_store_rec(W.pt_info, i0, cnt, sm, lane, o);
     }
   }
   double bm = block_max<real>(gmax);
@@ -290,13 +289,19 @@ void launch_pt_sums(const DevProblem& P, Scratch<real> W, double* out, cudaStrea
   k_pt_sums<real><<<std::min((P.n + 255) / 256, 4096), 256, 0, stream>>>(P, W.vp_acc, out);
 }
 
-__global__ void k_dc_to_float(const double* __restrict__ dc, float* __restrict__ dcf, int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    dcf[i] = (float)dc[i];
+template <typename real>
+__global__ void k_step_rows(int m, const real* __restrict__ ctab, const double* __restrict__ dc, real* __restrict__ edc) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 9 * (int64_t)m; i += (int64_t)gridDim.x * blockDim.x) {
+    const int j = (int)(i / 9), c = (int)(i - 9 * (int64_t)j);
+    edc[(size_t)VPI * j + c] = step_entry(jl_ptr(ctab, m, j), dc + 9 * (size_t)j, c);
+  }
 }
 
-void launch_dc_to_float(const double* dc, float* dcf, int64_t n, cudaStream_t stream) {
-  k_dc_to_float<<<(int)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, stream>>>(dc, dcf, n);
+template <typename real>
+void launch_step_rows(const DevProblem& P, const double* dc, real* edc, cudaStream_t stream) {
+  const real* ctab;
+  if constexpr (sizeof(real) == 4) ctab = P.ctab_f; else ctab = P.ctab_d;
+  k_step_rows<real><<<(int)std::min<int64_t>((9 * (int64_t)P.m + 255) / 256, 4096), 256, 0, stream>>>(P.m, ctab, dc, edc);
 }
 
 __global__ void k_failed_io(DevState* st, double* x, int to_double) {
@@ -314,13 +319,14 @@ void launch_failed_io(DevState* st, double* x, int to_double, cudaStream_t strea
 
 // ------------------------------------------------------------------------------------------------------
 // S' build (Eq. 10/13), in two passes.  With V' = L L^T the Cholesky factor of a virtual point's damped
-// block and G_o = L^-1 Jp,o^T Jc,o (3x9) for each of its observations, E' C'^-1 E'^T = G^T G, so
-//   off-diagonal camera blocks   S(a, b) = - sum_v G_a^T G_b                       (k_pair_build)
-//   diagonal camera block        S(a, a) = sum_o [Jc^T Jc + lambda diag(Jc^T Jc) - G_o^T G_o]  (k_cam_pass)
+// block and, for each of its observations, Pm_o = L^-1 Jp,o^T (3x2), the Schur term of two observations is
+// E' C'^-1 E'^T = Jc,a^T (Pm_a^T Pm_b) Jc,b with a 2x2 middle, so
+//   off-diagonal camera blocks   S(a, b) = - sum_v Jc,a^T (Pm_a^T Pm_b) Jc,b          (k_pair_build)
+//   diagonal camera block        S(a, a) = sum_o [Jc^T (I - Pm_o^T Pm_o) Jc + lambda diag(Jc^T Jc)]  (k_cam_pass)
 //   right-hand side              b(a)    = - sum_o Jc^T (f_o + Jp,o y_v),  y_v = V'^-1 w'_v
 //   camera gradient              v(a)    = - sum_o Jc^T f_o
-// For a virtual point with one observation, Jc^T Jc - G^T G = Jc^T (I - Jp V'^-1 Jp^T) Jc cancels by a
-// factor ~ lambda; it is evaluated in the equivalent Woodbury form Jc^T (I + Jp Lambda^-1 Jp^T)^-1 Jc with
+// For a virtual point with one observation, I - Pm^T Pm = I - Jp V'^-1 Jp^T cancels by a
+// factor ~ lambda; it is evaluated in the equivalent Woodbury form (I + Jp Lambda^-1 Jp^T)^-1 with
 // Lambda = lambda diag(Jp^T Jp), and without correction b(a) gets -Jc^T (I + Jp Lambda^-1 Jp^T)^-1 f_o.
 //
 // k_cam_pass: one warp per 32 observations of one camera (each camera's observation list is padded to
@@ -329,46 +335,12 @@ void launch_failed_io(DevState* st, double* x, int to_double, cudaStream_t strea
 // with a transposed reduction (62 shuffles leave lane L with the sums of terms L and 32 + L; a tree sum of
 // 32 terms, error <= 5 ulp of the sum of magnitudes) and adds them atomically into the FP64 S', b' and v
 // (zeroed before the launch): FP32 terms, FP64 accumulation across warps.  The per-observation arithmetic
-// stays off the FP64 pipe, which on this GPU runs at 1/64 of the FP32 rate.  It also stores G_o of every
-// observation of a multi-observation virtual point for the pair pass, unless the pair pass recomputes G_o.
-// In FP32 both passes evaluate the Jacobian rows with every operation rounded on its own (stba_strict.cuh):
-// the diagonal and off-diagonal blocks of a virtual point then come from bitwise the same J_c, J_p and G_o
-// whether G_o is stored or recomputed, and the FP32 S' does not change with the compiler's choice of
-// fused multiply-adds in the surrounding code.
-// G_o is stored column by column, four reals per camera-parameter column c (G[0][c], G[1][c], G[2][c], 0),
-// so that the pair pass reads a column with one 16-byte (FP32) load.
-constexpr int GSTRIDE = 36;   // reals per stored G_o
-
-// one stored G column from 16-byte aligned shared memory
-template <typename real>
-__device__ __forceinline__ void load_gcol_s(const real* p, real (&v)[3]) {
-  if constexpr (sizeof(real) == 4) {
-    const float4 t = *reinterpret_cast<const float4*>(p);
-    v[0] = t.x;
-    v[1] = t.y;
-    v[2] = t.z;
-  } else {
-    const double2 t = *reinterpret_cast<const double2*>(p);
-    v[0] = t.x;
-    v[1] = t.y;
-    v[2] = p[2];
-  }
-}
-
-template <typename real>
-__device__ __forceinline__ void load_gcol(const real* p, real (&v)[3]) {
-  if constexpr (sizeof(real) == 4) {
-    const float4 t = __ldg(reinterpret_cast<const float4*>(p));
-    v[0] = t.x;
-    v[1] = t.y;
-    v[2] = t.z;
-  } else {
-    const double2 t = __ldg(reinterpret_cast<const double2*>(p));
-    v[0] = t.x;
-    v[1] = t.y;
-    v[2] = __ldg(p + 2);
-  }
-}
+// stays off the FP64 pipe, which on this GPU runs at 1/64 of the FP32 rate.  With stored pair rows it also
+// stores (Pm_o, the tilde rows of Jc,o) of every observation of a multi-observation virtual point.
+// Both passes evaluate the same rows (stba_camtab.cuh; in FP32 with every operation rounded on its own): the
+// diagonal and off-diagonal blocks of a virtual point come from bitwise the same J_c and J_p whether they are
+// stored or recomputed, and the FP32 S' does not change with the compiler's choice of fused multiply-adds.
+constexpr int ROWREC = 24;   // reals per stored observation: Pm (6), tilde rows of J_c (18)
 
 // On return lane L holds the sum over the warp's lanes of v[L].  Each halving step keeps one half of the
 // values (lanes whose bit s is set keep the upper half) and adds the partner's copy of it.
@@ -388,64 +360,27 @@ __device__ __forceinline__ real warp_transpose_sum32(real (&v)[32]) {
   return v[0];
 }
 
-// P = L^-1 Jp^T (3 x 2) and G = P Jc (3 x 9) of one observation, with every product and sum rounded by explicit
-// fma / mul intrinsics, so that the camera pass and the pair pass form bitwise the same G from the same inputs
-// (the S' of a virtual point then stays consistent between its diagonal and off-diagonal camera blocks).
+// Pm = L^-1 Jp^T (3 x 2) of one observation, with every product and sum rounded by explicit fma / mul intrinsics,
+// so that the camera pass and the pair pass form bitwise the same values from the same inputs (the S' of a
+// virtual point then stays consistent between its diagonal and off-diagonal camera blocks).
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 
 template <typename real>
-__device__ __forceinline__ void g_of_obs(const real* Li, const real (&Jc)[2][9], const real (&Jp)[2][3], real (&Pm)[3][2],
-                                         real (&G)[3][9]) {
+__device__ __forceinline__ void pm_of_obs(const real* Li, const real (&Jp)[2][3], real (&Pm)[3][2]) {
 #pragma unroll
   for (int t = 0; t < 2; ++t) {
     Pm[0][t] = mul_rn(Li[0], Jp[t][0]);
     Pm[1][t] = fma_rn(Li[2], Jp[t][1], mul_rn(Li[1], Jp[t][0]));
     Pm[2][t] = fma_rn(Li[5], Jp[t][2], fma_rn(Li[4], Jp[t][1], mul_rn(Li[3], Jp[t][0])));
   }
-#pragma unroll
-  for (int c = 0; c < 9; ++c)
-#pragma unroll
-    for (int s = 0; s < 3; ++s) G[s][c] = fma_rn(Pm[s][1], Jc[1][c], mul_rn(Pm[s][0], Jc[0][c]));
 }
 
-// J_c and J_p of the observation at sorted position o, seen by camera C, scaled by the Huber weight of the
-// stored residual f_o (returned, scaled, in r).  STRICT (FP32 only): every operation rounded on its own, so
-// that the camera pass and the pair pass form bitwise the same rows.
-template <typename real, bool STRICT>
-__device__ __forceinline__ void obs_jacobian_at(const DevProblem& P, const Cam<real>& C, int o, int pt, real uo,
-                                                real vo, real (&r)[2], real (&Jc)[2][9], real (&Jp)[2][3]) {
-  static_assert(!STRICT || sizeof(real) == 4, "the strict rounding mode is FP32 only");
-  real X[3];
-  load_point_w(P, pt, X);
-  if constexpr (STRICT)
-    project_jacobian_strict(C, X, uo, vo, Jc, Jp);
-  else
-    project_jacobian<real, true>(C, X, uo, vo, r, Jc, Jp);
-  r[0] = res_ptr<real>(P)[2 * (size_t)o];
-  r[1] = res_ptr<real>(P)[2 * (size_t)o + 1];
-  real sw;
-  if constexpr (STRICT)
-    sw = huber_sqrt_weight_strict(P.huber_a, r[0], r[1]);
-  else
-    sw = huber_sqrt_weight<real>(P.huber_a, r[0], r[1]);
-  scale_rows(sw, r, Jc, Jp);
-}
-
-template <typename real, bool STRICT>
-__device__ __forceinline__ void obs_jacobian(const DevProblem& P, const Cam<real>& C, int o, real (&r)[2],
-                                             real (&Jc)[2][9], real (&Jp)[2][3]) {
-  real uo, vo;
-  load_uv(P, o, uo, vo);
-  obs_jacobian_at<real, STRICT>(P, C, o, P.obs_pt[o], uo, vo, r, Jc, Jp);
-}
-
-// STRICT (the FP32 pass): the Jacobian rows with every operation rounded on its own, as in the pair pass.
-template <typename real, bool STRICT>
-__global__ void __launch_bounds__(256, sizeof(real) == 4 ? 4 : 3) k_cam_pass(DevProblem P, Scratch<real> W, CamSlots CS, real* Gbuf,
-                                                  const DevState* st) {
+template <typename real>
+__global__ void __launch_bounds__(256, sizeof(real) == 4 ? 4 : 3) k_cam_pass(DevProblem P, Scratch<real> W, CamSlots CS,
+                                                                             real* rowbuf, const DevState* st) {
   const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (gw >= CS.nwarps) return;   // uniform per warp
   const int lane = threadIdx.x & 31;
@@ -458,25 +393,19 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 4 : 3) k_cam_pass(Dev
 #pragma unroll
   for (int c = 0; c < 9; ++c) Jc[0][c] = Jc[1][c] = 0;
   if (o >= 0) {
-    const Cam<real> C = load_cam_w<real>(P, j);
-    // point, virtual point and observation of the slot, stored in slot order with the camera lists
-    const size_t sl = 32 * (size_t)gw + lane;
-    const int2 pv = CS.pv[sl];
-    const int v = pv.y & INT_MAX;
-    const bool single = pv.y < 0;
-    real uo, vo;
-    if constexpr (sizeof(real) == 4) {
-      const float2 t = CS.uvf[sl];
-      uo = t.x;
-      vo = t.y;
-    } else {
-      const double2 t = CS.uvd[sl];
-      uo = t.x;
-      vo = t.y;
-    }
-    real Jp[2][3];
-    obs_jacobian_at<real, STRICT>(P, C, o, pv.x, uo, vo, r, Jc, Jp);
-    const real* vi = W.vp_info + 9 * (size_t)v;
+    const CamRow<real> C = load_camrow<real>(P, j);
+    // virtual point of the slot (its record holds the point), stored in slot order with the camera lists
+    const int pvs = CS.pv[32 * (size_t)gw + lane].y;
+    const int v = pvs & INT_MAX;
+    const bool single = pvs < 0;
+    real vi[VPI], Jp[2][3], Jl[9];
+    load_vec16<VPI>(W.vp_info + (size_t)VPI * v, vi);
+    const real X[3] = {vi[VPI_X], vi[VPI_X + 1], vi[VPI_X + 2]};
+    load_jl(P, j, Jl);
+    proj_rows<real, true>(C, X, Jc, Jp);   // tilde rows
+    r[0] = res_ptr<real>(P)[2 * (size_t)o];
+    r[1] = res_ptr<real>(P)[2 * (size_t)o + 1];
+    scale_rows(row_weight(P, r[0], r[1]), r, Jc, Jp);
     // Both cases reduce to Jc^T N Jc with a 2x2 N:
     //   single observation  N = (I + Jp Lambda^-1 Jp^T)^-1                 (Woodbury, no cancellation)
     //   several             N = I - Jp V'^-1 Jp^T = I - P^T P, P = L^-1 Jp^T  (V' = L L^T)
@@ -496,34 +425,41 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 4 : 3) k_cam_pass(Dev
       N01 = -K01 * idet;
       N11 = (real(1) + K00) * idet;
       if (corr) {
-        br[0] = r[0] + Jp[0][0] * vi[6] + Jp[0][1] * vi[7] + Jp[0][2] * vi[8];
-        br[1] = r[1] + Jp[1][0] * vi[6] + Jp[1][1] * vi[7] + Jp[1][2] * vi[8];
+        br[0] = r[0] + Jp[0][0] * vi[VPI_Y] + Jp[0][1] * vi[VPI_Y + 1] + Jp[0][2] * vi[VPI_Y + 2];
+        br[1] = r[1] + Jp[1][0] * vi[VPI_Y] + Jp[1][1] * vi[VPI_Y + 1] + Jp[1][2] * vi[VPI_Y + 2];
       } else {
         br[0] = N00 * r[0] + N01 * r[1];
         br[1] = N01 * r[0] + N11 * r[1];
       }
     } else {
-      real Pm[3][2], Gm[3][9];   // P = L^-1 Jp^T (3x2), G = P Jc
-      g_of_obs<real>(vi, Jc, Jp, Pm, Gm);
+      real Pm[3][2];
+      pm_of_obs<real>(vi, Jp, Pm);
       N00 = real(1) - (Pm[0][0] * Pm[0][0] + Pm[1][0] * Pm[1][0] + Pm[2][0] * Pm[2][0]);
       N01 = -(Pm[0][0] * Pm[0][1] + Pm[1][0] * Pm[1][1] + Pm[2][0] * Pm[2][1]);
       N11 = real(1) - (Pm[0][1] * Pm[0][1] + Pm[1][1] * Pm[1][1] + Pm[2][1] * Pm[2][1]);
-      // G = L^-1 Jp^T Jc = P Jc (3x9), stored by columns with 16-byte vector stores (unless the pair pass
-      // recomputes it)
-      real* Gs = Gbuf + (size_t)GSTRIDE * P.obs_base[o];   // indexed like the camera graph's pairs
+      if (!P.pair_recompute) {   // the pair pass's rows, with 16-byte stores, indexed like the camera graph's pairs
+        real v24[ROWREC];
 #pragma unroll
-      for (int c = 0; c < 9 && !P.pair_recompute; ++c) {
-        const real g0 = Gm[0][c], g1 = Gm[1][c], g2 = Gm[2][c];
+        for (int t = 0; t < 6; ++t) v24[t] = Pm[t >> 1][t & 1];
+#pragma unroll
+        for (int c = 0; c < 9; ++c) {
+          v24[6 + 2 * c] = Jc[0][c];
+          v24[7 + 2 * c] = Jc[1][c];
+        }
+        real* dst = rowbuf + (size_t)ROWREC * P.obs_base[o];
         if constexpr (sizeof(real) == 4) {
-          reinterpret_cast<float4*>(Gs)[c] = make_float4(g0, g1, g2, 0.f);
+#pragma unroll
+          for (int k = 0; k < ROWREC / 4; ++k)
+            reinterpret_cast<float4*>(dst)[k] = make_float4(v24[4 * k], v24[4 * k + 1], v24[4 * k + 2], v24[4 * k + 3]);
         } else {
-          reinterpret_cast<double2*>(Gs)[2 * c] = make_double2(g0, g1);
-          reinterpret_cast<double2*>(Gs)[2 * c + 1] = make_double2(g2, 0.0);
+#pragma unroll
+          for (int k = 0; k < ROWREC / 2; ++k) reinterpret_cast<double2*>(dst)[k] = make_double2(v24[2 * k], v24[2 * k + 1]);
         }
       }
-      br[0] = r[0] + Jp[0][0] * vi[6] + Jp[0][1] * vi[7] + Jp[0][2] * vi[8];
-      br[1] = r[1] + Jp[1][0] * vi[6] + Jp[1][1] * vi[7] + Jp[1][2] * vi[8];
+      br[0] = r[0] + Jp[0][0] * vi[VPI_Y] + Jp[0][1] * vi[VPI_Y + 1] + Jp[0][2] * vi[VPI_Y + 2];
+      br[1] = r[1] + Jp[1][0] * vi[VPI_Y] + Jp[1][1] * vi[VPI_Y + 1] + Jp[1][2] * vi[VPI_Y + 2];
     }
+    apply_jl<real>(Jl, Jc);
   }
   // terms: 0..44 diagonal block (packed lower, row-major), 45..53 b', 54..62 v, 63 unused
   real NJ[2][9];
@@ -577,170 +513,276 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 4 : 3) k_cam_pass(Dev
 }
 
 // k_pair_build: the off-diagonal blocks S'_k(la, lb) = -sum over the points seen by both cameras x > y of
-// one cluster of G_x^T G_y (Eq. 10, 13).  The observation pairs of the camera graph are listed once, at
-// create, by edge (x, y) and cut into chunks of at most PAIR_CHUNK; under a cluster assignment an edge
+// one cluster of Jc,x^T (Pm_x^T Pm_y) Jc,y (Eq. 10, 13).  The observation pairs of the camera graph are listed
+// once, at create, by edge (x, y) and cut into chunks (pair_chunk); under a cluster assignment an edge
 // contributes exactly when both cameras are in one cluster (its two observations of a point are then in
 // one virtual point), and a chunk adds to one block only.  The re-ordering of an assignment lists the
-// chunks whose edge lies inside a cluster; a fixed grid of warps walks that list.  A warp's work is a
-// sequence of pieces of CH pairs (the chunks it takes, cut into pieces); the G rows of the next piece are
-// copied into shared memory (cp.async, one row per lane) while 27 lanes accumulate the current one: lane
-// (g, rb, cb) takes every third pair (slot g) and the 3 x 3 sub-block (rb, cb) of the 9 x 9 block, in
-// registers; the three slots are summed by two shuffles and the block is added once per chunk into the
-// FP64 S'_k.
+// chunks whose edge lies inside a cluster; the warps of a fixed grid take them one by one from that list.  A warp works on pieces of
+// PB_CH pairs: lane (side, j) forms the rows of its pair's observation by camera x (side 0) or y (side 1) from
+// the camera's table, the point and L_v^-1 (both lanes of a pair share them); the y lane takes Pm_x by shuffle
+// and forms M = Pm_x^T Pm_y (2x2) and M Jt_y (2x9).  The rows go to shared memory, and 27 lanes accumulate: lane
+// (g, rb, cb) takes every third pair (slot g) and the 3 x 3 sub-block (rb, cb), in FP32 as packed pairs of FMAs
+// over the rank index.  The three slots are summed by two shuffles, the block is multiplied by the cameras' Jl
+// (J_c = Jt E) and written once per chunk to the FP64 S'_k: stored when the chunk is its edge's only one (the
+// edge's block has no other writer), else added atomically.
+// Bound by the L1 / shared-memory pipe (ncu: 85 % of its wavefronts): per 16 pairs about 65 wavefronts of row reads,
+// 26 of row writes, 80 of the gathers of the 48-byte virtual-point records.  Hence rank-2 rows (3x9 blocks
+// G = L^-1 Jp^T Jc of both sides move half as many words again), 16-byte records and loads, 24 warps per SM
+// (80 registers; 32 warps spill: 150 us against 135 us for 2.9M pairs).  S' build stage, before -> now:
+// 1000 cameras, 2.9M pairs 316 -> 177 us; 2000 sequential cameras, 10.5M pairs 913 -> 483; 6000 cameras, 12M
+// pairs 1802 -> 774; FP64, 300 cameras, 0.5M pairs 2702 -> 574 (stored rows: bound by the FP64 pipe).
 constexpr int PB_WARPS = 8;
+constexpr int PB_CH = 16;   // pairs per piece: one per lane and side
+template <typename real> constexpr int pb_ctas() { return sizeof(real) == 4 ? 3 : 2; }   // resident CTAs per SM
 
-template <typename real> struct PairStage {
-  static constexpr int CH = 64 / (int)sizeof(real);                   // pairs per piece
-  static constexpr int PIECES = 2;                                      // double buffer
-  static constexpr size_t bytes = sizeof(real) * (size_t)PB_WARPS * PIECES * CH * 2 * GSTRIDE;
+// Shared-memory rows of a piece: per pair and side three groups (camera-parameter triples) of 3 columns x 2 ranks,
+// 16-byte aligned; the pair stride spreads the 16-byte stores of 8 consecutive lanes over all banks.
+template <typename real> struct PairRows {
+  static constexpr int GROUP = sizeof(real) == 4 ? 8 : 6, SIDE = 3 * GROUP, PAIR = sizeof(real) == 4 ? 52 : 50;
+  static constexpr size_t bytes = sizeof(real) * (size_t)PB_WARPS * PB_CH * PAIR;
 };
 
-__device__ __forceinline__ void cp_async_16(void* smem_dst, const void* gsrc) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gsrc) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
-
-// G_o = L_v^-1 Jp,o^T Jc,o (3 x 9) of the observation at sorted position pos by camera cam, written by columns
-// (G[0][c], G[1][c], G[2][c], 0) to dst: the camera pass's arithmetic (Jacobians at the current x, Huber
-// weights from the stored residual, L_v^-1 of the virtual point's damped block); STRICT as in the camera pass.
-template <typename real, bool STRICT>
-__device__ __forceinline__ void obs_G(const DevProblem& P, const Scratch<real>& W, int cam, int pos, real* dst) {
-  const Cam<real> C = load_cam_w<real>(P, cam);
-  real r[2], Jc[2][9], Jp[2][3];
-  obs_jacobian<real, STRICT>(P, C, pos, r, Jc, Jp);
-  real Pm[3][2], Gm[3][9];
-  g_of_obs<real>(W.vp_info + 9 * (size_t)P.obs_vp[pos], Jc, Jp, Pm, Gm);
+// 3 columns x 2 ranks of one group
+template <typename real>
+__device__ __forceinline__ void store_group(real* dst, const real (&v)[6]) {
+  if constexpr (sizeof(real) == 4) {
+    *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+    *reinterpret_cast<float2*>(dst + 4) = make_float2(v[4], v[5]);
+  } else {
 #pragma unroll
-  for (int c = 0; c < 9; ++c) {
-    const real g0 = Gm[0][c], g1 = Gm[1][c], g2 = Gm[2][c];
-    if constexpr (sizeof(real) == 4) {
-      reinterpret_cast<float4*>(dst)[c] = make_float4(g0, g1, g2, 0.f);
-    } else {
-      reinterpret_cast<double2*>(dst)[2 * c] = make_double2(g0, g1);
-      reinterpret_cast<double2*>(dst)[2 * c + 1] = make_double2(g2, 0.0);
+    for (int k = 0; k < 3; ++k) *reinterpret_cast<double2*>(dst + 2 * k) = make_double2(v[2 * k], v[2 * k + 1]);
+  }
+}
+template <typename real>
+__device__ __forceinline__ void load_group(const real* src, real (&v)[6]) {
+  if constexpr (sizeof(real) == 4) {
+    const float4 a = *reinterpret_cast<const float4*>(src);
+    const float2 b = *reinterpret_cast<const float2*>(src + 4);
+    v[0] = a.x;
+    v[1] = a.y;
+    v[2] = a.z;
+    v[3] = a.w;
+    v[4] = b.x;
+    v[5] = b.y;
+  } else {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const double2 t = *reinterpret_cast<const double2*>(src + 2 * k);
+      v[2 * k] = t.x;
+      v[2 * k + 1] = t.y;
     }
   }
 }
 
+// Accumulator of a 2-term product sum: FP32 as one packed pair of FMAs (the two ranks side by side, added at the
+// end), FP64 as two FMAs.
+template <typename real> struct Acc2;
+template <> struct Acc2<float> {
+  unsigned long long v;
+  __device__ __forceinline__ void zero() { v = 0ull; }
+  __device__ __forceinline__ void add(float a0, float a1, float b0, float b1) {
+    asm("{\n.reg .b64 a, b;\nmov.b64 a, {%1, %2};\nmov.b64 b, {%3, %4};\nfma.rn.f32x2 %0, a, b, %0;\n}"
+        : "+l"(v)
+        : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
+  }
+  __device__ __forceinline__ float sum() const {
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+    return lo + hi;
+  }
+};
+template <> struct Acc2<double> {
+  double v;
+  __device__ __forceinline__ void zero() { v = 0.0; }
+  __device__ __forceinline__ void add(double a0, double a1, double b0, double b1) { v = fma(a1, b1, fma(a0, b0, v)); }
+  __device__ __forceinline__ double sum() const { return v; }
+};
+
 template <typename real, bool RECOMPUTE>
-__global__ void __launch_bounds__(32 * PB_WARPS) k_pair_build(DevProblem P, Scratch<real> W, PairChunks B,
-                                                              const real* __restrict__ Gbuf) {
-  constexpr int CH = PairStage<real>::CH;
-  constexpr int ROWQ = GSTRIDE * (int)sizeof(real) / 16;   // 16-byte pieces of one G row
+__global__ void __launch_bounds__(32 * PB_WARPS, pb_ctas<real>())
+    k_pair_build(DevProblem P, Scratch<real> W, PairChunks B, const real* __restrict__ rowbuf, DevState* st) {
+  using PR = PairRows<real>;
   extern __shared__ __align__(16) unsigned char pb_smem[];
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  real* stage = reinterpret_cast<real*>(pb_smem) + (size_t)wib * 2 * CH * 2 * GSTRIDE;   // [2][CH][2][GSTRIDE]
+  real* stage = reinterpret_cast<real*>(pb_smem) + (size_t)wib * PB_CH * PR::PAIR;
   const long long nactive = *B.nactive;
-  const long long wstride = ((long long)gridDim.x * blockDim.x) >> 5;
-  long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-  if (w >= nactive) return;   // uniform per warp
+  // chunks are handed out by a counter (zeroed with the iteration): their sizes vary, and a fixed stride leaves the
+  // most loaded warp half as much again as the average
+  auto take = [&]() {
+    unsigned w = 0;
+    if (lane == 0) w = atomicAdd(&st->pair_next, 1u);
+    return (long long)__shfl_sync(FULL_MASK, w, 0);
+  };
+  const long long w0 = take();
+  if (w0 >= nactive) return;   // uniform per warp
   // lanes 0..26: pair slot g = lane / 9 of every three, and the 3 x 3 sub-block (rb, cb) of the 9 x 9 block
   const int g = lane / 9, sub = lane - 9 * (lane / 9), rb = sub / 3, cb = sub - 3 * (sub / 3);
-  const bool act = lane < 27;
-  const int j = lane % CH, side = lane / CH;
-  // the piece (chunk record, first pair) being copied and the one being accumulated
-  int4 ch = B.chunks[B.active[w]];
+  const int j = lane % PB_CH, side = lane / PB_CH;
+  int4 ch = B.chunks[B.active[w0]];
+  long long wn = take();   // the warp's next chunk
+  int4 chn = B.chunks[B.active[min(wn, nactive - 1)]];
   int c0 = 0;
-  auto issue = [&](const int4& chunk, int first, int buf) {
-    const int cn = min(CH, chunk.w - first);
-    if (side < 2 && j < cn) {
-      const int2 pr = B.pairs[chunk.z + first + j];
-      real* dst = stage + ((size_t)(buf * CH + j) * 2 + side) * GSTRIDE;
-      if constexpr (RECOMPUTE) {   // computed here: no G buffer, about 90 bytes read per pair instead of 288
-        const int b = side ? pr.y : pr.x;
-        obs_G<real, sizeof(real) == 4>(P, W, side ? chunk.y : chunk.x, P.base_pos[b], dst);
-      } else {
-        const real* src = Gbuf + (size_t)GSTRIDE * (side ? pr.y : pr.x);
-#pragma unroll
-        for (int q = 0; q < ROWQ; ++q)
-          cp_async_16(dst + q * (16 / (int)sizeof(real)), src + q * (16 / (int)sizeof(real)));
-      }
-    }
-    cp_async_commit();
+  // the pair of this lane in the piece at (chunk, first), and the virtual point of its observations
+  auto pair_of = [&](const int4& chunk, int first) {
+    return B.pairs[chunk.z + min(first + j, (chunk.w & PAIR_COUNT_MASK) - 1)];
   };
-  issue(ch, 0, 0);
-  int buf = 0;
-  real acc[3][3];
+  int2 pr = pair_of(ch, 0);
+  int vp = RECOMPUTE ? P.base_vp[pr.x] : 0;
+  Acc2<real> acc[3][3];
 #pragma unroll
-  for (int x = 0; x < 3; ++x) acc[x][0] = acc[x][1] = acc[x][2] = real(0);
+  for (int x = 0; x < 3; ++x)
+#pragma unroll
+    for (int y = 0; y < 3; ++y) acc[x][y].zero();
   for (;;) {
     // the next piece: the rest of this chunk, else the warp's next chunk
+    const int count = ch.w & PAIR_COUNT_MASK;
     int4 nch = ch;
-    int n0 = c0 + CH;
+    int n0 = c0 + PB_CH;
     bool more = true;
-    if (n0 >= ch.w) {
-      const long long nw = w + wstride;
-      if (nw < nactive) {
-        nch = B.chunks[B.active[nw]];
-        n0 = 0;
-      } else {
-        more = false;
+    if (n0 >= count) {
+      nch = chn;
+      n0 = 0;
+      more = wn < nactive;
+    }
+    // rows of this lane's observation (a lane past the chunk's end repeats its last pair; it is not accumulated)
+    real Pm[3][2], Jt[2][9];
+    if constexpr (RECOMPUTE) {
+      const CamRow<real> C = load_camrow<real>(P, side ? ch.y : ch.x);
+      real vi[VPI], Jp[2][3];   // L_v^-1 and the point
+      load_vec16<VPI>(W.vp_info + (size_t)VPI * vp, vi);
+      const real X[3] = {vi[VPI_X], vi[VPI_X + 1], vi[VPI_X + 2]};
+      proj_rows<real, true>(C, X, Jt, Jp);
+      if (P.huber_a > 0.0) {
+        const size_t pos = (size_t)P.base_pos[side ? pr.y : pr.x];
+        real r[2] = {res_ptr<real>(P)[2 * pos], res_ptr<real>(P)[2 * pos + 1]};
+        scale_rows(row_weight(P, r[0], r[1]), r, Jt, Jp);
+      }
+      pm_of_obs<real>(vi, Jp, Pm);
+    } else {
+      real v24[ROWREC];
+      load_vec16<ROWREC>(rowbuf + (size_t)ROWREC * (side ? pr.y : pr.x), v24);
+#pragma unroll
+      for (int t = 0; t < 6; ++t) Pm[t >> 1][t & 1] = v24[t];
+#pragma unroll
+      for (int c = 0; c < 9; ++c) {
+        Jt[0][c] = v24[6 + 2 * c];
+        Jt[1][c] = v24[7 + 2 * c];
       }
     }
-    if (more) {
-      issue(nch, n0, buf ^ 1);
-      cp_async_wait<1>();
-    } else {
-      cp_async_wait<0>();
+    // the next piece's pairs (their virtual points follow below, once these have arrived)
+    int2 prn = pr;
+    if (more) prn = pair_of(nch, n0);
+    // y lanes: rows M Jt_y with M = Pm_x^T Pm_y
+    real M[2][2] = {{0, 0}, {0, 0}};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const real a0 = __shfl_sync(FULL_MASK, Pm[k][0], j), a1 = __shfl_sync(FULL_MASK, Pm[k][1], j);
+      M[0][0] += a0 * Pm[k][0];
+      M[0][1] += a0 * Pm[k][1];
+      M[1][0] += a1 * Pm[k][0];
+      M[1][1] += a1 * Pm[k][1];
+    }
+    real* dst = stage + (size_t)j * PR::PAIR + side * PR::SIDE;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      real v6[6];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const real u0 = Jt[0][3 * b + c], u1 = Jt[1][3 * b + c];
+        v6[2 * c] = side ? M[0][0] * u0 + M[0][1] * u1 : u0;
+        v6[2 * c + 1] = side ? M[1][0] * u0 + M[1][1] * u1 : u1;
+      }
+      store_group<real>(dst + b * PR::GROUP, v6);
     }
     __syncwarp();
-    if (act) {
-      const int cn = min(CH, ch.w - c0);
-      const real* base = stage + (size_t)buf * CH * 2 * GSTRIDE;
+    if (RECOMPUTE && more) vp = P.base_vp[prn.x];
+    if (lane < 27) {
+      const int cn = min(PB_CH, count - c0);
       for (int jj = g; jj < cn; jj += 3) {   // pair slot g of every three
-        const real* ga = base + (size_t)jj * 2 * GSTRIDE;
-        const real* gb = ga + GSTRIDE;
-        real a[3][3], b[3][3];
-#pragma unroll
-        for (int x = 0; x < 3; ++x) {
-          load_gcol_s(ga + 4 * (3 * rb + x), a[x]);
-          load_gcol_s(gb + 4 * (3 * cb + x), b[x]);
-        }
+        real a[6], b[6];
+        load_group<real>(stage + (size_t)jj * PR::PAIR + rb * PR::GROUP, a);
+        load_group<real>(stage + (size_t)jj * PR::PAIR + PR::SIDE + cb * PR::GROUP, b);
 #pragma unroll
         for (int x = 0; x < 3; ++x)
 #pragma unroll
-          for (int y = 0; y < 3; ++y) acc[x][y] += a[x][0] * b[y][0] + a[x][1] * b[y][1] + a[x][2] * b[y][2];
+          for (int y = 0; y < 3; ++y) acc[x][y].add(a[2 * x], a[2 * x + 1], b[2 * y], b[2 * y + 1]);
       }
     }
-    __syncwarp();   // every lane is done with this buffer before it is refilled
-    if (c0 + CH >= ch.w) {   // the chunk is complete: sum the three pair slots, one add per block entry
+    __syncwarp();   // every lane is done with the rows before they are overwritten
+    if (c0 + PB_CH >= count) {   // the chunk is complete: sum the three pair slots, write the block
+      real s[3][3];
 #pragma unroll
       for (int x = 0; x < 3; ++x)
 #pragma unroll
         for (int y = 0; y < 3; ++y) {
           // lane L < 9 adds slots 1 and 2 from lanes L + 9 and L + 18 (source lanes wrap mod 32 for the rest)
-          const real v = acc[x][y];
-          acc[x][y] = v + __shfl_sync(FULL_MASK, v, lane + 9) + __shfl_sync(FULL_MASK, v, lane + 18);
+          const real v = acc[x][y].sum();
+          s[x][y] = v + __shfl_sync(FULL_MASK, v, lane + 9) + __shfl_sync(FULL_MASK, v, lane + 18);
+          acc[x][y].zero();
         }
       if (lane < 9) {
-        const int k = P.cam_cluster[ch.x];
-        const int la = P.cam_local[ch.x], lb = P.cam_local[ch.y];   // la > lb: local order follows camera order
-        const int np = P.cluster_np[k];
-        double* dst = W.S + P.S_off[k] + (size_t)(9 * la + 3 * rb) * np + 9 * lb + 3 * cb;
+        // the rotation rows and columns: J_c = Jt E
+        real Jl[9], t[3][3];
+        if (rb == 0) {
+          load_jl(P, ch.x, Jl);
+#pragma unroll
+          for (int x = 0; x < 3; ++x)
+#pragma unroll
+            for (int y = 0; y < 3; ++y) t[x][y] = Jl[x] * s[0][y] + Jl[3 + x] * s[1][y] + Jl[6 + x] * s[2][y];
+#pragma unroll
+          for (int x = 0; x < 3; ++x)
+#pragma unroll
+            for (int y = 0; y < 3; ++y) s[x][y] = t[x][y];
+        }
+        if (cb == 0) {
+          load_jl(P, ch.y, Jl);
+#pragma unroll
+          for (int x = 0; x < 3; ++x)
+#pragma unroll
+            for (int y = 0; y < 3; ++y) t[x][y] = s[x][0] * Jl[y] + s[x][1] * Jl[3 + y] + s[x][2] * Jl[6 + y];
+#pragma unroll
+          for (int x = 0; x < 3; ++x)
+#pragma unroll
+            for (int y = 0; y < 3; ++y) s[x][y] = t[x][y];
+        }
 #pragma unroll
         for (int x = 0; x < 3; ++x)
 #pragma unroll
-          for (int y = 0; y < 3; ++y) atomicAdd(dst + (size_t)x * np + y, -(double)acc[x][y]);
+          for (int y = 0; y < 3; ++y) stage[9 * (3 * rb + x) + 3 * cb + y] = s[x][y];
       }
+      __syncwarp();
+      const int k = P.cam_cluster[ch.x];
+      const int la = P.cam_local[ch.x], lb = P.cam_local[ch.y];   // la > lb: local order follows camera order
+      const int np = P.cluster_np[k];
+      double* dstS = W.S + P.S_off[k] + (size_t)(9 * la) * np + 9 * lb;
+      if (lane < 27) {   // three rows of the block per instruction
 #pragma unroll
-      for (int x = 0; x < 3; ++x) acc[x][0] = acc[x][1] = acc[x][2] = real(0);
+        for (int t = 0; t < 3; ++t) {
+          const int row = 3 * t + g;
+          double* d = dstS + (size_t)row * np + sub;
+          const double v = -(double)stage[9 * row + sub];
+          if (ch.w & PAIR_WHOLE_EDGE)
+            *d = v;
+          else
+            atomicAdd(d, v);
+        }
+      }
+      __syncwarp();   // the rows are overwritten next
       if (!more) break;
-      w += wstride;
+      wn = take();
+      chn = B.chunks[B.active[min(wn, nactive - 1)]];
     }
     ch = nch;
     c0 = n0;
-    buf ^= 1;
+    pr = prn;
   }
 }
 
 template <typename real>
-void launch_rcs_build(const DevProblem& P, Scratch<real> W, CamSlots CS, PairChunks B, real* Gbuf, DevState* st,
+void launch_rcs_build(const DevProblem& P, Scratch<real> W, CamSlots CS, PairChunks B, real* rowbuf, DevState* st,
                       cudaStream_t stream, cudaStream_t side, cudaEvent_t fork, cudaEvent_t join) {
   const bool pairs = B.nchunks > 0 && P.l < P.m;
-  // a pair pass that recomputes G_o depends on nothing the camera pass writes (they add to different
+  // a pair pass that recomputes its rows depends on nothing the camera pass writes (they add to different
   // blocks of S'), so with a second stream the two run side by side
   const bool beside = pairs && P.pair_recompute && side != nullptr;
   if (beside) {
@@ -748,14 +790,13 @@ void launch_rcs_build(const DevProblem& P, Scratch<real> W, CamSlots CS, PairChu
     cudaStreamWaitEvent(side, fork, 0);
   }
   cudaStream_t ps = beside ? side : stream;
-  // FP32: both passes take the strict Jacobian rows, so that stored and recomputed G_o are bitwise equal
-  k_cam_pass<real, sizeof(real) == 4><<<(CS.nwarps + 7) / 8, 256, 0, stream>>>(P, W, CS, Gbuf, st);
-  if (pairs) {   // a fixed grid walks the list of chunks inside clusters
-    const int grid = std::min((B.nchunks + PB_WARPS - 1) / PB_WARPS, 3 * num_sms());
+  k_cam_pass<real><<<(CS.nwarps + 7) / 8, 256, 0, stream>>>(P, W, CS, rowbuf, st);
+  if (pairs) {   // a fixed grid takes the chunks inside clusters
+    const int grid = std::min((B.nchunks + PB_WARPS - 1) / PB_WARPS, pb_ctas<real>() * num_sms());
     if (P.pair_recompute)
-      k_pair_build<real, true><<<grid, 32 * PB_WARPS, PairStage<real>::bytes, ps>>>(P, W, B, Gbuf);
+      k_pair_build<real, true><<<grid, 32 * PB_WARPS, PairRows<real>::bytes, ps>>>(P, W, B, rowbuf, st);
     else
-      k_pair_build<real, false><<<grid, 32 * PB_WARPS, PairStage<real>::bytes, ps>>>(P, W, B, Gbuf);
+      k_pair_build<real, false><<<grid, 32 * PB_WARPS, PairRows<real>::bytes, ps>>>(P, W, B, rowbuf, st);
   }
   if (beside) {
     cudaEventRecord(join, side);
@@ -765,7 +806,7 @@ void launch_rcs_build(const DevProblem& P, Scratch<real> W, CamSlots CS, PairChu
 
 // ------------------------------------------------------------------------------------------------------
 template <typename real>
-__global__ void __launch_bounds__(256) k_point_rhs(DevProblem P, const double* dc, const float* dcf, real* t_acc) {
+__global__ void __launch_bounds__(256) k_point_rhs(DevProblem P, const real* __restrict__ edc, real* t_acc) {
   const int o = blockIdx.x * blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31;
   const bool act = o < P.q;
@@ -774,19 +815,17 @@ __global__ void __launch_bounds__(256) k_point_rhs(DevProblem P, const double* d
   if (act) {
     pt = P.obs_pt[o];
     const int cam = P.obs_cam[o];
-    Cam<real> C = load_cam_w<real>(P, cam);
+    const CamRow<real> C = gather_camrow<real>(P, cam);
     real X[3];
     load_point_w(P, pt, X);
-    real uo, vo;
-    load_uv(P, o, uo, vo);
-    real r[2], Jc[2][9], Jp[2][3];
-    project_jacobian<real, true>(C, X, uo, vo, r, Jc, Jp);
+    real Jt[2][9], Jp[2][3], d[12];
+    load_vec16<12>(edc + (size_t)VPI * cam, d);   // J_c dc = Jt (E dc)
+    proj_rows<real, true>(C, X, Jt, Jp);
     real jd0 = 0, jd1 = 0;
 #pragma unroll
     for (int c = 0; c < 9; ++c) {
-      const real dcc = (sizeof(real) == 4) ? (real)dcf[9 * (size_t)cam + c] : (real)dc[9 * (size_t)cam + c];
-      jd0 += Jc[0][c] * dcc;
-      jd1 += Jc[1][c] * dcc;
+      jd0 += Jt[0][c] * d[c];
+      jd1 += Jt[1][c] * d[c];
     }
     // with a robust loss both Jacobians carry sqrt(rho'): the product carries rho'
     real wgt = real(1);
@@ -1168,7 +1207,7 @@ void launch_apply(const DevProblem& P, const double* dc, const double* dp, doubl
 template <typename real>
 void launch_point_rhs(const DevProblem& P, Scratch<real> W, cudaStream_t stream) {
   int blocks = (P.q + 255) / 256;
-  k_point_rhs<real><<<blocks, 256, 0, stream>>>(P, W.dc, W.dcf, W.t_acc);
+  k_point_rhs<real><<<blocks, 256, 0, stream>>>(P, W.edc, W.t_acc);
 }
 
 template <typename real>
@@ -1187,35 +1226,50 @@ void launch_cost(const DevProblem& P, const double* dc, const double* dp, double
 }
 
 
-__global__ void k_params_to_float(int m, int n, const double* __restrict__ cams, const double* __restrict__ pts,
-                                  float* __restrict__ cams_f, float* __restrict__ pts_f) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 9 * m + 3 * n; i += gridDim.x * blockDim.x) {
-    if (i < 9 * m)
+// Once per linearisation: the camera tables (blocks 0 .. cam_blocks - 1, one warp each: the FP64 sincos and
+// divisions of a camera run at 1/64 rate, so 32 cameras per SM) and, in mixed precision, the FP32 copies of the
+// cameras and points (the other blocks).
+template <typename real>
+__global__ void __launch_bounds__(256) k_params(int m, int n, int cam_blocks, const double* __restrict__ cams,
+                                                const double* __restrict__ pts, real* __restrict__ ctab,
+                                                float* __restrict__ cams_f, float* __restrict__ pts_f) {
+  if ((int)blockIdx.x < cam_blocks) {
+    const int j = 32 * blockIdx.x + threadIdx.x;
+    if (threadIdx.x < 32 && j < m) write_camtab<real>(cams + 9 * (size_t)j, m, j, ctab);
+    return;
+  }
+  for (int64_t i = ((int64_t)blockIdx.x - cam_blocks) * blockDim.x + threadIdx.x; i < 9 * (int64_t)m + 3 * (int64_t)n;
+       i += ((int64_t)gridDim.x - cam_blocks) * blockDim.x) {
+    if (i < 9 * (int64_t)m)
       cams_f[i] = (float)cams[i];
     else
-      pts_f[i - 9 * m] = (float)pts[i - 9 * m];
+      pts_f[i - 9 * (int64_t)m] = (float)pts[i - 9 * (int64_t)m];
   }
 }
 
-void launch_params_to_float(const DevProblem& P, float* cams_f, float* pts_f, cudaStream_t stream) {
-  const int total = 9 * P.m + 3 * P.n;
-  k_params_to_float<<<std::min((total + 255) / 256, 2048), 256, 0, stream>>>(P.m, P.n, P.cams, P.pts, cams_f, pts_f);
+template <typename real>
+void launch_params(const DevProblem& P, real* ctab, float* cams_f, float* pts_f, cudaStream_t stream) {
+  const int cam_blocks = (P.m + 31) / 32;
+  const int64_t total = 9 * (int64_t)P.m + 3 * (int64_t)P.n;
+  const int copy_blocks = cams_f ? (int)std::min<int64_t>((total + 255) / 256, 2048) : 0;
+  k_params<real><<<cam_blocks + copy_blocks, 256, 0, stream>>>(P.m, P.n, cam_blocks, P.cams, P.pts, ctab, cams_f, pts_f);
 }
 
 void configure_kernels(int max_np) {
   configure_solve_kernels(max_np);
   cudaFuncSetAttribute(k_pair_build<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)PairStage<float>::bytes);
+                       (int)PairRows<float>::bytes);
   cudaFuncSetAttribute(k_pair_build<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)PairStage<float>::bytes);
+                       (int)PairRows<float>::bytes);
   cudaFuncSetAttribute(k_pair_build<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)PairStage<double>::bytes);
+                       (int)PairRows<double>::bytes);
   cudaFuncSetAttribute(k_pair_build<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)PairStage<double>::bytes);
+                       (int)PairRows<double>::bytes);
 }
 
 #define INSTANTIATE(real)                                                                                  \
   template void launch_iter_begin<real>(DevState*, const Settings&, cudaStream_t);                        \
+  template void launch_params<real>(const DevProblem&, real*, float*, float*, cudaStream_t);              \
   template void launch_vp_reduce<real>(const DevProblem&, Scratch<real>, cudaStream_t);                   \
   template void launch_vp_finalize<real>(const DevProblem&, Scratch<real>, DevState*, const long long*,   \
                                          cudaStream_t, const double*);                                     \
@@ -1225,6 +1279,7 @@ void configure_kernels(int max_np) {
   template void launch_point_update<real>(const DevProblem&, Scratch<real>, cudaStream_t);                \
   template void launch_finalize<real>(const DevProblem&, Scratch<real>, DevState*, const Settings&, int,  \
                                       cudaStream_t);                                                      \
+  template void launch_step_rows<real>(const DevProblem&, const double*, real*, cudaStream_t);            \
   template void launch_point_rhs<real>(const DevProblem&, Scratch<real>, cudaStream_t);                  \
   template void launch_cost<real>(const DevProblem&, const double*, const double*, double*, float*, float*, \
                                   double*, DevState*, real*, cudaStream_t);                               \

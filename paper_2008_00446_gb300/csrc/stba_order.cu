@@ -145,6 +145,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(ReorderArgs A, cons
     run += v[t];
     const int vp = run - 1;
     A.obs_vp[o] = vp;
+    if (A.base_vp) A.base_vp[A.obs_base[o]] = vp;
     if (v[t]) {
       A.vp_off[vp] = o;
       const int i = A.obs_pt[o];
@@ -229,8 +230,6 @@ __global__ void k_cam_place(ReorderArgs A, const int* __restrict__ flag, const i
   const size_t sl = 32 * (size_t)A.cam_warp_off[j] + idx;
   A.slots[sl] = o;
   A.slot_pv[sl] = make_int2(A.ept[e], flag[e] ? (A.obs_vp[o] | INT_MIN) : A.obs_vp[o]);
-  if (A.slot_uvf) A.slot_uvf[sl] = A.euvf[e];
-  if (A.slot_uvd) A.slot_uvd[sl] = A.euvd[e];
 }
 
 // chunks of the camera graph whose two cameras share a cluster
