@@ -87,14 +87,16 @@ typedef struct {
                                cores; STBA_FACTOR_UPDATE_TENSOR = tcgen05 tensor cores, TF32 operands split
                                in three products for FP32 accuracy (the FP32 factor of STBA_MIXED with tile
                                64 only; other settings return STBA_ERR_INVALID_ARG). */
-  int32_t factor_panel;     /* panel of each tile step of the cluster factorisation: 0 = default (for the
-                               FP32 factor with tile 64: STBA_FACTOR_PANEL_SPLIT when the tiles of all
-                               clusters outnumber the SMs, i.e. a step runs in several waves, else _STACKED;
+  int32_t factor_panel;     /* panel of each tile step of the cluster factorisation: 0 = default (with CUDA-core
+                               updates of the FP32 factor with tile 64: STBA_FACTOR_PANEL_SPLIT when the tiles of
+                               all clusters outnumber the SMs, i.e. a step runs in several waves, else _STACKED;
                                _STACKED otherwise);
-                               STBA_FACTOR_PANEL_STACKED = one kernel per step factors the stacked panel of
-                               the diagonal tile and each tile below it (the diagonal tile redundantly per
-                               tile row); STBA_FACTOR_PANEL_SPLIT = the diagonal tile is factored and
-                               inverted once per cluster, the tiles below are its products with the inverse;
+                               STBA_FACTOR_PANEL_STACKED = the stacked panel of the diagonal tile and each tile
+                               below it (the diagonal tile redundantly per tile row); with the tensor-core update
+                               it runs in one launch with the update of the step before;
+                               STBA_FACTOR_PANEL_SPLIT = the diagonal tile is factored and inverted once per
+                               cluster, the tiles below are its products with the inverse (CUDA-core updates;
+                               with the tensor-core update the panel is stacked, which is faster at every size);
                                STBA_FACTOR_PANEL_PERSISTENT = one launch factors every cluster, a thread-block
                                cluster of 8 CTAs per camera cluster running all its tile steps with cluster
                                barriers between them (SPLIT and PERSISTENT: the FP32 factor of STBA_MIXED
@@ -302,10 +304,10 @@ stba_status stba_cluster_sgc(stba_ctx* ctx, int32_t gamma, double beta, uint64_t
  * the cluster factorisation on the current parameters and cluster assignment, restores the parameters,
  * damping and cost after each trial, and keeps the fastest for the following iterations.  Candidates
  * (STBA_MIXED; FP64 has one):
- *   0 = tile 64, split panel, tensor-core trailing update     1 = tile 64, split panel, CUDA-core update
+ *   0 = tile 64, split panel, tensor-core update (as 5)       1 = tile 64, split panel, CUDA-core update
  *   2 = tile 64, stacked panel, CUDA-core update              3 = tile 32, stacked panel, CUDA-core update
  *   4 = tile 64, persistent (one launch of 8-CTA clusters)  5 = tile 64, stacked panel, tensor-core update
- *                                                              (the default on problems of one wave of panels)
+ *                                                              (the default)
  * *choice (optional) receives the index kept (-1 for the single FP64 configuration or the FP64 factor of
  * factor_fp64), ms[0..5] (optional, 6 floats) the
  * time per iteration of each candidate (-1 when not tried).  Synchronises the context stream.  Errors:

@@ -505,9 +505,10 @@ stba_status set_clusters_host(stba_ctx* c, const std::vector<int>& cl) {
     }
   }
   CK(cudaMemcpyAsync(c->cl_owned, c->h_owned.data(), (size_t)l * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-  // panel of the FP32 factor with tile 64: the split panel pays off once a tile step's tiles outnumber the SMs
-  // (several waves of panel CTAs per step; each of them would factor its diagonal tile again), the stacked
-  // panel when they fit in one wave (a single kernel per step on the critical path)
+  // panel of the FP32 factor with tile 64 and CUDA-core updates: the split panel pays off once a tile step's tiles
+  // outnumber the SMs (several waves of panel CTAs per step; each of them would factor its diagonal tile again), the
+  // stacked panel when they fit in one wave (a single kernel per step on the critical path).  The tensor-core steps
+  // (k_step_tc) are always stacked.
   c->persistent = c->mixed && TF == 64 && c->panel_choice == STBA_FACTOR_PANEL_PERSISTENT;
   // CTAs per cluster solve: 8 while the solves' CTAs fit in about two waves (more CTAs share each tile step's
   // products), 4 beyond (cheaper barriers and exchanges once the solves queue for SMs anyway)
@@ -515,7 +516,7 @@ stba_status set_clusters_host(stba_ctx* c, const std::vector<int>& cl) {
   if (c->mixed && TF == 64 && c->panel_choice != STBA_FACTOR_PANEL_STACKED && !c->persistent) {
     int64_t tiles = 0;
     for (int k = 0; k < l; ++k) tiles += c->h_np[k] / TF;
-    c->split_panel = c->panel_choice == STBA_FACTOR_PANEL_SPLIT || tiles > num_sms();
+    c->split_panel = !c->update_tc && (c->panel_choice == STBA_FACTOR_PANEL_SPLIT || tiles > num_sms());
   } else {
     c->split_panel = 0;
   }
@@ -574,9 +575,11 @@ stba_status set_clusters_host(stba_ctx* c, const std::vector<int>& cl) {
     c->ev_update.push_back(e2);
   }
   {
-    int factor_launches = 3;
+    // tensor-core steps: scaling, one launch per step; else scaling, copy, inverses, panels and updates
+    const bool steps = c->update_tc && !c->persistent;
+    int factor_launches = steps ? 1 : 3;
     for (int kt = 0; kt < max_nt; ++kt)
-      factor_launches += (c->h_panel_off[kt + 1] > c->h_panel_off[kt]) + (c->h_update_off[kt + 1] > c->h_update_off[kt]);
+      factor_launches += steps ? 1 : (c->h_panel_off[kt + 1] > c->h_panel_off[kt]) + (c->h_update_off[kt + 1] > c->h_update_off[kt]);
     const int build_launches = 1 + (c->pchunks.nchunks > 0 && l < m ? 1 : 0);
     const int solve_launches = 2 + c->set.refine_steps * (2 + (res_items.empty() ? 0 : 1));
     // iter_begin, vp_reduce, pt_acc, vp_finalize | build | factor | solve, count | rhs, update, cam_rt,

@@ -11,8 +11,10 @@
 //   panel   for every tile row i >= kt: apply step kt - 1's update to tiles (kt, kt) and (i, kt), factor
 //           the diagonal tile with its inverse (redundantly in each CTA); the CTA of i = kt stores
 //           L_kt,kt and L_kt,kt^-1 (for the solves), the others L_i,kt = A_i,kt L_kt,kt^-T;
-//   update  for every kt + 1 < j <= i: A_i,j -= L_i,kt L_j,kt^T, on a second stream, overlapping the
-//           next panel.
+//   update  for every kt + 1 < j <= i: A_i,j -= L_i,kt L_j,kt^T.
+// The FP32 factor with tile 64 (the default) runs panel kt + 1 and update kt as one launch of k_step_tc, on the
+// tensor cores, reading S' itself where a tile is first touched.  The other factors (FP64, tile 32, CUDA-core
+// updates) copy the scaled matrix first and run the updates on a second stream, overlapping the next panel.
 // FP64 factor (FP64 mode): a pivot that is not positive and finite marks the cluster as failed, and the
 // LM step is rejected (lambda *= 3).  FP32 factor (mixed mode): a pivot that rounding has made vanish
 // (below 2^-20 of the unit scaled diagonal; legitimate pivots of the damped system are about lambda or
@@ -724,11 +726,13 @@ __global__ void __launch_bounds__(256) k_chol_update(F* L, DevProblem P, const i
 // FP32 accuracy from TF32 operands: every value x is split into hi = tf32(x) and lo = tf32(x - hi), and
 // D = A_hi B_lo + A_lo B_hi + A_hi B_hi (3xTF32; the dropped A_lo B_lo is below FP32 rounding), 24 MMAs
 // of K = 8 issued by one thread.  The operands are converted by all threads into the no-swizzle K-major
-// core-matrix layout (stba_tc.cuh); while the MMAs run, each thread loads the 32 old values it will
-// update (one row, 32 columns), then subtracts its 32 accumulator columns read from TMEM.  The wait for
+// core-matrix layout (stba_tc.cuh); the product goes from TMEM through shared memory, so that the updated values are
+// read and written 256 contiguous bytes per row.  The wait for
 // the MMAs is bounded: a CTA that gives up marks the cluster failed (the LM step is rejected), frees its
 // tensor memory and returns.  When i0 + 1 is past the cluster's last tile, the second half of A is zero and
 // its rows are not written.
+// Bound by its loads and the read-modify-write of the updated tiles (one row per lane and 16 bytes per access, as
+// before, took 71 % of the L1 pipe and 20 us for 400 tile pairs).
 constexpr int TCU_THREADS = 256;
 constexpr size_t TCU_SMEM = sizeof(uint32_t) * (2 * 128 * 64 + 2 * 64 * 64);   // A hi/lo, B hi/lo: 96 KB
 constexpr int TCU_MAX_POLLS = 1 << 26;
@@ -741,30 +745,49 @@ __device__ __forceinline__ void split_store(uint32_t* hi, uint32_t* lo, int off,
                  tc::to_tf32(v.z - __uint_as_float(h2)), tc::to_tf32(v.w - __uint_as_float(h3)));
 }
 
-__global__ void __launch_bounds__(TCU_THREADS, 2) k_chol_update_tc(float* L, DevProblem P, const int2* items, int kt,
-                                                                  int* fail_flags) {
-  constexpr int T = 64;
-  extern __shared__ __align__(128) uint32_t tsm[];
+// One CTA's work in a tile step: cluster, tile row (panel) or (i0 << 16) | j (update), and the cluster's layout.
+struct TileTask {
+  int k, tile, np, nk;
+  int64_t S_off, v_off;
+};
+
+// Four values of row `row`, columns col .. col + 3 of cluster k's scaled matrix, from the FP64 S' (the first touch of a
+// tile reads S' itself: no scaled copy is made for the tensor-core factorisation).
+__device__ __forceinline__ float4 scaled4(const double* __restrict__ Sk, const double* __restrict__ sk, int np, int row,
+                                          int col) {
+  const double2* p = reinterpret_cast<const double2*>(Sk + (size_t)row * np + col);
+  const double2 a = p[0], b = p[1];
+  const double sr = sk[row];
+  return make_float4((float)(a.x * sr * sk[col]), (float)(a.y * sr * sk[col + 1]), (float)(b.x * sr * sk[col + 2]),
+                     (float)(b.y * sr * sk[col + 3]));
+}
+
+// FIRST: step 0, whose old values come from S' (every tile this kernel ever updates is in its list there).
+template <bool FIRST>
+__device__ __forceinline__ void update_pair_tc(uint32_t* tsm, float* L, const double* __restrict__ S,
+                                               const double* __restrict__ scale, const TileTask& task, int kt,
+                                               int* fail_flags) {
+  constexpr int T = 64, LDS_ = 68;   // staging rows of the product: 16-byte aligned, no bank conflicts
   uint32_t* Ah = tsm;   // 128 x 64 TF32, core-matrix layout
   uint32_t* Al = tsm + 128 * 64;
   uint32_t* Bh = tsm + 2 * 128 * 64;   // 64 x 64
   uint32_t* Bl = Bh + 64 * 64;
+  float* stage = reinterpret_cast<float*>(tsm);   // over A, once the MMAs are done
   __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t taddr_s;
-  const int2 it = items[blockIdx.x];
-  const int k = it.x, i0 = it.y >> 16, j = it.y & 0xffff;
-  const int np = P.cluster_np[k];
-  float* A = L + P.S_off[k];
+  const int k = task.k, i0 = task.tile >> 16, j = task.tile & 0xffff;
+  const int np = task.np;
+  float* A = L + task.S_off;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rows_valid = min(128, np - i0 * T);   // 64 or 128
   const float* srcA = A + (size_t)(i0 * T) * np + kt * T;
   const float* srcB = A + (size_t)(j * T) * np + kt * T;
   // 16-byte chunk q = tid + 256 u: row (q >> 7) * 8 + (q & 7), columns 4 ((q >> 3) & 15) ..: the 8 threads of a
-  // shared-memory store phase write one whole core matrix (no bank conflicts).  Every load of the thread (its
-  // 12 operand chunks and the 32 old values it will update) is issued before any of them is used.
-  const int R = 32 * (warp & 3) + lane, c0 = 32 * (warp >> 2);   // epilogue: row R, columns c0 .. c0 + 31
-  const bool valid = R < rows_valid;
-  float* dst = A + (size_t)(i0 * T + R) * np + j * T + c0;
+  // shared-memory store phase write one whole core matrix (no bank conflicts).  The updated values: 16 lanes per row
+  // (256 contiguous bytes), rows 16 v + tid / 16.  Every load of the thread (its 12 operand chunks and, but for step
+  // 0, the 32 old values it will update) is issued before any of them is used.
+  const int r16 = tid >> 4, c4 = 4 * (tid & 15);
+  float* dst = A + (size_t)(i0 * T + r16) * np + j * T + c4;
   float4 va[8], vb[4], old[8];
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
@@ -779,8 +802,12 @@ __global__ void __launch_bounds__(TCU_THREADS, 2) k_chol_update_tc(float* L, Dev
     const int r = ((q >> 7) << 3) | (q & 7), kc = (q >> 3) & 15;
     vb[u] = *reinterpret_cast<const float4*>(srcB + (size_t)r * np + 4 * kc);
   }
+  if constexpr (!FIRST) {
 #pragma unroll
-  for (int v = 0; v < 8; ++v) old[v] = valid ? *reinterpret_cast<const float4*>(dst + 4 * v) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int v = 0; v < 8; ++v)
+      old[v] = 16 * v + r16 < rows_valid ? *reinterpret_cast<const float4*>(dst + (size_t)(16 * v) * np)
+                                         : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
     const int q = tid + TCU_THREADS * u;
@@ -810,26 +837,364 @@ __global__ void __launch_bounds__(TCU_THREADS, 2) k_chol_update_tc(float* L, Dev
                      idesc, (pass | ks) != 0);
     tc::mma_commit(&mbar);
   }
-  // thread (lane quarter warp & 3, column half warp >> 2): row R of the 128, columns c0 .. c0 + 31 of tile j
+  if constexpr (FIRST) {   // while the MMAs run
+    const double* Sk = S + task.S_off;
+    const double* sk = scale + task.v_off;
+#pragma unroll
+    for (int v = 0; v < 8; ++v)
+      old[v] = 16 * v + r16 < rows_valid ? scaled4(Sk, sk, np, i0 * T + 16 * v + r16, j * T + c4)
+                                         : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  // thread (lane quarter warp & 3, column half warp >> 2): row R of the product, 32 columns, to the staging rows
   const bool done = __all_sync(0xffffffffu, tc::mbar_wait_bounded(&mbar, 0, TCU_MAX_POLLS));
   if (done) {
     tc::fence_after_sync();
     float d[32];
+    const int R = 32 * (warp & 3) + lane, c0 = 32 * (warp >> 2);
     tc::tmem_ld32(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0, d);
-    if (valid) {
 #pragma unroll
-      for (int v = 0; v < 8; ++v)
-        *reinterpret_cast<float4*>(dst + 4 * v) =
-            make_float4(old[v].x - d[4 * v], old[v].y - d[4 * v + 1], old[v].z - d[4 * v + 2], old[v].w - d[4 * v + 3]);
-    }
+    for (int v = 0; v < 8; ++v)
+      *reinterpret_cast<float4*>(stage + R * LDS_ + c0 + 4 * v) = make_float4(d[4 * v], d[4 * v + 1], d[4 * v + 2], d[4 * v + 3]);
   } else if (lane == 0) {
     atomicExch(fail_flags + k, 1);
   }
   tc::fence_before_sync();
-  __syncthreads();
+  const int all_done = __syncthreads_and(done);
   if (warp == 0) tc::tmem_dealloc(tmem, 64);
+  if (!all_done) return;
+#pragma unroll
+  for (int v = 0; v < 8; ++v) {
+    if (16 * v + r16 >= rows_valid) break;
+    const float4 d = *reinterpret_cast<const float4*>(stage + (16 * v + r16) * LDS_ + c4);
+    *reinterpret_cast<float4*>(dst + (size_t)(16 * v) * np) =
+        make_float4(old[v].x - d.x, old[v].y - d.y, old[v].z - d.z, old[v].w - d.w);
+  }
 }
 
+// ------------------------------------------------------------------------------------------------------
+// Panel of tile step kt with the tensor-core update (FP32 factor, T = 64): one CTA per tile row i >= kt of a
+// cluster works on the stacked tile [A_kt,kt; A_i,kt] (128 rows; the CTA of i = kt takes the identity as its lower
+// half, whose rows then come out as L_kt,kt^-T: the inverse the solves need, at no extra step).
+//   1. step kt - 1's update, [A_kt; A_i] -= [L_kt,kt-1; L_i,kt-1] L_kt,kt-1^T, is one 128 x 64 x 64 product on the
+//      tensor cores (3xTF32 as update_pair_tc; B is the first half of A), the old values loaded meanwhile;
+//   2. LL^T of the stack in blocks of 8 columns, left-looking: thread r < 128 owns row r.  Between two barriers warp
+//      4 applies the last block's rank-8 term to the 8 x 8 diagonal block and its lane 0 factors it, while every
+//      row below finishes the same block column in its registers and takes the terms of all earlier blocks off
+//      the next one; between the next two barriers the rows are solved against the factored block and stored.
+// The chain is the 64 pivots (about 55 cycles each in chol8_fast) plus two barriers and one 8-step substitution per
+// block.  A row's operands are its own smem row (16-byte loads, 68-float rows: no bank conflicts) and the diagonal
+// rows, which all lanes read at one address, so that a block moves a quarter of the shared-memory words of the
+// right-looking rank-8 updates of k_chol_panel, which bound it.
+// Panel alone on an SM: 9.6 us (loads and operands 2.5, product 0.65, sweep 5.9; k_chol_panel took 20), beside an
+// update CTA about 13.  One 512-thread CTA per SM with two tasks, so that a panel has its SM to itself, was slower
+// (12 clusters of 83 cameras 265 us against 228: an SM then waits for both tasks).
+constexpr int PTC_THREADS = 256;
+constexpr int PTC_LD = 68;
+constexpr size_t PTC_SMEM = sizeof(float) * 128 * PTC_LD + sizeof(uint32_t) * 2 * 128 * 64;   // tile, A hi / lo: 98 KB
+
+__device__ __forceinline__ float rsqrt_normal(float x) {   // x normal and positive (pivots are >= 2^-20)
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// LL^T of the 8 x 8 block at T (rows of PTC_LD floats), by one thread in registers; reciprocal pivots to rinv.
+// The pivot rules of chol8 (FP32).
+__device__ __forceinline__ void chol8_fast(float* T, int row0, int nk, float* rinv, int* fail, int* boosted) {
+  float d[8][8];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const float4 a = *reinterpret_cast<const float4*>(T + r * PTC_LD);
+    d[r][0] = a.x;
+    d[r][1] = a.y;
+    d[r][2] = a.z;
+    d[r][3] = a.w;
+    if (r >= 4) {
+      const float4 b = *reinterpret_cast<const float4*>(T + r * PTC_LD + 4);
+      d[r][4] = b.x;
+      d[r][5] = b.y;
+      d[r][6] = b.z;
+      d[r][7] = b.w;
+    }
+  }
+  int bad = 0, nboost = 0;
+  float ri[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    float pv = d[j][j];
+    const bool pad = row0 + j >= nk, fin = isfinite(pv), low = pv < 1.f / 1048576;
+    bad |= !pad && !fin;
+    nboost += !pad && fin && low;
+    pv = (pad || !fin) ? 1.f : (low ? 1.f / 4096 : pv);
+    const float is = rsqrt_normal(pv);
+    d[j][j] = pv * is;
+    ri[j] = is;
+#pragma unroll
+    for (int r = j + 1; r < 8; ++r) d[r][j] *= is;
+#pragma unroll
+    for (int c = j + 1; c < 8; ++c)
+#pragma unroll
+      for (int r = c; r < 8; ++r) d[r][c] -= d[r][j] * d[c][j];
+  }
+#pragma unroll
+  for (int r = 1; r < 8; ++r) {
+    *reinterpret_cast<float4*>(T + r * PTC_LD) =
+        make_float4(d[r][0], r > 1 ? d[r][1] : 0.f, r > 2 ? d[r][2] : 0.f, r > 3 ? d[r][3] : 0.f);
+    if (r > 4)
+      *reinterpret_cast<float4*>(T + r * PTC_LD + 4) =
+          make_float4(d[r][4], r > 5 ? d[r][5] : 0.f, r > 6 ? d[r][6] : 0.f, 0.f);   // below the diagonal only
+  }
+  reinterpret_cast<float4*>(rinv)[0] = make_float4(ri[0], ri[1], ri[2], ri[3]);
+  reinterpret_cast<float4*>(rinv)[1] = make_float4(ri[4], ri[5], ri[6], ri[7]);
+  if (bad) *fail = 1;
+  if (nboost && boosted) atomicAdd(boosted, nboost);
+}
+
+__device__ __forceinline__ float dot4(float4 a, float4 b, float s) {   // s - a.b
+  s = fmaf(-a.x, b.x, s);
+  s = fmaf(-a.y, b.y, s);
+  s = fmaf(-a.z, b.z, s);
+  return fmaf(-a.w, b.w, s);
+}
+
+// the barrier of the sweep: the four row warps and the pivot warp
+__device__ __forceinline__ void sweep_barrier() {
+  __syncwarp();
+  asm volatile("bar.sync 1, 160;\n" ::: "memory");
+}
+
+__device__ __forceinline__ void panel_tc(uint32_t* psm, float* L, float* Dinv, const double* __restrict__ S,
+                                         const double* __restrict__ scale, const TileTask& task, int kt,
+                                         int* fail_flags, int* boosted, int64_t v_total) {
+  constexpr int T = 64, LD = PTC_LD, NB = T / 8;
+  uint32_t* Ah = psm;   // 128 x 64 TF32, core-matrix layout: rows of L_kt,kt-1, then of L_i,kt-1
+  uint32_t* Al = psm + 128 * 64;
+  float* W = reinterpret_cast<float*>(psm + 2 * 128 * 64);   // [128][LD] the stacked tile
+  __shared__ __align__(8) uint64_t mbar;
+  __shared__ uint32_t taddr_s;
+  __shared__ __align__(16) float rinv[8];
+  const int k = task.k, i = task.tile;
+  const bool diag = i == kt;
+  const int np = task.np, nk = task.nk;
+  float* A = L + task.S_off;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // the stacked tile's old values: 16 lanes per row; columns 0 and 1 come from S' (no update has touched them)
+  const int r16 = tid >> 4, c4 = 4 * (tid & 15);
+#pragma unroll
+  for (int v = 0; v < 8; ++v) {
+    const int r = 16 * v + r16, grow = r < T ? kt * T + r : i * T + r - T;
+    float* w = W + r * LD + c4;
+    if (v >= 4 && diag) {   // the identity
+      const int e = r - T - c4;
+      *reinterpret_cast<float4*>(w) = make_float4(e == 0 ? 1.f : 0.f, e == 1 ? 1.f : 0.f, e == 2 ? 1.f : 0.f, e == 3 ? 1.f : 0.f);
+    } else if (kt <= 1) {
+      *reinterpret_cast<float4*>(w) = scaled4(S + task.S_off, scale + task.v_off, np, grow, kt * T + c4);
+    } else {
+      cp_async16(w, A + (size_t)grow * np + kt * T + c4);
+    }
+  }
+  bool done = true;
+  if (kt > 0) {
+    float4 va[8];   // chunks as in update_pair_tc
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int q = tid + PTC_THREADS * u;
+      const int r = ((q >> 7) << 3) | (q & 7), kc = (q >> 3) & 15;
+      const float* src = A + (size_t)(r < T ? kt * T + r : i * T + r - T) * np + (kt - 1) * T + 4 * kc;
+      va[u] = (r < T || !diag) ? *reinterpret_cast<const float4*>(src) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int q = tid + PTC_THREADS * u;
+      split_store(Ah, Al, tc::core_off<64>(((q >> 7) << 3) | (q & 7), 4 * ((q >> 3) & 15)), va[u]);
+    }
+    tc::fence_async_smem();
+    if (tid == 0) tc::mbar_init(&mbar, 1);
+    if (warp == 0) tc::tmem_alloc(&taddr_s, 64);
+    cp_async_wait_all();
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem = taddr_s;
+    if (tid == 0) {
+      constexpr uint32_t idesc = tc::idesc_tf32(128, 64);
+      const uint32_t pa[3] = {tc::smem_u32(Ah), tc::smem_u32(Al), tc::smem_u32(Ah)};
+      const uint32_t pb[3] = {tc::smem_u32(Al), tc::smem_u32(Ah), tc::smem_u32(Ah)};   // rows 0 .. 63
+#pragma unroll
+      for (int pass = 0; pass < 3; ++pass)
+#pragma unroll
+        for (int ks = 0; ks < 8; ++ks)
+          tc::mma_tf32(tmem, tc::smem_desc(pa[pass] + ks * 256, 128, 2048), tc::smem_desc(pb[pass] + ks * 256, 128, 2048),
+                       idesc, (pass | ks) != 0);
+      tc::mma_commit(&mbar);
+    }
+    done = __all_sync(FULL_MASK, tc::mbar_wait_bounded(&mbar, 0, TCU_MAX_POLLS));
+    if (done) {
+      tc::fence_after_sync();
+      float d[32];
+      const int R = 32 * (warp & 3) + lane, c0 = 32 * (warp >> 2);   // a row and half of its columns
+      tc::tmem_ld32(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0, d);
+      if (R < T || !diag) {
+#pragma unroll
+        for (int v = 0; v < 8; ++v) {
+          float4* w = reinterpret_cast<float4*>(W + R * LD + c0 + 4 * v);
+          float4 a = *w;
+          a.x -= d[4 * v];
+          a.y -= d[4 * v + 1];
+          a.z -= d[4 * v + 2];
+          a.w -= d[4 * v + 3];
+          *w = a;
+        }
+      }
+    }
+    tc::fence_before_sync();
+  }
+  const int all_done = __syncthreads_and(done);
+  if (kt > 0 && warp == 0) tc::tmem_dealloc(taddr_s, 64);
+  if (!all_done) {   // the wait gave up: the cluster fails, the step is rejected
+    if (tid == 0) atomicExch(fail_flags + k, 1);
+    return;
+  }
+  if (warp > 4) return;   // the sweep: row warps 0 .. 3, pivot warp 4
+  float* my = W + tid * LD;   // row threads
+  float x[8], nx[8], o[8];
+  float* Di = Dinv + (size_t)task.v_off * T + (size_t)kt * T * T;
+  float* DiT = Di + v_total * T;
+  float* Xg = nullptr;   // where this row's solved blocks go
+  if (warp == 2 || warp == 3) Xg = diag ? DiT + (tid - T) * T : A + (size_t)(i * T + tid - T) * np + kt * T;
+  auto load8 = [](const float* p, float (&v)[8]) {
+    const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
+    v[0] = a.x;
+    v[1] = a.y;
+    v[2] = a.z;
+    v[3] = a.w;
+    v[4] = b.x;
+    v[5] = b.y;
+    v[6] = b.z;
+    v[7] = b.w;
+  };
+#pragma unroll
+  for (int c = 0; c < 8; ++c) x[c] = nx[c] = o[c] = 0.f;
+#pragma unroll 1
+  for (int b = 0; b < NB; ++b) {
+    const int n0 = 8 * b, n1 = n0 + 8;
+    const float* last = W + n0 * LD + n0 - 8;   // rows of the diagonal block, columns of the last block
+    if (warp == 4) {
+      // lane (r, c / 2): entries (r, c), (r, c + 1) of the diagonal block
+      float* blk = W + n0 * LD + n0;
+      if (b > 0) {
+        const int r = lane >> 2, c = 2 * (lane & 3);
+        float lr[8], l0[8], l1[8];
+        load8(last + r * LD, lr);
+        load8(last + c * LD, l0);
+        load8(last + (c + 1) * LD, l1);
+        float2 v = *reinterpret_cast<float2*>(blk + r * LD + c);
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+          v.x = fmaf(-lr[t], l0[t], v.x);
+          v.y = fmaf(-lr[t], l1[t], v.y);
+        }
+        *reinterpret_cast<float2*>(blk + r * LD + c) = v;
+        __syncwarp();
+      }
+      if (lane == 0) chol8_fast(blk, kt * T + n0, nk, rinv, fail_flags + k, diag ? boosted : nullptr);
+    } else if (tid >= n1) {
+      // block column b of this row, all terms
+      if (b > 0) {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const float4 l0 = *reinterpret_cast<const float4*>(last + c * LD), l1 = *reinterpret_cast<const float4*>(last + c * LD + 4);
+          x[c] = dot4(make_float4(o[4], o[5], o[6], o[7]), l1, dot4(make_float4(o[0], o[1], o[2], o[3]), l0, nx[c]));
+        }
+      } else {
+        load8(my, x);
+      }
+      // block column b + 1, the terms of blocks 0 .. b - 1
+      if (b + 1 < NB) {
+        load8(my + n1, nx);
+        const float* next = W + n1 * LD;
+#pragma unroll 2
+        for (int t = 0; t < n0; t += 4) {
+          const float4 a = *reinterpret_cast<const float4*>(my + t);
+#pragma unroll
+          for (int c = 0; c < 8; ++c) nx[c] = dot4(a, *reinterpret_cast<const float4*>(next + c * LD + t), nx[c]);
+        }
+        if (tid < n1 + 8) {   // a row of the next diagonal block: for the pivot warp
+          *reinterpret_cast<float4*>(my + n1) = make_float4(nx[0], nx[1], nx[2], nx[3]);
+          *reinterpret_cast<float4*>(my + n1 + 4) = make_float4(nx[4], nx[5], nx[6], nx[7]);
+        }
+      }
+    }
+    sweep_barrier();
+    if (warp < 4 && tid >= n1) {
+      float ri[8];
+      load8(rinv, ri);
+#pragma unroll
+      for (int c = 0; c < 8; ++c) o[c] = x[c];
+      const float* lb = W + n0 * LD + n0;
+      float lc[8][8];
+#pragma unroll
+      for (int c = 1; c < 8; ++c) {
+        const float4 a = *reinterpret_cast<const float4*>(lb + c * LD);
+        lc[c][0] = a.x;
+        lc[c][1] = a.y;
+        lc[c][2] = a.z;
+        lc[c][3] = a.w;
+        if (c > 4) {
+          const float4 e = *reinterpret_cast<const float4*>(lb + c * LD + 4);
+          lc[c][4] = e.x;
+          lc[c][5] = e.y;
+          lc[c][6] = e.z;
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        o[t] *= ri[t];
+#pragma unroll
+        for (int c = t + 1; c < 8; ++c) o[c] = fmaf(-o[t], lc[c][t], o[c]);
+      }
+      const float4 a = make_float4(o[0], o[1], o[2], o[3]), e = make_float4(o[4], o[5], o[6], o[7]);
+      *reinterpret_cast<float4*>(my + n0) = a;
+      *reinterpret_cast<float4*>(my + n0 + 4) = e;
+      if (Xg) {
+        *reinterpret_cast<float4*>(Xg + n0) = a;
+        *reinterpret_cast<float4*>(Xg + n0 + 4) = e;
+        if (diag) {
+#pragma unroll
+          for (int c = 0; c < 8; ++c) Di[(n0 + c) * T + tid - T] = o[c];
+        }
+      }
+    }
+    sweep_barrier();
+  }
+}
+
+// One launch per tile step: the CTAs of panel kt + 1 first (their chain sets the step's time), then the trailing update
+// of step kt; both read column kt, finished by the launch before.  kt = -1: panel 0 alone; FIRST: kt = 0.  The next
+// step's CTAs start under programmatic dependent launch: they read their task while this step's last CTAs finish.
+// Factorisation stage, before (panel and update launches on two streams, scaled copy, inverses of the diagonal
+// tiles) -> now: 12 clusters of 83 cameras 357 -> 212 us, 10 of 100 404 -> 243, 13 uneven of up to 297 2186 -> 1195,
+// one of 400 1560 -> 857, 67 of 90 1057 -> 797.  Of it: the panel 98 us of 357 (12 clusters), update epilogue and no
+// scaled copy 2 (13 uneven: 190 of 2186), one launch per step 28, dependent launch 16.  Panels stacked with the
+// tiles below them also where they outnumber the SMs: a separate launch for the diagonal tiles (the split panel)
+// would put the update before the tiles below (67 clusters: 819 us split on two streams, 815 one launch).
+template <bool FIRST>
+__global__ void __launch_bounds__(PTC_THREADS, 2) k_step_tc(float* L, float* Dinv, const double* __restrict__ S,
+                                                            const double* __restrict__ scale, DevProblem P,
+                                                            const int2* panels, int npanels, const int2* updates,
+                                                            int kt, int* fail_flags, int* boosted, int64_t v_total) {
+  extern __shared__ __align__(128) uint32_t step_smem[];
+  const bool panel = (int)blockIdx.x < npanels;
+  const int2 it = panel ? panels[blockIdx.x] : updates[blockIdx.x - npanels];
+  const TileTask task{it.x, it.y, P.cluster_np[it.x], P.cluster_n[it.x], P.S_off[it.x], P.v_off[it.x]};
+  // the next step's CTAs may take free SMs and read their own tasks; what the launch before wrote, from here on
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (panel)
+    panel_tc(step_smem, L, Dinv, S, scale, task, kt + 1, fail_flags, boosted, v_total);
+  else
+    update_pair_tc<FIRST>(step_smem, L, S, scale, task, kt, fail_flags);
+}
 
 // ------------------------------------------------------------------------------------------------------
 // Persistent factorisation (FP32 factor, T = 64): one thread-block cluster of FCS CTAs per camera cluster
@@ -1395,11 +1760,13 @@ void launch_factor_t(const DevProblem& P, const double* S, const FactorBuffers& 
   dim3 g1(std::max(1, std::min(plan.max_np / 256 + 1, 64)), P.l);
   k_diag_scale<Sreal><<<g1, 256, 0, stream>>>(P, S, fb.scale);
   dim3 g2(std::min(plan.max_np, 1024), P.l);
+  bool tcf = false;   // tensor-core panels and updates: they read S' themselves, no scaled copy
+  if constexpr (sizeof(F) == 4 && T == 64) tcf = plan.update_tc && !plan.persistent;
   // the first tile column now (the first panels read it); with more tile steps, the rest of the copy runs
   // on the side stream beside panel 0, and panel 1 waits for it
-  bool copy_beside = plan.nsteps > 1 && plan.ev_copy != nullptr;
+  bool copy_beside = !tcf && plan.nsteps > 1 && plan.ev_copy != nullptr;
   if constexpr (sizeof(F) == 4 && T == 64) copy_beside = copy_beside && !plan.persistent;
-  k_scaled_copy<Sreal, F><<<g2, 256, 0, stream>>>(P, S, fb.scale, L, 0, copy_beside ? T : INT_MAX);
+  if (!tcf) k_scaled_copy<Sreal, F><<<g2, 256, 0, stream>>>(P, S, fb.scale, L, 0, copy_beside ? T : INT_MAX);
   // panels on `stream`; the trailing updates (all tiles but the next column, which the next panel updates
   // itself) on the side stream, so that update kt overlaps panel kt + 1.  Panel kt + 2 waits for update kt.
   if constexpr (sizeof(F) == 4 && T == 64) {
@@ -1419,6 +1786,32 @@ void launch_factor_t(const DevProblem& P, const double* S, const FactorBuffers& 
         cfg.numAttrs = 1;
         cudaLaunchKernelEx(&cfg, k_chol_cluster<T>, reinterpret_cast<float*>(L), reinterpret_cast<float*>(Dinv), P,
                            plan.cluster_items, fb.fail_flags, fb.boosted, fb.v_total);
+      }
+      return;
+    }
+  }
+  if constexpr (sizeof(F) == 4 && T == 64) {
+    if (tcf) {
+      constexpr size_t smem = std::max(PTC_SMEM, TCU_SMEM);
+      for (int kt = -1; kt + 1 < plan.nsteps; ++kt) {
+        const int npn = plan.h_panel_off[kt + 2] - plan.h_panel_off[kt + 1];
+        const int nu = kt < 0 ? 0 : plan.h_update_off[kt + 1] - plan.h_update_off[kt];
+        if (npn + nu == 0) continue;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(npn + nu);
+        cfg.blockDim = dim3(PTC_THREADS);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = stream;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = kt >= 0 ? 1 : 0;   // panel 0 follows kernels that do not signal
+        cudaLaunchKernelEx(&cfg, kt == 0 ? k_step_tc<true> : k_step_tc<false>, reinterpret_cast<float*>(L),
+                           reinterpret_cast<float*>(Dinv), S, (const double*)fb.scale, P,
+                           plan.panel_items + plan.h_panel_off[kt + 1], npn,
+                           plan.update_items + (kt < 0 ? 0 : plan.h_update_off[kt]), kt, fb.fail_flags, fb.boosted,
+                           fb.v_total);
       }
       return;
     }
@@ -1455,22 +1848,14 @@ void launch_factor_t(const DevProblem& P, const double* S, const FactorBuffers& 
     cudaStreamWaitEvent(side, plan.ev_panel[kt], 0);
     const int nu = plan.h_update_off[kt + 1] - plan.h_update_off[kt];
     if (nu > 0) {
-      if constexpr (sizeof(F) == 4 && T == 64) {
-        if (plan.update_tc) {
-          launch_prio(k_chol_update_tc, nu, TCU_SMEM, side, plan.prio_low, reinterpret_cast<float*>(L), P,
-                      plan.update_items + plan.h_update_off[kt], kt, fb.fail_flags);
-        } else {
-          launch_prio(k_chol_update<F, T>, nu, 0, side, plan.prio_low, L, P, plan.update_items + plan.h_update_off[kt], kt);
-        }
-      } else {
-        launch_prio(k_chol_update<F, T>, nu, 0, side, plan.prio_low, L, P, plan.update_items + plan.h_update_off[kt], kt);
-      }
+      launch_prio(k_chol_update<F, T>, nu, 0, side, plan.prio_low, L, P, plan.update_items + plan.h_update_off[kt], kt);
     }
     cudaEventRecord(plan.ev_update[kt], side);
   }
   cudaEventRecord(plan.ev_join, side);
   cudaStreamWaitEvent(stream, plan.ev_join, 0);
-  if (plan.n_diag_items > 0 && !plan.split)   // the split panel's diagonal kernels wrote the inverses
+  // the split panel's diagonal kernels wrote the inverses
+  if (plan.n_diag_items > 0 && !plan.split)
     k_diag_inverse<F, T><<<plan.n_diag_items, 256, 0, stream>>>(reinterpret_cast<const F*>(fb.Ldiag), Dinv, P,
                                                                 plan.diag_items, fb.v_total);
 }
@@ -1554,7 +1939,8 @@ void configure_solve_kernels(int max_np) {
   raise_smem_attr((const void*)k_chol_panel<float, 64>, (int)panel_smem<float, 64>());
   raise_smem_attr((const void*)k_chol_panel<float, 32>, (int)panel_smem<float, 32>());
   raise_smem_attr((const void*)k_chol_panel<double, 32>, (int)panel_smem<double, 32>());
-  raise_smem_attr((const void*)k_chol_update_tc, (int)TCU_SMEM);
+  raise_smem_attr((const void*)k_step_tc<true>, (int)std::max(PTC_SMEM, TCU_SMEM));
+  raise_smem_attr((const void*)k_step_tc<false>, (int)std::max(PTC_SMEM, TCU_SMEM));
   raise_smem_attr((const void*)k_chol_diag<float, 64>, (int)DiagLayout<float, 64>::bytes);
   raise_smem_attr((const void*)k_chol_trsm<float, 64>, (int)TrsmLayout<float, 64>::bytes);
   // room for three stages wherever solve_stages may choose them

@@ -1,0 +1,37 @@
+"""The cluster factorisation and solve at the edges of the 64-wide tiles: clusters of 1 to 5 tiles, full, one short
+and one over, an odd and an even number of tile rows below a step (the update works on pairs), all in one problem
+and alone, with the tensor-core steps (default) and the CUDA-core factor.  Every cluster's step against a dense
+FP64 solve of the device's own S'_k.  Bar 1e-6 of each camera row: at lambda = 0.09 the scaled system has no
+eigenvalue below about 0.08 and none above about 20, so the FP32 solution is within 250 x 10 x 6e-8 = 1.5e-4 of the
+exact one and one FP64 refinement step squares that."""
+import numpy as np
+import pytest
+
+import scenes
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2008_00446_gb300 import stba  # noqa: E402
+
+from elementwise import rows  # noqa: E402
+
+SIZES = [1, 7, 8, 14, 15, 21, 22, 28, 29, 35]   # 9, 63, 72, 126, 135, 189, 198, 252, 261, 315 unknowns
+
+
+@pytest.mark.parametrize("update", [0, 1])
+@pytest.mark.parametrize("sizes", [SIZES] + [[s] for s in SIZES if s > 1])
+def test_cluster_steps_at_tile_edges(sizes, update):
+    m = sum(sizes)
+    cl = np.repeat(np.arange(len(sizes)), sizes).astype(np.int32)
+    s = scenes.make_tiny_scene(m=m, n=30 * max(m, 4), seed=m, clusters=cl, drop=0.5 if m < 40 else 0.9)
+    with stba.stba_create(s.cameras, s.points, s.obs_cam, s.obs_pt, s.obs_uv, cl, lambda0=0.09,
+                          precision=stba.STBA_MIXED, factor_update=update) as ctx:
+        info = stba.stba_lm_iteration(ctx)
+        assert info["failed_clusters"] == 0
+        dc, _ = stba.stba_last_step(ctx)
+        for k in range(len(sizes)):
+            S, b = stba.stba_get_cluster_system(ctx, k)
+            x = np.linalg.solve(S, b)
+            e = rows(dc[cl == k].ravel(), x, 9)
+            assert e < 1e-6, (k, sizes[k], e)
