@@ -562,7 +562,8 @@ stba_status set_clusters_host(stba_ctx* c, const std::vector<int>& cl) {
     if (c->h_owned[k]) cluster_items.push_back(k);
   for (int k = 0; k < l && !c->use_pcg; ++k)
     if (c->h_owned[k])
-      for (int rb = 0; rb < (c->h_nk[k] + 31) / 32; ++rb) res_items.push_back(make_int2(k, rb));
+      for (int rb = 0; rb < (c->h_nk[k] + 31) / 32; ++rb)
+        for (int j0 = 0; j0 <= rb; j0 += RES_TILES) res_items.push_back(make_int2(k, rb | (j0 / RES_TILES) << 16));
   for (int k = 0; k < l && !c->use_pcg; ++k)
     if (c->h_owned[k])
       for (int t = 0; t < c->h_np[k] / TF; ++t) diag_items.push_back(make_int2(k, t));

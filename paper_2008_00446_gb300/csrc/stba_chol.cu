@@ -21,13 +21,14 @@
 // more) is raised to 2^-12 and counted -- static pivoting, as in Li & Demmel's SuperLU_DIST -- and the
 // FP64 iterative refinement that follows solves the unmodified system.  A non-finite pivot fails.
 //
-// Solves: one CTA per cluster; with the inverted diagonal tiles every tile step is two parallel
-// matrix-vector products.  Refinement: r = b - S x in FP64 over many CTAs (S symmetric, lower stored),
+// Solves (k_tri_push): a thread-block cluster of CTAs per camera cluster; with the inverted diagonal tiles every
+// tile step is two parallel matrix-vector products.  Refinement: r = b - S x in FP64 over many CTAs (S symmetric, lower stored),
 // then x += D^-1/2 (L L^T)^-1 D^-1/2 r.
 #include <cooperative_groups.h>
 
 #include <map>
 #include <mutex>
+#include <type_traits>
 
 #include "stba_internal.cuh"
 #include "stba_tc.cuh"
@@ -1583,6 +1584,252 @@ __global__ void __launch_bounds__(256) k_tri_solve(DevProblem P, const F* L, con
   cluster.sync();   // keep this CTA's shared memory alive until every peer has read it
 }
 
+// ------------------------------------------------------------------------------------------------------
+// The same solve as a data flow (clusters whose accumulators fit in shared memory: up to about 280 tile rows of the
+// FP32 factor with 8 CTAs; k_tri_solve beyond): tile row i belongs to CTA i mod CS
+// of the cluster's CS CTAs.  Forward, the owner of row k finishes t_k = r_k - sum_j L_kj y_j, forms y_k = D_k^-1 t_k and
+// sends it to every CTA with asynchronous stores counted by that CTA's mbarrier of step k; whoever has y_k subtracts
+// L_ik y_k from its rows i > k, row k + 1 first, whose owner then goes on to y_k+1 before its other rows.  The
+// backward pass is the same on reversed indices with L_ki^T and D_k^-T.  A step's chain is two 64 x 64 products by
+// 256 threads and one remote store: about 0.5 us, against 2.4 us with a cluster barrier, a gather of the partial
+// products from all CTAs and five block barriers per step.  Nothing depends on a tile's address on the vector, so
+// each thread keeps its elements of the next NB tiles in registers (loads in flight while it waits for y_k).
+// NB = 4 tiles of the FP32 factor (64 registers; 3 and 4 alike at 15 tile rows, 4 better beyond, 5 spills).
+// Solve stage with one refinement step, before (k_tri_solve, one residual CTA per tile row) -> now: 12 clusters of 83
+// cameras 180 -> 73 us, 10 of 100 194 -> 77, 13 uneven of up to 297 753 -> 290, one of 400 1053 -> 317, 67 of 90
+// 350 -> 202; FP64, 4 clusters of 94 387 -> 220.
+template <typename F, int T> struct PushLayout {
+  static constexpr int V = 16 / (int)sizeof(F);          // elements per 16-byte load
+  static constexpr int PARTS = 256 / T;                  // row products: threads per row
+  static constexpr int NL = T * T / 256 / V;             // 16-byte loads of a tile per thread
+  static constexpr int CG = T / V, RPN = 256 / CG;       // column products: column groups, row parts of NL rows
+  static constexpr int NB = NL == 1 ? 6 : 4;             // tiles in registers or in flight per thread
+  static size_t bytes(int nt, int cs) {
+    const int slots = (nt + cs - 1) / cs;
+    return 16 * (size_t)nt + sizeof(F) * ((size_t)nt * T + (size_t)slots * (T + 256 * V) + 9 * (size_t)T) + 16;
+  }
+};
+constexpr int PUSH_MAX_POLLS = 1 << 22;
+
+template <typename F, int N>
+__device__ __forceinline__ void load16s(const F* p, F* v) {   // one 16-byte load (N = 4 floats or 2 doubles)
+  if constexpr (sizeof(F) == 4) {
+    const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+    v[0] = t.x;
+    v[1] = t.y;
+    v[2] = t.z;
+    v[3] = t.w;
+  } else {
+    const double2 t = __ldg(reinterpret_cast<const double2*>(p));
+    v[0] = t.x;
+    v[1] = t.y;
+  }
+}
+
+template <typename F, int T, typename Rreal, int CS>
+__global__ void __launch_bounds__(256, T == 64 ? 2 : 3) k_tri_push(DevProblem P, const F* __restrict__ L, const F* __restrict__ Dinv,
+                                                     const double* __restrict__ scale, const Rreal* __restrict__ rhs,
+                                                     double* x, double* rcopy, int accumulate, int64_t v_total,
+                                                     int max_nt, int* fail_flags) {
+  namespace cg = cooperative_groups;
+  using PL = PushLayout<F, T>;
+  constexpr int V = PL::V, PARTS = PL::PARTS, NL = PL::NL, CG = PL::CG, NB = PL::NB;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank();
+  const int k = blockIdx.x / CS;
+  if (P.sharded && !P.cluster_owned[k]) return;   // the whole thread-block cluster leaves, before any barrier
+  const int np = P.cluster_np[k], nt = np / T;
+  const F* A = L + P.S_off[k];
+  const F* Di = Dinv + (size_t)P.v_off[k] * T;
+  const F* DiT = Di + v_total * T;
+  const double* sk = scale + P.v_off[k];
+  const Rreal* rk = rhs + P.v_off[k];
+  double* xk = x + P.v_off[k];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int slots = (max_nt + CS - 1) / CS;
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(smem_raw);        // [2][max_nt]: y_k, then x_k, has arrived
+  F* vec = reinterpret_cast<F*>(smem_raw + 16 * (size_t)max_nt);   // [max_nt][T] y, overwritten by x
+  F* own = vec + (size_t)max_nt * T;                               // [slots][T] r, then y, of this CTA's rows
+  F* acc = own + (size_t)slots * T;                                // [slots][256][V] per-thread sums of products
+  F* red = acc + (size_t)slots * 256 * V;                          // [8][T]
+  F* tv = red + 8 * T;                                             // [T]
+  for (int i = tid; i < 2 * nt; i += 256) {
+    const int b = i < nt ? i : max_nt + i - nt;
+    tc::mbar_init(mbar + b, 1);
+    tc::mbar_arrive_expect(mbar + b, (uint32_t)(T * sizeof(F)));
+  }
+  const int nown = rank < nt ? (nt - 1 - rank) / CS + 1 : 0;
+  for (int e = tid; e < nown * T; e += 256) {
+    const int g = (rank + CS * (e / T)) * T + e % T;
+    own[e] = (F)((double)rk[g] * sk[g]);
+    if (rcopy) rcopy[P.v_off[k] + g] = (double)rk[g];
+  }
+  for (int e = tid; e < nown * 256 * V; e += 256) acc[e] = F(0);
+  __syncthreads();
+  cluster.sync();   // every CTA's barriers are set up before the first remote store
+  const int row = tid / PARTS, part = tid - row * PARTS;   // row products
+  const int cgp = tid % CG, rp = tid / CG;                 // column products: rows rp NL ..
+  bool dead = false;
+  uint32_t rvec[(CS + PARTS - 1) / PARTS], rbar[(CS + PARTS - 1) / PARTS];   // the peers this thread sends to
+#pragma unroll
+  for (int u = 0; u < (CS + PARTS - 1) / PARTS; ++u) {
+    const uint32_t peer = (uint32_t)min(part + PARTS * u, CS - 1);
+    rvec[u] = tc::map_rank(tc::smem_u32(vec), peer);
+    rbar[u] = tc::map_rank(tc::smem_u32(mbar), peer);
+  }
+  // one pass; indices i of the pass run upwards: the tile row i (forward) or nt - 1 - i (backward)
+  auto pass = [&](auto fwd_c) {
+    constexpr bool FWD = decltype(fwd_c)::value;
+    const int me = FWD ? rank : ((nt - 1 - rank) % CS + CS) % CS;   // this CTA's pass indices are me mod CS
+    if (nown == 0) return;
+    const int last = me + CS * ((nt - 1 - me) / CS);
+    // tasks: update of index i by the vector piece of index kk (i > kk), or the diagonal product of index i (diag)
+    struct Task {
+      int i, kk;
+      bool diag, end;
+    };
+    auto first_of = [&](int kk) {   // the first task of step kk
+      Task t{0, kk, false, kk >= last};
+      const int d = ((me - (kk + 1)) % CS + CS) % CS;
+      t.i = kk + 1 + d;
+      return t;
+    };
+    auto next = [&](const Task& t) {
+      if (t.end) return t;
+      if (!t.diag && t.i == t.kk + 1) return Task{t.i, t.kk, true, false};
+      if (t.diag && t.kk < 0) return first_of(0);
+      return t.i + CS < nt ? Task{t.i + CS, t.kk, false, false} : first_of(t.kk + 1);
+    };
+    auto at = [&](int i) { return FWD ? i : nt - 1 - i; };
+    auto fetch = [&](const Task& t, F (&b)[NL * V]) {
+      if (t.end) return;
+      if (t.diag || FWD) {
+        const F* src = t.diag ? (FWD ? Di : DiT) + (size_t)at(t.i) * T * T + (size_t)row * T
+                              : A + (size_t)(at(t.i) * T + row) * np + at(t.kk) * T;
+#pragma unroll
+        for (int u = 0; u < NL; ++u) load16s<F, V>(src + V * (part + PARTS * u), b + V * u);
+      } else {
+        const F* src = A + (size_t)(at(t.kk) * T + rp * NL) * np + at(t.i) * T + V * cgp;
+#pragma unroll
+        for (int u = 0; u < NL; ++u) load16s<F, V>(src + (size_t)u * np, b + V * u);
+      }
+    };
+    auto row_dot = [&](const F (&cur)[NL * V], const F* v) {   // this thread's part of its row's product with v
+      F s = F(0);
+#pragma unroll
+      for (int u = 0; u < NL; ++u)
+#pragma unroll
+        for (int e = 0; e < V; ++e) s += cur[V * u + e] * v[V * (part + PARTS * u) + e];
+      return s;
+    };
+    auto row_sum = [&](F s) {   // over the threads of a row
+#pragma unroll
+      for (int d = PARTS / 2; d > 0; d >>= 1) s += __shfl_xor_sync(FULL_MASK, s, d);
+      return s;
+    };
+    // the tiles of the next NB tasks, in flight or in registers; buffer b serves tasks b, b + NB, ..
+    F buf[NB][NL * V];
+    Task tk[NB];
+    tk[0] = me == 0 ? Task{0, -1, true, false} : first_of(0);
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      if (b > 0) tk[b] = next(tk[b - 1]);
+#pragma unroll
+      for (int u = 0; u < NL * V; ++u) buf[b][u] = F(0);
+      fetch(tk[b], buf[b]);
+    }
+    Task tn = next(tk[NB - 1]);
+    int have = -1;   // the last step whose piece has arrived
+    auto work = [&](const Task& t0, const F (&cur)[NL * V]) {
+      const int slot = (at(t0.i) - rank) / CS;
+      if (t0.diag) {
+        F t;
+        if constexpr (FWD) {
+          t = own[slot * T + row] - row_sum(acc[(slot * 256 + tid) * V]);
+          if (part == 0) tv[row] = t;
+        } else {
+          F a[V];
+#pragma unroll
+          for (int e = 0; e < V; ++e) a[e] = acc[(slot * 256 + tid) * V + e];
+#pragma unroll
+          for (int d = CG; d < 32; d <<= 1)
+#pragma unroll
+            for (int e = 0; e < V; ++e) a[e] += __shfl_xor_sync(FULL_MASK, a[e], d);
+          if (lane < CG) {
+#pragma unroll
+            for (int e = 0; e < V; ++e) red[warp * T + V * cgp + e] = a[e];
+          }
+          __syncthreads();
+          if (tid < T) {
+            F s = F(0);
+#pragma unroll
+            for (int w = 0; w < 8; ++w) s += red[w * T + tid];
+            tv[tid] = own[slot * T + tid] - s;
+          }
+        }
+        __syncthreads();
+        const F y = row_sum(row_dot(cur, tv));
+        const int g = at(t0.i) * T + row;
+#pragma unroll
+        for (int u = 0; u < (CS + PARTS - 1) / PARTS; ++u)
+          if (part + PARTS * u < CS)
+            tc::st_async(rvec[u] + (uint32_t)(g * sizeof(F)), y, rbar[u] + (uint32_t)(8 * ((FWD ? 0 : max_nt) + at(t0.i))));
+        if (part == 0) {
+          if constexpr (FWD) {
+            own[slot * T + row] = y;
+          } else {
+            const double v = (double)y * sk[g];
+            xk[g] = accumulate ? xk[g] + v : v;
+          }
+        }
+      } else {
+        if (t0.kk > have) {
+          if (!dead) dead = !tc::mbar_wait_bounded(mbar + (FWD ? 0 : max_nt) + at(t0.kk), 0, PUSH_MAX_POLLS);
+          have = t0.kk;
+        }
+        const F* v = vec + (size_t)at(t0.kk) * T;
+        F* a = acc + (size_t)(slot * 256 + tid) * V;
+        if constexpr (FWD) {
+          a[0] += row_dot(cur, v);
+        } else {
+          F s[V];
+#pragma unroll
+          for (int e = 0; e < V; ++e) s[e] = a[e];
+#pragma unroll
+          for (int u = 0; u < NL; ++u) {
+            const F xv = v[rp * NL + u];
+#pragma unroll
+            for (int e = 0; e < V; ++e) s[e] += cur[V * u + e] * xv;
+          }
+#pragma unroll
+          for (int e = 0; e < V; ++e) a[e] = s[e];
+        }
+      }
+    };
+    for (bool more = true; more;) {
+#pragma unroll
+      for (int b = 0; b < NB; ++b) {
+        if (tk[b].end) {
+          more = false;
+          break;
+        }
+        work(tk[b], buf[b]);
+        tk[b] = tn;
+        fetch(tn, buf[b]);
+        tn = next(tn);
+      }
+    }
+  };
+  pass(std::true_type{});
+  __syncthreads();   // y of this CTA's rows, before the backward pass reads it
+  for (int e = tid; e < nown * 256 * V; e += 256) acc[e] = F(0);   // thread-private up to the reductions, but indexed by
+  __syncthreads();                                                 // another layout here
+  pass(std::false_type{});
+  if (dead) atomicExch(fail_flags + k, 1);   // a piece never came: the step is rejected
+  cluster.sync();   // no CTA leaves while a peer may still store into it
+}
+
 // Device figures, read by configure_solve_kernels.
 static int g_num_sms = 0, g_smem_optin = 0;
 
@@ -1600,14 +1847,14 @@ int solve_stages(int l, int max_np, int cs) {
   return one_wave && solve_cta_bytes<F, T>(3, max_np) <= (size_t)g_smem_optin ? 3 : 2;
 }
 
+// r = rhs copied to rcopy (unless null) along the way
 template <typename F, int T, typename Rreal>
 void launch_tri_solve(const DevProblem& P, const F* L, const F* Dinv, const double* scale, const Rreal* rhs,
-                      double* x, int accumulate, int max_np, int64_t v_total, int cs, cudaStream_t stream) {
+                      double* x, double* rcopy, int accumulate, int max_np, int64_t v_total, int cs, int* fail_flags,
+                      cudaStream_t stream) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(P.l * cs);
   cfg.blockDim = dim3(256);
-  const int nst = solve_stages<F, T>(P.l, max_np, cs);
-  cfg.dynamicSmemBytes = nst * SolveLayout<F, T>::stage_bytes + sizeof(F) * (size_t)max_np;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1616,16 +1863,24 @@ void launch_tri_solve(const DevProblem& P, const F* L, const F* Dinv, const doub
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cs == 2)
-    cudaLaunchKernelEx(&cfg, k_tri_solve<F, T, Rreal, 2>, P, L, Dinv, scale, rhs, x, accumulate, v_total, nst);
-  else if (cs == 4)
-    cudaLaunchKernelEx(&cfg, k_tri_solve<F, T, Rreal, 4>, P, L, Dinv, scale, rhs, x, accumulate, v_total, nst);
-  else
-    cudaLaunchKernelEx(&cfg, k_tri_solve<F, T, Rreal, 8>, P, L, Dinv, scale, rhs, x, accumulate, v_total, nst);
+  const int max_nt = max_np / T;
+  const size_t push = PushLayout<F, T>::bytes(max_nt, cs);
+  if (push <= (size_t)g_smem_optin) {
+    cfg.dynamicSmemBytes = push;
+    auto* kern = cs == 2 ? k_tri_push<F, T, Rreal, 2> : cs == 4 ? k_tri_push<F, T, Rreal, 4> : k_tri_push<F, T, Rreal, 8>;
+    cudaLaunchKernelEx(&cfg, kern, P, L, Dinv, scale, rhs, x, rcopy, accumulate, v_total, max_nt, fail_flags);
+    return;
+  }
+  // clusters too large for the accumulators
+  if (rcopy) cudaMemcpyAsync(rcopy, rhs, (size_t)v_total * sizeof(double), cudaMemcpyDeviceToDevice, stream);
+  const int nst = solve_stages<F, T>(P.l, max_np, cs);
+  cfg.dynamicSmemBytes = nst * SolveLayout<F, T>::stage_bytes + sizeof(F) * (size_t)max_np;
+  auto* kern = cs == 2 ? k_tri_solve<F, T, Rreal, 2> : cs == 4 ? k_tri_solve<F, T, Rreal, 4> : k_tri_solve<F, T, Rreal, 8>;
+  cudaLaunchKernelEx(&cfg, kern, P, L, Dinv, scale, rhs, x, accumulate, v_total, nst);
 }
 
 // r = b - S x (FP64) with S symmetric, lower triangle stored; r was set to b before.  One CTA per
-// (cluster, 32-row tile row I); its 4 warps take the tiles (I, J), J <= I, in turn.  A warp stages the
+// (cluster, 32-row tile row I, RES_TILES of its tiles); its 4 warps take the tiles (I, J), J <= I, in turn.  A warp stages the
 // 32 x 32 tile in shared memory with coalesced row loads, then lane l forms both the row sum of tile row l
 // (S_IJ x_J, kept in registers over the warp's tiles) and the column sum of tile column l (S_IJ^T x_I,
 // added atomically to r_J; on the diagonal tile only below the diagonal).
@@ -1639,7 +1894,7 @@ __global__ void __launch_bounds__(32 * RES_WARPS) k_residual(DevProblem P, const
   __shared__ double xi[32];
   __shared__ double red[RES_WARPS][32];
   const int2 it = items[blockIdx.x];
-  const int k = it.x, I = it.y;
+  const int k = it.x, I = it.y & 0xffff, J0 = RES_TILES * (it.y >> 16);
   const int np = P.cluster_np[k], nk = P.cluster_n[k];
   const Sreal* Sk = S + P.S_off[k];
   const double* xk = x + P.v_off[k];
@@ -1649,7 +1904,8 @@ __global__ void __launch_bounds__(32 * RES_WARPS) k_residual(DevProblem P, const
   if (warp == 0) xi[lane] = (i0 + lane < nk) ? xk[i0 + lane] : 0.0;
   __syncthreads();
   double rowacc = 0.0;
-  for (int J = warp; J <= I; J += RES_WARPS) {
+  const int J1 = min(I, J0 + RES_TILES - 1);
+  for (int J = J0 + warp; J <= J1; J += RES_WARPS) {
     const int j0 = 32 * J;
     const int col = j0 + lane;
     for (int rr = 0; rr < 32; ++rr) {
@@ -1679,12 +1935,6 @@ __global__ void __launch_bounds__(32 * RES_WARPS) k_residual(DevProblem P, const
     for (int w = 0; w < RES_WARPS; ++w) t += red[w][lane];
     if (i0 + lane < nk) atomicAdd(rk + i0 + lane, -t);
   }
-}
-
-template <typename Rreal>
-__global__ void k_copy_vec(const Rreal* src, double* dst, int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    dst[i] = (double)src[i];
 }
 
 // sharded: another process's clusters scatter zeros (their steps arrive by the exchange of dc)
@@ -1866,14 +2116,13 @@ void launch_solve_t(const DevProblem& P, const double* S, const double* b, const
   using Sreal = double;
   const F* L = reinterpret_cast<const F*>(fb.L);
   const F* Dinv = reinterpret_cast<const F*>(fb.Dinv);
-  launch_tri_solve<F, T, Sreal>(P, L, Dinv, fb.scale, b, fb.x, 0, plan.max_np, fb.v_total, plan.solve_cs, stream);
-  const int nblk = (int)std::min<int64_t>(fb.v_total / 256 + 1, (int64_t)num_sms() * 8);
-  for (int s = 0; s < refine_steps; ++s) {
-    k_copy_vec<Sreal><<<nblk, 256, 0, stream>>>(b, fb.r, fb.v_total);
+  for (int s = 0; s <= refine_steps; ++s) {   // x = S~^-1 b, then x += S~^-1 (b - S x)
+    launch_tri_solve<F, T, Sreal>(P, L, Dinv, fb.scale, s ? fb.r : b, fb.x, s < refine_steps && s == 0 ? fb.r : nullptr,
+                                  s > 0, plan.max_np, fb.v_total, plan.solve_cs, fb.fail_flags, stream);
+    if (s == refine_steps) break;
+    if (s > 0) cudaMemcpyAsync(fb.r, b, (size_t)fb.v_total * sizeof(double), cudaMemcpyDeviceToDevice, stream);
     if (plan.n_res_items > 0)
       k_residual<Sreal><<<plan.n_res_items, 32 * RES_WARPS, 0, stream>>>(P, S, fb.x, fb.r, plan.res_items);
-    launch_tri_solve<F, T, double>(P, L, Dinv, fb.scale, fb.r, fb.x, 1, plan.max_np, fb.v_total, plan.solve_cs,
-                                   stream);
   }
   k_scatter_dc<<<P.l, 256, 0, stream>>>(P, fb.x, dc);
 }
@@ -1882,19 +2131,19 @@ void launch_solve_t(const DevProblem& P, const double* S, const double* b, const
 template <typename F>
 void launch_factor(const DevProblem& P, const double* S, const FactorBuffers& fb, const CholPlan& plan,
                    cudaStream_t stream) {
-  if (sizeof(F) == 4 && plan.tile == 64)
-    launch_factor_t<F, 64>(P, S, fb, plan, stream);
-  else
-    launch_factor_t<F, 32>(P, S, fb, plan, stream);
+  if constexpr (sizeof(F) == 4) {
+    if (plan.tile == 64) return launch_factor_t<F, 64>(P, S, fb, plan, stream);
+  }
+  launch_factor_t<F, 32>(P, S, fb, plan, stream);
 }
 
 template <typename F>
 void launch_solve(const DevProblem& P, const double* S, const double* b, const FactorBuffers& fb,
                   const CholPlan& plan, int refine_steps, double* dc, cudaStream_t stream) {
-  if (sizeof(F) == 4 && plan.tile == 64)
-    launch_solve_t<F, 64>(P, S, b, fb, plan, refine_steps, dc, stream);
-  else
-    launch_solve_t<F, 32>(P, S, b, fb, plan, refine_steps, dc, stream);
+  if constexpr (sizeof(F) == 4) {
+    if (plan.tile == 64) return launch_solve_t<F, 64>(P, S, b, fb, plan, refine_steps, dc, stream);
+  }
+  launch_solve_t<F, 32>(P, S, b, fb, plan, refine_steps, dc, stream);
 }
 
 size_t solve_smem_bytes(bool mixed, int tile, int max_np) {   // with the smallest stage count
@@ -1951,6 +2200,20 @@ void configure_solve_kernels(int max_np) {
                   sizeof(float) * max_np;
   const int d32 = stages(solve_cta_bytes<double, 32>(3, max_np)) * SolveLayout<double, 32>::stage_bytes +
                   sizeof(double) * max_np;
+  auto push = [&](auto* kern, size_t bytes) {
+    if (bytes <= (size_t)optin) raise_smem_attr((const void*)kern, (int)bytes);
+  };
+#define PUSH_ATTR(F, T, CS) push(k_tri_push<F, T, double, CS>, PushLayout<F, T>::bytes(max_np / T, CS))
+  PUSH_ATTR(float, 64, 2);
+  PUSH_ATTR(float, 64, 4);
+  PUSH_ATTR(float, 64, 8);
+  PUSH_ATTR(float, 32, 2);
+  PUSH_ATTR(float, 32, 4);
+  PUSH_ATTR(float, 32, 8);
+  PUSH_ATTR(double, 32, 2);
+  PUSH_ATTR(double, 32, 4);
+  PUSH_ATTR(double, 32, 8);
+#undef PUSH_ATTR
   raise_smem_attr((const void*)k_tri_solve<float, 64, double, 8>, f64);
   raise_smem_attr((const void*)k_tri_solve<float, 32, double, 8>, f32);
   raise_smem_attr((const void*)k_tri_solve<double, 32, double, 8>, d32);

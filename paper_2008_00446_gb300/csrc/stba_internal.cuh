@@ -256,10 +256,13 @@ int num_sms();
 size_t solve_smem_bytes(bool mixed, int tile, int max_np);
 
 // Cholesky (stba_chol.cu)
+// 32 x 32 tiles per CTA of the refinement residual: a whole tile row per CTA left the last rows' CTAs running alone
+// (solve stage with 4 / 8 / 16 tiles: 12 clusters of 83 cameras 79 / 73 / 81 us, one of 400 321 / 317 / 321)
+constexpr int RES_TILES = 8;
 struct CholPlan {
   const int2* panel_items;   // (cluster, tile row i) for every step, concatenated
   const int2* update_items;  // (cluster, (i << 16) | j) for every step, concatenated
-  const int2* res_items;     // (cluster, 32-row block) of the refinement residual
+  const int2* res_items;     // (cluster, 32-row block | (its RES_TILES tiles' index << 16)) of the refinement residual
   int n_res_items;
   const int2* diag_items;    // (cluster, diagonal tile) for the inverses of the diagonal tiles
   int n_diag_items;

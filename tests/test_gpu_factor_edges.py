@@ -35,3 +35,29 @@ def test_cluster_steps_at_tile_edges(sizes, update):
             x = np.linalg.solve(S, b)
             e = rows(dc[cl == k].ravel(), x, 9)
             assert e < 1e-6, (k, sizes[k], e)
+
+
+@pytest.mark.parametrize("m", [650, 680])
+def test_solve_at_the_shared_memory_limit(m):
+    """One cluster solved by two CTAs: 92 tile rows, the most whose accumulators the data-flow solve holds, and 96,
+    which take the solve with cluster barriers.  Backward error below 1e-8: the FP32 solution's is about 1e-6 at
+    worst (6000 unknowns, 6e-8 per rounding), and the FP64 refinement step multiplies it by the FP32 factor's own
+    relative error, below 1e-2 here."""
+    rng = np.random.default_rng(m)
+    base = scenes.make_tiny_scene(m=m, n=200, seed=3, drop=0.97)
+    n = 4 * m                                        # every point seen by 4 cameras of a window around it
+    oc = np.sort((np.arange(n)[:, None] * m // n + rng.permuted(np.tile(np.arange(8), (n, 1)), axis=1)[:, :4]) % m, 1)
+    op = np.repeat(np.arange(n), 4).astype(np.int32)
+    oc = oc.ravel().astype(np.int32)
+    pts = rng.uniform(-0.3, 0.3, (n, 3))
+    from oracle import camera as ocam
+    uv = ocam.residuals(base.cameras_true, pts, oc, op, np.zeros((len(oc), 2))) + rng.normal(0, 1, (len(oc), 2))
+    with stba.stba_create(base.cameras, pts, oc, op, uv, np.zeros(m, np.int32), lambda0=0.09,
+                          precision=stba.STBA_MIXED, solve_cluster=2) as ctx:
+        info = stba.stba_lm_iteration(ctx)
+        assert info["failed_clusters"] == 0
+        dc, _ = stba.stba_last_step(ctx)
+        S, b = stba.stba_get_cluster_system(ctx, 0)
+    x = dc.ravel()
+    e = np.abs(S @ x - b).max() / (np.abs(S) @ np.abs(x) + np.abs(b)).max()
+    assert e < 1e-8, e
