@@ -97,7 +97,7 @@ struct stba_ctx {
   int *key = nullptr, *tile_sum = nullptr;
   long long* counts = nullptr;
   // buffers sized by the cluster layout, kept while the next layout fits
-  GrowBuf g_panel, g_update, g_res, g_diag, g_S, g_b, g_L, g_Dinv, g_Ldiag, g_scale, g_x, g_r, g_blob;
+  GrowBuf g_panel, g_update, g_res, g_diag, g_S, g_b, g_L, g_Dinv, g_Ldiag, g_split, g_scale, g_x, g_r, g_blob;
   // pinned staging of the per-assignment arrays (two, used in turn; an event marks each one's copy)
   void* stage_h[2] = {nullptr, nullptr};
   size_t stage_bytes[2] = {0, 0};
@@ -678,6 +678,8 @@ stba_status set_clusters_host(stba_ctx* c, const std::vector<int>& cl) {
     if ((s = ensure(c, c->g_L, &L_, (size_t)c->S_total * rs)) != STBA_OK) return s;
     if ((s = ensure(c, c->g_Dinv, &Dinv_, 2 * (size_t)c->v_total * TF * rs)) != STBA_OK) return s;
     if ((s = ensure(c, c->g_Ldiag, &Ldiag_, (size_t)c->v_total * TF * rs)) != STBA_OK) return s;
+    c->fbuf.split = nullptr;
+    if (c->update_tc && (s = ensure(c, c->g_split, &c->fbuf.split, 2 * 128 * (size_t)c->v_total)) != STBA_OK) return s;
     if ((s = ensure(c, c->g_scale, &c->fbuf.scale, (size_t)c->v_total)) != STBA_OK) return s;
     if ((s = ensure(c, c->g_x, &c->fbuf.x, (size_t)c->v_total)) != STBA_OK) return s;
     if ((s = ensure(c, c->g_r, &c->fbuf.r, (size_t)c->v_total)) != STBA_OK) return s;
@@ -1352,7 +1354,7 @@ void stba_destroy(stba_ctx* c) {
   free_list(c, c->allocs);
   free_list(c, c->tape_allocs);
   for (GrowBuf* g : {&c->g_panel, &c->g_update, &c->g_res, &c->g_diag, &c->g_S, &c->g_b, &c->g_L, &c->g_Dinv,
-                     &c->g_Ldiag, &c->g_scale, &c->g_x, &c->g_r, &c->g_blob})
+                     &c->g_Ldiag, &c->g_split, &c->g_scale, &c->g_x, &c->g_r, &c->g_blob})
     if (g->ptr) cudaFree(g->ptr);
   for (int i = 0; i < 2; ++i) {
     if (c->stage_h[i]) cudaFreeHost(c->stage_h[i]);
@@ -2003,7 +2005,7 @@ stba_status stba_problem_info(stba_ctx* c, int64_t* out, int32_t n) {
   }
   size_t grown = 0;
   for (const GrowBuf* g : {&c->g_panel, &c->g_update, &c->g_res, &c->g_diag, &c->g_S, &c->g_b, &c->g_L, &c->g_Dinv,
-                           &c->g_Ldiag, &c->g_scale, &c->g_x, &c->g_r, &c->g_blob})
+                           &c->g_Ldiag, &c->g_split, &c->g_scale, &c->g_x, &c->g_r, &c->g_blob})
     grown += g->bytes;
   const int64_t vals[12] = {c->m, c->n, c->q, c->l, c->nv, maxn, (int64_t)(c->bytes_base + grown),
                             c->build_items, c->launches_per_iter, c->n_pairs, (int64_t)c->factor_flops,

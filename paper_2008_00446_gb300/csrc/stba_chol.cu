@@ -726,14 +726,16 @@ __global__ void __launch_bounds__(256) k_chol_update(F* L, DevProblem P, const i
 // one 128 x 64 x 64 product D = A B^T by tcgen05.mma (kind::tf32, FP32 accumulation in tensor memory).
 // FP32 accuracy from TF32 operands: every value x is split into hi = tf32(x) and lo = tf32(x - hi), and
 // D = A_hi B_lo + A_lo B_hi + A_hi B_hi (3xTF32; the dropped A_lo B_lo is below FP32 rounding), 24 MMAs
-// of K = 8 issued by one thread.  The operands are converted by all threads into the no-swizzle K-major
-// core-matrix layout (stba_tc.cuh); the product goes from TMEM through shared memory, so that the updated values are
-// read and written 256 contiguous bytes per row.  The wait for
-// the MMAs is bounded: a CTA that gives up marks the cluster failed (the LM step is rejected), frees its
-// tensor memory and returns.  When i0 + 1 is past the cluster's last tile, the second half of A is zero and
+// of K = 8 issued by one thread.  The split operands were written by the panel that made the column, in the no-swizzle
+// K-major core-matrix layout (stba_tc.cuh), 32 KB per tile, so that six bulk copies bring them in and no thread
+// converts anything; the product goes from TMEM through shared memory, so that the updated values are
+// read and written 256 contiguous bytes per row.  The waits for the copies and
+// the MMAs are bounded: a CTA that gives up marks the cluster failed (the LM step is rejected), frees its
+// tensor memory and returns.  When i0 + 1 is past the cluster's last tile, the second half of A is undefined and
 // its rows are not written.
-// Bound by its loads and the read-modify-write of the updated tiles (one row per lane and 16 bytes per access, as
-// before, took 71 % of the L1 pipe and 20 us for 400 tile pairs).
+// Bound by L2 traffic (96 KB of operands, 64 KB of updated values per tile pair).  With operands loaded, split and
+// stored by the threads the factorisation stage took 1194 us instead of 922 (13 uneven clusters), 853 instead of 707
+// (one of 400 cameras); with one row per lane and 16 bytes per access on top, the L1 pipe was 71 % busy.
 constexpr int TCU_THREADS = 256;
 constexpr size_t TCU_SMEM = sizeof(uint32_t) * (2 * 128 * 64 + 2 * 64 * 64);   // A hi/lo, B hi/lo: 96 KB
 constexpr int TCU_MAX_POLLS = 1 << 26;
@@ -752,6 +754,12 @@ struct TileTask {
   int64_t S_off, v_off;
 };
 
+// A step CTA's barriers (operands loaded, MMAs done) and tensor memory.
+struct StepShared {
+  uint64_t mbar_load, mbar;
+  uint32_t taddr;
+};
+
 // Four values of row `row`, columns col .. col + 3 of cluster k's scaled matrix, from the FP64 S' (the first touch of a
 // tile reads S' itself: no scaled copy is made for the tensor-core factorisation).
 __device__ __forceinline__ float4 scaled4(const double* __restrict__ Sk, const double* __restrict__ sk, int np, int row,
@@ -764,90 +772,74 @@ __device__ __forceinline__ float4 scaled4(const double* __restrict__ Sk, const d
 }
 
 // FIRST: step 0, whose old values come from S' (every tile this kernel ever updates is in its list there).
+// The split operands of a tile column: hi and lo parts of every tile, in the core-matrix layout, SPLIT_TILE words per
+// tile at its row offset; written by the panel that makes the column, read by the next launch (two columns in turn).
+constexpr int SPLIT_TILE = 2 * 64 * 64;
+__device__ __forceinline__ uint32_t* split_tile(uint32_t* split, int64_t v_total, int64_t v_off, int tile, int kt) {
+  return split + (size_t)(kt & 1) * v_total * 128 + (size_t)(v_off + tile * 64) * 128;
+}
+
 template <bool FIRST>
-__device__ __forceinline__ void update_pair_tc(uint32_t* tsm, float* L, const double* __restrict__ S,
-                                               const double* __restrict__ scale, const TileTask& task, int kt,
-                                               int* fail_flags) {
+__device__ __forceinline__ void update_pair_tc(uint32_t* tsm, StepShared& hs, float* L, uint32_t* split,
+                                               const double* __restrict__ S, const double* __restrict__ scale,
+                                               const TileTask& task, int kt, int* fail_flags, int64_t v_total) {
   constexpr int T = 64, LDS_ = 68;   // staging rows of the product: 16-byte aligned, no bank conflicts
   uint32_t* Ah = tsm;   // 128 x 64 TF32, core-matrix layout
   uint32_t* Al = tsm + 128 * 64;
   uint32_t* Bh = tsm + 2 * 128 * 64;   // 64 x 64
   uint32_t* Bl = Bh + 64 * 64;
   float* stage = reinterpret_cast<float*>(tsm);   // over A, once the MMAs are done
-  __shared__ __align__(8) uint64_t mbar;
-  __shared__ uint32_t taddr_s;
   const int k = task.k, i0 = task.tile >> 16, j = task.tile & 0xffff;
   const int np = task.np;
-  float* A = L + task.S_off;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rows_valid = min(128, np - i0 * T);   // 64 or 128
-  const float* srcA = A + (size_t)(i0 * T) * np + kt * T;
-  const float* srcB = A + (size_t)(j * T) * np + kt * T;
-  // 16-byte chunk q = tid + 256 u: row (q >> 7) * 8 + (q & 7), columns 4 ((q >> 3) & 15) ..: the 8 threads of a
-  // shared-memory store phase write one whole core matrix (no bank conflicts).  The updated values: 16 lanes per row
-  // (256 contiguous bytes), rows 16 v + tid / 16.  Every load of the thread (its 12 operand chunks and, but for step
-  // 0, the 32 old values it will update) is issued before any of them is used.
-  const int r16 = tid >> 4, c4 = 4 * (tid & 15);
-  float* dst = A + (size_t)(i0 * T + r16) * np + j * T + c4;
-  float4 va[8], vb[4], old[8];
-#pragma unroll
-  for (int u = 0; u < 8; ++u) {
-    const int q = tid + TCU_THREADS * u;
-    const int r = ((q >> 7) << 3) | (q & 7), kc = (q >> 3) & 15;
-    va[u] = r < rows_valid ? *reinterpret_cast<const float4*>(srcA + (size_t)r * np + 4 * kc)
-                           : make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int q = tid + TCU_THREADS * u;
-    const int r = ((q >> 7) << 3) | (q & 7), kc = (q >> 3) & 15;
-    vb[u] = *reinterpret_cast<const float4*>(srcB + (size_t)r * np + 4 * kc);
-  }
-  if constexpr (!FIRST) {
-#pragma unroll
-    for (int v = 0; v < 8; ++v)
-      old[v] = 16 * v + r16 < rows_valid ? *reinterpret_cast<const float4*>(dst + (size_t)(16 * v) * np)
-                                         : make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-#pragma unroll
-  for (int u = 0; u < 8; ++u) {
-    const int q = tid + TCU_THREADS * u;
-    split_store(Ah, Al, tc::core_off<64>(((q >> 7) << 3) | (q & 7), 4 * ((q >> 3) & 15)), va[u]);
-  }
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int q = tid + TCU_THREADS * u;
-    split_store(Bh, Bl, tc::core_off<64>(((q >> 7) << 3) | (q & 7), 4 * ((q >> 3) & 15)), vb[u]);
-  }
-  tc::fence_async_smem();
-  if (tid == 0) tc::mbar_init(&mbar, 1);
-  if (warp == 0) tc::tmem_alloc(&taddr_s, 64);
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tmem = taddr_s;
+  const uint32_t tmem = hs.taddr;
+  // operands by the copy engine; the second half of A stays undefined past the last tile (its rows are not used)
   if (tid == 0) {
-    constexpr uint32_t idesc = tc::idesc_tf32(128, 64);
-    const uint32_t pa[3] = {tc::smem_u32(Ah), tc::smem_u32(Al), tc::smem_u32(Ah)};
-    const uint32_t pb[3] = {tc::smem_u32(Bl), tc::smem_u32(Bh), tc::smem_u32(Bh)};
+    const bool two = rows_valid == 128;
+    tc::fence_async_all();
+    tc::mbar_arrive_expect(&hs.mbar_load, (two ? 6u : 4u) * 16384u);
+    const uint32_t* a0 = split_tile(split, v_total, task.v_off, i0, kt);
+    const uint32_t* b = split_tile(split, v_total, task.v_off, j, kt);
+    tc::bulk_load(Ah, a0, 16384, &hs.mbar_load);
+    tc::bulk_load(Al, a0 + 4096, 16384, &hs.mbar_load);
+    tc::bulk_load(Bh, b, 16384, &hs.mbar_load);
+    tc::bulk_load(Bl, b + 4096, 16384, &hs.mbar_load);
+    if (two) {
+      tc::bulk_load(Ah + 4096, a0 + SPLIT_TILE, 16384, &hs.mbar_load);
+      tc::bulk_load(Al + 4096, a0 + SPLIT_TILE + 4096, 16384, &hs.mbar_load);
+    }
+    if (tc::mbar_wait_bounded(&hs.mbar_load, 0, TCU_MAX_POLLS)) {
+      tc::fence_after_sync();
+      constexpr uint32_t idesc = tc::idesc_tf32(128, 64);
+      const uint32_t pa[3] = {tc::smem_u32(Ah), tc::smem_u32(Al), tc::smem_u32(Ah)};
+      const uint32_t pb[3] = {tc::smem_u32(Bl), tc::smem_u32(Bh), tc::smem_u32(Bh)};
 #pragma unroll
-    for (int pass = 0; pass < 3; ++pass)
+      for (int pass = 0; pass < 3; ++pass)
 #pragma unroll
-      for (int ks = 0; ks < 8; ++ks)
-        tc::mma_tf32(tmem, tc::smem_desc(pa[pass] + ks * 256, 128, 2048), tc::smem_desc(pb[pass] + ks * 256, 128, 2048),
-                     idesc, (pass | ks) != 0);
-    tc::mma_commit(&mbar);
+        for (int ks = 0; ks < 8; ++ks)
+          tc::mma_tf32(tmem, tc::smem_desc(pa[pass] + ks * 256, 128, 2048), tc::smem_desc(pb[pass] + ks * 256, 128, 2048),
+                       idesc, (pass | ks) != 0);
+      tc::mma_commit(&hs.mbar);
+    }
   }
-  if constexpr (FIRST) {   // while the MMAs run
-    const double* Sk = S + task.S_off;
-    const double* sk = scale + task.v_off;
+  // the updated values: 16 lanes per row (256 contiguous bytes), rows 16 v + tid / 16
+  const int r16 = tid >> 4, c4 = 4 * (tid & 15);
+  float* dst = L + task.S_off + (size_t)(i0 * T + r16) * np + j * T + c4;
+  float4 old[8];
 #pragma unroll
-    for (int v = 0; v < 8; ++v)
-      old[v] = 16 * v + r16 < rows_valid ? scaled4(Sk, sk, np, i0 * T + 16 * v + r16, j * T + c4)
-                                         : make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int v = 0; v < 8; ++v) {
+    if (16 * v + r16 >= rows_valid) {
+      old[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else if constexpr (FIRST) {
+      old[v] = scaled4(S + task.S_off, scale + task.v_off, np, i0 * T + 16 * v + r16, j * T + c4);
+    } else {
+      old[v] = *reinterpret_cast<const float4*>(dst + (size_t)(16 * v) * np);
+    }
   }
+  __syncwarp();
   // thread (lane quarter warp & 3, column half warp >> 2): row R of the product, 32 columns, to the staging rows
-  const bool done = __all_sync(0xffffffffu, tc::mbar_wait_bounded(&mbar, 0, TCU_MAX_POLLS));
+  const bool done = __all_sync(0xffffffffu, tc::mbar_wait_bounded(&hs.mbar, 0, TCU_MAX_POLLS));
   if (done) {
     tc::fence_after_sync();
     float d[32];
@@ -886,8 +878,8 @@ __device__ __forceinline__ void update_pair_tc(uint32_t* tsm, float* L, const do
 // block.  A row's operands are its own smem row (16-byte loads, 68-float rows: no bank conflicts) and the diagonal
 // rows, which all lanes read at one address, so that a block moves a quarter of the shared-memory words of the
 // right-looking rank-8 updates of k_chol_panel, which bound it.
-// Panel alone on an SM: 9.6 us (loads and operands 2.5, product 0.65, sweep 5.9; k_chol_panel took 20), beside an
-// update CTA about 13.  One 512-thread CTA per SM with two tasks, so that a panel has its SM to itself, was slower
+// Panel alone on an SM: about 8.5 us (loads 1.5, product 0.65, sweep 5.9; k_chol_panel took 20), beside an
+// update CTA about 12.  Warps 5 .. 7 write each finished block out (factor, split operands, inverse).  One 512-thread CTA per SM with two tasks, so that a panel has its SM to itself, was slower
 // (12 clusters of 83 cameras 265 us against 228: an SM then waits for both tasks).
 constexpr int PTC_THREADS = 256;
 constexpr int PTC_LD = 68;
@@ -959,26 +951,32 @@ __device__ __forceinline__ float dot4(float4 a, float4 b, float s) {   // s - a.
 }
 
 // the barrier of the sweep: the four row warps and the pivot warp
-__device__ __forceinline__ void sweep_barrier() {
-  __syncwarp();
-  asm volatile("bar.sync 1, 160;\n" ::: "memory");
-}
-
-__device__ __forceinline__ void panel_tc(uint32_t* psm, float* L, float* Dinv, const double* __restrict__ S,
-                                         const double* __restrict__ scale, const TileTask& task, int kt,
-                                         int* fail_flags, int* boosted, int64_t v_total) {
+__device__ __forceinline__ void panel_tc(uint32_t* psm, StepShared& hs, float* L, float* Dinv, uint32_t* split,
+                                         const double* __restrict__ S, const double* __restrict__ scale,
+                                         const TileTask& task, int kt, int* fail_flags, int* boosted, int64_t v_total) {
   constexpr int T = 64, LD = PTC_LD, NB = T / 8;
   uint32_t* Ah = psm;   // 128 x 64 TF32, core-matrix layout: rows of L_kt,kt-1, then of L_i,kt-1
   uint32_t* Al = psm + 128 * 64;
   float* W = reinterpret_cast<float*>(psm + 2 * 128 * 64);   // [128][LD] the stacked tile
-  __shared__ __align__(8) uint64_t mbar;
-  __shared__ uint32_t taddr_s;
   __shared__ __align__(16) float rinv[8];
   const int k = task.k, i = task.tile;
   const bool diag = i == kt;
   const int np = task.np, nk = task.nk;
   float* A = L + task.S_off;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t tmem = hs.taddr;
+  if (kt > 0 && tid == 0) {   // the operands by the copy engine
+    tc::fence_async_all();
+    tc::mbar_arrive_expect(&hs.mbar_load, (diag ? 2u : 4u) * 16384u);
+    const uint32_t* a0 = split_tile(split, v_total, task.v_off, kt, kt - 1);
+    tc::bulk_load(Ah, a0, 16384, &hs.mbar_load);
+    tc::bulk_load(Al, a0 + 4096, 16384, &hs.mbar_load);
+    if (!diag) {   // else rows 64 .. stay undefined: their product is not used
+      const uint32_t* a1 = split_tile(split, v_total, task.v_off, i, kt - 1);
+      tc::bulk_load(Ah + 4096, a1, 16384, &hs.mbar_load);
+      tc::bulk_load(Al + 4096, a1 + 4096, 16384, &hs.mbar_load);
+    }
+  }
   // the stacked tile's old values: 16 lanes per row; columns 0 and 1 come from S' (no update has touched them)
   const int r16 = tid >> 4, c4 = 4 * (tid & 15);
 #pragma unroll
@@ -996,28 +994,8 @@ __device__ __forceinline__ void panel_tc(uint32_t* psm, float* L, float* Dinv, c
   }
   bool done = true;
   if (kt > 0) {
-    float4 va[8];   // chunks as in update_pair_tc
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int q = tid + PTC_THREADS * u;
-      const int r = ((q >> 7) << 3) | (q & 7), kc = (q >> 3) & 15;
-      const float* src = A + (size_t)(r < T ? kt * T + r : i * T + r - T) * np + (kt - 1) * T + 4 * kc;
-      va[u] = (r < T || !diag) ? *reinterpret_cast<const float4*>(src) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int q = tid + PTC_THREADS * u;
-      split_store(Ah, Al, tc::core_off<64>(((q >> 7) << 3) | (q & 7), 4 * ((q >> 3) & 15)), va[u]);
-    }
-    tc::fence_async_smem();
-    if (tid == 0) tc::mbar_init(&mbar, 1);
-    if (warp == 0) tc::tmem_alloc(&taddr_s, 64);
-    cp_async_wait_all();
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-    const uint32_t tmem = taddr_s;
-    if (tid == 0) {
+    if (tid == 0 && tc::mbar_wait_bounded(&hs.mbar_load, 0, TCU_MAX_POLLS)) {
+      tc::fence_after_sync();
       constexpr uint32_t idesc = tc::idesc_tf32(128, 64);
       const uint32_t pa[3] = {tc::smem_u32(Ah), tc::smem_u32(Al), tc::smem_u32(Ah)};
       const uint32_t pb[3] = {tc::smem_u32(Al), tc::smem_u32(Ah), tc::smem_u32(Ah)};   // rows 0 .. 63
@@ -1027,9 +1005,11 @@ __device__ __forceinline__ void panel_tc(uint32_t* psm, float* L, float* Dinv, c
         for (int ks = 0; ks < 8; ++ks)
           tc::mma_tf32(tmem, tc::smem_desc(pa[pass] + ks * 256, 128, 2048), tc::smem_desc(pb[pass] + ks * 256, 128, 2048),
                        idesc, (pass | ks) != 0);
-      tc::mma_commit(&mbar);
+      tc::mma_commit(&hs.mbar);
     }
-    done = __all_sync(FULL_MASK, tc::mbar_wait_bounded(&mbar, 0, TCU_MAX_POLLS));
+    cp_async_wait_all();
+    __syncthreads();   // the old values are in place
+    done = __all_sync(FULL_MASK, tc::mbar_wait_bounded(&hs.mbar, 0, TCU_MAX_POLLS));
     if (done) {
       tc::fence_after_sync();
       float d[32];
@@ -1051,18 +1031,35 @@ __device__ __forceinline__ void panel_tc(uint32_t* psm, float* L, float* Dinv, c
     tc::fence_before_sync();
   }
   const int all_done = __syncthreads_and(done);
-  if (kt > 0 && warp == 0) tc::tmem_dealloc(taddr_s, 64);
+  if (warp == 0) tc::tmem_dealloc(tmem, 64);
   if (!all_done) {   // the wait gave up: the cluster fails, the step is rejected
     if (tid == 0) atomicExch(fail_flags + k, 1);
     return;
   }
-  if (warp > 4) return;   // the sweep: row warps 0 .. 3, pivot warp 4
   float* my = W + tid * LD;   // row threads
   float x[8], nx[8], o[8];
   float* Di = Dinv + (size_t)task.v_off * T + (size_t)kt * T * T;
   float* DiT = Di + v_total * T;
-  float* Xg = nullptr;   // where this row's solved blocks go
-  if (warp == 2 || warp == 3) Xg = diag ? DiT + (tid - T) * T : A + (size_t)(i * T + tid - T) * np + kt * T;
+  uint32_t* Xs = diag ? nullptr : split_tile(split, v_total, task.v_off, i, kt);
+  float* Xg = diag ? DiT : A + (size_t)(i * T) * np + kt * T;   // where the lower rows go
+  const size_t Xld = diag ? (size_t)T : (size_t)np;
+  // warps 5 .. 7: the lower rows' solved columns n0 .. n0 + 7 from shared memory to the factor (or the inverse) and
+  // to the split operands
+  auto store_block = [&](int n0) {
+    for (int c = tid - 160; c < 128; c += 96) {
+      const int r = c & 63, col = n0 + 4 * (c >> 6);
+      const float4 v = *reinterpret_cast<const float4*>(W + (T + r) * LD + col);
+      *reinterpret_cast<float4*>(Xg + r * Xld + col) = v;
+      if (diag) {
+        Di[(col + 0) * T + r] = v.x;
+        Di[(col + 1) * T + r] = v.y;
+        Di[(col + 2) * T + r] = v.z;
+        Di[(col + 3) * T + r] = v.w;
+      } else {
+        split_store(Xs, Xs + 4096, tc::core_off<64>(r, col), v);
+      }
+    }
+  };
   auto load8 = [](const float* p, float (&v)[8]) {
     const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
     v[0] = a.x;
@@ -1099,6 +1096,8 @@ __device__ __forceinline__ void panel_tc(uint32_t* psm, float* L, float* Dinv, c
         __syncwarp();
       }
       if (lane == 0) chol8_fast(blk, kt * T + n0, nk, rinv, fail_flags + k, diag ? boosted : nullptr);
+    } else if (warp > 4) {
+      if (b > 0) store_block(n0 - 8);
     } else if (tid >= n1) {
       // block column b of this row, all terms
       if (b > 0) {
@@ -1126,7 +1125,7 @@ __device__ __forceinline__ void panel_tc(uint32_t* psm, float* L, float* Dinv, c
         }
       }
     }
-    sweep_barrier();
+    __syncthreads();
     if (warp < 4 && tid >= n1) {
       float ri[8];
       load8(rinv, ri);
@@ -1157,44 +1156,48 @@ __device__ __forceinline__ void panel_tc(uint32_t* psm, float* L, float* Dinv, c
       const float4 a = make_float4(o[0], o[1], o[2], o[3]), e = make_float4(o[4], o[5], o[6], o[7]);
       *reinterpret_cast<float4*>(my + n0) = a;
       *reinterpret_cast<float4*>(my + n0 + 4) = e;
-      if (Xg) {
-        *reinterpret_cast<float4*>(Xg + n0) = a;
-        *reinterpret_cast<float4*>(Xg + n0 + 4) = e;
-        if (diag) {
-#pragma unroll
-          for (int c = 0; c < 8; ++c) Di[(n0 + c) * T + tid - T] = o[c];
-        }
-      }
     }
-    sweep_barrier();
+    __syncthreads();
   }
+  if (warp > 4) store_block(T - 8);
 }
 
 // One launch per tile step: the CTAs of panel kt + 1 first (their chain sets the step's time), then the trailing update
 // of step kt; both read column kt, finished by the launch before.  kt = -1: panel 0 alone; FIRST: kt = 0.  The next
 // step's CTAs start under programmatic dependent launch: they read their task while this step's last CTAs finish.
 // Factorisation stage, before (panel and update launches on two streams, scaled copy, inverses of the diagonal
-// tiles) -> now: 12 clusters of 83 cameras 357 -> 212 us, 10 of 100 404 -> 243, 13 uneven of up to 297 2186 -> 1195,
-// one of 400 1560 -> 857, 67 of 90 1057 -> 797.  Of it: the panel 98 us of 357 (12 clusters), update epilogue and no
-// scaled copy 2 (13 uneven: 190 of 2186), one launch per step 28, dependent launch 16.  Panels stacked with the
+// tiles) -> now: 12 clusters of 83 cameras 357 -> 209 us, 10 of 100 404 -> 229, 13 uneven of up to 297 2186 -> 922,
+// one of 400 1560 -> 707, 67 of 90 1057 -> 681.  Of it: the panel 98 us of 357 (12 clusters), update epilogue and no
+// scaled copy 2 (13 uneven: 190 of 2186), one launch per step 28, dependent launch 16, split operands 4 (13 uneven:
+// 272).  Panels stacked with the
 // tiles below them also where they outnumber the SMs: a separate launch for the diagonal tiles (the split panel)
 // would put the update before the tiles below (67 clusters: 819 us split on two streams, 815 one launch).
 template <bool FIRST>
-__global__ void __launch_bounds__(PTC_THREADS, 2) k_step_tc(float* L, float* Dinv, const double* __restrict__ S,
+__global__ void __launch_bounds__(PTC_THREADS, 2) k_step_tc(float* L, float* Dinv, uint32_t* split,
+                                                            const double* __restrict__ S,
                                                             const double* __restrict__ scale, DevProblem P,
                                                             const int2* panels, int npanels, const int2* updates,
                                                             int kt, int* fail_flags, int* boosted, int64_t v_total) {
   extern __shared__ __align__(128) uint32_t step_smem[];
+  __shared__ __align__(16) StepShared hs;
   const bool panel = (int)blockIdx.x < npanels;
   const int2 it = panel ? panels[blockIdx.x] : updates[blockIdx.x - npanels];
   const TileTask task{it.x, it.y, P.cluster_np[it.x], P.cluster_n[it.x], P.S_off[it.x], P.v_off[it.x]};
-  // the next step's CTAs may take free SMs and read their own tasks; what the launch before wrote, from here on
+  if (threadIdx.x == 0) {
+    tc::mbar_init(&hs.mbar_load, 1);
+    tc::mbar_init(&hs.mbar, 1);
+  }
+  if (threadIdx.x < 32) tc::tmem_alloc(&hs.taddr, 64);
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  // the next step's CTAs may take free SMs and prepare as above; what the launch before wrote, from here on
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (panel)
-    panel_tc(step_smem, L, Dinv, S, scale, task, kt + 1, fail_flags, boosted, v_total);
+    panel_tc(step_smem, hs, L, Dinv, split, S, scale, task, kt + 1, fail_flags, boosted, v_total);
   else
-    update_pair_tc<FIRST>(step_smem, L, S, scale, task, kt, fail_flags);
+    update_pair_tc<FIRST>(step_smem, hs, L, split, S, scale, task, kt, fail_flags, v_total);
 }
 
 // ------------------------------------------------------------------------------------------------------
@@ -2058,7 +2061,7 @@ void launch_factor_t(const DevProblem& P, const double* S, const FactorBuffers& 
         cfg.attrs = attr;
         cfg.numAttrs = kt >= 0 ? 1 : 0;   // panel 0 follows kernels that do not signal
         cudaLaunchKernelEx(&cfg, kt == 0 ? k_step_tc<true> : k_step_tc<false>, reinterpret_cast<float*>(L),
-                           reinterpret_cast<float*>(Dinv), S, (const double*)fb.scale, P,
+                           reinterpret_cast<float*>(Dinv), fb.split, S, (const double*)fb.scale, P,
                            plan.panel_items + plan.h_panel_off[kt + 1], npn,
                            plan.update_items + (kt < 0 ? 0 : plan.h_update_off[kt]), kt, fb.fail_flags, fb.boosted,
                            fb.v_total);

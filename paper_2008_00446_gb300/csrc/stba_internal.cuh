@@ -294,6 +294,7 @@ struct FactorBuffers {
                     // their transposes follow at offset v_total * T
   void* Ldiag;      // factored diagonal tiles L_kk (same tile layout as Dinv).  Kept out of L: every CTA of a
                     // panel step reads the unfactored A_kk from L, so it must not be overwritten in place
+  uint32_t* split;  // [2][v_total][128] TF32 hi / lo operands of two tile columns (tensor-core steps), else null
   double* scale;    // [v_total] Jacobi scaling s_i = S_ii^-1/2
   double* x;        // [v_total] solution
   double* r;        // [v_total] refinement residual
