@@ -41,6 +41,8 @@ struct stba_ctx {
   stba_options opt{};
   Settings set{};
   cudaStream_t stream = nullptr;
+  cudaStream_t mark_stream = nullptr;           // the stage events of a captured iteration
+  cudaEvent_t ev_mark = nullptr;
   cudaStream_t cap_stream = nullptr;
   // re-ordering graphs of the two buffer states (argument bytes -> executable graph)
   std::vector<unsigned char> reorder_key[2];
@@ -50,6 +52,8 @@ struct stba_ctx {
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   cudaEvent_t ev_rfork = nullptr, ev_rjoin = nullptr;   // the re-ordering's side branch (chunk listing)
   cudaEvent_t ev_sfork = nullptr, ev_sjoin = nullptr;   // the S' build's side branch (pair pass)
+  cudaEvent_t ev_zfork = nullptr, ev_zjoin = nullptr;   // the zeros of S' beside the linearisation
+  cudaEvent_t ev_cfork = nullptr, ev_cjoin = nullptr;   // the cost's camera table beside the point step
   cudaEvent_t ev_copy = nullptr;                        // the factorisation's scaled copy beside panel 0
   std::vector<cudaEvent_t> ev_panel, ev_update;  // one per tile step (grown, never shrunk)
   std::string err;
@@ -582,10 +586,10 @@ stba_status set_clusters_host(stba_ctx* c, const std::vector<int>& cl) {
     for (int kt = 0; kt < max_nt; ++kt)
       factor_launches += steps ? 1 : (c->h_panel_off[kt + 1] > c->h_panel_off[kt]) + (c->h_update_off[kt + 1] > c->h_update_off[kt]);
     const int build_launches = 1 + (c->pchunks.nchunks > 0 && l < m ? 1 : 0);
-    const int solve_launches = 2 + c->set.refine_steps * (2 + (res_items.empty() ? 0 : 1));
-    // iter_begin, vp_reduce, pt_acc, vp_finalize | build | factor | solve, count | rhs, update, cam_rt,
-    // (cam_df, point_df,) cost, finalize, apply
-    c->launches_per_iter = 4 + build_launches + factor_launches + solve_launches + 1 + 6 + (c->mixed ? 3 : 0);
+    const int solve_launches = 1 + c->set.refine_steps * (1 + (res_items.empty() ? 0 : 1));
+    // begin, vp_reduce, pt_acc, vp_finalize | build | factor | solve, scatter | cost_cams, rhs, update, cost,
+    // finalize, apply
+    c->launches_per_iter = 4 + build_launches + factor_launches + solve_launches + 1 + 6;
     c->factor_flops = 0;
     for (int k = 0; k < l; ++k) c->factor_flops += std::pow((double)c->h_nk[k], 3) / 3.0;
   }
@@ -714,33 +718,83 @@ stba_status set_clusters_host(stba_ctx* c, const std::vector<int>& cl) {
 
 // ------------------------------------------------------------------------------------------------------
 void record_stage(stba_ctx* c, int i) {
-  // inside a capture the record becomes an event node of the graph, so every replay times its stages
-  cudaEventRecordWithFlags(c->ev[i], c->stream, c->capturing ? cudaEventRecordExternal : cudaEventRecordDefault);
+  // inside a capture the record becomes an event node of the graph, so every replay times its stages; on a branch
+  // of its own, as a node between two kernels would keep them a launch gap apart
+  if (!c->capturing) {
+    cudaEventRecord(c->ev[i], c->stream);
+    return;
+  }
+  cudaEventRecord(c->ev_mark, c->stream);
+  cudaStreamWaitEvent(c->mark_stream, c->ev_mark, 0);
+  cudaEventRecordWithFlags(c->ev[i], c->mark_stream, cudaEventRecordExternal);
+  if (i == NSTAGES) {
+    cudaEventRecord(c->ev_mark, c->mark_stream);
+    cudaStreamWaitEvent(c->stream, c->ev_mark, 0);
+  }
+}
+
+// What an iteration starts from; the vectors of the cluster solver when `clusters`.
+template <typename real>
+void enqueue_begin(stba_ctx* c, const DevProblem& P, const Scratch<real>& W, bool clusters, cudaStream_t s) {
+  const int64_t rw = sizeof(real) / 4;
+  ZeroList Z = {};
+  Z.p[0] = (uint32_t*)c->t_acc;
+  Z.words[0] = 3 * c->n * rw;
+  if (clusters) {
+    Z.p[1] = (uint32_t*)c->b;
+    Z.words[1] = 2 * c->v_total;
+    Z.p[2] = (uint32_t*)c->vgrad;
+    Z.words[2] = 9 * c->m * rw;
+    Z.p[3] = (uint32_t*)c->fail_flags;
+    Z.words[3] = c->fail_flags ? c->l : 0;
+  }
+  launch_begin<real>(P, W, (real*)c->ctab, c->cams_f, c->pts_f, c->st, c->set, c->counts, Z, s);
+}
+
+// The cost at x + dx, and accept / reject.  The camera table depends on dc alone: in a captured iteration it is
+// formed on a side branch beside the point step (enqueue_cost_cams before the point step, joined here).
+template <typename real>
+void enqueue_cost_cams(stba_ctx* c, const DevProblem& P) {
+  if (c->capturing) {
+    cudaEventRecord(c->ev_cfork, c->stream);
+    cudaStreamWaitEvent(c->side_stream, c->ev_cfork, 0);
+    launch_cost_cams<real>(P, c->dc, c->cam_rt, c->cam_df, c->side_stream);
+    cudaEventRecord(c->ev_cjoin, c->side_stream);
+  } else {
+    launch_cost_cams<real>(P, c->dc, c->cam_rt, c->cam_df, c->stream);
+  }
+}
+
+template <typename real>
+void enqueue_control(stba_ctx* c, const DevProblem& P) {
+  cudaStream_t s = c->stream;
+  if (c->capturing) cudaStreamWaitEvent(s, c->ev_cjoin, 0);
+  launch_cost<real>(P, c->dp, c->cam_rt, c->cam_df, c->pt_df, c->partial, c->st, (real*)c->res_cand, s);
+  launch_finalize<real>(P, c->partial, c->st, c->set, 1, s);
+  launch_apply<real>(P, c->dc, c->dp, c->cams, c->pts, (const real*)c->res_cand, (real*)c->res_cur, c->st, s);
 }
 
 // The LM step at the current parameters and c->st->lambda: S', the cluster factors, dc and dp (stages 0-3
-// and the point update of Algorithm 1).  With stages, records the stage events 0..4.
+// and the point update of Algorithm 1).  With stages, records the stage events 0..4 and forms the camera table of
+// the cost.
 template <typename real>
 void enqueue_step(stba_ctx* c, bool stages) {
   const DevProblem P = dev_problem(c);
   const Scratch<real> W = scratch<real>(c);
   cudaStream_t s = c->stream;
-  const size_t rs = sizeof(real);
   auto mark = [&](int i) {
     if (stages) record_stage(c, i);
   };
   mark(0);
-  // stage 0: linearisation and virtual points
-  launch_iter_begin<real>(c->st, c->set, s);
-  launch_params<real>(P, (real*)c->ctab, c->cams_f, c->pts_f, s);
-  launch_zero_vp(c->vp_acc, c->counts, (int)rs, s);   // 9 nv reals, nv from the device counter
-  cudaMemsetAsync(c->S, 0, (size_t)c->S_total * sizeof(double), s);
-  cudaMemsetAsync(c->b, 0, (size_t)c->v_total * sizeof(double), s);
-  cudaMemsetAsync(c->vgrad, 0, 9 * (size_t)c->m * rs, s);
-  cudaMemsetAsync(c->t_acc, 0, 3 * (size_t)c->n * rs, s);
-  cudaMemsetAsync(c->fail_flags, 0, (size_t)c->l * sizeof(int), s);
+  // stage 0: linearisation and virtual points, the zeros of S' on the side stream beside them
+  cudaEventRecord(c->ev_zfork, s);
+  cudaStreamWaitEvent(c->side_stream, c->ev_zfork, 0);
+  cudaMemsetAsync(c->S, 0, (size_t)c->S_total * sizeof(double), c->side_stream);
+  cudaEventRecord(c->ev_zjoin, c->side_stream);
+  enqueue_begin<real>(c, P, W, true, s);
   launch_vp_reduce<real>(P, W, s);
   launch_vp_finalize<real>(P, W, c->st, c->counts, s);
+  cudaStreamWaitEvent(s, c->ev_zjoin, 0);
   mark(1);
   // stage 1: S' and b'
   launch_rcs_build<real>(P, W, c->cslots, c->pchunks, (real*)c->rowbuf, c->st, s, c->side_stream, c->ev_sfork,
@@ -754,26 +808,21 @@ void enqueue_step(stba_ctx* c, bool stages) {
   mark(3);
   // stage 3: cluster solves with FP64 refinement
   if (c->f32f)
-    launch_solve<float>(P, W.S, W.b, c->fbuf, c->cplan, c->set.refine_steps, c->dc, s);
+    launch_solve<float>(P, W.S, W.b, c->fbuf, c->cplan, c->set.refine_steps, s);
   else
-    launch_solve<double>(P, W.S, W.b, c->fbuf, c->cplan, c->set.refine_steps, c->dc, s);
-  launch_count_failures(c->fail_flags, c->l, c->st, s);
+    launch_solve<double>(P, W.S, W.b, c->fbuf, c->cplan, c->set.refine_steps, s);
+  launch_scatter_step<real>(P, c->fbuf.x, c->fail_flags, c->max_np, c->st, c->dc, (real*)c->edc, s);
   mark(4);
   // stage 4: points, cost, control
-  launch_step_rows<real>(P, c->dc, (real*)c->edc, s);
+  if (stages) enqueue_cost_cams<real>(c, P);
   launch_point_rhs<real>(P, W, s);
-  launch_point_update<real>(P, W, s);
+  launch_point_update<real>(P, W, c->pt_df, s);
 }
 
 template <typename real>
 void enqueue_iteration(stba_ctx* c) {
-  const DevProblem P = dev_problem(c);
-  const Scratch<real> W = scratch<real>(c);
-  cudaStream_t s = c->stream;
   enqueue_step<real>(c, true);
-  launch_cost<real>(P, c->dc, c->dp, c->cam_rt, c->cam_df, c->pt_df, c->partial, c->st, (real*)c->res_cand, s);
-  launch_finalize<real>(P, W, c->st, c->set, 1, s);
-  launch_apply<real>(P, c->dc, c->dp, c->cams, c->pts, (const real*)c->res_cand, (real*)c->res_cur, c->st, s);
+  enqueue_control<real>(c, dev_problem(c));
   record_stage(c, 5);
 }
 
@@ -785,15 +834,8 @@ int enqueue_pcg_iteration(stba_ctx* c) {
   const Scratch<real> W = scratch<real>(c);
   cudaStream_t s = c->stream;
   record_stage(c, 0);
-  launch_iter_begin<real>(c->st, c->set, s);
-  launch_params<real>(P, (real*)c->ctab, c->cams_f, c->pts_f, s);
-  launch_zero_vp(c->vp_acc, c->counts, (int)sizeof(real), s);
-  cudaMemsetAsync(c->t_acc, 0, 3 * (size_t)c->n * sizeof(real), s);
-  if (c->use_spcg) {
-    launch_spcg_zero(P, W.S, s);
-    cudaMemsetAsync(c->b, 0, (size_t)c->v_total * sizeof(double), s);
-    cudaMemsetAsync(c->vgrad, 0, 9 * (size_t)c->m * sizeof(real), s);
-  }
+  enqueue_begin<real>(c, P, W, c->use_spcg, s);
+  if (c->use_spcg) launch_spcg_zero(P, W.S, s);
   launch_vp_reduce<real>(P, W, s);
   launch_vp_finalize<real>(P, W, c->st, c->counts, s);
   record_stage(c, 1);
@@ -807,11 +849,10 @@ int enqueue_pcg_iteration(stba_ctx* c) {
   record_stage(c, 3);
   const int iters = pcg_iterate<real>(P, W, c->cslots, c->pcg, c->opt.pcg_max_iter, c->opt.pcg_tol, c->st, s);
   record_stage(c, 4);
+  enqueue_cost_cams<real>(c, P);
   launch_point_rhs<real>(P, W, s);
-  launch_point_update<real>(P, W, s);
-  launch_cost<real>(P, c->dc, c->dp, c->cam_rt, c->cam_df, c->pt_df, c->partial, c->st, (real*)c->res_cand, s);
-  launch_finalize<real>(P, W, c->st, c->set, 1, s);
-  launch_apply<real>(P, c->dc, c->dp, c->cams, c->pts, (const real*)c->res_cand, (real*)c->res_cur, c->st, s);
+  launch_point_update<real>(P, W, c->pt_df, s);
+  enqueue_control<real>(c, P);
   record_stage(c, 5);
   return iters;
 }
@@ -819,11 +860,9 @@ int enqueue_pcg_iteration(stba_ctx* c) {
 template <typename real>
 void enqueue_cost(stba_ctx* c) {
   const DevProblem P = dev_problem(c);
-  const Scratch<real> W = scratch<real>(c);
-  launch_iter_begin<real>(c->st, c->set, c->stream);
-  launch_cost<real>(P, nullptr, nullptr, c->cam_rt, c->cam_df, c->pt_df, c->partial, c->st, (real*)c->res_cur,
-                    c->stream);
-  launch_finalize<real>(P, W, c->st, c->set, 0, c->stream);
+  launch_iter_begin(c->st, c->set, c->stream);
+  launch_cost_x<real>(P, c->cam_rt, c->cam_df, c->pt_df, c->partial, c->st, (real*)c->res_cur, c->stream);
+  launch_finalize<real>(P, c->partial, c->st, c->set, 0, c->stream);
 }
 
 stba_status run_cost(stba_ctx* c, double* F) {
@@ -887,16 +926,9 @@ stba_status run_sharded_iteration(stba_ctx* c) {
   const Scratch<real> W = scratch<real>(c);
   cudaStream_t s = c->stream;
   stba_status st;
-  const size_t rs = sizeof(real);
   record_stage(c, 0);
-  launch_iter_begin<real>(c->st, c->set, s);
-  launch_params<real>(P, (real*)c->ctab, c->cams_f, c->pts_f, s);
-  launch_zero_vp(c->vp_acc, c->counts, (int)rs, s);
   cudaMemsetAsync(c->S, 0, (size_t)c->S_total * sizeof(double), s);
-  cudaMemsetAsync(c->b, 0, (size_t)c->v_total * sizeof(double), s);
-  cudaMemsetAsync(c->vgrad, 0, 9 * (size_t)c->m * rs, s);
-  cudaMemsetAsync(c->t_acc, 0, 3 * (size_t)c->n * rs, s);
-  cudaMemsetAsync(c->fail_flags, 0, (size_t)c->l * sizeof(int), s);
+  enqueue_begin<real>(c, P, W, true, s);
   launch_vp_reduce<real>(P, W, s);   // this process's observations only
   launch_pt_sums<real>(P, W, c->xch, s);
   if ((st = shard_exchange(c, c->xch, 9 * (int64_t)c->n, 0)) != STBA_OK) return st;
@@ -910,10 +942,10 @@ stba_status run_sharded_iteration(stba_ctx* c) {
     launch_factor<double>(P, W.S, c->fbuf, c->cplan, s);
   record_stage(c, 3);
   if (c->f32f)
-    launch_solve<float>(P, W.S, W.b, c->fbuf, c->cplan, c->set.refine_steps, c->dc, s);
+    launch_solve<float>(P, W.S, W.b, c->fbuf, c->cplan, c->set.refine_steps, s);
   else
-    launch_solve<double>(P, W.S, W.b, c->fbuf, c->cplan, c->set.refine_steps, c->dc, s);
-  launch_count_failures(c->fail_flags, c->l, c->st, s);
+    launch_solve<double>(P, W.S, W.b, c->fbuf, c->cplan, c->set.refine_steps, s);
+  launch_scatter_step<real>(P, c->fbuf.x, c->fail_flags, c->max_np, c->st, c->dc, (real*)nullptr, s);
   double* nfail = c->xch + 9 * (size_t)c->n;
   launch_failed_io(c->st, nfail, 1, s);
   if ((st = shard_exchange(c, c->dc, 9 * (int64_t)c->m, 0)) != STBA_OK) return st;
@@ -922,11 +954,10 @@ stba_status run_sharded_iteration(stba_ctx* c) {
   launch_failed_io(c->st, nfail, 0, s);
   launch_step_rows<real>(P, c->dc, (real*)c->edc, s);
   record_stage(c, 4);
+  enqueue_cost_cams<real>(c, P);
   launch_point_rhs<real>(P, W, s);
-  launch_point_update<real>(P, W, s);
-  launch_cost<real>(P, c->dc, c->dp, c->cam_rt, c->cam_df, c->pt_df, c->partial, c->st, (real*)c->res_cand, s);
-  launch_finalize<real>(P, W, c->st, c->set, 1, s);
-  launch_apply<real>(P, c->dc, c->dp, c->cams, c->pts, (const real*)c->res_cand, (real*)c->res_cur, c->st, s);
+  launch_point_update<real>(P, W, c->pt_df, s);
+  enqueue_control<real>(c, P);
   record_stage(c, 5);
   CK(cudaGetLastError());
   c->have_stage_times = true;
@@ -1069,10 +1100,9 @@ void enqueue_adjoint_step(stba_ctx* c, double lam, int corrected, const AdjointB
   // the number of virtual points on the host)
   refresh_counts(c);
   launch_set_lambda(c->st, lam, c->stream);
-  launch_iter_begin<real>(c->st, c->set, c->stream);
+  launch_iter_begin(c->st, c->set, c->stream);
   const DevProblem P = dev_problem(c);
-  launch_cost<real>(P, nullptr, nullptr, c->cam_rt, c->cam_df, c->pt_df, c->partial, c->st, (real*)c->res_cur,
-                    c->stream);
+  launch_cost_x<real>(P, c->cam_rt, c->cam_df, c->pt_df, c->partial, c->st, (real*)c->res_cur, c->stream);
   enqueue_step<real>(c, false);
   launch_adjoint_step<real>(P, scratch<real>(c), c->clist, c->fbuf, c->cplan, c->set.refine_steps, c->obs_perm, lam,
                             corrected, A, c->stream);
@@ -1366,6 +1396,8 @@ void stba_destroy(stba_ctx* c) {
   for (cudaGraphExec_t& e : c->reorder_exec)
     if (e) cudaGraphExecDestroy(e);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
+  if (c->mark_stream) cudaStreamDestroy(c->mark_stream);
+  if (c->ev_mark) cudaEventDestroy(c->ev_mark);
   if (c->side_stream) cudaStreamDestroy(c->side_stream);
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
   if (c->ev_join) cudaEventDestroy(c->ev_join);
@@ -1373,6 +1405,8 @@ void stba_destroy(stba_ctx* c) {
   if (c->ev_rjoin) cudaEventDestroy(c->ev_rjoin);
   if (c->ev_sfork) cudaEventDestroy(c->ev_sfork);
   if (c->ev_sjoin) cudaEventDestroy(c->ev_sjoin);
+  for (cudaEvent_t e : {c->ev_zfork, c->ev_zjoin, c->ev_cfork, c->ev_cjoin})
+    if (e) cudaEventDestroy(e);
   if (c->ev_copy) cudaEventDestroy(c->ev_copy);
   for (auto e : c->ev_panel) cudaEventDestroy(e);
   for (auto e : c->ev_update) cudaEventDestroy(e);
@@ -1502,7 +1536,9 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
   }
   // all host-side validation is done; from here on the device is needed
   c->stream = (cudaStream_t)cuda_stream;
-  if (cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
+  if (cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaStreamCreateWithFlags(&c->mark_stream, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->ev_mark, cudaEventDisableTiming) != cudaSuccess) {
     cudaGetLastError();
     return bail(fail(c, STBA_ERR_CUDA, "cannot create a CUDA stream (is a GPU visible?)"));
   }
@@ -1515,6 +1551,10 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
       cudaEventCreateWithFlags(&c->ev_rjoin, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_sfork, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_sjoin, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->ev_zfork, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->ev_zjoin, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->ev_cfork, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->ev_cjoin, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_copy, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->stage_ev[0], cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->stage_ev[1], cudaEventDisableTiming) != cudaSuccess)

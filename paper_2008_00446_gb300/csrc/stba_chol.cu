@@ -30,6 +30,7 @@
 #include <mutex>
 #include <type_traits>
 
+#include "stba_device.cuh"
 #include "stba_internal.cuh"
 #include "stba_tc.cuh"
 
@@ -44,6 +45,7 @@ int factor_tile(bool mixed) { return mixed ? 64 : 32; }
 // s_i = 1 / sqrt(S_ii) (1 on padding)
 template <typename Sreal>
 __global__ void k_diag_scale(DevProblem P, const Sreal* S, double* scale) {
+  chain_begin();
   const int k = blockIdx.y;
   if (P.sharded && !P.cluster_owned[k]) return;
   const int np = P.cluster_np[k], nk = P.cluster_n[k];
@@ -1637,6 +1639,7 @@ __global__ void __launch_bounds__(256, T == 64 ? 2 : 3) k_tri_push(DevProblem P,
   namespace cg = cooperative_groups;
   using PL = PushLayout<F, T>;
   constexpr int V = PL::V, PARTS = PL::PARTS, NL = PL::NL, CG = PL::CG, NB = PL::NB;
+  chain_begin();
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank();
   const int k = blockIdx.x / CS;
@@ -1854,22 +1857,25 @@ int solve_stages(int l, int max_np, int cs) {
 template <typename F, int T, typename Rreal>
 void launch_tri_solve(const DevProblem& P, const F* L, const F* Dinv, const double* scale, const Rreal* rhs,
                       double* x, double* rcopy, int accumulate, int max_np, int64_t v_total, int cs, int* fail_flags,
-                      cudaStream_t stream) {
+                      bool after_kernel, cudaStream_t stream) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(P.l * cs);
   cfg.blockDim = dim3(256);
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = cs;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   const int max_nt = max_np / T;
   const size_t push = PushLayout<F, T>::bytes(max_nt, cs);
   if (push <= (size_t)g_smem_optin) {
     cfg.dynamicSmemBytes = push;
+    cfg.numAttrs = after_kernel && chained(P) ? 2 : 1;
     auto* kern = cs == 2 ? k_tri_push<F, T, Rreal, 2> : cs == 4 ? k_tri_push<F, T, Rreal, 4> : k_tri_push<F, T, Rreal, 8>;
     cudaLaunchKernelEx(&cfg, kern, P, L, Dinv, scale, rhs, x, rcopy, accumulate, v_total, max_nt, fail_flags);
     return;
@@ -1896,6 +1902,7 @@ __global__ void __launch_bounds__(32 * RES_WARPS) k_residual(DevProblem P, const
   __shared__ double xs[RES_WARPS][32];
   __shared__ double xi[32];
   __shared__ double red[RES_WARPS][32];
+  chain_begin();
   const int2 it = items[blockIdx.x];
   const int k = it.x, I = it.y & 0xffff, J0 = RES_TILES * (it.y >> 16);
   const int np = P.cluster_np[k], nk = P.cluster_n[k];
@@ -1940,32 +1947,6 @@ __global__ void __launch_bounds__(32 * RES_WARPS) k_residual(DevProblem P, const
   }
 }
 
-// sharded: another process's clusters scatter zeros (their steps arrive by the exchange of dc)
-__global__ void k_scatter_dc(DevProblem P, const double* x, double* dc) {
-  const int k = blockIdx.x;
-  const int nk = P.cluster_n[k], cbase = P.cluster_cam_off[k];
-  const bool own = !P.sharded || P.cluster_owned[k];
-  const double* xk = x + P.v_off[k];
-  for (int i = threadIdx.x; i < nk; i += blockDim.x) {
-    const int cam = P.cluster_cams[cbase + i / 9];
-    const double v = own ? xk[i] : 0.0;
-    dc[9 * (size_t)cam + i % 9] = v;
-  }
-}
-
-__global__ void k_count_failures(const int* fail_flags, int l, DevState* st) {
-  int c = 0;
-  for (int i = threadIdx.x; i < l; i += blockDim.x) c += fail_flags[i] != 0;
-  for (int d = 16; d > 0; d >>= 1) c += __shfl_xor_sync(FULL_MASK, c, d);
-  __shared__ int red[32];
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = c;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int t = 0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += red[i];
-    st->failed = t;
-  }
-}
 
 // ------------------------------------------------------------------------------------------------------
 // Host launchers
@@ -2004,6 +1985,12 @@ size_t panel_smem(int npn = 0) {
   return npn <= g_num_sms ? std::max(PanelLayout<F, T>::bytes, g_panel_min_smem) : PanelLayout<F, T>::bytes;
 }
 
+// whether the factorisation runs as tensor-core steps (k_step_tc)
+template <typename F, int T>
+bool tensor_steps(const CholPlan& plan) {
+  return sizeof(F) == 4 && T == 64 && plan.update_tc && !plan.persistent;
+}
+
 template <typename F, int T>
 void launch_factor_t(const DevProblem& P, const double* S, const FactorBuffers& fb, const CholPlan& plan,
                      cudaStream_t stream) {
@@ -2013,8 +2000,7 @@ void launch_factor_t(const DevProblem& P, const double* S, const FactorBuffers& 
   dim3 g1(std::max(1, std::min(plan.max_np / 256 + 1, 64)), P.l);
   k_diag_scale<Sreal><<<g1, 256, 0, stream>>>(P, S, fb.scale);
   dim3 g2(std::min(plan.max_np, 1024), P.l);
-  bool tcf = false;   // tensor-core panels and updates: they read S' themselves, no scaled copy
-  if constexpr (sizeof(F) == 4 && T == 64) tcf = plan.update_tc && !plan.persistent;
+  const bool tcf = tensor_steps<F, T>(plan);   // they read S' themselves, no scaled copy
   // the first tile column now (the first panels read it); with more tile steps, the rest of the copy runs
   // on the side stream beside panel 0, and panel 1 waits for it
   bool copy_beside = !tcf && plan.nsteps > 1 && plan.ev_copy != nullptr;
@@ -2059,7 +2045,7 @@ void launch_factor_t(const DevProblem& P, const double* S, const FactorBuffers& 
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
-        cfg.numAttrs = kt >= 0 ? 1 : 0;   // panel 0 follows kernels that do not signal
+        cfg.numAttrs = 1;
         cudaLaunchKernelEx(&cfg, kt == 0 ? k_step_tc<true> : k_step_tc<false>, reinterpret_cast<float*>(L),
                            reinterpret_cast<float*>(Dinv), fb.split, S, (const double*)fb.scale, P,
                            plan.panel_items + plan.h_panel_off[kt + 1], npn,
@@ -2115,19 +2101,23 @@ void launch_factor_t(const DevProblem& P, const double* S, const FactorBuffers& 
 
 template <typename F, int T>
 void launch_solve_t(const DevProblem& P, const double* S, const double* b, const FactorBuffers& fb,
-                    const CholPlan& plan, int refine_steps, double* dc, cudaStream_t stream) {
+                    const CholPlan& plan, int refine_steps, cudaStream_t stream) {
   using Sreal = double;
   const F* L = reinterpret_cast<const F*>(fb.L);
   const F* Dinv = reinterpret_cast<const F*>(fb.Dinv);
   for (int s = 0; s <= refine_steps; ++s) {   // x = S~^-1 b, then x += S~^-1 (b - S x)
     launch_tri_solve<F, T, Sreal>(P, L, Dinv, fb.scale, s ? fb.r : b, fb.x, s < refine_steps && s == 0 ? fb.r : nullptr,
-                                  s > 0, plan.max_np, fb.v_total, plan.solve_cs, fb.fail_flags, stream);
+                                  s > 0, plan.max_np, fb.v_total, plan.solve_cs, fb.fail_flags,
+                                  s ? plan.n_res_items > 0 : tensor_steps<F, T>(plan), stream);
     if (s == refine_steps) break;
     if (s > 0) cudaMemcpyAsync(fb.r, b, (size_t)fb.v_total * sizeof(double), cudaMemcpyDeviceToDevice, stream);
-    if (plan.n_res_items > 0)
-      k_residual<Sreal><<<plan.n_res_items, 32 * RES_WARPS, 0, stream>>>(P, S, fb.x, fb.r, plan.res_items);
+    if (plan.n_res_items > 0) {
+      if (s == 0)
+        launch_after(chained(P), k_residual<Sreal>, plan.n_res_items, 32 * RES_WARPS, stream, P, S, fb.x, fb.r, plan.res_items);
+      else
+        k_residual<Sreal><<<plan.n_res_items, 32 * RES_WARPS, 0, stream>>>(P, S, fb.x, fb.r, plan.res_items);
+    }
   }
-  k_scatter_dc<<<P.l, 256, 0, stream>>>(P, fb.x, dc);
 }
 
 // the tile size of the plan: FP32 factors 32 or 64 (chosen by stba_autotune), FP64 factors 32
@@ -2142,11 +2132,11 @@ void launch_factor(const DevProblem& P, const double* S, const FactorBuffers& fb
 
 template <typename F>
 void launch_solve(const DevProblem& P, const double* S, const double* b, const FactorBuffers& fb,
-                  const CholPlan& plan, int refine_steps, double* dc, cudaStream_t stream) {
+                  const CholPlan& plan, int refine_steps, cudaStream_t stream) {
   if constexpr (sizeof(F) == 4) {
-    if (plan.tile == 64) return launch_solve_t<F, 64>(P, S, b, fb, plan, refine_steps, dc, stream);
+    if (plan.tile == 64) return launch_solve_t<F, 64>(P, S, b, fb, plan, refine_steps, stream);
   }
-  launch_solve_t<F, 32>(P, S, b, fb, plan, refine_steps, dc, stream);
+  launch_solve_t<F, 32>(P, S, b, fb, plan, refine_steps, stream);
 }
 
 size_t solve_smem_bytes(bool mixed, int tile, int max_np) {   // with the smallest stage count
@@ -2228,17 +2218,13 @@ void configure_solve_kernels(int max_np) {
   raise_smem_attr((const void*)k_tri_solve<double, 32, double, 2>, d32);
 }
 
-void launch_count_failures(const int* fail_flags, int l, DevState* st, cudaStream_t stream) {
-  k_count_failures<<<1, 256, 0, stream>>>(fail_flags, l, st);
-}
-
 template void launch_factor<float>(const DevProblem&, const double*, const FactorBuffers&, const CholPlan&,
                                    cudaStream_t);
 template void launch_factor<double>(const DevProblem&, const double*, const FactorBuffers&, const CholPlan&,
                                     cudaStream_t);
 template void launch_solve<float>(const DevProblem&, const double*, const double*, const FactorBuffers&,
-                                  const CholPlan&, int, double*, cudaStream_t);
+                                  const CholPlan&, int, cudaStream_t);
 template void launch_solve<double>(const DevProblem&, const double*, const double*, const FactorBuffers&,
-                                   const CholPlan&, int, double*, cudaStream_t);
+                                   const CholPlan&, int, cudaStream_t);
 
 }  // namespace stba

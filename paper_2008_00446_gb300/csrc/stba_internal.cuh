@@ -201,14 +201,20 @@ template <typename real>
 void launch_reorder(const ReorderArgs& A, int* key, int* tile_sum, long long* counts, const real* res_old,
                     real* res_new, cudaStream_t stream);
 
-// zeroes the virtual-point accumulators (9 nv reals of real_bytes each; nv = counts[0] on the device)
-void launch_zero_vp(void* vp_acc, const long long* counts, int real_bytes, cudaStream_t stream);
-
 constexpr int RED_BLOCKS = 456;    // 3 x 152 SMs: fixed grid of the deterministic reductions
 constexpr int RED_THREADS = 256;
 
-template <typename real>
+// resets the iteration's state; launch_begin does it with everything else an iteration starts from
 void launch_iter_begin(DevState* st, const Settings& s, cudaStream_t stream);
+struct ZeroList {   // 32-bit words that an iteration starts from zero (unused entries: no words)
+  static constexpr int N = 4;
+  uint32_t* p[N];
+  int64_t words[N];
+};
+// camera tables, FP32 copies of the cameras and points (mixed precision; else null), zeroed accumulators
+template <typename real>
+void launch_begin(const DevProblem& P, Scratch<real> W, real* ctab, float* cams_f, float* pts_f, DevState* st,
+                  const Settings& s, const long long* counts, const ZeroList& Z, cudaStream_t stream);
 template <typename real>
 void launch_vp_reduce(const DevProblem& P, Scratch<real> W, cudaStream_t stream);
 template <typename real>
@@ -229,20 +235,27 @@ void launch_rcs_build(const DevProblem& P, Scratch<real> W, CamSlots CS, PairChu
                       cudaEvent_t join = nullptr);
 template <typename real>
 void launch_point_rhs(const DevProblem& P, Scratch<real> W, cudaStream_t stream);
-// camera tables, and FP32 copies of the cameras and points (mixed precision; else null): once per linearisation
+// x (padded, per cluster) -> dc [m][9]; with edc, E dc too; with st, counts the failed clusters into st->failed
 template <typename real>
-void launch_params(const DevProblem& P, real* ctab, float* cams_f, float* pts_f, cudaStream_t stream);
+void launch_scatter_step(const DevProblem& P, const double* x, const int* fail_flags, int max_np, DevState* st,
+                         double* dc, real* edc, cudaStream_t stream);
+// dp and the partial sums of the stop tests; mixed precision: pt_df [n][6] gets p + dp as double-float
 template <typename real>
-void launch_point_update(const DevProblem& P, Scratch<real> W, cudaStream_t stream);
-// k_cam_rt + k_cost: rt is a [m][15] FP64 scratch (R, t, f, k1, k2 of x + dx); residuals go to rout.  In mixed
-// mode with a step, the cost runs in double-float arithmetic with the scratch tables cam_df [m][28] and
-// pt_df [n][6] (floats).
+void launch_point_update(const DevProblem& P, Scratch<real> W, float* pt_df, cudaStream_t stream);
+// The cost at x + dx: k_cost_cams fills the camera table of c + dc (rt [m][15] FP64; mixed precision: cam_df
+// [m][28] floats, double-float), then k_cost the residuals (rout) and partial sums, in mixed precision in
+// double-float arithmetic from cam_df and pt_df.  launch_cost_x: all of it at x itself.
 template <typename real>
-void launch_cost(const DevProblem& P, const double* dc, const double* dp, double* rt, float* cam_df, float* pt_df,
+void launch_cost_cams(const DevProblem& P, const double* dc, double* rt, float* cam_df, cudaStream_t stream);
+template <typename real>
+void launch_cost(const DevProblem& P, const double* dp, const double* rt, const float* cam_df, const float* pt_df,
                  double* partial, DevState* st, real* rout, cudaStream_t stream);
-// with_step = 1: stop tests and accept / reject of the step in W.dc / W.dp; 0: F(x) -> st->F.
 template <typename real>
-void launch_finalize(const DevProblem& P, Scratch<real> W, DevState* st, const Settings& s, int with_step,
+void launch_cost_x(const DevProblem& P, double* rt, float* cam_df, float* pt_df, double* partial, DevState* st,
+                   real* rout, cudaStream_t stream);
+// with_step = 1: stop tests and accept / reject of the step; 0: F(x) -> st->F.
+template <typename real>
+void launch_finalize(const DevProblem& P, const double* partial, DevState* st, const Settings& s, int with_step,
                      cudaStream_t stream);
 template <typename real>
 void launch_apply(const DevProblem& P, const double* dc, const double* dp, double* cams, double* pts,
@@ -306,11 +319,10 @@ int factor_tile(bool mixed);
 template <typename F>
 void launch_factor(const DevProblem& P, const double* S, const FactorBuffers& fb, const CholPlan& plan,
                    cudaStream_t stream);
-// x = S'^-1 b per cluster, scattered to dc [m][9]
+// fb.x = S'^-1 b per cluster (launch_scatter_step gives the cameras' order)
 template <typename F>
 void launch_solve(const DevProblem& P, const double* S, const double* b, const FactorBuffers& fb,
-                  const CholPlan& plan, int refine_steps, double* dc, cudaStream_t stream);
-void launch_count_failures(const int* fail_flags, int l, DevState* st, cudaStream_t stream);
+                  const CholPlan& plan, int refine_steps, cudaStream_t stream);
 
 // Adjoint of one accepted step (stba_adjoint.cu).  With the forward step at x_t recomputed in W and fb
 // (dc, dp, vp_info, pt_info, S', the cluster factors), maps the upstream adjoint (a_c, a_p) of x_{t+1} in

@@ -31,27 +31,27 @@
 namespace stba {
 
 // ------------------------------------------------------------------------------------------------------
-template <typename real>
-__global__ void k_iter_begin(DevState* st, Settings s) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    st->lambda_used = st->lambda;
-    st->corrected = (s.correction && st->lambda >= s.correction_lambda) ? 1 : 0;
-    st->grad_max_bits = 0ull;
-    st->failed = 0;
-    st->nonfinite = 0;
-    st->boosted = 0;
-    st->pair_next = 0;
-  }
+__device__ __forceinline__ void reset_state(DevState* st, const Settings& s) {
+  st->lambda_used = st->lambda;
+  st->corrected = (s.correction && st->lambda >= s.correction_lambda) ? 1 : 0;
+  st->grad_max_bits = 0ull;
+  st->failed = 0;
+  st->nonfinite = 0;
+  st->boosted = 0;
+  st->pair_next = 0;
 }
 
-template <typename real>
-void launch_iter_begin(DevState* st, const Settings& s, cudaStream_t stream) {
-  k_iter_begin<real><<<1, 32, 0, stream>>>(st, s);
+// the state alone, for the cost at x (an iteration resets it in k_begin)
+__global__ void k_iter_begin(DevState* st, Settings s) {
+  if (threadIdx.x == 0 && blockIdx.x == 0) reset_state(st, s);
 }
+
+void launch_iter_begin(DevState* st, const Settings& s, cudaStream_t stream) { k_iter_begin<<<1, 32, 0, stream>>>(st, s); }
 
 // ------------------------------------------------------------------------------------------------------
 template <typename real>
 __global__ void __launch_bounds__(256) k_vp_reduce(DevProblem P, real* vp_acc) {
+  chain_begin();
   const int o = blockIdx.x * blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31;
   // sharded: only the observations of this process's clusters (a virtual point lies in one cluster, so its
@@ -100,26 +100,46 @@ __global__ void __launch_bounds__(256) k_vp_reduce(DevProblem P, real* vp_acc) {
 template <typename real>
 void launch_vp_reduce(const DevProblem& P, Scratch<real> W, cudaStream_t stream) {
   int blocks = (P.q + 255) / 256;
-  k_vp_reduce<real><<<blocks, 256, 0, stream>>>(P, W.vp_acc);
+  launch_after(chained(P), k_vp_reduce<real>, blocks, 256, stream, P, W.vp_acc);
 }
 
 // ------------------------------------------------------------------------------------------------------
-template <typename real>
-__device__ __forceinline__ double block_max(double v) {
-  __shared__ double red[32];
+// FP64 arithmetic runs at 2 lanes a cycle and SM here, so a warp's FP64 instruction costs 16 cycles however few
+// of its lanes matter, and shuffle trees in every warp of a CTA add up (8 warps x 5 steps: 640 cycles a value).
+// The reductions below keep the tree in as few warps as possible, and maxima in the integer pipe: values >= 0
+// order like their bits.
+__device__ __forceinline__ unsigned long long warp_max_bits(float v) {   // v >= 0, not NaN; the max as FP64 bits
+  const float m = __uint_as_float(__reduce_max_sync(FULL_MASK, __float_as_uint(v)));
+  return (unsigned long long)__double_as_longlong((double)m);
+}
+__device__ __forceinline__ unsigned long long warp_max_bits(double v) {
+  unsigned long long b = (unsigned long long)__double_as_longlong(v);
 #pragma unroll
-  for (int d = 16; d > 0; d >>= 1) v = fmax(v, __shfl_xor_sync(FULL_MASK, v, d));
-  int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) red[w] = v;
-  __syncthreads();
-  double r = 0.0;
-  if (w == 0) {
-    r = lane < (int)(blockDim.x >> 5) ? red[lane] : 0.0;
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) r = fmax(r, __shfl_xor_sync(FULL_MASK, r, d));
+  for (int d = 16; d > 0; d >>= 1) {
+    const unsigned long long o = __shfl_xor_sync(FULL_MASK, b, d);
+    b = o > b ? o : b;
   }
-  return r;
+  return b;
+}
+
+// Sums of NV values over a 256-thread CTA, valid in lane 0 of warp c for value c: warp c adds the eight rows of
+// its value, then its 32 lanes (13 warp instructions a value instead of 40).
+template <int NV>
+__device__ __forceinline__ double cta_sums(const double (&v)[NV], double (&buf)[NV][RED_THREADS]) {
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int c = 0; c < NV; ++c) buf[c][threadIdx.x] = v[c];
+  __syncthreads();
+  double s = 0.0;
+  if (w < NV) {
+    double a[RED_THREADS / 32];
+#pragma unroll
+    for (int i = 0; i < RED_THREADS / 32; ++i) a[i] = buf[w][32 * i + lane];
+    s = ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(FULL_MASK, s, d);
+  }
+  return s;
 }
 
 // Per point, the sums over its virtual points of V_v and w'_v: C and w of the physical point (Eq. 15).  A warp
@@ -129,6 +149,7 @@ __device__ __forceinline__ double block_max(double v) {
 template <typename real>
 __global__ void __launch_bounds__(256) k_pt_acc(DevProblem P, const real* __restrict__ vp_acc,
                                                 real* __restrict__ pt_acc) {
+  chain_begin();
   __shared__ __align__(16) real stage[8][288];
   const int lane = threadIdx.x & 31;
   real* sm = stage[threadIdx.x >> 5];
@@ -167,13 +188,14 @@ template <typename real>
 __global__ void __launch_bounds__(256) k_vp_finalize(DevProblem P, Scratch<real> W, DevState* st,
                                                      const double* __restrict__ pt_sums,
                                                      const long long* __restrict__ counts) {
+  chain_begin();
   __shared__ __align__(16) real stage[8][32 * VPI];
   const real lam = (real)st->lambda_used;
   const bool corr = st->corrected != 0;
   const long long nv = counts[0];
   const int lane = threadIdx.x & 31;
   real* sm = stage[threadIdx.x >> 5];
-  double gmax = 0.0;
+  real gmax = real(0);
   // C_i (6 packed) and w_i (3) of point i, read directly (corrected steps)
   auto point_sums = [&](int i, real (&a)[9]) {
     if (pt_sums) {
@@ -250,13 +272,21 @@ __global__ void __launch_bounds__(256) k_vp_finalize(DevProblem P, Scratch<real>
         o[6] = a[6];
         o[7] = a[7];
         o[8] = a[8];
-        gmax = fmax(gmax, fmax(fabs((double)a[6]), fmax(fabs((double)a[7]), fabs((double)a[8]))));
+        gmax = fmax(gmax, fmax(fabs(a[6]), fmax(fabs(a[7]), fabs(a[8]))));
       }
       warp_store_rec(W.pt_info, i0, cnt, sm, lane, o);
     }
   }
-  double bm = block_max<real>(gmax);
-  if (threadIdx.x == 0) atomicMax(&st->grad_max_bits, (unsigned long long)__double_as_longlong(bm));
+  __shared__ unsigned long long wmax[8];
+  const unsigned long long wm = warp_max_bits(gmax);
+  if (lane == 0) wmax[threadIdx.x >> 5] = wm;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned long long b = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) b = wmax[i] > b ? wmax[i] : b;
+    atomicMax(&st->grad_max_bits, b);
+  }
 }
 
 template <typename real>
@@ -266,10 +296,13 @@ void launch_vp_finalize(const DevProblem& P, Scratch<real> W, DevState* st, cons
   const long long nmax = (long long)P.q + P.n + 31;
   const long long cap = 8LL * num_sms();
   if (!pt_sums)
-    k_pt_acc<real><<<(int)std::min<long long>(((long long)P.n + 255) / 256, cap), 256, 0, stream>>>(P, W.vp_acc,
-                                                                                                 W.pt_acc);
-  k_vp_finalize<real><<<(int)std::min<long long>((nmax + 255) / 256, cap), 256, 0, stream>>>(P, W, st, pt_sums,
-                                                                                            counts);
+    launch_after(chained(P), k_pt_acc<real>, (int)std::min<long long>(((long long)P.n + 255) / 256, cap), 256, stream,
+                 P, W.vp_acc, W.pt_acc);
+  const int grid = (int)std::min<long long>((nmax + 255) / 256, cap);
+  if (pt_sums)   // after an exchange, not a kernel
+    k_vp_finalize<real><<<grid, 256, 0, stream>>>(P, W, st, pt_sums, counts);
+  else
+    launch_after(chained(P), k_vp_finalize<real>, grid, 256, stream, P, W, st, pt_sums, counts);
 }
 
 template <typename real>
@@ -805,8 +838,40 @@ void launch_rcs_build(const DevProblem& P, Scratch<real> W, CamSlots CS, PairChu
 }
 
 // ------------------------------------------------------------------------------------------------------
+// Double-float numbers: a value is an unevaluated sum hi + lo of two floats.
+__device__ __forceinline__ float2 df_two_sum(float a, float b) {
+  const float s = a + b;
+  const float bb = s - a;
+  return make_float2(s, (a - (s - bb)) + (b - bb));
+}
+__device__ __forceinline__ float2 df_fast_two_sum(float a, float b) {   // |a| >= |b|
+  const float s = a + b;
+  return make_float2(s, b - (s - a));
+}
+__device__ __forceinline__ float2 df_add(float2 x, float2 y) {
+  const float2 s = df_two_sum(x.x, y.x);
+  return df_fast_two_sum(s.x, s.y + (x.y + y.y));
+}
+__device__ __forceinline__ float2 df_sub(float2 x, float2 y) { return df_add(x, make_float2(-y.x, -y.y)); }
+__device__ __forceinline__ float2 df_mul(float2 x, float2 y) {
+  const float p = x.x * y.x;
+  const float e = fmaf(x.x, y.y, fmaf(x.y, y.x, fmaf(x.x, y.x, -p)));
+  return df_fast_two_sum(p, e);
+}
+__device__ __forceinline__ float2 df_rcp(float2 y) {   // one Newton correction of the FP32 reciprocal
+  const float q = __frcp_rn(y.x);
+  const float2 r = df_sub(make_float2(1.f, 0.f), df_mul(make_float2(q, 0.f), y));
+  return df_fast_two_sum(q, r.x * q);
+}
+__device__ __forceinline__ float2 df_split(double d) {
+  const float hi = __double2float_rn(d);
+  return make_float2(hi, __double2float_rn(d - (double)hi));
+}
+
+// ------------------------------------------------------------------------------------------------------
 template <typename real>
 __global__ void __launch_bounds__(256) k_point_rhs(DevProblem P, const real* __restrict__ edc, real* t_acc) {
+  chain_begin();
   const int o = blockIdx.x * blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31;
   const bool act = o < P.q;
@@ -842,10 +907,16 @@ __global__ void __launch_bounds__(256) k_point_rhs(DevProblem P, const real* __r
 
 // dp = C^-1 (w - t) per point; the same grid also forms the partial sums of the stop tests: |dp|^2, |p|^2,
 // |dc|^2, |c|^2 and max |v| (camera gradient), one partial per block at partial[RED_BLOCKS * (1..5) + block].
+// With pdf (mixed precision) it also writes the candidate p + dp as double-float numbers for k_cost_df.
+// Bound by the FP64 pipe: the sums were four shuffle trees in each of the eight warps (14 us at 1000 photos with
+// a separate 8 us kernel for the double-float points; the fused kernel takes 15.6 us).
 template <typename real>
-__global__ void __launch_bounds__(256) k_point_update(DevProblem P, const real* pt_info, const real* t_acc,
-                                                      const double* dc, const real* vgrad, double* dp,
-                                                      double* partial) {
+__global__ void __launch_bounds__(RED_THREADS) k_point_update(DevProblem P, const real* __restrict__ pt_info,
+                                                              const real* __restrict__ t_acc,
+                                                              const double* __restrict__ dc,
+                                                              const real* __restrict__ vgrad, double* __restrict__ dp,
+                                                              float2* __restrict__ pdf, double* __restrict__ partial) {
+  chain_begin();
   double s_dp = 0.0, s_p = 0.0, s_dc = 0.0, s_c = 0.0;
   real gmax = real(0);   // max |v| in the working precision (exact)
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P.n; i += gridDim.x * blockDim.x) {
@@ -859,9 +930,15 @@ __global__ void __launch_bounds__(256) k_point_update(DevProblem P, const real* 
     out[0] = d0;
     out[1] = d1;
     out[2] = d2;
-    s_dp += (double)d0 * d0 + (double)d1 * d1 + (double)d2 * d2;
+    const double e[3] = {(double)d0, (double)d1, (double)d2};
     const double* p = P.pts + 3 * (size_t)i;
-    s_p += p[0] * p[0] + p[1] * p[1] + p[2] * p[2];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double pc = p[c];
+      s_dp += e[c] * e[c];
+      s_p += pc * pc;
+      if constexpr (sizeof(real) == 4) pdf[3 * (size_t)i + c] = df_split(pc + e[c]);
+    }
   }
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 9 * P.m; i += gridDim.x * blockDim.x) {
     const double d = dc[i], c = P.cams[i];
@@ -869,33 +946,19 @@ __global__ void __launch_bounds__(256) k_point_update(DevProblem P, const real* 
     s_c += c * c;
     gmax = fmax(gmax, fabs(vgrad[i]));
   }
-  __shared__ double red[4][8];
-  __shared__ real redm[8];
-  for (int d = 16; d > 0; d >>= 1) {
-    s_dp += __shfl_xor_sync(FULL_MASK, s_dp, d);
-    s_p += __shfl_xor_sync(FULL_MASK, s_p, d);
-    s_dc += __shfl_xor_sync(FULL_MASK, s_dc, d);
-    s_c += __shfl_xor_sync(FULL_MASK, s_c, d);
-    gmax = fmax(gmax, __shfl_xor_sync(FULL_MASK, gmax, d));
-  }
+  __shared__ double buf[4][RED_THREADS];
+  __shared__ unsigned long long wmax[RED_THREADS / 32];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) {
-    red[0][w] = s_dp;
-    red[1][w] = s_p;
-    red[2][w] = s_dc;
-    red[3][w] = s_c;
-    redm[w] = gmax;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a[4] = {0, 0, 0, 0};
-    real mx = real(0);
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) {
-      for (int c = 0; c < 4; ++c) a[c] += red[c][i];
-      mx = fmax(mx, redm[i]);
-    }
-    for (int c = 0; c < 4; ++c) partial[(1 + c) * RED_BLOCKS + blockIdx.x] = a[c];
-    partial[5 * RED_BLOCKS + blockIdx.x] = (double)mx;
+  const unsigned long long wm = warp_max_bits(gmax);
+  if (lane == 0) wmax[w] = wm;
+  const double v[4] = {s_dp, s_p, s_dc, s_c};
+  const double a = cta_sums<4>(v, buf);
+  if (lane == 0 && w < 4) partial[(1 + w) * RED_BLOCKS + blockIdx.x] = a;
+  if (threadIdx.x == 32 * 4) {
+    unsigned long long b = 0;
+#pragma unroll
+    for (int i = 0; i < RED_THREADS / 32; ++i) b = wmax[i] > b ? wmax[i] : b;
+    partial[5 * RED_BLOCKS + blockIdx.x] = __longlong_as_double((long long)b);
   }
 }
 
@@ -903,28 +966,48 @@ __global__ void __launch_bounds__(256) k_point_update(DevProblem P, const real* 
 // Residuals in FP64 (both precisions): the cost F(x + dx) and the accept test need them to FP64 accuracy,
 // and the stored residuals drive the next linearisation (FP32 projections of pixel coordinates of a few
 // hundred px carry ~3e-5 px of rounding, which the conditioning of S' amplifies in the step).
-// k_cam_rt precomputes per camera R(w + dw) (Rodrigues in FP64), t + dt and the intrinsics.
-__global__ void k_cam_rt(int m, const double* cams, const double* dc, double* rt) {
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < m; j += gridDim.x * blockDim.x) {
-    double c[9];
+// k_cost_cams: per camera R(w + dw) (Rodrigues in FP64), t + dt and the intrinsics, as 15 FP64 numbers, or in
+// mixed precision split into double-float (CAM_DF floats).  A long FP64 chain per camera and 16 cycles a warp
+// instruction: one warp a CTA, so that the cameras spread over the SMs (four warps a CTA and the split in a
+// kernel of its own: 7.9 + 5.3 us at 1000 cameras; 8.4 us now, beside the point step).
+constexpr int CAM_DF = 28;   // floats per camera: R (9 x 2), t (3 x 2), f (2), k1, k2
+
+template <typename real>
+__global__ void __launch_bounds__(32) k_cost_cams(int m, const double* __restrict__ cams, const double* __restrict__ dc,
+                                                  double* __restrict__ rt, float* __restrict__ cdf) {
+  const int j = 32 * blockIdx.x + threadIdx.x;
+  if (j >= m) return;
+  double c[9];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) c[i] = cams[9 * (size_t)j + i] + (dc ? dc[9 * (size_t)j + i] : 0.0);
-    const double s = c[0] * c[0] + c[1] * c[1] + c[2] * c[2];
-    double a, b, da, db;
-    rodrigues_coeffs(s, a, b, da, db);
-    const double* w = c;
-    double* o = rt + 15 * (size_t)j;
-    o[0] = 1.0 + b * (w[0] * w[0] - s);
-    o[1] = -a * w[2] + b * w[0] * w[1];
-    o[2] = a * w[1] + b * w[0] * w[2];
-    o[3] = a * w[2] + b * w[0] * w[1];
-    o[4] = 1.0 + b * (w[1] * w[1] - s);
-    o[5] = -a * w[0] + b * w[1] * w[2];
-    o[6] = -a * w[1] + b * w[0] * w[2];
-    o[7] = a * w[0] + b * w[1] * w[2];
-    o[8] = 1.0 + b * (w[2] * w[2] - s);
+  for (int i = 0; i < 9; ++i) c[i] = cams[9 * (size_t)j + i] + (dc ? dc[9 * (size_t)j + i] : 0.0);
+  const double s = c[0] * c[0] + c[1] * c[1] + c[2] * c[2];
+  double a, b, da, db;
+  rodrigues_coeffs(s, a, b, da, db);
+  const double* w = c;
+  double o[15];
+  o[0] = 1.0 + b * (w[0] * w[0] - s);
+  o[1] = -a * w[2] + b * w[0] * w[1];
+  o[2] = a * w[1] + b * w[0] * w[2];
+  o[3] = a * w[2] + b * w[0] * w[1];
+  o[4] = 1.0 + b * (w[1] * w[1] - s);
+  o[5] = -a * w[0] + b * w[1] * w[2];
+  o[6] = -a * w[1] + b * w[0] * w[2];
+  o[7] = a * w[0] + b * w[1] * w[2];
+  o[8] = 1.0 + b * (w[2] * w[2] - s);
 #pragma unroll
-    for (int i = 0; i < 6; ++i) o[9 + i] = c[3 + i];
+  for (int i = 0; i < 6; ++i) o[9 + i] = c[3 + i];
+  if constexpr (sizeof(real) == 4) {
+    float4* out = reinterpret_cast<float4*>(cdf + CAM_DF * (size_t)j);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      const float2 u = df_split(o[2 * i]), v = df_split(o[2 * i + 1]);
+      out[i] = make_float4(u.x, u.y, v.x, v.y);
+    }
+    const float2 f = df_split(o[12]);
+    out[6] = make_float4(f.x, f.y, (float)o[13], (float)o[14]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 15; ++i) rt[15 * (size_t)j + i] = o[i];
   }
 }
 
@@ -932,6 +1015,7 @@ __global__ void k_cam_rt(int m, const double* cams, const double* dc, double* rt
 template <typename real>
 __global__ void __launch_bounds__(RED_THREADS) k_cost(DevProblem P, const double* rt, const double* dp,
                                                       double* partial, DevState* st, real* rout) {
+  chain_begin();
   double s = 0.0;
   int bad = 0;
   for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < P.q; o += gridDim.x * blockDim.x) {
@@ -960,18 +1044,11 @@ __global__ void __launch_bounds__(RED_THREADS) k_cost(DevProblem P, const double
     rout[2 * (size_t)o] = (real)r0;
     rout[2 * (size_t)o + 1] = (real)r1;
   }
-  __shared__ double red[RED_THREADS / 32];
-  for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(FULL_MASK, s, d);
-  bad = __any_sync(FULL_MASK, bad);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) red[w] = s;
-  if (lane == 0 && bad) st->nonfinite = 1;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0;
-    for (int i = 0; i < RED_THREADS / 32; ++i) a += red[i];
-    partial[blockIdx.x] = a;
-  }
+  __shared__ double buf[1][RED_THREADS];
+  if (__any_sync(FULL_MASK, bad) && (threadIdx.x & 31) == 0) st->nonfinite = 1;
+  const double v[1] = {s};
+  const double a = cta_sums<1>(v, buf);
+  if (threadIdx.x == 0) partial[blockIdx.x] = a;
 }
 
 // ------------------------------------------------------------------------------------------------------
@@ -979,65 +1056,17 @@ __global__ void __launch_bounds__(RED_THREADS) k_cost(DevProblem P, const double
 // hi + lo of two floats, ~48-bit significand; Dekker's and Knuth's error-free transformations, with the
 // product error taken by an FMA).  The FP64 pipe of this GPU runs at 1/64 of the FP32 rate; double-float
 // keeps the residuals accurate to ~1e-12 px at pixel offsets of a few hundred px on the FP32 pipe.
-// Per camera the FP64 table of k_cam_rt is split into double-float (R, t, f; k1 and k2 as floats, since
-// they scale the small distortion term only); per point the candidate p + dp is split in k_point_df.
-__device__ __forceinline__ float2 df_two_sum(float a, float b) {
-  const float s = a + b;
-  const float bb = s - a;
-  return make_float2(s, (a - (s - bb)) + (b - bb));
-}
-__device__ __forceinline__ float2 df_fast_two_sum(float a, float b) {   // |a| >= |b|
-  const float s = a + b;
-  return make_float2(s, b - (s - a));
-}
-__device__ __forceinline__ float2 df_add(float2 x, float2 y) {
-  const float2 s = df_two_sum(x.x, y.x);
-  return df_fast_two_sum(s.x, s.y + (x.y + y.y));
-}
-__device__ __forceinline__ float2 df_sub(float2 x, float2 y) { return df_add(x, make_float2(-y.x, -y.y)); }
-__device__ __forceinline__ float2 df_mul(float2 x, float2 y) {
-  const float p = x.x * y.x;
-  const float e = fmaf(x.x, y.y, fmaf(x.y, y.x, fmaf(x.x, y.x, -p)));
-  return df_fast_two_sum(p, e);
-}
-__device__ __forceinline__ float2 df_rcp(float2 y) {   // one Newton correction of the FP32 reciprocal
-  const float q = __frcp_rn(y.x);
-  const float2 r = df_sub(make_float2(1.f, 0.f), df_mul(make_float2(q, 0.f), y));
-  return df_fast_two_sum(q, r.x * q);
-}
-__device__ __forceinline__ float2 df_split(double d) {
-  const float hi = __double2float_rn(d);
-  return make_float2(hi, __double2float_rn(d - (double)hi));
-}
-
-constexpr int CAM_DF = 28;   // floats per camera: R (9 x 2), t (3 x 2), f (2), k1, k2
-
-__global__ void k_cam_df(int m, const double* __restrict__ rt, float* __restrict__ cdf) {
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < m; j += gridDim.x * blockDim.x) {
-    const double* c = rt + 15 * (size_t)j;
-    float* o = cdf + CAM_DF * (size_t)j;
-#pragma unroll
-    for (int i = 0; i < 13; ++i) {
-      const float2 v = df_split(c[i]);
-      o[2 * i] = v.x;
-      o[2 * i + 1] = v.y;
-    }
-    o[26] = (float)c[13];
-    o[27] = (float)c[14];
-  }
-}
-
-__global__ void k_point_df(int n, const double* __restrict__ pts, const double* __restrict__ dp,
-                           float* __restrict__ pdf) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 3 * n; i += gridDim.x * blockDim.x) {
-    const float2 v = df_split(dp ? pts[i] + dp[i] : pts[i]);
-    reinterpret_cast<float2*>(pdf)[i] = v;
-  }
+// Per camera the table of k_cost_cams holds double-float numbers (R, t, f; k1 and k2 as floats, since they
+// scale the small distortion term only); per point k_point_update splits the candidate p + dp (k_point_df the
+// points of x itself).
+__global__ void k_point_df(int n, const double* __restrict__ pts, float2* __restrict__ pdf) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 3 * n; i += gridDim.x * blockDim.x) pdf[i] = df_split(pts[i]);
 }
 
 __global__ void __launch_bounds__(RED_THREADS) k_cost_df(DevProblem P, const float* __restrict__ cdf,
                                                          const float* __restrict__ pdf, double* partial,
                                                          DevState* st, float* rout) {
+  chain_begin();
   float2 acc = make_float2(0.f, 0.f);
   double acc_rho = 0.0;
   int bad = 0;
@@ -1080,66 +1109,68 @@ __global__ void __launch_bounds__(RED_THREADS) k_cost_df(DevProblem P, const flo
     rout[2 * (size_t)o + 1] = r1.x + r1.y;
   }
   double s = (double)acc.x + (double)acc.y + acc_rho;
-  __shared__ double red[RED_THREADS / 32];
-  for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(FULL_MASK, s, d);
-  bad = __any_sync(FULL_MASK, bad);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) red[w] = s;
-  if (lane == 0 && bad) st->nonfinite = 1;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0;
-    for (int i = 0; i < RED_THREADS / 32; ++i) a += red[i];
-    partial[blockIdx.x] = a;
-  }
+  __shared__ double buf[1][RED_THREADS];
+  if (__any_sync(FULL_MASK, bad) && (threadIdx.x & 31) == 0) st->nonfinite = 1;
+  const double v[1] = {s};
+  const double a = cta_sums<1>(v, buf);
+  if (threadIdx.x == 0) partial[blockIdx.x] = a;
 }
 
 // ------------------------------------------------------------------------------------------------------
-// Stop tests and accept / reject (Algorithm 1), one block; fixed-order sums of the partials.
+// Stop tests and accept / reject (Algorithm 1), one CTA of one warp per partial sum (fixed order).  32 warps
+// took 16 us on the FP64 pipe of the one SM; six warps and paired square roots take 5.3 us.
+constexpr int FIN_WARPS = 6;
 template <typename real>
-__global__ void __launch_bounds__(1024) k_finalize(DevProblem P, const real* vgrad, const double* dc,
-                                                   const double* partial, DevState* st, Settings s,
-                                                   int with_step) {
-  __shared__ double red[4][32];
-  double F_new = 0, dpn = 0, pn = 0, dcn = 0, cn = 0, gmax = 0;
-  for (int i = threadIdx.x; i < RED_BLOCKS; i += blockDim.x) {
-    F_new += partial[i];
-    if (with_step) {
-      dpn += partial[RED_BLOCKS + i];
-      pn += partial[2 * RED_BLOCKS + i];
-      dcn += partial[3 * RED_BLOCKS + i];
-      cn += partial[4 * RED_BLOCKS + i];
-      gmax = fmax(gmax, partial[5 * RED_BLOCKS + i]);
-    }
-  }
-  double vals[4] = {F_new, dpn + dcn, pn + cn, gmax};
+__global__ void __launch_bounds__(32 * FIN_WARPS) k_finalize(const double* __restrict__ partial, DevState* st,
+                                                             Settings s, int with_step) {
+  chain_begin();
+  __shared__ double red[FIN_WARPS];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int PER = (RED_BLOCKS + 31) / 32;
+  double x[PER];
 #pragma unroll
-  for (int c = 0; c < 3; ++c)
-    for (int d = 16; d > 0; d >>= 1) vals[c] += __shfl_xor_sync(FULL_MASK, vals[c], d);
-  for (int d = 16; d > 0; d >>= 1) vals[3] = fmax(vals[3], __shfl_xor_sync(FULL_MASK, vals[3], d));
-  if (lane == 0)
-    for (int c = 0; c < 4; ++c) red[c][w] = vals[c];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double tot[4] = {0, 0, 0, 0};
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) {
-      tot[0] += red[0][i];
-      tot[1] += red[1][i];
-      tot[2] += red[2][i];
-      tot[3] = fmax(tot[3], red[3][i]);
+  for (int i = 0; i < PER; ++i) {
+    const int e = 32 * i + lane;
+    x[i] = e < RED_BLOCKS && (w == 0 || with_step) ? partial[w * RED_BLOCKS + e] : 0.0;
+  }
+  if (w < FIN_WARPS - 1) {
+    double a = x[0], b = x[1];
+#pragma unroll
+    for (int i = 2; i < PER; i += 2) {
+      a += x[i];
+      if (i + 1 < PER) b += x[i + 1];
     }
+    a += b;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) a += __shfl_xor_sync(FULL_MASK, a, d);
+    if (lane == 0) red[w] = a;
+  } else {
+    unsigned long long b = 0;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const unsigned long long o = (unsigned long long)__double_as_longlong(x[i]);
+      b = o > b ? o : b;
+    }
+    b = warp_max_bits(__longlong_as_double((long long)b));
+    if (lane == 0) red[w] = __longlong_as_double((long long)b);
+  }
+  __syncthreads();
+  if (w != 0) return;
+  // |dx|^2 = |dp|^2 + |dc|^2 in lane 0, |x|^2 in lane 1: one square root for both
+  const double root = sqrt(lane == 0 ? red[1] + red[3] : red[2] + red[4]);
+  const double xn = __shfl_sync(FULL_MASK, root, 1);
+  if (lane == 0) {
     if (!with_step) {
-      st->F = tot[0];
-      st->info.F_before = tot[0];
+      st->F = red[0];
+      st->info.F_before = red[0];
       return;
     }
-    double Fn = tot[0];
+    double Fn = red[0];
     const double F = st->F;
     const double lam = st->lambda_used;
     if (st->failed > 0 || st->nonfinite || !isfinite(Fn)) Fn = __longlong_as_double(0x7ff0000000000000ll);
-    const double grad = fmax(tot[3], __longlong_as_double((long long)st->grad_max_bits));
-    const double dxn = sqrt(tot[1]), xn = sqrt(tot[2]);
+    const double grad = fmax(red[5], __longlong_as_double((long long)st->grad_max_bits));
+    const double dxn = root;
     int stop = 0;
     if (s.ftol > 0 && F > 0 && fabs(F - Fn) / F < s.ftol) stop = 1;
     if (s.gtol > 0 && grad < s.gtol) stop = 1;
@@ -1170,6 +1201,7 @@ __global__ void __launch_bounds__(1024) k_finalize(DevProblem P, const real* vgr
 template <typename real>
 __global__ void k_apply(int m, int n, int q, const double* dc, const double* dp, double* cams, double* pts,
                         const real* r_cand, real* r_cur, const DevState* st) {
+  chain_begin();
   if (!st->info.accepted) return;
   const int total = 9 * m + 3 * n;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
@@ -1184,15 +1216,15 @@ __global__ void k_apply(int m, int n, int q, const double* dc, const double* dp,
 // ------------------------------------------------------------------------------------------------------
 // launchers
 template <typename real>
-void launch_point_update(const DevProblem& P, Scratch<real> W, cudaStream_t stream) {
-  k_point_update<real><<<RED_BLOCKS, RED_THREADS, 0, stream>>>(P, W.pt_info, W.t_acc, W.dc, W.vgrad, W.dp,
-                                                               W.partial);
+void launch_point_update(const DevProblem& P, Scratch<real> W, float* pt_df, cudaStream_t stream) {
+  launch_after(chained(P), k_point_update<real>, RED_BLOCKS, RED_THREADS, stream, P, W.pt_info, W.t_acc, W.dc, W.vgrad, W.dp,
+               reinterpret_cast<float2*>(pt_df), W.partial);
 }
 
 template <typename real>
-void launch_finalize(const DevProblem& P, Scratch<real> W, DevState* st, const Settings& s, int with_step,
+void launch_finalize(const DevProblem& P, const double* partial, DevState* st, const Settings& s, int with_step,
                      cudaStream_t stream) {
-  k_finalize<real><<<1, 1024, 0, stream>>>(P, W.vgrad, W.dc, W.partial, st, s, with_step);
+  launch_after(chained(P), k_finalize<real>, 1, 32 * FIN_WARPS, stream, partial, st, s, with_step);
 }
 
 template <typename real>
@@ -1201,58 +1233,110 @@ void launch_apply(const DevProblem& P, const double* dc, const double* dp, doubl
   int total = std::max(9 * P.m + 3 * P.n, 2 * P.q);
   int blocks = (total + 255) / 256;
   if (blocks > 2048) blocks = 2048;
-  k_apply<real><<<blocks, 256, 0, stream>>>(P.m, P.n, P.q, dc, dp, cams, pts, r_cand, r_cur, st);
+  launch_after(chained(P), k_apply<real>, blocks, 256, stream, P.m, P.n, P.q, dc, dp, cams, pts, r_cand, r_cur, st);
 }
 
 template <typename real>
 void launch_point_rhs(const DevProblem& P, Scratch<real> W, cudaStream_t stream) {
   int blocks = (P.q + 255) / 256;
-  k_point_rhs<real><<<blocks, 256, 0, stream>>>(P, W.edc, W.t_acc);
+  launch_after(chained(P), k_point_rhs<real>, blocks, 256, stream, P, W.edc, W.t_acc);
 }
 
 template <typename real>
-void launch_cost(const DevProblem& P, const double* dc, const double* dp, double* rt, float* cam_df, float* pt_df,
+void launch_cost_cams(const DevProblem& P, const double* dc, double* rt, float* cam_df, cudaStream_t stream) {
+  k_cost_cams<real><<<(P.m + 31) / 32, 32, 0, stream>>>(P.m, P.cams, dc, rt, cam_df);
+}
+
+// FP32 working precision: always the double-float kernels (cam_df, pt_df and the double-float observations are
+// required; the FP64 observations are not kept in that mode)
+template <typename real>
+void launch_cost(const DevProblem& P, const double* dp, const double* rt, const float* cam_df, const float* pt_df,
                  double* partial, DevState* st, real* rout, cudaStream_t stream) {
-  k_cam_rt<<<(P.m + 127) / 128, 128, 0, stream>>>(P.m, P.cams, dc, rt);
-  // FP32 working precision: always the double-float kernels (cam_df, pt_df and the double-float observations
-  // are required; the FP64 observations are not kept in that mode); dc, dp null: F(x) itself
-  if constexpr (sizeof(real) == 4) {
-    k_cam_df<<<(P.m + 127) / 128, 128, 0, stream>>>(P.m, rt, cam_df);
-    k_point_df<<<std::min((3 * P.n + 255) / 256, 2048), 256, 0, stream>>>(P.n, P.pts, dp, pt_df);
-    k_cost_df<<<RED_BLOCKS, RED_THREADS, 0, stream>>>(P, cam_df, pt_df, partial, st, (float*)rout);
-  } else {
+  if constexpr (sizeof(real) == 4)
+    k_cost_df<<<RED_BLOCKS, RED_THREADS, 0, stream>>>(P, cam_df, pt_df, partial, st, rout);
+  else
     k_cost<real><<<RED_BLOCKS, RED_THREADS, 0, stream>>>(P, rt, dp, partial, st, rout);
-  }
 }
 
-
-// Once per linearisation: the camera tables (blocks 0 .. cam_blocks - 1, one warp each: the FP64 sincos and
-// divisions of a camera run at 1/64 rate, so 32 cameras per SM) and, in mixed precision, the FP32 copies of the
-// cameras and points (the other blocks).
 template <typename real>
-__global__ void __launch_bounds__(256) k_params(int m, int n, int cam_blocks, const double* __restrict__ cams,
-                                                const double* __restrict__ pts, real* __restrict__ ctab,
-                                                float* __restrict__ cams_f, float* __restrict__ pts_f) {
+void launch_cost_x(const DevProblem& P, double* rt, float* cam_df, float* pt_df, double* partial, DevState* st,
+                   real* rout, cudaStream_t stream) {
+  launch_cost_cams<real>(P, nullptr, rt, cam_df, stream);
+  if constexpr (sizeof(real) == 4)
+    k_point_df<<<(int)std::min<int64_t>((3 * (int64_t)P.n + 255) / 256, 2048), 256, 0, stream>>>(
+        P.n, P.pts, reinterpret_cast<float2*>(pt_df));
+  launch_cost<real>(P, nullptr, rt, cam_df, pt_df, partial, st, rout, stream);
+}
+
+// The camera step from the padded cluster vectors x, in the cameras' order, with E dc (edc, if given) and the
+// count of failed clusters (st, if given).  sharded: another process's clusters give zeros (their steps arrive
+// by the exchange of dc).  One launch for what were three (5.2 + 3.5 + 2.8 us at 1000 cameras, 4.5 us now).
+template <typename real>
+__global__ void __launch_bounds__(256) k_scatter_step(DevProblem P, const double* __restrict__ x,
+                                                      const int* __restrict__ fail_flags, DevState* st,
+                                                      const real* __restrict__ ctab, double* __restrict__ dc,
+                                                      real* __restrict__ edc) {
+  chain_begin();
+  const int k = blockIdx.x;
+  const int i = blockIdx.y * blockDim.x + threadIdx.x;
+  if (st && i == 0 && fail_flags[k] != 0) atomicAdd(&st->failed, 1);
+  if (i >= P.cluster_n[k]) return;
+  const int cam = P.cluster_cams[P.cluster_cam_off[k] + i / 9], c = i % 9;
+  const bool own = !P.sharded || P.cluster_owned[k];
+  const double* xc = x + P.v_off[k] + (i - c);
+  dc[9 * (size_t)cam + c] = own ? xc[c] : 0.0;
+  if (edc) edc[(size_t)VPI * cam + c] = step_entry(jl_ptr(ctab, P.m, cam), xc, c);
+}
+
+template <typename real>
+void launch_scatter_step(const DevProblem& P, const double* x, const int* fail_flags, int max_np, DevState* st,
+                         double* dc, real* edc, cudaStream_t stream) {
+  const real* ctab;
+  if constexpr (sizeof(real) == 4) ctab = P.ctab_f; else ctab = P.ctab_d;
+  launch_after(chained(P), k_scatter_step<real>, dim3(P.l, (max_np + 255) / 256), 256, stream, P, x, fail_flags, st, ctab, dc, edc);
+}
+
+// The start of an iteration in one launch: the device state, the camera tables (blocks 0 .. cam_blocks - 1, one
+// warp each: the FP64 sincos and divisions of a camera run at 1/64 rate, so 32 cameras per SM), in mixed
+// precision the FP32 copies of the cameras and points, the zeros of the virtual-point accumulators (9 nv reals,
+// nv from the device counter) and of the vectors in Z (the other blocks).  Two kernels, a zeroing kernel and
+// four memsets in a row before: linearisation stage 28 -> 17 us at 10 cameras.
+template <typename real>
+__global__ void __launch_bounds__(256) k_begin(int m, int n, int cam_blocks, const double* __restrict__ cams,
+                                               const double* __restrict__ pts, real* __restrict__ ctab,
+                                               float* __restrict__ cams_f, float* __restrict__ pts_f, DevState* st,
+                                               Settings s, real* __restrict__ vp_acc,
+                                               const long long* __restrict__ counts, ZeroList Z) {
+  chain_begin();
   if ((int)blockIdx.x < cam_blocks) {
     const int j = 32 * blockIdx.x + threadIdx.x;
     if (threadIdx.x < 32 && j < m) write_camtab<real>(cams + 9 * (size_t)j, m, j, ctab);
+    if (blockIdx.x == 0 && threadIdx.x == 32) reset_state(st, s);
     return;
   }
-  for (int64_t i = ((int64_t)blockIdx.x - cam_blocks) * blockDim.x + threadIdx.x; i < 9 * (int64_t)m + 3 * (int64_t)n;
-       i += ((int64_t)gridDim.x - cam_blocks) * blockDim.x) {
-    if (i < 9 * (int64_t)m)
-      cams_f[i] = (float)cams[i];
-    else
-      pts_f[i - 9 * (int64_t)m] = (float)pts[i - 9 * (int64_t)m];
+  const int64_t first = ((int64_t)blockIdx.x - cam_blocks) * blockDim.x + threadIdx.x;
+  const int64_t step = ((int64_t)gridDim.x - cam_blocks) * blockDim.x;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int64_t nz = (9 * counts[0] * (int64_t)sizeof(real) + 15) / 16;   // the buffer is padded to 16 bytes
+  for (int64_t i = first; i < nz; i += step) reinterpret_cast<float4*>(vp_acc)[i] = zero;
+#pragma unroll
+  for (int z = 0; z < ZeroList::N; ++z)
+    for (int64_t i = first; i < Z.words[z]; i += step) Z.p[z][i] = 0;
+  if (cams_f) {
+    for (int64_t i = first; i < 9 * (int64_t)m; i += step) cams_f[i] = (float)cams[i];
+    for (int64_t i = first; i < 3 * (int64_t)n; i += step) pts_f[i] = (float)pts[i];
   }
 }
 
 template <typename real>
-void launch_params(const DevProblem& P, real* ctab, float* cams_f, float* pts_f, cudaStream_t stream) {
+void launch_begin(const DevProblem& P, Scratch<real> W, real* ctab, float* cams_f, float* pts_f, DevState* st,
+                  const Settings& s, const long long* counts, const ZeroList& Z, cudaStream_t stream) {
   const int cam_blocks = (P.m + 31) / 32;
-  const int64_t total = 9 * (int64_t)P.m + 3 * (int64_t)P.n;
-  const int copy_blocks = cams_f ? (int)std::min<int64_t>((total + 255) / 256, 2048) : 0;
-  k_params<real><<<cam_blocks + copy_blocks, 256, 0, stream>>>(P.m, P.n, cam_blocks, P.cams, P.pts, ctab, cams_f, pts_f);
+  int64_t work = 9 * (int64_t)P.m + 3 * (int64_t)P.n;
+  for (int z = 0; z < ZeroList::N; ++z) work = std::max<int64_t>(work, Z.words[z]);
+  const int rest = (int)std::min<int64_t>((work + 255) / 256, 8 * (int64_t)num_sms());
+  k_begin<real><<<cam_blocks + rest, 256, 0, stream>>>(P.m, P.n, cam_blocks, P.cams, P.pts, ctab, cams_f, pts_f, st, s,
+                                                       W.vp_acc, counts, Z);
 }
 
 void configure_kernels(int max_np) {
@@ -1268,24 +1352,28 @@ void configure_kernels(int max_np) {
 }
 
 #define INSTANTIATE(real)                                                                                  \
-  template void launch_iter_begin<real>(DevState*, const Settings&, cudaStream_t);                        \
-  template void launch_params<real>(const DevProblem&, real*, float*, float*, cudaStream_t);              \
+  template void launch_begin<real>(const DevProblem&, Scratch<real>, real*, float*, float*, DevState*,    \
+                                   const Settings&, const long long*, const ZeroList&, cudaStream_t);     \
   template void launch_vp_reduce<real>(const DevProblem&, Scratch<real>, cudaStream_t);                   \
   template void launch_vp_finalize<real>(const DevProblem&, Scratch<real>, DevState*, const long long*,   \
                                          cudaStream_t, const double*);                                     \
   template void launch_pt_sums<real>(const DevProblem&, Scratch<real>, double*, cudaStream_t);              \
   template void launch_rcs_build<real>(const DevProblem&, Scratch<real>, CamSlots, PairChunks, real*,     \
                                        DevState*, cudaStream_t, cudaStream_t, cudaEvent_t, cudaEvent_t);  \
-  template void launch_point_update<real>(const DevProblem&, Scratch<real>, cudaStream_t);                \
-  template void launch_finalize<real>(const DevProblem&, Scratch<real>, DevState*, const Settings&, int,  \
+  template void launch_scatter_step<real>(const DevProblem&, const double*, const int*, int, DevState*,   \
+                                          double*, real*, cudaStream_t);                                  \
+  template void launch_point_update<real>(const DevProblem&, Scratch<real>, float*, cudaStream_t);        \
+  template void launch_finalize<real>(const DevProblem&, const double*, DevState*, const Settings&, int,  \
                                       cudaStream_t);                                                      \
   template void launch_step_rows<real>(const DevProblem&, const double*, real*, cudaStream_t);            \
   template void launch_point_rhs<real>(const DevProblem&, Scratch<real>, cudaStream_t);                  \
-  template void launch_cost<real>(const DevProblem&, const double*, const double*, double*, float*, float*, \
-                                  double*, DevState*, real*, cudaStream_t);                               \
+  template void launch_cost_cams<real>(const DevProblem&, const double*, double*, float*, cudaStream_t);  \
+  template void launch_cost<real>(const DevProblem&, const double*, const double*, const float*,          \
+                                  const float*, double*, DevState*, real*, cudaStream_t);                 \
+  template void launch_cost_x<real>(const DevProblem&, double*, float*, float*, double*, DevState*, real*, \
+                                    cudaStream_t);                                                        \
   template void launch_apply<real>(const DevProblem&, const double*, const double*, double*, double*,     \
-                                   const real*, real*, DevState*, cudaStream_t);                          \
-
+                                   const real*, real*, DevState*, cudaStream_t);
 
 INSTANTIATE(float)
 INSTANTIATE(double)

@@ -271,10 +271,6 @@ void launch_list_chunks(const PairChunks& B, const int* cam_cluster, const int* 
   k_chunk_list<<<g, 256, 0, stream>>>(n, B.flag, B.excl, const_cast<int*>(B.active));
 }
 
-void launch_zero_vp(void* vp_acc, const long long* counts, int real_bytes, cudaStream_t stream) {
-  k_zero_vp<<<2 * RED_BLOCKS, 256, 0, stream>>>(reinterpret_cast<float4*>(vp_acc), counts, real_bytes, 9);
-}
-
 void launch_zero_vp3(void* p, const long long* counts, int real_bytes, cudaStream_t stream) {
   k_zero_vp<<<2 * RED_BLOCKS, 256, 0, stream>>>(reinterpret_cast<float4*>(p), counts, real_bytes, 3);
 }
