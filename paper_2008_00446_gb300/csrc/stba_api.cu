@@ -546,10 +546,24 @@ stba_status set_clusters_host(stba_ctx* c, const std::vector<int>& cl) {
           panel.push_back(make_int2(k, kt));
           c->h_diag_count[kt]++;
         }
+    // FP64: a row tile in two halves, a CTA each, while the halves of the step's tiles fit on the SMs at once: the
+    // FP64 pipe of one SM bounds a panel CTA (with chol8_warp: factor stage of 4 clusters of 75 cameras 1894 ->
+    // 1454 us, of 3 clusters of 10 cameras 152 -> 113 us); beyond, they would queue for the SMs
+    int rows = 0;
+    for (int k = 0; k < l; ++k)
+      if (c->h_owned[k]) rows += std::max(c->h_np[k] / TF - kt, 0);
+    const bool halves = !c->f32f && 2 * rows <= num_sms();
     for (int k = 0; k < l; ++k) {
       const int ntk = c->h_np[k] / TF;
       if (ntk <= kt || !c->h_owned[k]) continue;   // sharded: the other processes' clusters
-      for (int i = c->split_panel ? kt + 1 : kt; i < ntk; ++i) panel.push_back(make_int2(k, i));
+      for (int i = c->split_panel ? kt + 1 : kt; i < ntk; ++i) {
+        if (halves && i > kt) {
+          panel.push_back(make_int2(k, i | (1 << 16)));
+          panel.push_back(make_int2(k, i | (2 << 16)));
+        } else {
+          panel.push_back(make_int2(k, i));
+        }
+      }
       for (int j = kt + 2; j < ntk; ++j) {   // column kt + 1 is updated by panel kt + 1 itself
         if (c->update_tc)   // tile pairs (i0, i0 + 1) x j, from the diagonal tile down
           for (int i0 = j; i0 < ntk; i0 += 2) update.push_back(make_int2(k, (i0 << 16) | j));

@@ -169,6 +169,52 @@ __device__ __forceinline__ void chol8(F (*Ad)[LDA], int b0, int row0, int nk, F*
   if (nboost && boosted) atomicAdd(boosted, nboost);
 }
 
+// The FP64 factorisation of the block by one warp: an FP64 instruction occupies the SM's pipe for 16 cycles whether
+// one lane or 32 need it, and one thread's 28 reciprocal roots, products and updates a column made chol8 the longest
+// part of a panel (53 us a panel of 4 clusters of 75 cameras; 34 with this, the diagonal product on its lower cells
+// only and row tiles in halves).  Lane 4 r + p holds entries (r, p) and (r, p + 4): two updates a column for the
+// whole block.  The same operations on every entry as in chol8, and its pivot rules.
+template <int LDA>
+__device__ __forceinline__ void chol8_warp(double (*Ad)[LDA], int b0, int row0, int nk, double* rinv, int* fail) {
+  const int lane = threadIdx.x & 31, r = lane >> 2, p = lane & 3;
+  double d0 = p <= r ? Ad[b0 + r][b0 + p] : 0.0, d1 = p + 4 <= r ? Ad[b0 + r][b0 + p + 4] : 0.0;
+  int bad = 0;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const double col = j < 4 ? d0 : d1;
+    double pv = __shfl_sync(FULL_MASK, col, 4 * j + (j & 3));
+    if (row0 + b0 + j >= nk) {
+      pv = 1.0;
+    } else if (!(isfinite(pv) && pv > 0.0)) {
+      bad = 1;
+      pv = 1.0;
+    }
+    const double is = rsqrt_w(pv);
+    // L_rj of this lane's row, and L_cj for its two columns c
+    const double rj = __shfl_sync(FULL_MASK, col, (lane & ~3) | (j & 3));
+    const double lr = (r == j ? pv : rj) * is;
+    const double l0 = __shfl_sync(FULL_MASK, lr, 4 * p), l1 = __shfl_sync(FULL_MASK, lr, 4 * p + 16);
+    if (lane == 0) rinv[j] = is;
+    if (p == (j & 3) && r >= j) {
+      if (j < 4) d0 = lr; else d1 = lr;
+    }
+    if (j < 3 && p > j) d0 -= lr * l0;
+    if (p + 4 > j) d1 -= lr * l1;
+  }
+  if (p <= r) Ad[b0 + r][b0 + p] = d0;
+  if (p + 4 <= r) Ad[b0 + r][b0 + p + 4] = d1;
+  if (bad && lane == 0) *fail = 1;
+}
+
+// the block's factorisation by warp 0 (FP32: by its first thread); called by the whole warp
+template <typename F, int LDA>
+__device__ __forceinline__ void chol8_warp0(F (*Ad)[LDA], int b0, int row0, int nk, F* rinv, int* fail, int* boosted) {
+  if constexpr (sizeof(F) == 8)
+    chol8_warp<LDA>(Ad, b0, row0, nk, rinv, fail);
+  else if (threadIdx.x == 0)
+    chol8<F, LDA>(Ad, b0, row0, nk, rinv, fail, boosted);
+}
+
 // ------------------------------------------------------------------------------------------------------
 // Panel of tile step kt, one CTA per tile row i >= kt of a cluster (512 threads: the diagonal tile's work on
 // threads 0..255, the row tile's on threads 256..511, wherever the two are independent):
@@ -203,15 +249,27 @@ __global__ void __launch_bounds__(PANEL_THREADS) k_chol_panel(F* L, F* Ldiag, De
   F(*LiT)[LDV] = LkT + T;
   __shared__ F rinv2[2][8];   // reciprocal pivots of block b in rinv2[b & 1]
   const int2 it = items[blockIdx.x];
-  const int k = it.x, i = it.y;
+  const int k = it.x, i = it.y & 0xffff, part = it.y >> 16;   // part: 0 the whole row tile, 1 or 2 its upper or lower half
   const bool diag = (i == kt);
+  const int x0 = part == 2 ? T / 2 : 0, xrows = diag ? 0 : part ? T / 2 : T;   // rows of the row tile in this CTA
   const int np = P.cluster_np[k], nk = P.cluster_n[k];
   F* A = L + P.S_off[k];
   const int tid = threadIdx.x;
-  // fused update: threads 0..255 form the diagonal tile's product, threads 256..511 the row tile's
-  const int half = tid >> 8, bi = tid & 15, bj = (tid & 255) >> 4;
+  // R x R cells of a product: threads 0..255 take the diagonal tile's lower ones, threads 256..511 the row tile's
+  const int half = tid >> 8, nci = xrows / R;
+  int bi = 0, bj = 0;
+  bool cell_act;
+  if (half == 0) {
+    while ((bi + 1) * (bi + 2) / 2 <= tid) ++bi;
+    bj = tid - bi * (bi + 1) / 2;
+    cell_act = bi < 16;
+  } else {
+    bi = nci ? (tid & 255) % nci : 0;
+    bj = nci ? (tid & 255) / nci : 16;
+    cell_act = bj < 16;
+  }
   const size_t base_kk = (size_t)(kt * T) * np + kt * T;
-  const size_t base_ik = (size_t)(i * T) * np + kt * T;
+  const size_t base_ik = (size_t)(i * T + x0) * np + kt * T;
   // 1. loads; the upper part of the diagonal tile is never stored, so it is set to zero
   for (int idx = tid; idx < T * T; idx += PANEL_THREADS) {
     const int r = idx / T, c = idx - (idx / T) * T;
@@ -219,17 +277,17 @@ __global__ void __launch_bounds__(PANEL_THREADS) k_chol_panel(F* L, F* Ldiag, De
       cp_async_elem(&Ad[r][c], A + base_kk + (size_t)r * np + c);
     else
       Ad[r][c] = F(0);
-    if (!diag) cp_async_elem(&Ax[r][c], A + base_ik + (size_t)r * np + c);
+    if (r < xrows) cp_async_elem(&Ax[r][c], A + base_ik + (size_t)r * np + c);
     if (kt > 0) {
       cp_async_elem(&LkT[c][r], A + base_kk - T + (size_t)r * np + c);
-      if (!diag) cp_async_elem(&LiT[c][r], A + base_ik - T + (size_t)r * np + c);
+      if (r < xrows) cp_async_elem(&LiT[c][r], A + base_ik - T + (size_t)r * np + c);
     }
   }
   cp_async_wait_all();
   __syncthreads();
   if (kt > 0) {
     // half 0: A_kt,kt -= L_kt,kt-1 L_kt,kt-1^T (lower part); half 1: A_i,kt -= L_i,kt-1 L_kt,kt-1^T
-    if (half == 0 || !diag) {
+    if (cell_act) {
       F acc[R][R];
 #pragma unroll
       for (int a = 0; a < R; ++a)
@@ -263,14 +321,14 @@ __global__ void __launch_bounds__(PANEL_THREADS) k_chol_panel(F* L, F* Ldiag, De
   //    applies block b's rank-8 update to the next 8 x 8 diagonal block and lane 0 factors it, while warps
   //    1..7 apply the update to the rest of the diagonal tile and warps 8..15 to the row tile (look-ahead
   //    of one block).
-  if (tid == 0) chol8<F, LDA>(Ad, 0, kt * T, nk, rinv2[0], fail_flags + k, diag ? boosted : nullptr);
+  if (tid < 32) chol8_warp0<F, LDA>(Ad, 0, kt * T, nk, rinv2[0], fail_flags + k, diag ? boosted : nullptr);
   __syncthreads();
   for (int b = 0; b < NB; ++b) {
     const int b0 = 8 * b;
     const F* rinv = rinv2[b & 1];
     // block column below the diagonal block: L_rb L_bb^T = A_rb, one row per thread (Ad rows, then Ax rows)
     const int rows_d = T - b0 - 8;
-    const int rows_tot = rows_d + (diag ? 0 : T);
+    const int rows_tot = rows_d + xrows;
     if (tid < rows_tot) {
       F* row = (tid < rows_d) ? &Ad[b0 + 8 + tid][0] : &Ax[tid - rows_d][0];
       F o8[8];
@@ -299,15 +357,15 @@ __global__ void __launch_bounds__(PANEL_THREADS) k_chol_panel(F* L, F* Ldiag, De
         Ad[n0 + rr][n0 + cc] -= s;
       }
       __syncwarp();
-      if (tid == 0) chol8<F, LDA>(Ad, n0, kt * T, nk, rinv2[(b + 1) & 1], fail_flags + k, diag ? boosted : nullptr);
+      chol8_warp0<F, LDA>(Ad, n0, kt * T, nk, rinv2[(b + 1) & 1], fail_flags + k, diag ? boosted : nullptr);
     } else {
       // rank-8 update of the other columns right of the block, register-blocked R x R cells: warps 1..7
       // take the diagonal tile's cells, warps 8..15 the row tile's
       const bool xpart = tid >= 256;
-      for (int cell = xpart ? tid - 256 : tid - 32; cell < 256; cell += xpart ? 256 : 224) {
-        const int ci = cell & 15, cj = cell >> 4;
+      for (int cell = xpart ? tid - 256 : tid - 32; cell < (xpart ? 16 * nci : 256); cell += xpart ? 256 : 224) {
+        const int ci = xpart ? cell % nci : cell & 15, cj = xpart ? cell / nci : cell >> 4;
         const int c0 = cj * R, r0 = ci * R;
-        if (c0 + R <= n0 || (xpart && diag)) continue;
+        if (c0 + R <= n0) continue;
         F lc[R][8];
 #pragma unroll
         for (int cc = 0; cc < R; ++cc)
@@ -362,7 +420,7 @@ __global__ void __launch_bounds__(PANEL_THREADS) k_chol_panel(F* L, F* Ldiag, De
     }
     return;
   }
-  for (int idx = tid; idx < T * T; idx += PANEL_THREADS) {
+  for (int idx = tid; idx < xrows * T; idx += PANEL_THREADS) {
     const int r = idx / T, c = idx - (idx / T) * T;
     A[base_ik + (size_t)r * np + c] = Ax[r][c];
   }
@@ -456,7 +514,7 @@ __device__ __forceinline__ void factor_diag_tile(F (*Ad)[T + 1], F (*rinv2)[8], 
                                                  int* boosted) {
   constexpr int R = T / 16, LDA = T + 1, NB = T / 8;
   const int tid = threadIdx.x;
-  if (tid == 0) chol8<F, LDA>(Ad, 0, row0, nk, rinv2[0], fail, boosted);
+  if (tid < 32) chol8_warp0<F, LDA>(Ad, 0, row0, nk, rinv2[0], fail, boosted);
   __syncthreads();
   for (int b = 0; b < NB; ++b) {
     const int b0 = 8 * b;
@@ -489,7 +547,7 @@ __device__ __forceinline__ void factor_diag_tile(F (*Ad)[T + 1], F (*rinv2)[8], 
         Ad[n0 + rr][n0 + cc] -= s;
       }
       __syncwarp();
-      if (tid == 0) chol8<F, LDA>(Ad, n0, row0, nk, rinv2[(b + 1) & 1], fail, boosted);
+      chol8_warp0<F, LDA>(Ad, n0, row0, nk, rinv2[(b + 1) & 1], fail, boosted);
     } else {
       for (int cell = tid - 32; cell < 256; cell += 224) {
         const int ci = cell & 15, cj = cell >> 4;

@@ -61,3 +61,24 @@ def test_solve_at_the_shared_memory_limit(m):
     x = dc.ravel()
     e = np.abs(S @ x - b).max() / (np.abs(S) @ np.abs(x) + np.abs(b)).max()
     assert e < 1e-8, e
+
+
+@pytest.mark.parametrize("sizes", [[1, 3, 4, 7, 8, 11, 14, 15], [3], [4], [7], [8], [300], [160, 150]])
+def test_fp64_panels_at_tile_edges(sizes):
+    """FP64 panels of 32 columns, a row tile per CTA or, while twice a step's tiles fit on the SMs, half a tile: clusters
+    of 1 to 5 tiles around the tile edges, one of 85 tiles and two of 45 and 43, which begin with whole tiles and go
+    over to halves.  Bar 1e-10 of each camera row: condition below 250 (of the system with unit diagonal, which the
+    reference solves too) x 2700 roundings of 1.1e-16."""
+    m = sum(sizes)
+    cl = np.repeat(np.arange(len(sizes)), sizes).astype(np.int32)
+    s = scenes.make_tiny_scene(m=m, n=max(30 * min(m, 20), 4), seed=m, clusters=cl, drop=0.5 if m < 100 else 0.9)
+    with stba.stba_create(s.cameras, s.points, s.obs_cam, s.obs_pt, s.obs_uv, cl, lambda0=0.09,
+                          precision=stba.STBA_FP64) as ctx:
+        info = stba.stba_lm_iteration(ctx)
+        assert info["failed_clusters"] == 0
+        dc, _ = stba.stba_last_step(ctx)
+        for k in range(len(sizes)):
+            S, b = stba.stba_get_cluster_system(ctx, k)
+            d = 1 / np.sqrt(np.diag(S))
+            e = rows(dc[cl == k].ravel(), d * np.linalg.solve(S * d[:, None] * d, b * d), 9)
+            assert e < 1e-10, (k, sizes[k], e)
