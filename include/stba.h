@@ -205,7 +205,8 @@ stba_status stba_last_step(stba_ctx* ctx, double* dc, double* dp);
  * the context) and, after it, its record (damping, accept flag, correction flag), with the cluster
  * assignment it used.  It also allocates the reverse pass's buffers (about 184 q + 216 m + 96 n bytes of
  * device memory), so that stba_adjoint allocates nothing.  A further iteration returns STBA_ERR_STATE;
- * stba_record restarts the tape and max_iter = 0 frees it (the buffers with it).  Errors:
+ * stba_record restarts the tape (in the buffers that it has, when they hold max_iter iterations and
+ * no more than four times as many) and max_iter = 0 frees it (the buffers with it).  Errors:
  * STBA_ERR_INVALID_ARG (max_iter < 0), STBA_ERR_OOM (the tape or the buffers do not fit; nothing is then
  * recorded). */
 stba_status stba_record(stba_ctx* ctx, int32_t max_iter);

@@ -129,7 +129,7 @@ struct stba_ctx {
 
   // tape of recorded iterations for stba_adjoint: x_t before every iteration, its record after it, and
   // the cluster assignment it used
-  int tape_cap = 0, tape_len = 0;
+  int tape_cap = 0, tape_len = 0, tape_alloc = 0;   // iterations it may hold, holds, has room for
   bool tape_broken = false;             // parameters or damping were replaced between recorded iterations
   double* tape_x = nullptr;             // [tape_cap][9m + 3n]
   stba_iter_info* tape_info = nullptr;  // [tape_cap]
@@ -1096,16 +1096,21 @@ stba_status run_iteration(stba_ctx* c) {
   return STBA_OK;
 }
 
+void reset_tape(stba_ctx* c) {
+  c->tape_cap = c->tape_len = 0;
+  c->tape_broken = false;
+  c->tape_clusters.clear();
+  c->tape_cluster_id.clear();
+}
+
 void free_tape(stba_ctx* c) {
   free_list(c, c->tape_allocs);
   c->tape_x = nullptr;
   c->tape_info = nullptr;
   c->adj = AdjointBuffers{};
   c->adj_save_x = nullptr;
-  c->tape_cap = c->tape_len = 0;
-  c->tape_broken = false;
-  c->tape_clusters.clear();
-  c->tape_cluster_id.clear();
+  c->tape_alloc = 0;
+  reset_tape(c);
 }
 
 template <typename real>
@@ -1950,6 +1955,13 @@ stba_status stba_last_step(stba_ctx* c, double* dc, double* dp) {
 stba_status stba_record(stba_ctx* c, int32_t max_iter) {
   if (!c || max_iter < 0) return STBA_ERR_INVALID_ARG;
   CK(cudaStreamSynchronize(c->stream));
+  // a tape at least as long and at most four times as long is used again: its 12 allocations and frees took
+  // 690 us of a recording's 8.5 ms (500 cameras, four iterations and their adjoint)
+  if (max_iter > 0 && c->tape_alloc >= max_iter && c->tape_alloc / 4 <= max_iter) {
+    reset_tape(c);
+    c->tape_cap = max_iter;
+    return STBA_OK;
+  }
   free_tape(c);
   if (max_iter == 0) return STBA_OK;
   const size_t nx = 9 * (size_t)c->m + 3 * (size_t)c->n;
@@ -1973,7 +1985,7 @@ stba_status stba_record(stba_ctx* c, int32_t max_iter) {
     free_tape(c);
     return s;
   }
-  c->tape_cap = max_iter;
+  c->tape_cap = c->tape_alloc = max_iter;
   return STBA_OK;
 }
 
