@@ -80,7 +80,6 @@ struct stba_ctx {
 
   // device arrays
   double *cams = nullptr, *pts = nullptr, *obs_uv = nullptr;
-  float* obs_uvf = nullptr;
   int *obs_cam = nullptr, *obs_vp = nullptr, *obs_pt = nullptr, *obs_perm = nullptr, *obs_base = nullptr;
   int *vp_off = nullptr, *vp_point = nullptr, *pt_vp_off = nullptr, *pt_off = nullptr;
   int *cam_local = nullptr, *cam_cluster = nullptr, *cluster_cams = nullptr, *cluster_cam_off = nullptr;
@@ -265,7 +264,6 @@ DevProblem dev_problem(const stba_ctx* c) {
   P.obs_pt = c->obs_pt;
   P.obs_base = c->obs_base;
   P.obs_uv = c->obs_uv;
-  P.obs_uvf = c->obs_uvf;
   P.obs_uvdf = c->obs_uvdf;
   P.cams_f = c->cams_f;
   P.pts_f = c->pts_f;
@@ -348,7 +346,7 @@ stba_status refresh_counts(stba_ctx* c) {
   CK(cudaMemcpyAsync(h, c->counts, sizeof h, cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   c->nv = (int)h[0];
-  c->n_pairs = h[1];
+  c->n_pairs = h[1] / 2;   // counted from both ends
   c->counts_known = true;
   return STBA_OK;
 }
@@ -391,11 +389,10 @@ static stba_status launch_reorder_graph(stba_ctx* c, const ReorderArgs& A, bool 
     CK(cudaGetLastError());
     return STBA_OK;
   }
-  // the argument bytes: ReorderArgs (padding after its three ints cleared) and the other arguments
-  static_assert(offsetof(ReorderArgs, obs_pt) == 16, "ReorderArgs: three ints, then pointers");
+  // the argument bytes: ReorderArgs and the other arguments
+  static_assert(offsetof(ReorderArgs, obs_pt) == 16, "ReorderArgs: four ints, then pointers: no padding");
   std::vector<unsigned char> key(sizeof(ReorderArgs));
   std::memcpy(key.data(), &A, sizeof A);
-  std::memset(key.data() + 12, 0, 4);
   const void* more[] = {c->key, c->tile_sum, c->counts, carry ? c->res_cur : nullptr, c->res_cand,
                         c->pchunks.chunks, c->pchunks.active, c->pchunks.nactive, c->pchunks.flag,
                         c->pchunks.excl, c->pchunks.tile_sum, c->cam_cluster, c->cl_owned};
@@ -1682,7 +1679,6 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
     const size_t Q = (size_t)q;
     std::vector<int> base_cam(Q), base_src(Q), base_pt(Q);
     std::vector<double> base_uv(2 * Q);
-    std::vector<float> base_uvf(c->mixed ? 2 * Q : 0);
     std::vector<float4> base_uvdf(c->mixed ? Q : 0);
     for (size_t bo = 0; bo < Q; ++bo) {
       const int src = c->base_order[bo];
@@ -1694,8 +1690,6 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
       base_uv[2 * bo + 1] = v;
       if (c->mixed) {
         const float uh = (float)u, vh = (float)v;
-        base_uvf[2 * bo] = uh;
-        base_uvf[2 * bo + 1] = vh;
         base_uvdf[bo] = make_float4(uh, (float)(u - (double)uh), vh, (float)(v - (double)vh));
       }
     }
@@ -1747,16 +1741,11 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
     if ((s = dalloc(c, &d_nsing, Q)) != STBA_OK) return bail(s);
     if ((s = upload(c, &d_cam_warp_off, cam_warp_off)) != STBA_OK) return bail(s);
     if ((s = upload(c, &d_warp_cam, warp_cam)) != STBA_OK) return bail(s);
-    A.base_uvf = nullptr;
     A.base_uvdf = nullptr;
     if (c->mixed) {
-      float* d_uvf;
       float4* d_uvdf;
-      if ((s = upload(c, &d_uvf, base_uvf)) != STBA_OK) return bail(s);
       if ((s = upload(c, &d_uvdf, base_uvdf)) != STBA_OK) return bail(s);
-      A.base_uvf = d_uvf;
       A.base_uvdf = d_uvdf;
-      if ((s = dalloc(c, &c->obs_uvf, 2 * Q)) != STBA_OK) return bail(s);
       if ((s = dalloc(c, &c->obs_uvdf, Q)) != STBA_OK) return bail(s);
     }
     int* const* ints_q[] = {&c->obs_cam, &c->obs_vp, &c->obs_perm, &c->obs_base, &c->vp_point, &c->inv[0], &c->inv[1],
@@ -1770,7 +1759,7 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
     if (!c->mixed && (s = dalloc(c, &c->obs_uv, 2 * Q)) != STBA_OK) return bail(s);
     if ((s = dalloc(c, &d_cam_obs, Q)) != STBA_OK) return bail(s);
     if ((s = dalloc(c, &d_slots, 32 * (size_t)nwarps)) != STBA_OK) return bail(s);
-    if ((s = dalloc(c, &c->tile_sum, Q / 2048 + 2)) != STBA_OK) return bail(s);
+    if ((s = dalloc(c, &c->tile_sum, reorder_tiles(q))) != STBA_OK) return bail(s);
     if ((s = dalloc(c, &c->counts, 4)) != STBA_OK) return bail(s);   // nv, pairs, singles, active chunks
     // failure flags at their largest size (l <= m); the other cluster arrays live in the assignment blob
     if ((s = dalloc(c, &c->fail_flags, (size_t)m)) != STBA_OK) return bail(s);
@@ -1813,6 +1802,7 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
     c->rowbuf = gb;
     A.base_vp = nullptr;   // read by a pair pass that recomputes its rows
     if (c->pair_recompute && !c->use_pcg && !c->use_spcg && (s = dalloc(c, &A.base_vp, Q)) != STBA_OK) return bail(s);
+    A.max_cam_obs = *std::max_element(c->h_cam_nobs.begin(), c->h_cam_nobs.end());
     A.obs_pt = c->obs_pt;
     A.pt_off = c->pt_off;
     A.base_cam = d_base_cam;
@@ -1823,7 +1813,6 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
     A.obs_cam = c->obs_cam;
     A.obs_perm = c->obs_perm;
     A.obs_uv = c->obs_uv;
-    A.obs_uvf = c->obs_uvf;
     A.obs_uvdf = c->obs_uvdf;
     A.obs_vp = c->obs_vp;
     A.vp_off = c->vp_off;

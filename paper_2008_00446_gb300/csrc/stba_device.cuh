@@ -41,19 +41,6 @@ inline void launch_after(bool chain, void (*kern)(KA...), dim3 grid, int block, 
 }
 
 template <typename real>
-__device__ __forceinline__ void load_uv(const DevProblem& P, int o, real& u, real& v) {
-  if constexpr (sizeof(real) == 8) {
-    double2 t = reinterpret_cast<const double2*>(P.obs_uv)[o];
-    u = t.x;
-    v = t.y;
-  } else {
-    float2 t = reinterpret_cast<const float2*>(P.obs_uvf)[o];
-    u = t.x;
-    v = t.y;
-  }
-}
-
-template <typename real>
 __device__ __forceinline__ void load_point(const double* p, real X[3]) {
   X[0] = (real)p[0];
   X[1] = (real)p[1];

@@ -28,7 +28,6 @@ struct DevProblem {
   const int* obs_pt;       // [q] point of each sorted observation
   const int* obs_base;     // [q] position of each sorted observation in the (point, camera) order
   const double* obs_uv;    // [q][2] FP64 observations (FP64 mode only; null in mixed precision)
-  const float* obs_uvf;    // [q][2] FP32 copy (mixed precision)
   const float4* obs_uvdf;  // [q] double-float copy (u_hi, u_lo, v_hi, v_lo) (mixed precision)
   const int* vp_off;       // [nv+1] observation range of each virtual point
   const int* vp_point;     // [nv] point of each virtual point
@@ -166,12 +165,12 @@ void sgc_sample_batch(const CameraGraph& g, int m, int gamma, double beta, uint6
 // Re-ordering for a new cluster assignment (stba_order.cu).  Base = the (point, camera) order of create.
 struct ReorderArgs {
   int q, n, m;
+  int max_cam_obs;          // the largest number of observations of a camera
   const int* obs_pt;        // [q] point of every position (the same in both orders)
   const int* pt_off;        // [n+1]
   const int* base_cam;      // [q] camera, original index and observation of every base position
   const int* base_src;
   const double* base_uv;    // [q][2]
-  const float* base_uvf;    // [q][2] or null
   const float4* base_uvdf;  // [q] or null
   const int* cam_cluster;   // [m] the new assignment
   const int* inv_old;       // [q] new position of every base position under the previous assignment
@@ -179,7 +178,6 @@ struct ReorderArgs {
   int* start;               // [q] 1 where a virtual point starts
   int *obs_base, *obs_cam, *obs_perm;
   double* obs_uv;
-  float* obs_uvf;
   float4* obs_uvdf;
   int *obs_vp, *vp_off, *vp_point, *pt_vp_off;
   int* base_vp;             // [q] virtual point of every base position, for the pair pass, or null
@@ -187,7 +185,7 @@ struct ReorderArgs {
   const int* cam_base;      // [q]   their base positions, ascending
   const int* ecam;          // [q]   the camera of every entry of cam_base
   const int* ept;           // [q]   the point of every entry of cam_base
-  int2* slot_pv;            // CamSlots::pv (written by k_cam_place)
+  int2* slot_pv;            // CamSlots::pv (written with the camera lists)
   int* eo;                  // [q]   the new position of every entry of cam_base (scratch of the assignment)
   int* nsing;               // [q]   per base position: its new position, bit 31 set when its virtual point
                             //       has no other observation (scratch of the assignment)
@@ -195,8 +193,9 @@ struct ReorderArgs {
   int* cam_obs;             // [q] new positions, single-observation virtual points first
   int* slots;               // [32 * warps] the same padded to whole warps (-1)
 };
-// key: [q] scratch; tile_sum: [q / 2048 + 1] scratch; A.start: [2 (q + 1)]; counts: [3] -> number of virtual
-// points, number of camera-pair instances, number of single-observation virtual points.  With res_old, the residuals are carried over into res_new in the new order.
+// key: [q] scratch; tile_sum: [reorder_tiles(q)] scratch; A.start: [2 (q + 1)]; counts: [3] -> number of virtual
+// points, twice the number of camera-pair instances, scratch.  With res_old, the residuals are carried over into res_new in the new order.
+size_t reorder_tiles(int64_t q);
 template <typename real>
 void launch_reorder(const ReorderArgs& A, int* key, int* tile_sum, long long* counts, const real* res_old,
                     real* res_new, cudaStream_t stream);
