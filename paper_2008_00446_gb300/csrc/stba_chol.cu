@@ -22,8 +22,8 @@
 // FP64 iterative refinement that follows solves the unmodified system.  A non-finite pivot fails.
 //
 // Solves (k_tri_push): a thread-block cluster of CTAs per camera cluster; with the inverted diagonal tiles every
-// tile step is two parallel matrix-vector products.  Refinement: r = b - S x in FP64 over many CTAs (S symmetric, lower stored),
-// then x += D^-1/2 (L L^T)^-1 D^-1/2 r.
+// tile step is two parallel matrix-vector products.  Refinement: r = b - S x in FP64 over many CTAs (S symmetric,
+// lower stored), then x += D^-1/2 (L L^T)^-1 D^-1/2 r.
 #include <cooperative_groups.h>
 
 #include <map>
@@ -2005,7 +2005,6 @@ __global__ void __launch_bounds__(32 * RES_WARPS) k_residual(DevProblem P, const
   }
 }
 
-
 // ------------------------------------------------------------------------------------------------------
 // Host launchers
 
@@ -2171,7 +2170,8 @@ void launch_solve_t(const DevProblem& P, const double* S, const double* b, const
     if (s > 0) cudaMemcpyAsync(fb.r, b, (size_t)fb.v_total * sizeof(double), cudaMemcpyDeviceToDevice, stream);
     if (plan.n_res_items > 0) {
       if (s == 0)
-        launch_after(chained(P), k_residual<Sreal>, plan.n_res_items, 32 * RES_WARPS, stream, P, S, fb.x, fb.r, plan.res_items);
+        launch_after(chained(P), k_residual<Sreal>, plan.n_res_items, 32 * RES_WARPS, stream, P, S, fb.x, fb.r,
+                     plan.res_items);
       else
         k_residual<Sreal><<<plan.n_res_items, 32 * RES_WARPS, 0, stream>>>(P, S, fb.x, fb.r, plan.res_items);
     }

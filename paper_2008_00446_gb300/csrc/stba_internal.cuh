@@ -68,7 +68,7 @@ struct DevState {
   int failed;            // clusters whose factorisation failed this iteration
   int corrected;         // correction active this iteration
   int nonfinite;         // a non-positive depth was met in the cost at x + dx
-  unsigned pair_next;    // next chunk of the pair pass (zeroed by k_iter_begin)
+  unsigned pair_next;    // next chunk of the pair pass (zeroed by k_begin)
   int boosted;           // FP32 pivots raised by static pivoting this iteration
   stba_iter_info info;   // record of the last finished iteration
 };

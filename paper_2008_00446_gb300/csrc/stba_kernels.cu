@@ -1,5 +1,6 @@
 // Per-iteration kernels of the STBA LM step (Algorithm 1), except the dense cluster factorisation.
 //
+//   k_begin          the state, the camera tables (stba_camtab.cuh), FP32 copies and the zeros of an iteration.
 //   k_vp_reduce      per observation, warp-segmented by virtual point: V = sum Jp^T Jp, w' = -sum Jp^T f
 //                    (Eq. 10: C' and w' of the split points).
 //   k_pt_acc         per point (a warp per 32 points): C and w of the physical point, summed over its
@@ -10,9 +11,10 @@
 //   k_cam_pass       per camera (a warp per 32 of its observations): the diagonal blocks of S'_k, b' and the
 //                    camera gradient (Eq. 10/13).
 //   k_pair_build     per camera pair of the camera graph inside a cluster: the off-diagonal blocks of S'_k.
+//   k_scatter_step   dc in the cameras' order from the cluster solves, E dc, failed clusters.
 //   k_point_rhs      per observation, warp-segmented by point: sum_o Jp^T Jc dc.
-//   k_point_update   per point: dp = C^-1 (w - E^T dc) (Eq. 6 = Eq. 15).
-//   k_cost(_df)      F(x + dx) with FP64 sums; k_finalize: stop tests and the accept rule of Algorithm 1.
+//   k_point_update   per point: dp = C^-1 (w - E^T dc) (Eq. 6 = Eq. 15), sums of the stop tests.
+//   k_cost_cams, k_cost(_df)   F(x + dx) with FP64 sums; k_finalize: stop tests and the accept rule of Algorithm 1.
 //
 // Correction closed form: A has no camera columns and H~ = diag(H_lambda) is diagonal, so
 // nu = (A H~^-1 A^T)^-1 A H~^-1 g makes H~^-1 (g - A^T nu) the H~-weighted projection of H~^-1 g on the
@@ -550,8 +552,8 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 4 : 3) k_cam_pass(Dev
 // once, at create, by edge (x, y) and cut into chunks (pair_chunk); under a cluster assignment an edge
 // contributes exactly when both cameras are in one cluster (its two observations of a point are then in
 // one virtual point), and a chunk adds to one block only.  The re-ordering of an assignment lists the
-// chunks whose edge lies inside a cluster; the warps of a fixed grid take them one by one from that list.  A warp works on pieces of
-// PB_CH pairs: lane (side, j) forms the rows of its pair's observation by camera x (side 0) or y (side 1) from
+// chunks whose edge lies inside a cluster; the warps of a fixed grid take them one by one from that list.  A warp
+// works on pieces of PB_CH pairs: lane (side, j) forms the rows of its pair's observation by camera x (side 0) or y (side 1) from
 // the camera's table, the point and L_v^-1 (both lanes of a pair share them); the y lane takes Pm_x by shuffle
 // and forms M = Pm_x^T Pm_y (2x2) and M Jt_y (2x9).  The rows go to shared memory, and 27 lanes accumulate: lane
 // (g, rb, cb) takes every third pair (slot g) and the 3 x 3 sub-block (rb, cb), in FP32 as packed pairs of FMAs
@@ -1293,7 +1295,8 @@ void launch_scatter_step(const DevProblem& P, const double* x, const int* fail_f
                          double* dc, real* edc, cudaStream_t stream) {
   const real* ctab;
   if constexpr (sizeof(real) == 4) ctab = P.ctab_f; else ctab = P.ctab_d;
-  launch_after(chained(P), k_scatter_step<real>, dim3(P.l, (max_np + 255) / 256), 256, stream, P, x, fail_flags, st, ctab, dc, edc);
+  launch_after(chained(P), k_scatter_step<real>, dim3(P.l, (max_np + 255) / 256), 256, stream, P, x, fail_flags, st,
+               ctab, dc, edc);
 }
 
 // The start of an iteration in one launch: the device state, the camera tables (blocks 0 .. cam_blocks - 1, one
