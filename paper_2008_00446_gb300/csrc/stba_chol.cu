@@ -1653,7 +1653,10 @@ __global__ void __launch_bounds__(256) k_tri_solve(DevProblem P, const F* L, con
 // of the cluster's CS CTAs.  Forward, the owner of row k finishes t_k = r_k - sum_j L_kj y_j, forms y_k = D_k^-1 t_k and
 // sends it to every CTA with asynchronous stores counted by that CTA's mbarrier of step k; whoever has y_k subtracts
 // L_ik y_k from its rows i > k, row k + 1 first, whose owner then goes on to y_k+1 before its other rows.  The
-// backward pass is the same on reversed indices with L_ki^T and D_k^-T.  A step's chain is two 64 x 64 products by
+// backward pass is the same on reversed indices with L_ki^T and D_k^-T.  Only the mbarrier it counts on tells that an
+// asynchronous store has arrived (a cluster barrier orders its issue), so after a pass every CTA waits for all nt
+// pieces, the ones that none of its rows needs too: x overwrites y only once every y has arrived everywhere, and no
+// CTA leaves while a store to it is under way.  A step's chain is two 64 x 64 products by
 // 256 threads and one remote store: about 0.5 us, against 2.4 us with a cluster barrier, a gather of the partial
 // products from all CTAs and five block barriers per step.  Nothing depends on a tile's address on the vector, so
 // each thread keeps its elements of the next NB tiles in registers (loads in flight while it waits for y_k).
@@ -1746,7 +1749,10 @@ __global__ void __launch_bounds__(256, T == 64 ? 2 : 3) k_tri_push(DevProblem P,
   auto pass = [&](auto fwd_c) {
     constexpr bool FWD = decltype(fwd_c)::value;
     const int me = FWD ? rank : ((nt - 1 - rank) % CS + CS) % CS;   // this CTA's pass indices are me mod CS
-    if (nown == 0) return;
+    if (nown == 0) {
+      if constexpr (!FWD) cluster.barrier_wait();
+      return;
+    }
     const int last = me + CS * ((nt - 1 - me) / CS);
     // tasks: update of index i by the vector piece of index kk (i > kk), or the diagonal product of index i (diag)
     struct Task {
@@ -1804,6 +1810,7 @@ __global__ void __launch_bounds__(256, T == 64 ? 2 : 3) k_tri_push(DevProblem P,
       fetch(tk[b], buf[b]);
     }
     Task tn = next(tk[NB - 1]);
+    if constexpr (!FWD) cluster.barrier_wait();   // every y has arrived in every CTA
     int have = -1;   // the last step whose piece has arrived
     auto work = [&](const Task& t0, const F (&cur)[NL * V]) {
       const int slot = (at(t0.i) - rank) / CS;
@@ -1885,13 +1892,21 @@ __global__ void __launch_bounds__(256, T == 64 ? 2 : 3) k_tri_push(DevProblem P,
       }
     }
   };
+  // all pieces of a pass (barriers first .. first + nt - 1) have arrived in this CTA
+  auto arrived = [&](int first) {
+    for (int i = tid; i < nt; i += 256)
+      if (!tc::mbar_wait_bounded(mbar + first + i, 0, PUSH_MAX_POLLS)) dead = true;
+  };
   pass(std::true_type{});
+  arrived(0);
+  cluster.barrier_arrive();   // waited for once the backward pass's first tiles are in flight
   __syncthreads();   // y of this CTA's rows, before the backward pass reads it
   for (int e = tid; e < nown * 256 * V; e += 256) acc[e] = F(0);   // thread-private up to the reductions, but indexed by
   __syncthreads();                                                 // another layout here
   pass(std::false_type{});
+  arrived(max_nt);
   if (dead) atomicExch(fail_flags + k, 1);   // a piece never came: the step is rejected
-  cluster.sync();   // no CTA leaves while a peer may still store into it
+  cluster.sync();
 }
 
 // Device figures, read by configure_solve_kernels.
