@@ -36,7 +36,8 @@ template <> struct RowNum<double> { using T = double; };
 __device__ __forceinline__ SF rcp_num(SF a) { return SF(__frcp_rn(a.v)); }
 __device__ __forceinline__ double rcp_num(double a) { return __drcp_rn(a); }
 
-// N reals (a multiple of 16 bytes) from a 16-byte aligned address through the read-only path
+// N reals (a multiple of 16 bytes) from a 16-byte aligned address through the read-only path: for kernels that are
+// not chained (chain_begin)
 template <int N, typename real>
 __device__ __forceinline__ void load_vec16(const real* p, real (&v)[N]) {
   if constexpr (sizeof(real) == 4) {
@@ -52,6 +53,28 @@ __device__ __forceinline__ void load_vec16(const real* p, real (&v)[N]) {
 #pragma unroll
     for (int k = 0; k < N / 2; ++k) {
       const double2 t = __ldg(reinterpret_cast<const double2*>(p) + k);
+      v[2 * k] = t.x;
+      v[2 * k + 1] = t.y;
+    }
+  }
+}
+
+// the same with ordinary loads: for chained kernels too
+template <int N, typename real>
+__device__ __forceinline__ void gather_vec16(const real* p, real (&v)[N]) {
+  if constexpr (sizeof(real) == 4) {
+#pragma unroll
+    for (int k = 0; k < N / 4; ++k) {
+      const float4 t = reinterpret_cast<const float4*>(p)[k];
+      v[4 * k] = t.x;
+      v[4 * k + 1] = t.y;
+      v[4 * k + 2] = t.z;
+      v[4 * k + 3] = t.w;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < N / 2; ++k) {
+      const double2 t = reinterpret_cast<const double2*>(p)[k];
       v[2 * k] = t.x;
       v[2 * k + 1] = t.y;
     }
@@ -89,7 +112,7 @@ template <typename real>
 __device__ __forceinline__ CamRow<real> gather_camrow(const DevProblem& P, int j) {
   using T = typename RowNum<real>::T;
   real v[12];
-  load_vec16<12>(ctab_ptr<real>(P) + (size_t)CTAB_R * P.m + (size_t)CTAB_Q * j, v);
+  gather_vec16<12>(ctab_ptr<real>(P) + (size_t)CTAB_R * P.m + (size_t)CTAB_Q * j, v);
   const T q[4] = {T(v[0]), T(v[1]), T(v[2]), T(v[3])};
   T Rm[9];
   quat_rotation(q, Rm);
@@ -116,7 +139,7 @@ __device__ __forceinline__ void load_jl(const DevProblem& P, int j, real (&Jl)[9
 }
 // entry c of E dc for one camera's step (9 entries): J_c dc = Jt (E dc)
 template <typename real>
-__device__ __forceinline__ real step_entry(const real* __restrict__ Jl, const double* __restrict__ dc, int c) {
+__device__ __forceinline__ real step_entry(const real* Jl, const double* dc, int c) {
   if (c >= 3) return (real)dc[c];
   return (real)((double)Jl[3 * c] * dc[0] + (double)Jl[3 * c + 1] * dc[1] + (double)Jl[3 * c + 2] * dc[2]);
 }

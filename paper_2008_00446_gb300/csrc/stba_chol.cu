@@ -822,7 +822,7 @@ struct StepShared {
 
 // Four values of row `row`, columns col .. col + 3 of cluster k's scaled matrix, from the FP64 S' (the first touch of a
 // tile reads S' itself: no scaled copy is made for the tensor-core factorisation).
-__device__ __forceinline__ float4 scaled4(const double* __restrict__ Sk, const double* __restrict__ sk, int np, int row,
+__device__ __forceinline__ float4 scaled4(const double* __restrict__ Sk, const double* sk, int np, int row,
                                           int col) {
   const double2* p = reinterpret_cast<const double2*>(Sk + (size_t)row * np + col);
   const double2 a = p[0], b = p[1];
@@ -841,7 +841,7 @@ __device__ __forceinline__ uint32_t* split_tile(uint32_t* split, int64_t v_total
 
 template <bool FIRST>
 __device__ __forceinline__ void update_pair_tc(uint32_t* tsm, StepShared& hs, float* L, uint32_t* split,
-                                               const double* __restrict__ S, const double* __restrict__ scale,
+                                               const double* __restrict__ S, const double* scale,
                                                const TileTask& task, int kt, int* fail_flags, int64_t v_total) {
   constexpr int T = 64, LDS_ = 68;   // staging rows of the product: 16-byte aligned, no bank conflicts
   uint32_t* Ah = tsm;   // 128 x 64 TF32, core-matrix layout
@@ -1012,7 +1012,7 @@ __device__ __forceinline__ float dot4(float4 a, float4 b, float s) {   // s - a.
 
 // the barrier of the sweep: the four row warps and the pivot warp
 __device__ __forceinline__ void panel_tc(uint32_t* psm, StepShared& hs, float* L, float* Dinv, uint32_t* split,
-                                         const double* __restrict__ S, const double* __restrict__ scale,
+                                         const double* __restrict__ S, const double* scale,
                                          const TileTask& task, int kt, int* fail_flags, int* boosted, int64_t v_total) {
   constexpr int T = 64, LD = PTC_LD, NB = T / 8;
   uint32_t* Ah = psm;   // 128 x 64 TF32, core-matrix layout: rows of L_kt,kt-1, then of L_i,kt-1
@@ -1235,7 +1235,7 @@ __device__ __forceinline__ void panel_tc(uint32_t* psm, StepShared& hs, float* L
 template <bool FIRST>
 __global__ void __launch_bounds__(PTC_THREADS, 2) k_step_tc(float* L, float* Dinv, uint32_t* split,
                                                             const double* __restrict__ S,
-                                                            const double* __restrict__ scale, DevProblem P,
+                                                            const double* scale, DevProblem P,
                                                             const int2* panels, int npanels, const int2* updates,
                                                             int kt, int* fail_flags, int* boosted, int64_t v_total) {
   extern __shared__ __align__(128) uint32_t step_smem[];
@@ -1680,21 +1680,21 @@ constexpr int PUSH_MAX_POLLS = 1 << 22;
 template <typename F, int N>
 __device__ __forceinline__ void load16s(const F* p, F* v) {   // one 16-byte load (N = 4 floats or 2 doubles)
   if constexpr (sizeof(F) == 4) {
-    const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+    const float4 t = *reinterpret_cast<const float4*>(p);
     v[0] = t.x;
     v[1] = t.y;
     v[2] = t.z;
     v[3] = t.w;
   } else {
-    const double2 t = __ldg(reinterpret_cast<const double2*>(p));
+    const double2 t = *reinterpret_cast<const double2*>(p);
     v[0] = t.x;
     v[1] = t.y;
   }
 }
 
 template <typename F, int T, typename Rreal, int CS>
-__global__ void __launch_bounds__(256, T == 64 ? 2 : 3) k_tri_push(DevProblem P, const F* __restrict__ L, const F* __restrict__ Dinv,
-                                                     const double* __restrict__ scale, const Rreal* __restrict__ rhs,
+__global__ void __launch_bounds__(256, T == 64 ? 2 : 3) k_tri_push(DevProblem P, const F* L, const F* Dinv,
+                                                     const double* scale, const Rreal* rhs,
                                                      double* x, double* rcopy, int accumulate, int64_t v_total,
                                                      int max_nt, int* fail_flags) {
   namespace cg = cooperative_groups;

@@ -13,6 +13,10 @@ namespace stba {
 // First statement of a kernel of the iteration's chain (launch_after): the next launch may be set up from here
 // on, and everything that the launches before wrote is visible after it.  Every thread of every CTA passes it,
 // so a launch that waits for this one has waited for all before it too.
+// A chained kernel's CTAs are resident while the launches before still write, so what these write is loaded with
+// ordinary loads alone: the read-only path (__ldg, const __restrict__ parameters) wants data that stays as it is for
+// the whole kernel and would allow the compiler to load before the wait.  It is left to what was complete before the
+// chain began (tests/test_chained_loads.py).
 __device__ __forceinline__ void chain_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -83,7 +87,7 @@ __device__ __forceinline__ void load_point_w(const DevProblem& P, int i, real X[
 // contiguous, 16-byte aligned span, moved with 16-byte vector accesses by the whole warp instead of nine
 // strided scalar accesses per lane.  Lanes >= cnt get / store nothing.
 template <typename real>
-__device__ __forceinline__ void warp_load_rec9(const real* __restrict__ g, long long r0, int cnt, real* sm, int lane,
+__device__ __forceinline__ void warp_load_rec9(const real* g, long long r0, int cnt, real* sm, int lane,
                                                real (&x)[9]) {
   const real* blk = g + 9 * r0;
   if (cnt == 32 && ((reinterpret_cast<size_t>(blk) & 15) == 0)) {

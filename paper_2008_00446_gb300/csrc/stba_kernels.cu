@@ -149,8 +149,7 @@ __device__ __forceinline__ double cta_sums(const double (&v)[NV], double (&buf)[
 // moves through shared memory 32 records at a time with coalesced loads, each lane adding up its own
 // point's records in order (no atomics: the sums do not depend on the launch).
 template <typename real>
-__global__ void __launch_bounds__(256) k_pt_acc(DevProblem P, const real* __restrict__ vp_acc,
-                                                real* __restrict__ pt_acc) {
+__global__ void __launch_bounds__(256) k_pt_acc(DevProblem P, const real* vp_acc, real* __restrict__ pt_acc) {
   chain_begin();
   __shared__ __align__(16) real stage[8][288];
   const int lane = threadIdx.x & 31;
@@ -188,7 +187,7 @@ __global__ void __launch_bounds__(256) k_pt_acc(DevProblem P, const real* __rest
 // is sharded.
 template <typename real>
 __global__ void __launch_bounds__(256) k_vp_finalize(DevProblem P, Scratch<real> W, DevState* st,
-                                                     const double* __restrict__ pt_sums,
+                                                     const double* pt_sums,
                                                      const long long* __restrict__ counts) {
   chain_begin();
   __shared__ __align__(16) real stage[8][32 * VPI];
@@ -872,7 +871,7 @@ __device__ __forceinline__ float2 df_split(double d) {
 
 // ------------------------------------------------------------------------------------------------------
 template <typename real>
-__global__ void __launch_bounds__(256) k_point_rhs(DevProblem P, const real* __restrict__ edc, real* t_acc) {
+__global__ void __launch_bounds__(256) k_point_rhs(DevProblem P, const real* edc, real* t_acc) {
   chain_begin();
   const int o = blockIdx.x * blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31;
@@ -886,7 +885,7 @@ __global__ void __launch_bounds__(256) k_point_rhs(DevProblem P, const real* __r
     real X[3];
     load_point_w(P, pt, X);
     real Jt[2][9], Jp[2][3], d[12];
-    load_vec16<12>(edc + (size_t)VPI * cam, d);   // J_c dc = Jt (E dc)
+    gather_vec16<12>(edc + (size_t)VPI * cam, d);   // J_c dc = Jt (E dc)
     proj_rows<real, true>(C, X, Jt, Jp);
     real jd0 = 0, jd1 = 0;
 #pragma unroll
@@ -913,17 +912,16 @@ __global__ void __launch_bounds__(256) k_point_rhs(DevProblem P, const real* __r
 // Bound by the FP64 pipe: the sums were four shuffle trees in each of the eight warps (14 us at 1000 photos with
 // a separate 8 us kernel for the double-float points; the fused kernel takes 15.6 us).
 template <typename real>
-__global__ void __launch_bounds__(RED_THREADS) k_point_update(DevProblem P, const real* __restrict__ pt_info,
-                                                              const real* __restrict__ t_acc,
-                                                              const double* __restrict__ dc,
-                                                              const real* __restrict__ vgrad, double* __restrict__ dp,
-                                                              float2* __restrict__ pdf, double* __restrict__ partial) {
+__global__ void __launch_bounds__(RED_THREADS) k_point_update(DevProblem P, const real* pt_info, const real* t_acc,
+                                                              const double* dc, const real* vgrad, double* dp,
+                                                              float2* pdf, double* partial) {
   chain_begin();
   double s_dp = 0.0, s_p = 0.0, s_dc = 0.0, s_c = 0.0;
   real gmax = real(0);   // max |v| in the working precision (exact)
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P.n; i += gridDim.x * blockDim.x) {
     const real* in = pt_info + 9 * (size_t)i;
     const real* t = t_acc + 3 * (size_t)i;
+    const double p[3] = {P.pts[3 * (size_t)i], P.pts[3 * (size_t)i + 1], P.pts[3 * (size_t)i + 2]};
     real g0 = in[6] - t[0], g1 = in[7] - t[1], g2 = in[8] - t[2];
     real d0 = in[0] * g0 + in[1] * g1 + in[2] * g2;
     real d1 = in[1] * g0 + in[3] * g1 + in[4] * g2;
@@ -933,7 +931,6 @@ __global__ void __launch_bounds__(RED_THREADS) k_point_update(DevProblem P, cons
     out[1] = d1;
     out[2] = d2;
     const double e[3] = {(double)d0, (double)d1, (double)d2};
-    const double* p = P.pts + 3 * (size_t)i;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const double pc = p[c];
@@ -1123,7 +1120,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_cost_df(DevProblem P, const flo
 // took 16 us on the FP64 pipe of the one SM; six warps and paired square roots take 5.3 us.
 constexpr int FIN_WARPS = 6;
 template <typename real>
-__global__ void __launch_bounds__(32 * FIN_WARPS) k_finalize(const double* __restrict__ partial, DevState* st,
+__global__ void __launch_bounds__(32 * FIN_WARPS) k_finalize(const double* partial, DevState* st,
                                                              Settings s, int with_step) {
   chain_begin();
   __shared__ double red[FIN_WARPS];
@@ -1274,9 +1271,9 @@ void launch_cost_x(const DevProblem& P, double* rt, float* cam_df, float* pt_df,
 // count of failed clusters (st, if given).  sharded: another process's clusters give zeros (their steps arrive
 // by the exchange of dc).  One launch for what were three (5.2 + 3.5 + 2.8 us at 1000 cameras, 4.5 us now).
 template <typename real>
-__global__ void __launch_bounds__(256) k_scatter_step(DevProblem P, const double* __restrict__ x,
-                                                      const int* __restrict__ fail_flags, DevState* st,
-                                                      const real* __restrict__ ctab, double* __restrict__ dc,
+__global__ void __launch_bounds__(256) k_scatter_step(DevProblem P, const double* x,
+                                                      const int* fail_flags, DevState* st,
+                                                      const real* ctab, double* __restrict__ dc,
                                                       real* __restrict__ edc) {
   chain_begin();
   const int k = blockIdx.x;

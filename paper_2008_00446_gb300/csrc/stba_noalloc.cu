@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(32) k_noalloc_rt(int m, const double* __restri
 // Bound by the FP64 pipe (2 lanes a cycle and SM): every sum is a chain of fused multiply-adds, the depth test
 // compares bits (a depth that is NaN makes the sum NaN by itself), and one warp adds up the CTA's sums.  The call at
 // 1000 cameras and 1.1 M observations: 80 us before (about 35 FP64 instructions an observation), 61 us now.
-__global__ void __launch_bounds__(NOALLOC_THREADS) k_noalloc_cost(int m, int n, int q, const double* __restrict__ rt,
+__global__ void __launch_bounds__(NOALLOC_THREADS) k_noalloc_cost(int m, int n, int q, const double* rt,
                                                                   const double* __restrict__ pts,
                                                                   const int* __restrict__ obs_cam,
                                                                   const int* __restrict__ obs_pt,
@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(NOALLOC_THREADS) k_noalloc_cost(int m, int n, 
 }
 
 constexpr int NOALLOC_FINAL = 128;
-__global__ void __launch_bounds__(NOALLOC_FINAL) k_noalloc_final(const double* __restrict__ partial, double* __restrict__ F) {
+__global__ void __launch_bounds__(NOALLOC_FINAL) k_noalloc_final(const double* partial, double* __restrict__ F) {
   chain_begin();
   __shared__ double red[NOALLOC_FINAL / 32];
   double s = 0.0;
