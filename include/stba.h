@@ -43,7 +43,7 @@ typedef enum {
   STBA_ERR_OOM = 3,         /* device allocation failed */
   STBA_ERR_NOT_SPD = 4,     /* reserved: a failed factorisation is reported in stba_iter_info instead */
   STBA_ERR_NONFINITE = 5,   /* non-finite input values, or a point behind a camera (depth <= 1e-9) */
-  STBA_ERR_TIMEOUT = 6,     /* reserved for bounded device waits */
+  STBA_ERR_TIMEOUT = 6,     /* a bounded device wait gave up (stba_measure_peaks; an LM step is rejected instead) */
   STBA_ERR_STATE = 7        /* wrong call order, or lambda above 1e16 */
 } stba_status;
 
@@ -315,6 +315,12 @@ stba_status stba_cluster_sgc(stba_ctx* ctx, int32_t gamma, double beta, uint64_t
  * STBA_ERR_STATE while iterations are being recorded (stba_record), STBA_ERR_INVALID_ARG for
  * iterations < 1. */
 stba_status stba_autotune(stba_ctx* ctx, int32_t iterations, int32_t* choice, float* ms);
+
+/* Limit of the device-side waits of the cluster factorisation and solves (for their own copies, tensor-core products
+ * and the pieces of a solve's other CTAs), 0 .. 4e9 ns; one second at create.  A wait that reaches it gives up: the
+ * cluster counts as failed and the LM step is rejected.  0 gives up whatever is not there at the first look, which
+ * makes the failure path testable.  Takes effect with the next iteration. */
+stba_status stba_set_wait_limit(stba_ctx* ctx, int64_t nanoseconds);
 
 /* Measured arithmetic peaks of the current GPU, the denominators of the factorisation's roofline.  The
  * paper has no counterpart: this is measurement infrastructure.  *fp32_tflops (optional): FP32 FMA rate of

@@ -148,6 +148,7 @@ struct stba_ctx {
   int update_tc = 0;                    // trailing updates on the tensor cores (FP32 factor, tile 64)
   int split_panel = 0;                  // split panel: diagonal-tile factor + inverse, then the tiles below
   int persistent = 0;                   // one persistent launch of 8-CTA clusters factors every cluster
+  uint32_t wait_ns = 1000000000u;       // limit of the device-side waits (stba_set_wait_limit)
   int solve_cs = 8;                     // CTAs per thread-block cluster of the cluster solves
   int panel_choice = STBA_FACTOR_PANEL_DEFAULT;   // option, or the autotuner's choice; DEFAULT decides per
                                                   // assignment (set_clusters_host)
@@ -287,6 +288,7 @@ DevProblem dev_problem(const stba_ctx* c) {
   P.base_vp = c->reorder.base_vp;
   P.base_pos = c->inv[c->inv_cur];
   P.pair_recompute = c->pair_recompute ? 1 : 0;
+  P.wait_ns = c->wait_ns;
   P.sharded = c->shard_world > 1 ? 1 : 0;
   P.cluster_owned = c->cl_owned;
   return P;
@@ -2105,6 +2107,13 @@ stba_status stba_get_cluster_system(stba_ctx* c, int32_t k, double* S, double* b
       std::memcpy(b, hb.data(), hb.size() * 8);
     }
   }
+  return STBA_OK;
+}
+
+stba_status stba_set_wait_limit(stba_ctx* c, int64_t nanoseconds) {
+  if (!c || nanoseconds < 0 || nanoseconds > 4000000000ll) return STBA_ERR_INVALID_ARG;
+  c->wait_ns = (uint32_t)nanoseconds;
+  c->graph_stale = true;   // a kernel argument: the next iteration's capture takes it
   return STBA_OK;
 }
 

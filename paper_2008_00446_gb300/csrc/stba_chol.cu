@@ -790,15 +790,14 @@ __global__ void __launch_bounds__(256) k_chol_update(F* L, DevProblem P, const i
 // K-major core-matrix layout (stba_tc.cuh), 32 KB per tile, so that six bulk copies bring them in and no thread
 // converts anything; the product goes from TMEM through shared memory, so that the updated values are
 // read and written 256 contiguous bytes per row.  The waits for the copies and
-// the MMAs are bounded: a CTA that gives up marks the cluster failed (the LM step is rejected), frees its
-// tensor memory and returns.  When i0 + 1 is past the cluster's last tile, the second half of A is undefined and
+// the MMAs are bounded: a CTA that gives up marks the cluster failed (the LM step is rejected), waits, bounded again,
+// for what it has in flight, frees its tensor memory and returns.  When i0 + 1 is past the cluster's last tile, the second half of A is undefined and
 // its rows are not written.
 // Bound by L2 traffic (96 KB of operands, 64 KB of updated values per tile pair).  With operands loaded, split and
 // stored by the threads the factorisation stage took 1194 us instead of 922 (13 uneven clusters), 853 instead of 707
 // (one of 400 cameras); with one row per lane and 16 bytes per access on top, the L1 pipe was 71 % busy.
 constexpr int TCU_THREADS = 256;
 constexpr size_t TCU_SMEM = sizeof(uint32_t) * (2 * 128 * 64 + 2 * 64 * 64);   // A hi/lo, B hi/lo: 96 KB
-constexpr int TCU_MAX_POLLS = 1 << 26;
 
 __device__ __forceinline__ void split_store(uint32_t* hi, uint32_t* lo, int off, float4 v) {
   const uint32_t h0 = tc::to_tf32(v.x), h1 = tc::to_tf32(v.y), h2 = tc::to_tf32(v.z), h3 = tc::to_tf32(v.w);
@@ -819,6 +818,18 @@ struct StepShared {
   uint64_t mbar_load, mbar;
   uint32_t taddr;
 };
+
+// The end of a step CTA that gave up: its copies (loads) and products (multiplied; thread 0's knowledge) end before its
+// shared and tensor memory are handed back.
+__device__ __forceinline__ void step_give_up(StepShared& hs, int* fail, bool loads, bool multiplied) {
+  if (threadIdx.x == 0) {
+    atomicExch(fail, 1);
+    if (loads) tc::mbar_wait_bounded(&hs.mbar_load, 0, tc::WAIT_NS);
+    if (multiplied) tc::mbar_wait_bounded(&hs.mbar, 0, tc::WAIT_NS);
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) tc::tmem_dealloc(hs.taddr, 64);
+}
 
 // Four values of row `row`, columns col .. col + 3 of cluster k's scaled matrix, from the FP64 S' (the first touch of a
 // tile reads S' itself: no scaled copy is made for the tensor-core factorisation).
@@ -842,7 +853,8 @@ __device__ __forceinline__ uint32_t* split_tile(uint32_t* split, int64_t v_total
 template <bool FIRST>
 __device__ __forceinline__ void update_pair_tc(uint32_t* tsm, StepShared& hs, float* L, uint32_t* split,
                                                const double* __restrict__ S, const double* scale,
-                                               const TileTask& task, int kt, int* fail_flags, int64_t v_total) {
+                                               const TileTask& task, int kt, int* fail_flags, int64_t v_total,
+                                               uint32_t wait_ns) {
   constexpr int T = 64, LDS_ = 68;   // staging rows of the product: 16-byte aligned, no bank conflicts
   uint32_t* Ah = tsm;   // 128 x 64 TF32, core-matrix layout
   uint32_t* Al = tsm + 128 * 64;
@@ -855,6 +867,7 @@ __device__ __forceinline__ void update_pair_tc(uint32_t* tsm, StepShared& hs, fl
   const int rows_valid = min(128, np - i0 * T);   // 64 or 128
   const uint32_t tmem = hs.taddr;
   // operands by the copy engine; the second half of A stays undefined past the last tile (its rows are not used)
+  bool multiplied = false;
   if (tid == 0) {
     const bool two = rows_valid == 128;
     tc::fence_async_all();
@@ -869,7 +882,8 @@ __device__ __forceinline__ void update_pair_tc(uint32_t* tsm, StepShared& hs, fl
       tc::bulk_load(Ah + 4096, a0 + SPLIT_TILE, 16384, &hs.mbar_load);
       tc::bulk_load(Al + 4096, a0 + SPLIT_TILE + 4096, 16384, &hs.mbar_load);
     }
-    if (tc::mbar_wait_bounded(&hs.mbar_load, 0, TCU_MAX_POLLS)) {
+    multiplied = tc::mbar_wait_bounded(&hs.mbar_load, 0, wait_ns);
+    if (multiplied) {
       tc::fence_after_sync();
       constexpr uint32_t idesc = tc::idesc_tf32(128, 64);
       const uint32_t pa[3] = {tc::smem_u32(Ah), tc::smem_u32(Al), tc::smem_u32(Ah)};
@@ -899,7 +913,7 @@ __device__ __forceinline__ void update_pair_tc(uint32_t* tsm, StepShared& hs, fl
   }
   __syncwarp();
   // thread (lane quarter warp & 3, column half warp >> 2): row R of the product, 32 columns, to the staging rows
-  const bool done = __all_sync(0xffffffffu, tc::mbar_wait_bounded(&hs.mbar, 0, TCU_MAX_POLLS));
+  const bool done = __all_sync(0xffffffffu, tc::mbar_wait_bounded(&hs.mbar, 0, wait_ns));
   if (done) {
     tc::fence_after_sync();
     float d[32];
@@ -908,13 +922,10 @@ __device__ __forceinline__ void update_pair_tc(uint32_t* tsm, StepShared& hs, fl
 #pragma unroll
     for (int v = 0; v < 8; ++v)
       *reinterpret_cast<float4*>(stage + R * LDS_ + c0 + 4 * v) = make_float4(d[4 * v], d[4 * v + 1], d[4 * v + 2], d[4 * v + 3]);
-  } else if (lane == 0) {
-    atomicExch(fail_flags + k, 1);
   }
   tc::fence_before_sync();
-  const int all_done = __syncthreads_and(done);
+  if (!__syncthreads_and(done)) return step_give_up(hs, fail_flags + k, true, multiplied);
   if (warp == 0) tc::tmem_dealloc(tmem, 64);
-  if (!all_done) return;
 #pragma unroll
   for (int v = 0; v < 8; ++v) {
     if (16 * v + r16 >= rows_valid) break;
@@ -1013,7 +1024,8 @@ __device__ __forceinline__ float dot4(float4 a, float4 b, float s) {   // s - a.
 // the barrier of the sweep: the four row warps and the pivot warp
 __device__ __forceinline__ void panel_tc(uint32_t* psm, StepShared& hs, float* L, float* Dinv, uint32_t* split,
                                          const double* __restrict__ S, const double* scale,
-                                         const TileTask& task, int kt, int* fail_flags, int* boosted, int64_t v_total) {
+                                         const TileTask& task, int kt, int* fail_flags, int* boosted, int64_t v_total,
+                                         uint32_t wait_ns) {
   constexpr int T = 64, LD = PTC_LD, NB = T / 8;
   uint32_t* Ah = psm;   // 128 x 64 TF32, core-matrix layout: rows of L_kt,kt-1, then of L_i,kt-1
   uint32_t* Al = psm + 128 * 64;
@@ -1052,9 +1064,10 @@ __device__ __forceinline__ void panel_tc(uint32_t* psm, StepShared& hs, float* L
       cp_async16(w, A + (size_t)grow * np + kt * T + c4);
     }
   }
-  bool done = true;
+  bool done = true, multiplied = false;
   if (kt > 0) {
-    if (tid == 0 && tc::mbar_wait_bounded(&hs.mbar_load, 0, TCU_MAX_POLLS)) {
+    if (tid == 0) multiplied = tc::mbar_wait_bounded(&hs.mbar_load, 0, wait_ns);
+    if (multiplied) {
       tc::fence_after_sync();
       constexpr uint32_t idesc = tc::idesc_tf32(128, 64);
       const uint32_t pa[3] = {tc::smem_u32(Ah), tc::smem_u32(Al), tc::smem_u32(Ah)};
@@ -1069,7 +1082,7 @@ __device__ __forceinline__ void panel_tc(uint32_t* psm, StepShared& hs, float* L
     }
     cp_async_wait_all();
     __syncthreads();   // the old values are in place
-    done = __all_sync(FULL_MASK, tc::mbar_wait_bounded(&hs.mbar, 0, TCU_MAX_POLLS));
+    done = __all_sync(FULL_MASK, tc::mbar_wait_bounded(&hs.mbar, 0, wait_ns));
     if (done) {
       tc::fence_after_sync();
       float d[32];
@@ -1090,12 +1103,9 @@ __device__ __forceinline__ void panel_tc(uint32_t* psm, StepShared& hs, float* L
     }
     tc::fence_before_sync();
   }
-  const int all_done = __syncthreads_and(done);
+  // a wait gave up: the cluster fails, the step is rejected
+  if (!__syncthreads_and(done)) return step_give_up(hs, fail_flags + k, true, multiplied);
   if (warp == 0) tc::tmem_dealloc(tmem, 64);
-  if (!all_done) {   // the wait gave up: the cluster fails, the step is rejected
-    if (tid == 0) atomicExch(fail_flags + k, 1);
-    return;
-  }
   float* my = W + tid * LD;   // row threads
   float x[8], nx[8], o[8];
   float* Di = Dinv + (size_t)task.v_off * T + (size_t)kt * T * T;
@@ -1255,9 +1265,9 @@ __global__ void __launch_bounds__(PTC_THREADS, 2) k_step_tc(float* L, float* Din
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (panel)
-    panel_tc(step_smem, hs, L, Dinv, split, S, scale, task, kt + 1, fail_flags, boosted, v_total);
+    panel_tc(step_smem, hs, L, Dinv, split, S, scale, task, kt + 1, fail_flags, boosted, v_total, P.wait_ns);
   else
-    update_pair_tc<FIRST>(step_smem, hs, L, split, S, scale, task, kt, fail_flags, v_total);
+    update_pair_tc<FIRST>(step_smem, hs, L, split, S, scale, task, kt, fail_flags, v_total, P.wait_ns);
 }
 
 // ------------------------------------------------------------------------------------------------------
@@ -1675,7 +1685,6 @@ template <typename F, int T> struct PushLayout {
     return 16 * (size_t)nt + sizeof(F) * ((size_t)nt * T + (size_t)slots * (T + 256 * V) + 9 * (size_t)T) + 16;
   }
 };
-constexpr int PUSH_MAX_POLLS = 1 << 22;
 
 template <typename F, int N>
 __device__ __forceinline__ void load16s(const F* p, F* v) {   // one 16-byte load (N = 4 floats or 2 doubles)
@@ -1856,7 +1865,7 @@ __global__ void __launch_bounds__(256, T == 64 ? 2 : 3) k_tri_push(DevProblem P,
         }
       } else {
         if (t0.kk > have) {
-          if (!dead) dead = !tc::mbar_wait_bounded(mbar + (FWD ? 0 : max_nt) + at(t0.kk), 0, PUSH_MAX_POLLS);
+          if (!dead) dead = !tc::mbar_wait_bounded(mbar + (FWD ? 0 : max_nt) + at(t0.kk), 0, P.wait_ns);
           have = t0.kk;
         }
         const F* v = vec + (size_t)at(t0.kk) * T;
@@ -1892,10 +1901,11 @@ __global__ void __launch_bounds__(256, T == 64 ? 2 : 3) k_tri_push(DevProblem P,
       }
     }
   };
-  // all pieces of a pass (barriers first .. first + nt - 1) have arrived in this CTA
+  // all pieces of a pass (barriers first .. first + nt - 1) have arrived in this CTA (a CTA that gave up a wait sends
+  // its pieces all the same)
   auto arrived = [&](int first) {
     for (int i = tid; i < nt; i += 256)
-      if (!tc::mbar_wait_bounded(mbar + first + i, 0, PUSH_MAX_POLLS)) dead = true;
+      if (!tc::mbar_wait_bounded(mbar + first + i, 0, tc::WAIT_NS)) dead = true;
   };
   pass(std::true_type{});
   arrived(0);

@@ -49,6 +49,7 @@ struct DevProblem {
   const int* base_vp;          // [q] virtual point of every base-order observation (null unless the pair pass reads it)
   const int* base_pos;         // [q] sorted position of every base-order observation (current assignment)
   int pair_recompute;          // 1: the pair pass recomputes its rows instead of reading the camera pass's copy
+  uint32_t wait_ns;            // limit of the factorisation's and solves' waits (stba_set_wait_limit)
   int sharded;                 // 1: this process owns only some clusters (stba_set_shard)
   const int* cluster_owned;    // [l] 1 where this process builds, factors and solves cluster k (all 1 unless
                                //     sharded)

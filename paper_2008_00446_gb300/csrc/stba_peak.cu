@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(128) k_peak_tf32(int n_mma, int* err) {
     }
     tc::mma_commit(&mbar);
   }
-  if (!tc::mbar_wait_bounded(&mbar, 0, 1 << 26) && threadIdx.x == 0) atomicExch(err, 1);
+  if (!tc::mbar_wait_bounded(&mbar, 0, tc::WAIT_NS) && threadIdx.x == 0) atomicExch(err, 1);
   tc::fence_before_sync();
   __syncthreads();
   if ((threadIdx.x >> 5) == 0) tc::tmem_dealloc(tmem, PEAK_N);

@@ -93,14 +93,32 @@ __device__ __forceinline__ void st_async(uint32_t addr, double v, uint32_t mbar)
                : "memory");
 }
 
-// Waits for phase `parity` of the mbarrier, at most `max_tries` polls; returns false if it gave up.
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* mbar, uint32_t parity, int max_tries) {
+__device__ __forceinline__ uint64_t global_ns() {   // the GPU's wall clock
+  uint64_t t;
+  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+  return t;
+}
+
+constexpr uint32_t WAIT_NS = 1000000000u;   // one second: the longest wait of a kernel for its own copies and products
+
+// Waits for phase `parity` of the mbarrier, at most `limit_ns` by the wall clock (a poll may suspend the thread for a
+// time that the hardware chooses, so a number of polls bounds no time); 0: one look.  Returns false if it gave up.
+__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* mbar, uint32_t parity, uint32_t limit_ns) {
   uint32_t ok = 0;
-  for (int it = 0; it < max_tries && !ok; ++it)
-    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-                 : "=r"(ok)
-                 : "r"(smem_u32(mbar)), "r"(parity)
-                 : "memory");
+  asm volatile("{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+               : "=r"(ok)
+               : "r"(smem_u32(mbar)), "r"(parity)
+               : "memory");
+  if (ok || limit_ns == 0) return ok != 0;
+  const uint64_t t0 = global_ns();
+  do {
+#pragma unroll 1
+    for (int it = 0; it < 64 && !ok; ++it)
+      asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+                   : "=r"(ok)
+                   : "r"(smem_u32(mbar)), "r"(parity)
+                   : "memory");
+  } while (!ok && global_ns() - t0 < limit_ns);
   return ok != 0;
 }
 

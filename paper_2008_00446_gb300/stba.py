@@ -32,7 +32,8 @@ EXPORTS = ["stba_default_options", "stba_create", "stba_set_clusters", "stba_lm_
            "stba_last_step", "stba_problem_info", "stba_get_cluster_system", "stba_set_timing",
            "stba_stage_times", "stba_destroy", "stba_status_string", "stba_last_error", "stba_cost_noalloc",
            "stba_record", "stba_adjoint", "stba_graph_create", "stba_graph_edges", "stba_graph_cluster",
-           "stba_graph_cluster_batch", "stba_graph_destroy", "stba_cluster_sgc", "stba_autotune", "stba_measure_peaks", "stba_set_shard", "stba_shard_owned"]
+           "stba_graph_cluster_batch", "stba_graph_destroy", "stba_cluster_sgc", "stba_autotune", "stba_measure_peaks", "stba_set_shard", "stba_shard_owned",
+           "stba_set_wait_limit"]
 
 
 # transport of the sharded iteration: (user, data, count, dtype 0 = FP64 / 1 = FP32, stream) -> 0 on success
@@ -120,6 +121,7 @@ def load(build_if_missing: bool = True):
         "stba_measure_peaks": (I32, [P, I32, ctypes.POINTER(D), ctypes.POINTER(D)]),
         "stba_set_shard": (I32, [P, I32, I32, ALLREDUCE_FN, P, I32]),
         "stba_shard_owned": (I32, [P, P, ctypes.POINTER(I32)]),
+        "stba_set_wait_limit": (I32, [P, I64]),
     }
     for name, (res, args) in sig.items():
         fn = getattr(L, name)
@@ -298,6 +300,11 @@ def stba_stage_times(ctx: Context):
     cnt = ctypes.c_int32()
     ctx._check(load().stba_stage_times(ctx.handle, ms, 16, ctypes.byref(cnt)))
     return list(ms)[: cnt.value]
+
+
+def stba_set_wait_limit(ctx: Context, nanoseconds: int):
+    """Limit of the device-side waits of the factorisation and solves (1 s at create; 0: one look)."""
+    ctx._check(load().stba_set_wait_limit(ctx.handle, int(nanoseconds)))
 
 
 def _noalloc_check(cameras, points, obs_cam, obs_pt, obs_uv, F_out):
