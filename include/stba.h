@@ -41,9 +41,10 @@ typedef enum {
   STBA_ERR_INVALID_ARG = 1, /* bad sizes, indices out of range, duplicate projections, empty cluster */
   STBA_ERR_CUDA = 2,        /* a CUDA runtime call failed */
   STBA_ERR_OOM = 3,         /* device allocation failed */
-  STBA_ERR_NOT_SPD = 4,     /* reserved: a failed factorisation is reported in stba_iter_info instead */
+  STBA_ERR_NOT_SPD = 4,     /* a factorisation failed in stba_adjoint (an LM step reports it in stba_iter_info) */
   STBA_ERR_NONFINITE = 5,   /* non-finite input values, or a point behind a camera (depth <= 1e-9) */
-  STBA_ERR_TIMEOUT = 6,     /* a bounded device wait gave up (stba_measure_peaks; an LM step is rejected instead) */
+  STBA_ERR_TIMEOUT = 6,     /* a bounded device wait gave up (stba_adjoint, stba_measure_peaks; an LM step
+                               is rejected instead) */
   STBA_ERR_STATE = 7        /* wrong call order, or lambda above 1e16 */
 } stba_status;
 
@@ -225,7 +226,8 @@ stba_status stba_record(stba_ctx* ctx, int32_t max_iter);
  * right-hand side, w~'_v = (h_v / H_i) o w_i (h_v = diag(V_v), H_i their sum over point i's copies, w_i the
  * physical w), including the dependence of h_v / H_i on the parameters.
  * Errors: STBA_ERR_STATE with the PCG solvers or the Huber loss, if nothing was recorded, or if
- * stba_set_params replaced the parameters during the recording.  On return the parameters, the cluster
+ * stba_set_params replaced the parameters during the recording; STBA_ERR_TIMEOUT or STBA_ERR_NOT_SPD if a device
+ * wait gave up, or a factorisation failed, while a step was recomputed (no output is then written).  On return the parameters, the cluster
  * assignment and the LM state are those before the call.  The call synchronises the stream and allocates
  * no memory (its buffers are held with the tape). */
 stba_status stba_adjoint(stba_ctx* ctx, const double* dL_dcams, const double* dL_dpts, double* dL_dobs,
@@ -318,7 +320,7 @@ stba_status stba_autotune(stba_ctx* ctx, int32_t iterations, int32_t* choice, fl
 
 /* Limit of the device-side waits of the cluster factorisation and solves (for their own copies, tensor-core products
  * and the pieces of a solve's other CTAs), 0 .. 4e9 ns; one second at create.  A wait that reaches it gives up: the
- * cluster counts as failed and the LM step is rejected.  0 gives up whatever is not there at the first look, which
+ * cluster counts as failed and the LM step is rejected; stba_adjoint returns STBA_ERR_TIMEOUT.  0 gives up whatever is not there at the first look, which
  * makes the failure path testable.  Takes effect with the next iteration. */
 stba_status stba_set_wait_limit(stba_ctx* ctx, int64_t nanoseconds);
 

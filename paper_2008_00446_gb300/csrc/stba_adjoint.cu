@@ -151,8 +151,12 @@ __global__ void __launch_bounds__(256) k_adj_vp(DevProblem P, const double* __re
 
 // Per virtual point: z_v = -C'_v^-1 (E'^T z_c)_v and the expanded point step dp'_v = C'_v^-1 (w'_v - (E'^T dc)_v)
 // = y_v - C'_v^-1 (E'^T dc)_v (uncorrected w').
+// It also notes for stba_adjoint why a cluster's factor or solve failed in this step, if one did.
 template <typename real>
-__global__ void k_adj_vp_final(int nv, const real* __restrict__ vp_info, double* __restrict__ vpz) {
+__global__ void k_adj_vp_final(int nv, const real* __restrict__ vp_info, double* __restrict__ vpz, int l,
+                               const int* __restrict__ fail_flags, int* failed) {
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < l; k += gridDim.x * blockDim.x)
+    if (fail_flags[k]) atomicOr(failed, fail_flags[k]);
   for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += gridDim.x * blockDim.x) {
     const real* in = vp_info + VPI * (size_t)v;
     double Li[6];
@@ -422,7 +426,8 @@ void launch_adjoint_step(const DevProblem& P, Scratch<real> W, CamLists CL, cons
   launch_scatter_step<real>(P, fb.x, fb.fail_flags, plan.max_np, nullptr, A.zc, nullptr, stream);
   cudaMemsetAsync(A.vpz, 0, 6 * (size_t)P.nv * sizeof(double), stream);
   k_adj_vp<real><<<(P.q + 255) / 256, 256, 0, stream>>>(P, A.zc, W.dc, A.vpz);
-  k_adj_vp_final<real><<<std::min((P.nv + 255) / 256, 4096), 256, 0, stream>>>(P.nv, W.vp_info, A.vpz);
+  k_adj_vp_final<real><<<std::min((P.nv + 255) / 256, 4096), 256, 0, stream>>>(P.nv, W.vp_info, A.vpz, P.l, fb.fail_flags,
+                                                                            A.failed);
   if (corrected) k_adj_zeta<real><<<pblocks, 256, 0, stream>>>(P, W.vp_acc, A.vpz, A.zeta, A.kappa);
   k_adj_obs<real><<<(P.q + ADJ_THREADS - 1) / ADJ_THREADS, ADJ_THREADS, 0, stream>>>(
       P, perm, lam, W.dc, W.dp, A.zc, A.u, A.vpz, corrected, A.zeta, A.kappa, A.T, A.qbar);

@@ -1971,6 +1971,7 @@ stba_status stba_record(stba_ctx* c, int32_t max_iter) {
                   (s = dalloc_into(c, &A.qbar, 2 * q, c->tape_allocs)) == STBA_OK &&
                   (s = dalloc_into(c, &A.zeta, 3 * (size_t)c->n, c->tape_allocs)) == STBA_OK &&
                   (s = dalloc_into(c, &A.kappa, 3 * q, c->tape_allocs)) == STBA_OK &&   // nv <= q
+                  (s = dalloc_into(c, &A.failed, 1, c->tape_allocs)) == STBA_OK &&
                   (s = dalloc_into(c, &c->adj_save_x, nx, c->tape_allocs)) == STBA_OK;
   if (!ok) {
     free_tape(c);
@@ -2010,6 +2011,7 @@ stba_status stba_adjoint(stba_ctx* c, const double* dL_dcams, const double* dL_d
     CK(cudaMemsetAsync(A.a_p, 0, 3 * (size_t)n * 8, c->stream));
   }
   CK(cudaMemsetAsync(A.qbar, 0, 2 * (size_t)q * 8, c->stream));
+  CK(cudaMemsetAsync(A.failed, 0, sizeof(int), c->stream));
   CK(cudaStreamSynchronize(c->stream));
   const std::vector<int> final_clusters = c->h_clusters;
   auto reverse_pass = [&]() -> stba_status {
@@ -2027,7 +2029,12 @@ stba_status stba_adjoint(stba_ctx* c, const double* dL_dcams, const double* dL_d
         enqueue_adjoint_step<double>(c, info[t].lambda_used, info[t].corrected, A);
       CK(cudaGetLastError());
     }
+    int failed = 0;
+    CK(cudaMemcpyAsync(&failed, A.failed, sizeof failed, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
+    if (failed & FAIL_WAIT)
+      return fail(c, STBA_ERR_TIMEOUT, "a device wait of a recomputed step's factorisation or solve gave up");
+    if (failed) return fail(c, STBA_ERR_NOT_SPD, "a cluster's factorisation failed while a recorded step was recomputed");
     // outputs (qbar is in the input order of the observations)
     if (dL_dcams0) CK(cudaMemcpyAsync(dL_dcams0, A.a_c, 9 * (size_t)m * 8, cudaMemcpyDefault, c->stream));
     if (dL_dpts0) CK(cudaMemcpyAsync(dL_dpts0, A.a_p, 3 * (size_t)n * 8, cudaMemcpyDefault, c->stream));

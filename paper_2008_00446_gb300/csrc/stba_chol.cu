@@ -165,7 +165,7 @@ __device__ __forceinline__ void chol8(F (*Ad)[LDA], int b0, int row0, int nk, F*
   for (int r = 0; r < 8; ++r)
 #pragma unroll
     for (int c = 0; c <= r; ++c) Ad[b0 + r][b0 + c] = d[r][c];
-  if (bad) *fail = 1;
+  if (bad) atomicOr(fail, FAIL_PIVOT);
   if (nboost && boosted) atomicAdd(boosted, nboost);
 }
 
@@ -203,7 +203,7 @@ __device__ __forceinline__ void chol8_warp(double (*Ad)[LDA], int b0, int row0, 
   }
   if (p <= r) Ad[b0 + r][b0 + p] = d0;
   if (p + 4 <= r) Ad[b0 + r][b0 + p + 4] = d1;
-  if (bad && lane == 0) *fail = 1;
+  if (bad && lane == 0) atomicOr(fail, FAIL_PIVOT);
 }
 
 // the block's factorisation by warp 0 (FP32: by its first thread); called by the whole warp
@@ -823,7 +823,7 @@ struct StepShared {
 // shared and tensor memory are handed back.
 __device__ __forceinline__ void step_give_up(StepShared& hs, int* fail, bool loads, bool multiplied) {
   if (threadIdx.x == 0) {
-    atomicExch(fail, 1);
+    atomicOr(fail, FAIL_WAIT);
     if (loads) tc::mbar_wait_bounded(&hs.mbar_load, 0, tc::WAIT_NS);
     if (multiplied) tc::mbar_wait_bounded(&hs.mbar, 0, tc::WAIT_NS);
   }
@@ -1010,7 +1010,7 @@ __device__ __forceinline__ void chol8_fast(float* T, int row0, int nk, float* ri
   }
   reinterpret_cast<float4*>(rinv)[0] = make_float4(ri[0], ri[1], ri[2], ri[3]);
   reinterpret_cast<float4*>(rinv)[1] = make_float4(ri[4], ri[5], ri[6], ri[7]);
-  if (bad) *fail = 1;
+  if (bad) atomicOr(fail, FAIL_PIVOT);
   if (nboost && boosted) atomicAdd(boosted, nboost);
 }
 
@@ -1915,7 +1915,7 @@ __global__ void __launch_bounds__(256, T == 64 ? 2 : 3) k_tri_push(DevProblem P,
   __syncthreads();                                                 // another layout here
   pass(std::false_type{});
   arrived(max_nt);
-  if (dead) atomicExch(fail_flags + k, 1);   // a piece never came: the step is rejected
+  if (dead) atomicOr(fail_flags + k, FAIL_WAIT);   // a piece never came: the step is rejected
   cluster.sync();
 }
 

@@ -301,6 +301,7 @@ struct CholPlan {
   int n_cluster_items;
   int solve_cs;                   // CTAs per thread-block cluster of the cluster solves (2, 4 or 8)
 };
+constexpr int FAIL_PIVOT = 1, FAIL_WAIT = 2;   // a lost pivot; a bounded device wait that gave up
 struct FactorBuffers {
   void* L;          // factor (F = float or double), same layout as S'
   void* Dinv;       // inverses of the diagonal tiles, T x T per tile, v_off[k] * T offset per cluster;
@@ -311,7 +312,7 @@ struct FactorBuffers {
   double* scale;    // [v_total] Jacobi scaling s_i = S_ii^-1/2
   double* x;        // [v_total] solution
   double* r;        // [v_total] refinement residual
-  int* fail_flags;  // [l]
+  int* fail_flags;  // [l] 0, or why the cluster's factor or solve failed (FAIL_PIVOT, FAIL_WAIT)
   int* boosted;     // counter of raised pivots (in DevState)
   int64_t v_total;
 };
@@ -338,6 +339,7 @@ struct AdjointBuffers {
   double* qbar;   // [q][2] observation adjoint, input order
   double* zeta;   // [n][3] corrected steps: h-weighted mean of the copies' z_v per point
   double* kappa;  // [nv][3] corrected steps: (z_v - zeta_i) o w_i / H_i per virtual point
+  int* failed;    // the fail_flags of every recomputed step's clusters, combined
 };
 template <typename real>
 void launch_adjoint_step(const DevProblem& P, Scratch<real> W, CamLists CL, const FactorBuffers& fb,

@@ -45,6 +45,29 @@ def test_waits_that_run_out_reject_the_step(precision, bar, use_graph):
             assert cols(a, b, w) < bar
 
 
+@pytest.mark.parametrize("precision,bar", [(stba.STBA_MIXED, 1e-3), (stba.STBA_FP64, 1e-8)])
+def test_waits_that_run_out_fail_the_adjoint(precision, bar):
+    """STBA_ERR_TIMEOUT with the parameters as they were; the gradients of a fresh recording once the limit is back
+    (bars of the adjoint's own tests: mixed 1e-3 of the largest entry; FP64 the order of the sums through two steps)."""
+    s = _scene()
+    g = np.random.default_rng(1).normal(size=(s.m, 9))
+    with _ctx(s, precision=precision) as ctx, _ctx(s, precision=precision) as ref:
+        for c in (ctx, ref):
+            stba.stba_record(c, 2)
+            for _ in range(2):
+                assert stba.stba_lm_iteration(c)["accepted"]
+        before = stba.stba_get_params(ctx)
+        stba.stba_set_wait_limit(ctx, 0)
+        with pytest.raises(stba.StbaError) as e:
+            stba.stba_adjoint(ctx, g)
+        assert e.value.status == 6
+        after = stba.stba_get_params(ctx)
+        assert np.array_equal(before[0], after[0]) and np.array_equal(before[1], after[1])
+        stba.stba_set_wait_limit(ctx, 1_000_000_000)
+        for a, b in zip(stba.stba_adjoint(ctx, g), stba.stba_adjoint(ref, g)):
+            assert np.max(np.abs(a - b)) <= bar * np.max(np.abs(b))
+
+
 def test_limits_out_of_range_are_refused():
     with _ctx(_scene((4, 4))) as ctx:
         for bad in (-1, 4_000_000_001):
