@@ -948,7 +948,10 @@ __device__ __forceinline__ void update_pair_tc(uint32_t* tsm, StepShared& hs, fl
 // The chain is the 64 pivots (about 55 cycles each in chol8_fast) plus two barriers and one 8-step substitution per
 // block.  A row's operands are its own smem row (16-byte loads, 68-float rows: no bank conflicts) and the diagonal
 // rows, which all lanes read at one address, so that a block moves a quarter of the shared-memory words of the
-// right-looking rank-8 updates of k_chol_panel, which bound it.
+// right-looking rank-8 updates of k_chol_panel, which bound it.  The terms of a block of columns are summed from zero
+// before they come off an entry (dot8): taken off one by one, they round eight times as often at the entry's
+// magnitude, and the unrefined step was 1.5 times as far from the exact one (120 cameras, lambda 0.05: 1.12e-6 against
+// 7.4e-7, which k_chol_panel has too), at the same time per step.
 // Panel alone on an SM: about 8.5 us (loads 1.5, product 0.65, sweep 5.9; k_chol_panel took 20), beside an
 // update CTA about 12.  Warps 5 .. 7 write each finished block out (factor, split operands, inverse).  One 512-thread CTA per SM with two tasks, so that a panel has its SM to itself, was slower
 // (12 clusters of 83 cameras 265 us against 228: an SM then waits for both tasks).
@@ -1014,11 +1017,18 @@ __device__ __forceinline__ void chol8_fast(float* T, int row0, int nk, float* ri
   if (nboost && boosted) atomicAdd(boosted, nboost);
 }
 
-__device__ __forceinline__ float dot4(float4 a, float4 b, float s) {   // s - a.b
-  s = fmaf(-a.x, b.x, s);
-  s = fmaf(-a.y, b.y, s);
-  s = fmaf(-a.z, b.z, s);
-  return fmaf(-a.w, b.w, s);
+// a.b over one block of eight columns, summed from zero: the terms of a block come off an entry with one rounding at
+// the entry's magnitude, not eight
+__device__ __forceinline__ float dot8(float4 a0, float4 a1, const float* b) {
+  const float4 b0 = *reinterpret_cast<const float4*>(b), b1 = *reinterpret_cast<const float4*>(b + 4);
+  float s = a0.x * b0.x;
+  s = fmaf(a0.y, b0.y, s);
+  s = fmaf(a0.z, b0.z, s);
+  s = fmaf(a0.w, b0.w, s);
+  s = fmaf(a1.x, b1.x, s);
+  s = fmaf(a1.y, b1.y, s);
+  s = fmaf(a1.z, b1.z, s);
+  return fmaf(a1.w, b1.w, s);
 }
 
 // the barrier of the sweep: the four row warps and the pivot warp
@@ -1157,12 +1167,13 @@ __device__ __forceinline__ void panel_tc(uint32_t* psm, StepShared& hs, float* L
         load8(last + c * LD, l0);
         load8(last + (c + 1) * LD, l1);
         float2 v = *reinterpret_cast<float2*>(blk + r * LD + c);
+        float s0 = 0.f, s1 = 0.f;
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
-          v.x = fmaf(-lr[t], l0[t], v.x);
-          v.y = fmaf(-lr[t], l1[t], v.y);
+          s0 = fmaf(lr[t], l0[t], s0);
+          s1 = fmaf(lr[t], l1[t], s1);
         }
-        *reinterpret_cast<float2*>(blk + r * LD + c) = v;
+        *reinterpret_cast<float2*>(blk + r * LD + c) = make_float2(v.x - s0, v.y - s1);
         __syncwarp();
       }
       if (lane == 0) chol8_fast(blk, kt * T + n0, nk, rinv, fail_flags + k, diag ? boosted : nullptr);
@@ -1171,11 +1182,9 @@ __device__ __forceinline__ void panel_tc(uint32_t* psm, StepShared& hs, float* L
     } else if (tid >= n1) {
       // block column b of this row, all terms
       if (b > 0) {
+        const float4 a0 = make_float4(o[0], o[1], o[2], o[3]), a1 = make_float4(o[4], o[5], o[6], o[7]);
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          const float4 l0 = *reinterpret_cast<const float4*>(last + c * LD), l1 = *reinterpret_cast<const float4*>(last + c * LD + 4);
-          x[c] = dot4(make_float4(o[4], o[5], o[6], o[7]), l1, dot4(make_float4(o[0], o[1], o[2], o[3]), l0, nx[c]));
-        }
+        for (int c = 0; c < 8; ++c) x[c] = nx[c] - dot8(a0, a1, last + c * LD);
       } else {
         load8(my, x);
       }
@@ -1183,11 +1192,11 @@ __device__ __forceinline__ void panel_tc(uint32_t* psm, StepShared& hs, float* L
       if (b + 1 < NB) {
         load8(my + n1, nx);
         const float* next = W + n1 * LD;
-#pragma unroll 2
-        for (int t = 0; t < n0; t += 4) {
-          const float4 a = *reinterpret_cast<const float4*>(my + t);
+#pragma unroll 1
+        for (int t = 0; t < n0; t += 8) {
+          const float4 a0 = *reinterpret_cast<const float4*>(my + t), a1 = *reinterpret_cast<const float4*>(my + t + 4);
 #pragma unroll
-          for (int c = 0; c < 8; ++c) nx[c] = dot4(a, *reinterpret_cast<const float4*>(next + c * LD + t), nx[c]);
+          for (int c = 0; c < 8; ++c) nx[c] -= dot8(a0, a1, next + c * LD + t);
         }
         if (tid < n1 + 8) {   // a row of the next diagonal block: for the pivot warp
           *reinterpret_cast<float4*>(my + n1) = make_float4(nx[0], nx[1], nx[2], nx[3]);
