@@ -819,6 +819,20 @@ struct StepShared {
   uint32_t taddr;
 };
 
+// A step's product accumulates in two halves of K (64 columns of tensor memory each), added in FP32: the tensor cores'
+// sums are less exact than FP32 additions at the accumulator's magnitude, which each half has to bear half as often at
+// half the size.  The unrefined step's distance from the exact one, with one accumulator -> with two (with FP32 panel
+// updates on the CUDA cores): 500 photos, lambda 0.01, 1.15e-6 -> 9.8e-7 (1.04e-6); 150 photos 1.22e-6 -> 1.05e-6
+// (1.10e-6); four accumulators 1.03e-6, but 10 % more time.
+constexpr uint32_t STEP_TMEM = 128;
+__device__ __forceinline__ void load_product(uint32_t taddr, float (&d)[32]) {
+  float e[32];
+  tc::tmem_ld32(taddr, d);
+  tc::tmem_ld32(taddr + 64, e);
+#pragma unroll
+  for (int u = 0; u < 32; ++u) d[u] += e[u];
+}
+
 // The end of a step CTA that gave up: its copies (loads) and products (multiplied; thread 0's knowledge) end before its
 // shared and tensor memory are handed back.
 __device__ __forceinline__ void step_give_up(StepShared& hs, int* fail, bool loads, bool multiplied) {
@@ -828,7 +842,7 @@ __device__ __forceinline__ void step_give_up(StepShared& hs, int* fail, bool loa
     if (multiplied) tc::mbar_wait_bounded(&hs.mbar, 0, tc::WAIT_NS);
   }
   __syncthreads();
-  if (threadIdx.x < 32) tc::tmem_dealloc(hs.taddr, 64);
+  if (threadIdx.x < 32) tc::tmem_dealloc(hs.taddr, STEP_TMEM);
 }
 
 // Four values of row `row`, columns col .. col + 3 of cluster k's scaled matrix, from the FP64 S' (the first touch of a
@@ -892,8 +906,8 @@ __device__ __forceinline__ void update_pair_tc(uint32_t* tsm, StepShared& hs, fl
       for (int pass = 0; pass < 3; ++pass)
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks)
-          tc::mma_tf32(tmem, tc::smem_desc(pa[pass] + ks * 256, 128, 2048), tc::smem_desc(pb[pass] + ks * 256, 128, 2048),
-                       idesc, (pass | ks) != 0);
+          tc::mma_tf32(tmem + 64 * (ks / 4), tc::smem_desc(pa[pass] + ks * 256, 128, 2048), tc::smem_desc(pb[pass] + ks * 256, 128, 2048),
+                       idesc, (pass | (ks & 3)) != 0);
       tc::mma_commit(&hs.mbar);
     }
   }
@@ -918,14 +932,14 @@ __device__ __forceinline__ void update_pair_tc(uint32_t* tsm, StepShared& hs, fl
     tc::fence_after_sync();
     float d[32];
     const int R = 32 * (warp & 3) + lane, c0 = 32 * (warp >> 2);
-    tc::tmem_ld32(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0, d);
+    load_product(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0, d);
 #pragma unroll
     for (int v = 0; v < 8; ++v)
       *reinterpret_cast<float4*>(stage + R * LDS_ + c0 + 4 * v) = make_float4(d[4 * v], d[4 * v + 1], d[4 * v + 2], d[4 * v + 3]);
   }
   tc::fence_before_sync();
   if (!__syncthreads_and(done)) return step_give_up(hs, fail_flags + k, true, multiplied);
-  if (warp == 0) tc::tmem_dealloc(tmem, 64);
+  if (warp == 0) tc::tmem_dealloc(tmem, STEP_TMEM);
 #pragma unroll
   for (int v = 0; v < 8; ++v) {
     if (16 * v + r16 >= rows_valid) break;
@@ -1086,8 +1100,8 @@ __device__ __forceinline__ void panel_tc(uint32_t* psm, StepShared& hs, float* L
       for (int pass = 0; pass < 3; ++pass)
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks)
-          tc::mma_tf32(tmem, tc::smem_desc(pa[pass] + ks * 256, 128, 2048), tc::smem_desc(pb[pass] + ks * 256, 128, 2048),
-                       idesc, (pass | ks) != 0);
+          tc::mma_tf32(tmem + 64 * (ks / 4), tc::smem_desc(pa[pass] + ks * 256, 128, 2048), tc::smem_desc(pb[pass] + ks * 256, 128, 2048),
+                       idesc, (pass | (ks & 3)) != 0);
       tc::mma_commit(&hs.mbar);
     }
     cp_async_wait_all();
@@ -1097,7 +1111,7 @@ __device__ __forceinline__ void panel_tc(uint32_t* psm, StepShared& hs, float* L
       tc::fence_after_sync();
       float d[32];
       const int R = 32 * (warp & 3) + lane, c0 = 32 * (warp >> 2);   // a row and half of its columns
-      tc::tmem_ld32(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0, d);
+      load_product(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0, d);
       if (R < T || !diag) {
 #pragma unroll
         for (int v = 0; v < 8; ++v) {
@@ -1115,7 +1129,7 @@ __device__ __forceinline__ void panel_tc(uint32_t* psm, StepShared& hs, float* L
   }
   // a wait gave up: the cluster fails, the step is rejected
   if (!__syncthreads_and(done)) return step_give_up(hs, fail_flags + k, true, multiplied);
-  if (warp == 0) tc::tmem_dealloc(tmem, 64);
+  if (warp == 0) tc::tmem_dealloc(tmem, STEP_TMEM);
   float* my = W + tid * LD;   // row threads
   float x[8], nx[8], o[8];
   float* Di = Dinv + (size_t)task.v_off * T + (size_t)kt * T * T;
@@ -1266,7 +1280,7 @@ __global__ void __launch_bounds__(PTC_THREADS, 2) k_step_tc(float* L, float* Din
     tc::mbar_init(&hs.mbar_load, 1);
     tc::mbar_init(&hs.mbar, 1);
   }
-  if (threadIdx.x < 32) tc::tmem_alloc(&hs.taddr, 64);
+  if (threadIdx.x < 32) tc::tmem_alloc(&hs.taddr, STEP_TMEM);
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
