@@ -170,19 +170,28 @@ __device__ __forceinline__ void load_p9(const real* __restrict__ p, int j, real 
   }
 }
 
-// Sum over the warp of v[0..N-1]; lane i < N receives sum i.
-template <int N, typename real>
-__device__ __forceinline__ real warp_sums_to_lanes(real (&v)[N]) {
+// Sums over the warp of v[0..8]; lane i < 9 receives sum i.  Transposed: every step halves the values a lane holds, 16
+// shuffles instead of 45.
+template <typename real>
+__device__ __forceinline__ real warp_sums9(const real (&v)[9]) {
   const int lane = threadIdx.x & 31;
-  real mine = real(0);
+  real x[8];
+  const bool up = (lane & 8) != 0;
 #pragma unroll
-  for (int i = 0; i < N; ++i) {
-    real x = v[i];
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) x += __shfl_xor_sync(FULL_MASK, x, d);
-    if (lane == i) mine = x;
+  for (int i = 0; i < 8; ++i) {
+    const real hi = i == 0 ? v[8] : real(0);
+    x[i] = (up ? hi : v[i]) + __shfl_xor_sync(FULL_MASK, up ? v[i] : hi, 8);
   }
-  return mine;
+#pragma unroll
+  for (int s = 4; s >= 1; s >>= 1) {
+    const bool u = (lane & s) != 0;
+#pragma unroll
+    for (int i = 0; i < s; ++i) {
+      const real send = u ? x[i] : x[i + s];
+      x[i] = (u ? x[i + s] : x[i]) + __shfl_xor_sync(FULL_MASK, send, s);
+    }
+  }
+  return x[0] + __shfl_xor_sync(FULL_MASK, x[0], 16);
 }
 
 // Per camera diagonal block of S (45 lower entries, without the damping), diag(B) and v = -J_c^T f.
@@ -395,8 +404,8 @@ __device__ __forceinline__ void add_pq(double v, double* __restrict__ pq) {
 }
 
 // The camera passes of a product: a warp takes `groups` consecutive groups of 32 slots (mostly of one camera),
-// the next group's Jacobians in flight while it works on one, and adds a camera's 9 sums up once per camera
-// instead of once per group.  Bound by the 96 bytes per observation of J (the previous product's other copy has
+// the next group's Jacobians in flight while it works on one; the sums of a group are added up in FP64 in lanes 0..8
+// and go to memory once per camera.  Bound by the 96 bytes per observation of J (the previous product's other copy has
 // displaced them from L2).  Per CG iteration of 1.1M observations / 280k observations: one group per warp and
 // no prefetch 89 / 44 us; 4 groups 85 / 41, 8 groups 80 / 42, 2 resident CTAs (3: 85 / 45): 8 groups once they
 // still leave 16 warps per SM, else 4.
@@ -423,14 +432,15 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 2 : 1)
     };
     fetch(g0);
     bool first = g0 == 0 || CS.warp_cam[g0 - 1] != CS.warp_cam[g0];   // the camera's first group is this warp's
-#pragma unroll
-    for (int c = 0; c < 9; ++c) v[c] = real(0);
+    double add = 0.0;
     for (int g = g0; g < g1; ++g) {
       const int j = CS.warp_cam[g];
       const int pt = pt_n;
       real Jc[2][9], Jp[2][3];
       unpack_j(Jn, Jc, Jp);
       if (g + 1 < g1) fetch(g + 1);
+#pragma unroll
+      for (int c = 0; c < 9; ++c) v[c] = real(0);
       if (pt >= 0) {
         const real* ui = u + 3 * (size_t)pt;
         real a0 = -(Jp[0][0] * ui[0] + Jp[0][1] * ui[1] + Jp[0][2] * ui[2]);
@@ -445,21 +455,19 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 2 : 1)
           }
         }
 #pragma unroll
-        for (int c = 0; c < 9; ++c) v[c] += Jc[0][c] * a0 + Jc[1][c] * a1;
+        for (int c = 0; c < 9; ++c) v[c] = Jc[0][c] * a0 + Jc[1][c] * a1;
       }
+      add += (double)warp_sums9(v);
       const int jn = g + 1 < g1 ? CS.warp_cam[g + 1] : -1;
       if (jn != j) {   // the camera's last group of this warp
-        const real s = warp_sums_to_lanes<9>(v);
         if (lane < 9) {
-          double add = (double)s;
           if (p) {
             if (first) add += st->lambda_used * Bdiag[9 * (size_t)j + lane] * (double)p[PSTRIDE * (size_t)j + lane];
             dot += add * pvec[9 * (size_t)j + lane];
           }
           atomicAdd(y + 9 * (size_t)j + lane, add);
         }
-#pragma unroll
-        for (int c = 0; c < 9; ++c) v[c] = real(0);
+        add = 0.0;
         first = true;
       }
     }
@@ -561,8 +569,7 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 2 : 1)
       act_n = CS.slots[sl] >= 0;
     };
     fetch(g0);
-#pragma unroll
-    for (int c = 0; c < 9; ++c) vsum[c] = real(0);
+    double add = 0.0;
     for (int g = g0; g < g1; ++g) {
       const int j = CS.warp_cam[g];
       const int vs = vs_n;
@@ -570,6 +577,8 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 2 : 1)
       real Jc[2][9], Jp[2][3];
       unpack_j(Jn, Jc, Jp);
       if (g + 1 < g1) fetch(g + 1);
+#pragma unroll
+      for (int c = 0; c < 9; ++c) vsum[c] = real(0);
       if (act) {
         real pj[9];
         load_p9(p, j, pj);
@@ -599,17 +608,16 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 2 : 1)
         }
 #pragma unroll
         for (int c = 0; c < 9; ++c)
-          vsum[c] += Jc[0][c] * b0 + Jc[1][c] * b1 + lam * (Jc[0][c] * Jc[0][c] + Jc[1][c] * Jc[1][c]) * pj[c];
+          vsum[c] = Jc[0][c] * b0 + Jc[1][c] * b1 + lam * (Jc[0][c] * Jc[0][c] + Jc[1][c] * Jc[1][c]) * pj[c];
       }
+      add += (double)warp_sums9(vsum);
       const int jn = g + 1 < g1 ? CS.warp_cam[g + 1] : -1;
       if (jn != j) {
-        const real sv = warp_sums_to_lanes<9>(vsum);
         if (lane < 9) {
-          dot += (double)sv * pvec[9 * (size_t)j + lane];
-          atomicAdd(y + 9 * (size_t)j + lane, (double)sv);
+          dot += add * pvec[9 * (size_t)j + lane];
+          atomicAdd(y + 9 * (size_t)j + lane, add);
         }
-#pragma unroll
-        for (int c = 0; c < 9; ++c) vsum[c] = real(0);
+        add = 0.0;
       }
     }
   }
