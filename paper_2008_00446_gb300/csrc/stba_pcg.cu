@@ -857,11 +857,11 @@ int pcg_iterate(const DevProblem& P, Scratch<real> W, CamSlots CS, const PcgBuff
   const int vec_blocks = std::min((m + CAMS_PER_BLOCK - 1) / CAMS_PER_BLOCK, RED_BLOCKS);
   int it = 0;
   const double tol2 = tol * tol;
-  // The GPU idles about 25 us at each reading of the residual (copy, synchronisation, the next launches); with
-  // eight iterations between readings the average overshoot of two more costs as much as the readings saved,
-  // and the system is solved no less exactly: 4 -> 8: 1000 cameras 4300 -> 4450 us, 500
-  // cameras, split 2390 -> 2300 us per LM step.
-  constexpr int CHECK_EVERY = 8;
+  // The GPU idles about 25 us at each reading of the residual (copy, synchronisation, the next launches); a solve
+  // runs on average half an interval past its tolerance.  An interval of 8 took 4404 us instead of 4186 for a step
+  // of 1000 cameras (full system), 2423 instead of 2472 for one of 500 cameras (split), and twice the products
+  // wherever four are enough.
+  constexpr int CHECK_EVERY = 4;
   while (it < max_iter) {
     const int upto = std::min(it + CHECK_EVERY, max_iter);
     for (; it < upto; ++it) {
