@@ -87,7 +87,8 @@ typedef struct {
                                STBA_FACTOR_UPDATE_SIMT); STBA_FACTOR_UPDATE_SIMT = FP32/FP64 FMA on the CUDA
                                cores; STBA_FACTOR_UPDATE_TENSOR = tcgen05 tensor cores, TF32 operands split
                                in three products for FP32 accuracy (the FP32 factor of STBA_MIXED with tile
-                               64 only; other settings return STBA_ERR_INVALID_ARG). */
+                               64 only; other settings return STBA_ERR_INVALID_ARG).  The split operands take
+                               1 KB per unknown; where that does not fit, the updates run on the CUDA cores. */
   int32_t factor_panel;     /* panel of each tile step of the cluster factorisation: 0 = default (with CUDA-core
                                updates of the FP32 factor with tile 64: STBA_FACTOR_PANEL_SPLIT when the tiles of
                                all clusters outnumber the SMs, i.e. a step runs in several waves, else _STACKED;
@@ -113,7 +114,8 @@ typedef struct {
                                STBA_PAIR_BLOCKS_STORED = the camera pass stores them (24 reals per
                                observation of device memory) and the pair pass reads them;
                                0 (default) = RECOMPUTE in mixed precision; in FP64 STORED while that takes at
-                               most a quarter of the free device memory at create, else RECOMPUTE.
+                               most a quarter of the free device memory at create, else RECOMPUTE; rows stored
+                               by default are given up when another allocation of the context needs the room.
                                Both give the same S': every pass evaluates the same rows (in FP32 with each
                                operation rounded on its own), up to the order of the FP64 atomic sums. */
   int32_t factor_fp64;      /* STBA_MIXED only: 1 = factor the cluster systems in FP64 (tile 32, CUDA cores)

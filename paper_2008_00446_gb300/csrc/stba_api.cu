@@ -89,9 +89,12 @@ struct stba_ctx {
   CamSlots cslots{};
   PairChunks pchunks{};
   CameraGraph cgraph;                   // camera graph with its observation pairs (host copy)
-  void* rowbuf = nullptr;               // stored rows of the pair pass (or a placeholder)
+  void* rowbuf = nullptr;               // stored rows of the pair pass, or null
   void* ctab = nullptr;                 // camera tables
   bool pair_recompute = true;
+  bool rows_optional = false;           // rowbuf was taken by default: freed when another allocation needs the room
+  int* base_vp = nullptr;               // [q] ReorderArgs::base_vp, whether the pair pass reads it or not
+  size_t rows_bytes = 0, jslot_bytes = 0;   // of rowbuf and pcg.Jslot while they may be freed
   // re-ordering for new assignments: fixed arguments, the two inverse maps (previous / current), scratch
   ReorderArgs reorder{};
   int* inv[2] = {nullptr, nullptr};
@@ -193,10 +196,46 @@ stba_status fail(stba_ctx* c, stba_status s, const char* fmt, ...) {
     if (e_ != cudaSuccess) return fail(c, STBA_ERR_CUDA, "%s: %s", #call, cudaGetErrorString(e_)); \
   } while (0)
 
+// Frees a buffer that the context holds for speed alone: the stored rows of the pair pass where they were the default's
+// choice (the rows are recomputed from then on), or the PCG solvers' Jacobians in slot order (gathered from then on).
+// Returns false when there is none.
+bool shed_buffer(stba_ctx* c) {
+  auto forget = [&](void* p, size_t bytes) {
+    c->allocs.erase(std::find(c->allocs.begin(), c->allocs.end(), p));
+    c->bytes_base -= bytes;
+    cudaFree(p);   // waits for the device
+  };
+  if (c->rows_optional) {
+    c->rows_optional = false;
+    forget(c->rowbuf, c->rows_bytes);
+    c->rowbuf = nullptr;
+    c->pair_recompute = true;
+    c->graph_stale = true;
+    c->reorder.base_vp = c->base_vp;   // read by the pair pass from now on
+    if (c->have_order) launch_base_vp(c->obs_base, c->obs_vp, c->reorder.base_vp, (int)c->q, c->stream);
+    return true;
+  }
+  if (c->pcg.Jslot && c->jslot_bytes) {
+    forget(c->pcg.Jslot, c->jslot_bytes);
+    c->pcg.Jslot = nullptr;
+    return true;
+  }
+  return false;
+}
+
+cudaError_t device_alloc(stba_ctx* c, void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  while (e == cudaErrorMemoryAllocation && shed_buffer(c)) {
+    cudaGetLastError();
+    e = cudaMalloc(p, bytes);
+  }
+  return e;
+}
+
 template <typename T>
 stba_status dalloc(stba_ctx* c, T** p, size_t count) {
   size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
-  cudaError_t e = cudaMalloc((void**)p, bytes);
+  cudaError_t e = device_alloc(c, (void**)p, bytes);
   if (e != cudaSuccess) {
     cudaGetLastError();
     *p = nullptr;
@@ -210,7 +249,7 @@ stba_status dalloc(stba_ctx* c, T** p, size_t count) {
 template <typename T>
 stba_status dalloc_into(stba_ctx* c, T** p, size_t count, std::vector<void*>& list) {
   size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
-  cudaError_t e = cudaMalloc((void**)p, bytes);
+  cudaError_t e = device_alloc(c, (void**)p, bytes);
   if (e != cudaSuccess) {
     cudaGetLastError();
     *p = nullptr;
@@ -323,7 +362,7 @@ stba_status ensure(stba_ctx* c, GrowBuf& g, T** p, size_t count) {
     g.ptr = nullptr;
     g.bytes = 0;
     const size_t want = bytes + bytes / 4;
-    if (cudaMalloc(&g.ptr, want) != cudaSuccess) {
+    if (device_alloc(c, &g.ptr, want) != cudaSuccess) {
       cudaGetLastError();
       g.ptr = nullptr;
       return fail(c, STBA_ERR_OOM, "cudaMalloc of %zu bytes failed", want);
@@ -696,7 +735,11 @@ stba_status set_clusters_host(stba_ctx* c, const std::vector<int>& cl) {
     if ((s = ensure(c, c->g_Dinv, &Dinv_, 2 * (size_t)c->v_total * TF * rs)) != STBA_OK) return s;
     if ((s = ensure(c, c->g_Ldiag, &Ldiag_, (size_t)c->v_total * TF * rs)) != STBA_OK) return s;
     c->fbuf.split = nullptr;
-    if (c->update_tc && (s = ensure(c, c->g_split, &c->fbuf.split, 2 * 128 * (size_t)c->v_total)) != STBA_OK) return s;
+    if (c->update_tc && ensure(c, c->g_split, &c->fbuf.split, 2 * 128 * (size_t)c->v_total) != STBA_OK) {
+      c->update_tc = 0;   // no room for the split operands (1 KB per unknown): CUDA-core updates from now on
+      const std::vector<int> again = cl;
+      return set_clusters_host(c, again);
+    }
     if ((s = ensure(c, c->g_scale, &c->fbuf.scale, (size_t)c->v_total)) != STBA_OK) return s;
     if ((s = ensure(c, c->g_x, &c->fbuf.x, (size_t)c->v_total)) != STBA_OK) return s;
     if ((s = ensure(c, c->g_r, &c->fbuf.r, (size_t)c->v_total)) != STBA_OK) return s;
@@ -1714,10 +1757,12 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
     }
     const int nwarps = cam_warp_off[m];
     if (c->use_pcg || c->use_spcg) {
-      char* js;
-      if ((s = dalloc(c, &js, 24 * 32 * (size_t)nwarps * (c->mixed ? sizeof(float) : sizeof(double)))) != STBA_OK)
-        return bail(s);
-      c->pcg.Jslot = js;
+      char* js;   // may be missing: the camera passes then gather J
+      const size_t bytes = 24 * 32 * (size_t)nwarps * (c->mixed ? sizeof(float) : sizeof(double));
+      if (dalloc(c, &js, bytes) == STBA_OK) {
+        c->pcg.Jslot = js;
+        c->jslot_bytes = bytes;
+      }
     }
     ReorderArgs& A = c->reorder;
     A.q = (int)q;
@@ -1793,8 +1838,13 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
       stored = 24 * Q * rs <= free_b / 4;
     }
     stored = stored && !c->use_pcg && !c->use_spcg;   // the PCG solvers form no off-diagonal blocks
+    const bool by_default = c->opt.pair_blocks == STBA_PAIR_BLOCKS_DEFAULT;
+    gb = nullptr;
+    if (stored && (s = dalloc(c, &gb, 24 * Q * rs)) != STBA_OK) {
+      if (!by_default) return bail(s);
+      stored = false;
+    }
     c->pair_recompute = !stored;
-    if ((s = dalloc(c, &gb, (stored ? 24 * Q : 1) * rs)) != STBA_OK) return bail(s);
     c->vp_acc = vpa;
     c->vp_info = vpi;
     c->pt_info = pti;
@@ -1802,8 +1852,14 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
     c->vgrad = vg;
     c->t_acc = ta;
     c->rowbuf = gb;
-    A.base_vp = nullptr;   // read by a pair pass that recomputes its rows
-    if (c->pair_recompute && !c->use_pcg && !c->use_spcg && (s = dalloc(c, &A.base_vp, Q)) != STBA_OK) return bail(s);
+    c->rows_optional = stored && by_default;
+    c->rows_bytes = 24 * Q * rs;
+    // read by a pair pass that recomputes its rows
+    A.base_vp = nullptr;
+    if (!c->use_pcg && !c->use_spcg) {
+      if ((s = dalloc(c, &c->base_vp, Q)) != STBA_OK) return bail(s);
+      if (c->pair_recompute) A.base_vp = c->base_vp;
+    }
     A.max_cam_obs = *std::max_element(c->h_cam_nobs.begin(), c->h_cam_nobs.end());
     A.obs_pt = c->obs_pt;
     A.pt_off = c->pt_off;

@@ -197,6 +197,8 @@ struct ReorderArgs {
 // key: [q] scratch; tile_sum: [reorder_tiles(q)] scratch; A.start: [2 (q + 1)]; counts: [3] -> number of virtual
 // points, twice the number of camera-pair instances, scratch.  With res_old, the residuals are carried over into res_new in the new order.
 size_t reorder_tiles(int64_t q);
+// base_vp (ReorderArgs) of the assignment in place
+void launch_base_vp(const int* obs_base, const int* obs_vp, int* base_vp, int q, cudaStream_t stream);
 template <typename real>
 void launch_reorder(const ReorderArgs& A, int* key, int* tile_sum, long long* counts, const real* res_old,
                     real* res_new, cudaStream_t stream);
@@ -351,7 +353,7 @@ void launch_set_lambda(DevState* st, double lam, cudaStream_t stream);
 struct PcgBuffers {
   void* J;          // [q rounded up to 32][24] J_c and J_p of every observation (working precision), in groups of
                     // 32 records interleaved by 16-byte pieces
-  void* Jslot;      // [32 * nwarps][24] the same in the order of the camera passes' slots
+  void* Jslot;      // [32 * nwarps][24] the same in the order of the camera passes' slots, or null (no room for it)
   double* Mblk;     // [m][45] diagonal blocks of S (lower, undamped B part)
   double* Bdiag;    // [m][9] diag(J_c^T J_c)
   double* Minv;     // [m][81] inverse damped diagonal blocks (the preconditioner)

@@ -405,6 +405,15 @@ __global__ void __launch_bounds__(256) k_zero_vp(float4* __restrict__ p, const l
 
 }  // namespace
 
+__global__ void k_base_vp(int q, const int* __restrict__ obs_base, const int* __restrict__ obs_vp, int* __restrict__ base_vp) {
+  const int o = blockIdx.x * blockDim.x + threadIdx.x;
+  if (o < q) base_vp[obs_base[o]] = obs_vp[o];
+}
+
+void launch_base_vp(const int* obs_base, const int* obs_vp, int* base_vp, int q, cudaStream_t stream) {
+  k_base_vp<<<(q + 255) / 256, 256, 0, stream>>>(q, obs_base, obs_vp, base_vp);
+}
+
 size_t reorder_tiles(int64_t q) {
   const size_t ntiles = (size_t)((q + SCAN_TILE - 1) / SCAN_TILE);
   return 3 * ntiles + ntiles / SUPER + 1;

@@ -196,7 +196,7 @@ __device__ __forceinline__ real warp_sums9(const real (&v)[9]) {
 
 // Per camera diagonal block of S (45 lower entries, without the damping), diag(B) and v = -J_c^T f.
 template <typename real>
-__global__ void __launch_bounds__(256) k_pcg_precond(DevProblem P, CamSlots CS, const real* __restrict__ J,
+__global__ void __launch_bounds__(256) k_pcg_precond(DevProblem P, CamSlots CS, bool gather, const real* __restrict__ J,
                                                      const real* __restrict__ pt_info, double* __restrict__ Mblk,
                                                      double* __restrict__ Bdiag, real* __restrict__ vgrad) {
   const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(256) k_pcg_precond(DevProblem P, CamSlots CS, 
 #pragma unroll
   for (int s = 0; s < 3; ++s) Jp[0][s] = Jp[1][s] = real(0);
   if (o >= 0) {
-    load_j(J, 32 * (size_t)gw + lane, Jc, Jp);   // rows already scaled by sqrt(rho') under a robust loss
+    load_j(J, gather ? (size_t)o : 32 * (size_t)gw + lane, Jc, Jp);   // rows already scaled by sqrt(rho') under a robust loss
     f[0] = res_ptr<real>(P)[2 * (size_t)o];
     f[1] = res_ptr<real>(P)[2 * (size_t)o + 1];
     const real sw = huber_sqrt_weight<real>(P.huber_a, f[0], f[1]);
@@ -413,7 +413,8 @@ static int cam_groups(int nwarps) { return nwarps >= 8 * 16 * num_sms() ? 8 : 4;
 
 // y_j += sum_{o in camera j} J_c^T (J_c p_j - J_p u_pt(o)) (+ lambda diag(B_j) p_j, added by the camera's first
 // group), and pq += p.y.  With p = null the J_c p term is absent (right-hand side pass).
-template <typename real>
+// GATHER: J is in observation order (there was no room for the copy in slot order).
+template <typename real, bool GATHER>
 __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 2 : 1)
     k_pcg_cam(CamSlots CS, int groups, const real* __restrict__ J, const real* __restrict__ p,
               const double* __restrict__ pvec, const real* __restrict__ u, const double* __restrict__ Bdiag,
@@ -426,9 +427,11 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 2 : 1)
     int pt_n = -1;   // point of the prefetched slot, -1 for a padding slot
     auto fetch = [&](int g) {
       const size_t sl = 32 * (size_t)g + lane;
-      load_j_vec(J, sl, Jn);   // unconditional (a padding slot's record is unused): not behind the load of the slot
+      const int o = CS.slots[sl];
+      // unconditional (a padding slot's record is unused): in slot order not behind the load of the slot
+      load_j_vec(J, GATHER ? (size_t)max(o, 0) : sl, Jn);
       const int pt = CS.pv[sl].x;
-      pt_n = CS.slots[sl] >= 0 ? pt : -1;
+      pt_n = o >= 0 ? pt : -1;
     };
     fetch(g0);
     bool first = g0 == 0 || CS.warp_cam[g0 - 1] != CS.warp_cam[g0];   // the camera's first group is this warp's
@@ -549,7 +552,7 @@ __global__ void k_spcg_u(const long long* __restrict__ counts, const real* __res
 // y_j += sum over the camera's observations of J_c^T N J_c p_j (single-observation virtual points, N =
 // (I + J_p Lambda^-1 J_p^T)^-1, Lambda = lambda diag(J_p^T J_p)) or J_c^T (J_c p_j - J_p u_v) (the others),
 // plus lambda diag(J_c^T J_c) p_j: S' p for the cameras of every cluster
-template <typename real>
+template <typename real, bool GATHER>
 __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 2 : 1)
     k_spcg_cam(CamSlots CS, int groups, const real* __restrict__ J, const real* __restrict__ p,
                const double* __restrict__ pvec, const real* __restrict__ u, const DevState* st,
@@ -564,9 +567,10 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 2 : 1)
     bool act_n = false;   // not a padding slot
     auto fetch = [&](int g) {
       const size_t sl = 32 * (size_t)g + lane;
-      load_j_vec(J, sl, Jn);   // unconditional, as in k_pcg_cam
+      const int o = CS.slots[sl];
+      load_j_vec(J, GATHER ? (size_t)max(o, 0) : sl, Jn);   // as in k_pcg_cam
       vs_n = CS.pv[sl].y;
-      act_n = CS.slots[sl] >= 0;
+      act_n = o >= 0;
     };
     fetch(g0);
     double add = 0.0;
@@ -811,7 +815,7 @@ void pcg_prepare(const DevProblem& P, Scratch<real> W, CamSlots CS, const PcgBuf
   const int pt_blocks = std::min((P.n + 255) / 256, 4096);
   const int vec_blocks = std::min((m + CAMS_PER_BLOCK - 1) / CAMS_PER_BLOCK, RED_BLOCKS);
   k_pcg_jac<real><<<obs_blocks, 256, 0, stream>>>(P, J);
-  k_pcg_slot_j<real><<<std::min(cam_blocks, num_sms() * 16), 256, 0, stream>>>(CS, J, Js);
+  if (Js) k_pcg_slot_j<real><<<std::min(cam_blocks, num_sms() * 16), 256, 0, stream>>>(CS, J, Js);
   cudaMemsetAsync(B.Bdiag, 0, 9 * (size_t)m * sizeof(double), stream);
   cudaMemsetAsync(B.pq, 0, PQ_SLOTS * sizeof(double), stream);
   const int inv_blocks = (m + INV_WARPS - 1) / INV_WARPS;
@@ -827,13 +831,14 @@ void pcg_prepare(const DevProblem& P, Scratch<real> W, CamSlots CS, const PcgBuf
   cudaMemsetAsync(B.Mblk, 0, 45 * (size_t)m * sizeof(double), stream);
   cudaMemsetAsync(W.vgrad, 0, 9 * (size_t)m * sizeof(real), stream);
   cudaMemsetAsync(B.tpt, 0, 3 * (size_t)P.n * sizeof(real), stream);
-  k_pcg_precond<real><<<cam_blocks, 256, 0, stream>>>(P, CS, Js, W.pt_info, B.Mblk, B.Bdiag, W.vgrad);
+  k_pcg_precond<real><<<cam_blocks, 256, 0, stream>>>(P, CS, !Js, Js ? Js : J, W.pt_info, B.Mblk, B.Bdiag, W.vgrad);
   k_pcg_invert<<<inv_blocks, 32 * INV_WARPS, 0, stream>>>(m, B.Mblk, B.Bdiag, st, B.Minv);
   // right-hand side b = v - E C^-1 w: the camera pass with p = 0 and u = C^-1 w
   k_pcg_uw<real><<<pt_blocks, 256, 0, stream>>>(P.n, W.pt_info, upt);
   cudaMemsetAsync(B.q, 0, (size_t)m9 * sizeof(double), stream);
-  k_pcg_cam<real><<<(cam_blocks + groups - 1) / groups, 256, 0, stream>>>(CS, groups, Js, nullptr, nullptr, upt,
-                                                                           B.Bdiag, st, B.q, B.pq);
+  const auto pcg_cam = Js ? k_pcg_cam<real, false> : k_pcg_cam<real, true>;
+  pcg_cam<<<(cam_blocks + groups - 1) / groups, 256, 0, stream>>>(CS, groups, Js ? Js : J, nullptr, nullptr, upt,
+                                                                  B.Bdiag, st, B.q, B.pq);
   k_pcg_init<real><<<vec_blocks, VEC_THREADS, 0, stream>>>(m, W.vgrad, B.q, B.Minv, B.x, B.r, B.p, pw, B.partial);
   k_pcg_start<<<1, VEC_THREADS, 0, stream>>>(B.partial, vec_blocks, B.scal);
 }
@@ -855,6 +860,9 @@ int pcg_iterate(const DevProblem& P, Scratch<real> W, CamSlots CS, const PcgBuff
   const int cam_blocks = (CS.nwarps + 7) / 8, groups = cam_groups(CS.nwarps);
   const int pt_blocks = std::min((P.n + 255) / 256, 4096);
   const int vec_blocks = std::min((m + CAMS_PER_BLOCK - 1) / CAMS_PER_BLOCK, RED_BLOCKS);
+  const auto pcg_cam = Js ? k_pcg_cam<real, false> : k_pcg_cam<real, true>;
+  const auto spcg_cam = Js ? k_spcg_cam<real, false> : k_spcg_cam<real, true>;
+  const real* Jc = Js ? Js : J;   // the camera passes' rows
   int it = 0;
   const double tol2 = tol * tol;
   // The GPU idles about 25 us at each reading of the residual (copy, synchronisation, the next launches); a solve
@@ -872,13 +880,12 @@ int pcg_iterate(const DevProblem& P, Scratch<real> W, CamSlots CS, const PcgBuff
         real* uvp = reinterpret_cast<real*>(B.uvp);
         k_spcg_Et<real><<<seg_blocks, 256, 0, stream>>>(P, J, pw, tvp);
         k_spcg_u<real><<<2 * RED_BLOCKS, 256, 0, stream>>>(B.counts, W.vp_info, tvp, uvp);
-        k_spcg_cam<real><<<(cam_blocks + groups - 1) / groups, 256, 0, stream>>>(CS, groups, Js, pw, B.p, uvp, st, B.q,
-                                                                                B.pq);
+        spcg_cam<<<(cam_blocks + groups - 1) / groups, 256, 0, stream>>>(CS, groups, Jc, pw, B.p, uvp, st, B.q, B.pq);
       } else {
         k_pcg_Et<real><<<seg_blocks, 256, 0, stream>>>(P, J, pw, tpt);
         k_pcg_u<real><<<pt_blocks, 256, 0, stream>>>(P.n, W.pt_info, tpt, upt);
-        k_pcg_cam<real><<<(cam_blocks + groups - 1) / groups, 256, 0, stream>>>(CS, groups, Js, pw, B.p, upt, B.Bdiag,
-                                                                                st, B.q, B.pq);
+        pcg_cam<<<(cam_blocks + groups - 1) / groups, 256, 0, stream>>>(CS, groups, Jc, pw, B.p, upt, B.Bdiag, st, B.q,
+                                                                        B.pq);
       }
       k_pcg_update<<<vec_blocks, VEC_THREADS, 0, stream>>>(m, B.pq, B.scal, parity, B.p, B.q, B.Minv, B.x, B.r, B.z,
                                                            B.partial);
