@@ -309,7 +309,8 @@ stba_status stba_cluster_sgc(stba_ctx* ctx, int32_t gamma, double beta, uint64_t
  * the cluster factorisation on the current parameters and cluster assignment, restores the parameters,
  * damping and cost after each trial, and keeps the fastest for the following iterations.  Candidates
  * (STBA_MIXED; FP64 has one):
- *   0 = tile 64, split panel, tensor-core update (as 5)       1 = tile 64, split panel, CUDA-core update
+ *   0 = tile 64, split panel, tensor-core update (the same    1 = tile 64, split panel, CUDA-core update
+ *       kernels as 5: timed once, never the choice)
  *   2 = tile 64, stacked panel, CUDA-core update              3 = tile 32, stacked panel, CUDA-core update
  *   4 = tile 64, persistent (one launch of 8-CTA clusters)  5 = tile 64, stacked panel, tensor-core update
  *                                                              (the default)

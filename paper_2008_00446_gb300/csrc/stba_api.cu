@@ -1366,7 +1366,7 @@ stba_status stba_autotune(stba_ctx* c, int32_t iterations, int32_t* choice, floa
   stba_status s = STBA_OK;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) ok = false;
-  for (int t = 0; t < NCAND && ok && s == STBA_OK; ++t) {
+  for (int t = 1; t < NCAND && ok && s == STBA_OK; ++t) {   // 0 is the configuration of 5 under another name
     c->tile = cand_tile[t];
     c->update_tc = cand_tc[t];
     c->panel_choice = cand_panel[t];
@@ -1386,6 +1386,7 @@ stba_status stba_autotune(stba_ctx* c, int32_t iterations, int32_t* choice, floa
       best = t;
     }
   }
+  if (ms) ms[0] = ms[5];
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   if (s == STBA_OK && ok && best >= 0) {
