@@ -121,8 +121,9 @@ struct stba_ctx {
   // scratch (real = float in mixed mode, double in FP64 mode)
   void *vp_acc = nullptr, *vp_info = nullptr, *pt_info = nullptr, *pt_acc = nullptr, *S = nullptr, *b = nullptr, *vgrad = nullptr,
        *t_acc = nullptr;
-  double *dc = nullptr, *dp = nullptr, *partial = nullptr, *cam_rt = nullptr;
-  float *cam_df = nullptr, *pt_df = nullptr;   // double-float tables of the mixed-mode cost
+  double *dc = nullptr, *dp = nullptr, *partial = nullptr;
+  double* cam_rt = nullptr;                    // camera table of the cost (FP64)
+  float *cam_df = nullptr, *pt_df = nullptr;   // double-float tables of the cost (mixed precision)
   float *cams_f = nullptr, *pts_f = nullptr;   // FP32 copies (mixed precision)
   void* edc = nullptr;                         // E dc per camera (working precision)
   float4* obs_uvdf = nullptr;
@@ -1626,7 +1627,6 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
   if ((s = dalloc(c, &c->dc, 9 * (size_t)m)) != STBA_OK) return bail(s);
   if ((s = dalloc(c, &c->dp, 3 * (size_t)n)) != STBA_OK) return bail(s);
   if ((s = dalloc(c, &c->partial, 6 * (size_t)RED_BLOCKS)) != STBA_OK) return bail(s);
-  if ((s = dalloc(c, &c->cam_rt, 15 * (size_t)m)) != STBA_OK) return bail(s);
   {
     char* ct;
     const size_t rs = c->mixed ? sizeof(float) : sizeof(double);
@@ -1635,9 +1635,10 @@ stba_status stba_create(const double* cameras, int64_t m, const double* points, 
     if ((s = dalloc(c, &ct, VPI * (size_t)m * rs)) != STBA_OK) return bail(s);
     c->edc = ct;
   }
-  if ((s = dalloc(c, &c->cam_df, 28 * (size_t)m)) != STBA_OK) return bail(s);
-  if ((s = dalloc(c, &c->pt_df, 6 * (size_t)n)) != STBA_OK) return bail(s);
+  if (!c->mixed && (s = dalloc(c, &c->cam_rt, 15 * (size_t)m)) != STBA_OK) return bail(s);
   if (c->mixed) {
+    if ((s = dalloc(c, &c->cam_df, 28 * (size_t)m)) != STBA_OK) return bail(s);
+    if ((s = dalloc(c, &c->pt_df, 6 * (size_t)n)) != STBA_OK) return bail(s);
     if ((s = dalloc(c, &c->cams_f, 9 * (size_t)m)) != STBA_OK) return bail(s);
     if ((s = dalloc(c, &c->pts_f, 3 * (size_t)n)) != STBA_OK) return bail(s);
   }

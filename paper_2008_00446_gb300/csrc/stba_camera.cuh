@@ -66,42 +66,6 @@ __device__ __forceinline__ Cam<real> load_cam(const double* c) {
   return C;
 }
 
-template <typename real>
-__device__ __forceinline__ Cam<real> load_cam_step(const double* c, const double* dc) {
-  Cam<real> C;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    C.w[k] = (real)(c[k] + dc[k]);
-    C.t[k] = (real)(c[3 + k] + dc[3 + k]);
-  }
-  C.f = (real)(c[6] + dc[6]);
-  C.k1 = (real)(c[7] + dc[7]);
-  C.k2 = (real)(c[8] + dc[8]);
-  return C;
-}
-
-// Residual only (cost evaluation).  Returns the depth Xc.z in *z.
-template <typename real>
-__device__ __forceinline__ void project_residual(const Cam<real>& C, const real X[3], real u_obs, real v_obs,
-                                                 real r[2], real* z) {
-  const real* w = C.w;
-  real s = w[0] * w[0] + w[1] * w[1] + w[2] * w[2];
-  real a, b, da, db;
-  rodrigues_coeffs(s, a, b, da, db);
-  real wx[3] = {w[1] * X[2] - w[2] * X[1], w[2] * X[0] - w[0] * X[2], w[0] * X[1] - w[1] * X[0]};
-  real wd = w[0] * X[0] + w[1] * X[1] + w[2] * X[2];
-  real Xc[3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) Xc[i] = X[i] + a * wx[i] + b * (w[i] * wd - s * X[i]) + C.t[i];
-  real iz = real(1) / Xc[2];
-  real x = Xc[0] * iz, y = Xc[1] * iz;
-  real r2 = x * x + y * y;
-  real d = real(1) + r2 * (C.k1 + C.k2 * r2);
-  r[0] = C.f * d * x - u_obs;
-  r[1] = C.f * d * y - v_obs;
-  *z = Xc[2];
-}
-
 // Residual and Jacobian blocks: Jc (2x9, row-major) and Jp (2x3).  With want_cam = false only Jp.
 template <typename real, bool want_cam>
 __device__ __forceinline__ void project_jacobian(const Cam<real>& C, const real X[3], real u_obs, real v_obs,

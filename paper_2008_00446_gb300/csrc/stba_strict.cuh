@@ -24,7 +24,6 @@ struct SF {
   friend __device__ __forceinline__ SF operator-(SF a, SF b) { return SF(__fsub_rn(a.v, b.v)); }
   friend __device__ __forceinline__ SF operator-(SF a) { return SF(-a.v); }
   friend __device__ __forceinline__ SFProd operator*(SF a, SF b);
-  friend __device__ __forceinline__ SF operator/(SF a, SF b) { return SF(__fdiv_rn(a.v, b.v)); }
 };
 
 // a * b, not yet rounded
@@ -42,8 +41,6 @@ struct SFProd {
   friend __device__ __forceinline__ SFProd operator*(SFProd p, SF c) { return SFProd{p.rounded(), c.v}; }
   friend __device__ __forceinline__ SFProd operator*(SF c, SFProd p) { return SFProd{c.v, p.rounded()}; }
   friend __device__ __forceinline__ SFProd operator*(SFProd p, SFProd q) { return SFProd{p.rounded(), q.rounded()}; }
-  friend __device__ __forceinline__ SF operator/(SFProd p, SF d) { return SF(__fdiv_rn(p.rounded(), d.v)); }
-  friend __device__ __forceinline__ SF operator/(SF n, SFProd p) { return SF(__fdiv_rn(n.v, p.rounded())); }
 };
 
 __device__ __forceinline__ SF::SF(const SFProd& p) : v(p.rounded()) {}
