@@ -105,8 +105,8 @@ typedef struct {
                                with tile 64 only; other settings return STBA_ERR_INVALID_ARG). */
   int32_t solve_cluster;    /* CTAs per thread-block cluster of each camera cluster's triangular solves
                                (2, 4 or 8; 0 = default: 8 while the clusters' solve CTAs fit in two waves on
-                               the SMs, else 4): more CTAs share a tile step's products, fewer make its
-                               cluster barrier and distributed-shared-memory exchange cheaper. */
+                               the SMs, else 4): more CTAs share a tile step's products, fewer leave SMs to
+                               the solves of other clusters. */
   int32_t pair_blocks;      /* off-diagonal camera blocks of S' (Eq. 10, 13), -sum over the observation pairs
                                of a virtual point of Jc_a^T (P_a^T P_b) Jc_b with P_o = L_v^-1 Jp,o^T:
                                STBA_PAIR_BLOCKS_RECOMPUTE = the pair pass recomputes P_o and Jc_o from the
@@ -229,9 +229,9 @@ stba_status stba_record(stba_ctx* ctx, int32_t max_iter);
  * physical w), including the dependence of h_v / H_i on the parameters.
  * Errors: STBA_ERR_STATE with the PCG solvers or the Huber loss, if nothing was recorded, or if
  * stba_set_params replaced the parameters during the recording; STBA_ERR_TIMEOUT or STBA_ERR_NOT_SPD if a device
- * wait gave up, or a factorisation failed, while a step was recomputed (no output is then written).  On return the parameters, the cluster
- * assignment and the LM state are those before the call.  The call synchronises the stream and allocates
- * no memory (its buffers are held with the tape). */
+ * wait gave up, or a factorisation failed, while a step was recomputed (no output is then written).  On return the
+ * parameters, the cluster assignment and the LM state are those before the call.  The call synchronises the stream
+ * and allocates no memory (its buffers are held with the tape). */
 stba_status stba_adjoint(stba_ctx* ctx, const double* dL_dcams, const double* dL_dpts, double* dL_dobs,
                          double* dL_dcams0, double* dL_dpts0);
 
@@ -323,8 +323,8 @@ stba_status stba_autotune(stba_ctx* ctx, int32_t iterations, int32_t* choice, fl
 
 /* Limit of the device-side waits of the cluster factorisation and solves (for their own copies, tensor-core products
  * and the pieces of a solve's other CTAs), 0 .. 4e9 ns; one second at create.  A wait that reaches it gives up: the
- * cluster counts as failed and the LM step is rejected; stba_adjoint returns STBA_ERR_TIMEOUT.  0 gives up whatever is not there at the first look, which
- * makes the failure path testable.  Takes effect with the next iteration. */
+ * cluster counts as failed and the LM step is rejected; stba_adjoint returns STBA_ERR_TIMEOUT.  0 gives up whatever
+ * is not there at the first look, which makes the failure path testable.  Takes effect with the next iteration. */
 stba_status stba_set_wait_limit(stba_ctx* ctx, int64_t nanoseconds);
 
 /* Measured arithmetic peaks of the current GPU, the denominators of the factorisation's roofline.  The

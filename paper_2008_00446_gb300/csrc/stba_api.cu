@@ -553,8 +553,10 @@ stba_status set_clusters_host(stba_ctx* c, const std::vector<int>& cl) {
   // stacked panel when they fit in one wave (a single kernel per step on the critical path).  The tensor-core steps
   // (k_step_tc) are always stacked.
   c->persistent = c->mixed && TF == 64 && c->panel_choice == STBA_FACTOR_PANEL_PERSISTENT;
-  // CTAs per cluster solve: 8 while the solves' CTAs fit in about two waves (more CTAs share each tile step's
-  // products), 4 beyond (cheaper barriers and exchanges once the solves queue for SMs anyway)
+  // CTAs per cluster solve: 8 while the solves' CTAs fit in two waves (more CTAs share each tile step's products), 4
+  // beyond, where the solves queue for SMs.  Solve stage with 8 / 4 / 2: one cluster of 400 cameras 332 / 555 / 1009
+  // us, 12 of 83 63 / 66 / 90, 30 of 100 137 / 137 / 178, 38 of 79 139 / 123 / 137, 60 of 50 102 / 88 / 88, 100 of 30
+  // 100 / 80 / 63; FP64, 20 of 50 139 / 125 / 174, 50 of 20 80 / 76 / 63
   c->solve_cs = c->opt.solve_cluster ? c->opt.solve_cluster : ((int64_t)l * 8 <= 2 * (int64_t)num_sms() ? 8 : 4);
   if (c->mixed && TF == 64 && c->panel_choice != STBA_FACTOR_PANEL_STACKED && !c->persistent) {
     int64_t tiles = 0;

@@ -791,8 +791,8 @@ __global__ void __launch_bounds__(256) k_chol_update(F* L, DevProblem P, const i
 // converts anything; the product goes from TMEM through shared memory, so that the updated values are
 // read and written 256 contiguous bytes per row.  The waits for the copies and
 // the MMAs are bounded: a CTA that gives up marks the cluster failed (the LM step is rejected), waits, bounded again,
-// for what it has in flight, frees its tensor memory and returns.  When i0 + 1 is past the cluster's last tile, the second half of A is undefined and
-// its rows are not written.
+// for what it has in flight, frees its tensor memory and returns.  When i0 + 1 is past the cluster's last tile, the
+// second half of A is undefined and its rows are not written.
 // Bound by L2 traffic (96 KB of operands, 64 KB of updated values per tile pair).  With operands loaded, split and
 // stored by the threads the factorisation stage took 1194 us instead of 922 (13 uneven clusters), 853 instead of 707
 // (one of 400 cameras); with one row per lane and 16 bytes per access on top, the L1 pipe was 71 % busy.
@@ -856,7 +856,6 @@ __device__ __forceinline__ float4 scaled4(const double* __restrict__ Sk, const d
                      (float)(b.y * sr * sk[col + 3]));
 }
 
-// FIRST: step 0, whose old values come from S' (every tile this kernel ever updates is in its list there).
 // The split operands of a tile column: hi and lo parts of every tile, in the core-matrix layout, SPLIT_TILE words per
 // tile at its row offset; written by the panel that makes the column, read by the next launch (two columns in turn).
 constexpr int SPLIT_TILE = 2 * 64 * 64;
@@ -864,6 +863,7 @@ __device__ __forceinline__ uint32_t* split_tile(uint32_t* split, int64_t v_total
   return split + (size_t)(kt & 1) * v_total * 128 + (size_t)(v_off + tile * 64) * 128;
 }
 
+// FIRST: step 0, whose old values come from S' (every tile this kernel ever updates is in its list there).
 template <bool FIRST>
 __device__ __forceinline__ void update_pair_tc(uint32_t* tsm, StepShared& hs, float* L, uint32_t* split,
                                                const double* __restrict__ S, const double* scale,
@@ -967,8 +967,9 @@ __device__ __forceinline__ void update_pair_tc(uint32_t* tsm, StepShared& hs, fl
 // magnitude, and the unrefined step was 1.5 times as far from the exact one (120 cameras, lambda 0.05: 1.12e-6 against
 // 7.4e-7, which k_chol_panel has too), at the same time per step.
 // Panel alone on an SM: about 8.5 us (loads 1.5, product 0.65, sweep 5.9; k_chol_panel took 20), beside an
-// update CTA about 12.  Warps 5 .. 7 write each finished block out (factor, split operands, inverse).  One 512-thread CTA per SM with two tasks, so that a panel has its SM to itself, was slower
-// (12 clusters of 83 cameras 265 us against 228: an SM then waits for both tasks).
+// update CTA about 12.  Warps 5 .. 7 write each finished block out (factor, split operands, inverse).  One 512-thread
+// CTA per SM with two tasks, so that a panel has its SM to itself, was slower (12 clusters of 83 cameras 265 us
+// against 228: an SM then waits for both tasks).
 constexpr int PTC_THREADS = 256;
 constexpr int PTC_LD = 68;
 constexpr size_t PTC_SMEM = sizeof(float) * 128 * PTC_LD + sizeof(uint32_t) * 2 * 128 * 64;   // tile, A hi / lo: 98 KB
@@ -1045,7 +1046,6 @@ __device__ __forceinline__ float dot8(float4 a0, float4 a1, const float* b) {
   return fmaf(a1.w, b1.w, s);
 }
 
-// the barrier of the sweep: the four row warps and the pivot warp
 __device__ __forceinline__ void panel_tc(uint32_t* psm, StepShared& hs, float* L, float* Dinv, uint32_t* split,
                                          const double* __restrict__ S, const double* scale,
                                          const TileTask& task, int kt, int* fail_flags, int* boosted, int64_t v_total,
@@ -1681,17 +1681,18 @@ __global__ void __launch_bounds__(256) k_tri_solve(DevProblem P, const F* L, con
 }
 
 // ------------------------------------------------------------------------------------------------------
-// The same solve as a data flow (clusters whose accumulators fit in shared memory: up to about 280 tile rows of the
-// FP32 factor with 8 CTAs; k_tri_solve beyond): tile row i belongs to CTA i mod CS
-// of the cluster's CS CTAs.  Forward, the owner of row k finishes t_k = r_k - sum_j L_kj y_j, forms y_k = D_k^-1 t_k and
+// The same solve as a data flow (clusters whose accumulators fit in shared memory: up to 94, 168 and 280 tile rows of
+// either factor with 2, 4 and 8 CTAs; k_tri_solve beyond): tile row i belongs to CTA i mod CS of the cluster's CS CTAs.
+// Forward, the owner of row k finishes t_k = r_k - sum_j L_kj y_j, forms y_k = D_k^-1 t_k and
 // sends it to every CTA with asynchronous stores counted by that CTA's mbarrier of step k; whoever has y_k subtracts
 // L_ik y_k from its rows i > k, row k + 1 first, whose owner then goes on to y_k+1 before its other rows.  The
 // backward pass is the same on reversed indices with L_ki^T and D_k^-T.  Only the mbarrier it counts on tells that an
 // asynchronous store has arrived (a cluster barrier orders its issue), so after a pass every CTA waits for all nt
 // pieces, the ones that none of its rows needs too: x overwrites y only once every y has arrived everywhere, and no
 // CTA leaves while a store to it is under way.  A step's chain is two 64 x 64 products by
-// 256 threads and one remote store: about 0.5 us, against 2.4 us with a cluster barrier, a gather of the partial
-// products from all CTAs and five block barriers per step.  Nothing depends on a tile's address on the vector, so
+// 256 threads and one remote store: 0.8 us (12 clusters of 83 cameras) to 1.4 us (one of 400, whose later steps also
+// have 7 rows per CTA to update), against 2.4 us with a cluster barrier, a gather of the partial products from all
+// CTAs and five block barriers per step.  Nothing depends on a tile's address on the vector, so
 // each thread keeps its elements of the next NB tiles in registers (loads in flight while it waits for y_k).
 // NB = 4 tiles of the FP32 factor (64 registers; 3 and 4 alike at 15 tile rows, 4 better beyond, 5 spills).
 // Solve stage with one refinement step, before (k_tri_solve, one residual CTA per tile row) -> now: 12 clusters of 83
@@ -1995,8 +1996,8 @@ void launch_tri_solve(const DevProblem& P, const F* L, const F* Dinv, const doub
 }
 
 // r = b - S x (FP64) with S symmetric, lower triangle stored; r was set to b before.  One CTA per
-// (cluster, 32-row tile row I, RES_TILES of its tiles); its 4 warps take the tiles (I, J), J <= I, in turn.  A warp stages the
-// 32 x 32 tile in shared memory with coalesced row loads, then lane l forms both the row sum of tile row l
+// (cluster, 32-row tile row I, RES_TILES of its tiles); its 4 warps take the tiles (I, J), J <= I, in turn.  A warp
+// stages the 32 x 32 tile in shared memory with coalesced row loads, then lane l forms both the row sum of tile row l
 // (S_IJ x_J, kept in registers over the warp's tiles) and the column sum of tile column l (S_IJ^T x_I,
 // added atomically to r_J; on the diagonal tile only below the diagonal).
 constexpr int RES_WARPS = 4;

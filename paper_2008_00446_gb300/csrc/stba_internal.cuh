@@ -135,7 +135,9 @@ void launch_list_chunks(const PairChunks& B, const int* cam_cluster, const int* 
 // Pairs per chunk: as many as leave eight chunks of the camera graph's pairs per resident warp of the pair pass
 // (24 warps on 152 SMs; chunks are handed out by a counter), between 64 and 128.  S' build stage with 64 / 128 /
 // 256 at most: 1000 cameras, 2.9M pairs inside clusters 183 / 177 / 185 us; 2000 sequential cameras, 10.5M pairs
-// 510 / 483 / 479; 6000 cameras, 12M pairs 868 / 774 / 774; 400 cameras in FP64, 0.5M pairs 574 / 625 / 605.
+// 510 / 483 / 479; 6000 cameras, 12M pairs 868 / 774 / 774; 400 cameras in FP64, 0.5M pairs 574 / 625 / 605.  FP32
+// sums run over a chunk: with up to 128 pairs of two products the off-diagonal blocks are closer to FP64 than with 64
+// pairs of three (2000 sequential cameras, lambda 0.05: 7.5e-8 of the unit diagonal against 1.3e-7).
 constexpr int PAIR_CHUNK_MIN = 64, PAIR_CHUNK_MAX = 128;
 inline int pair_chunk(int64_t pairs) {
   return (int)std::min<int64_t>(PAIR_CHUNK_MAX, std::max<int64_t>(PAIR_CHUNK_MIN, pairs / (8 * 24 * 152) / 16 * 16));
@@ -195,7 +197,8 @@ struct ReorderArgs {
   int* slots;               // [32 * warps] the same padded to whole warps (-1)
 };
 // key: [q] scratch; tile_sum: [reorder_tiles(q)] scratch; A.start: [2 (q + 1)]; counts: [3] -> number of virtual
-// points, twice the number of camera-pair instances, scratch.  With res_old, the residuals are carried over into res_new in the new order.
+// points, twice the number of camera-pair instances, scratch.  With res_old, the residuals are carried over into
+// res_new in the new order.
 size_t reorder_tiles(int64_t q);
 // base_vp (ReorderArgs) of the assignment in place
 void launch_base_vp(const int* obs_base, const int* obs_vp, int* base_vp, int q, cudaStream_t stream);

@@ -372,8 +372,12 @@ void launch_failed_io(DevState* st, double* x, int to_double, cudaStream_t strea
 // stays off the FP64 pipe, which on this GPU runs at 1/64 of the FP32 rate.  With stored pair rows it also
 // stores (Pm_o, the tilde rows of Jc,o) of every observation of a multi-observation virtual point.
 // Both passes evaluate the same rows (stba_camtab.cuh; in FP32 with every operation rounded on its own): the
-// diagonal and off-diagonal blocks of a virtual point come from bitwise the same J_c and J_p whether they are
-// stored or recomputed, and the FP32 S' does not change with the compiler's choice of fused multiply-adds.
+// diagonal and off-diagonal blocks of a virtual point come from bitwise the same Jt and J_p whether they are
+// stored or recomputed, and the FP32 S' does not change with the compiler's choice of fused multiply-adds.  The
+// constant factor Jl of the three rotation columns is rounded in per observation here and once per block in the pair
+// pass; with it per observation in both, the solution of S' x = b' is as far from FP64 as this way (lambda 1e-5 to
+// 0.05, ten systems of each of five kinds: medians within 7 %), and S' and b' themselves are closer to FP64 than
+// from rows that evaluate Rodrigues' formula (off-diagonal blocks of 1000 photos 3.9e-9 of the unit diagonal, 5.5e-9).
 constexpr int ROWREC = 24;   // reals per stored observation: Pm (6), tilde rows of J_c (18)
 
 // On return lane L holds the sum over the warp's lanes of v[L].  Each halving step keeps one half of the
@@ -552,9 +556,9 @@ __global__ void __launch_bounds__(256, sizeof(real) == 4 ? 4 : 3) k_cam_pass(Dev
 // contributes exactly when both cameras are in one cluster (its two observations of a point are then in
 // one virtual point), and a chunk adds to one block only.  The re-ordering of an assignment lists the
 // chunks whose edge lies inside a cluster; the warps of a fixed grid take them one by one from that list.  A warp
-// works on pieces of PB_CH pairs: lane (side, j) forms the rows of its pair's observation by camera x (side 0) or y (side 1) from
-// the camera's table, the point and L_v^-1 (both lanes of a pair share them); the y lane takes Pm_x by shuffle
-// and forms M = Pm_x^T Pm_y (2x2) and M Jt_y (2x9).  The rows go to shared memory, and 27 lanes accumulate: lane
+// works on pieces of PB_CH pairs: lane (side, j) forms the rows of its pair's observation by camera x (side 0) or y
+// (side 1) from the camera's table, the point and L_v^-1 (both lanes of a pair share them); the y lane takes Pm_x by
+// shuffle and forms M = Pm_x^T Pm_y (2x2) and M Jt_y (2x9).  The rows go to shared memory, and 27 lanes accumulate: lane
 // (g, rb, cb) takes every third pair (slot g) and the 3 x 3 sub-block (rb, cb), in FP32 as packed pairs of FMAs
 // over the rank index.  The three slots are summed by two shuffles, the block is multiplied by the cameras' Jl
 // (J_c = Jt E) and written once per chunk to the FP64 S'_k: stored when the chunk is its edge's only one (the

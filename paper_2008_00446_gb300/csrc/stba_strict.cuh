@@ -3,8 +3,8 @@
 // on its own (__fadd_rn, __fmul_rn, ...), and the compiler contracts or re-associates nothing.  The
 // arithmetic of an expression is then the same in every kernel that evaluates it.  The FP32 kernels that form
 // V_v, the diagonal and the off-diagonal blocks of S'_k (Eq. 10, 13) all evaluate the reprojection Jacobian
-// of an observation (Sec. 3; stba_camtab.cuh) on this type, so that they see bitwise the same J_c and J_p
-// whether the pair pass reads the camera pass's copy or recomputes it.
+// of an observation (Sec. 3; stba_camtab.cuh) on this type, so that they see bitwise the same rows, whether the
+// pair pass reads the camera pass's copy or recomputes it.
 #pragma once
 #include <cuda_runtime.h>
 
