@@ -1683,21 +1683,24 @@ __global__ void __launch_bounds__(256) k_tri_solve(DevProblem P, const F* L, con
 // ------------------------------------------------------------------------------------------------------
 // The same solve as a data flow (clusters whose accumulators fit in shared memory: up to 94, 168 and 280 tile rows of
 // either factor with 2, 4 and 8 CTAs; k_tri_solve beyond): tile row i belongs to CTA i mod CS of the cluster's CS CTAs.
-// Forward, the owner of row k finishes t_k = r_k - sum_j L_kj y_j, forms y_k = D_k^-1 t_k and
-// sends it to every CTA with asynchronous stores counted by that CTA's mbarrier of step k; whoever has y_k subtracts
+// Forward, the owner of row k finishes t_k = r_k - sum_j L_kj y_j, forms y_k = D_k^-1 t_k and sends it to every CTA with
+// a row below k, with asynchronous stores counted by that CTA's mbarrier of step k; whoever has y_k subtracts
 // L_ik y_k from its rows i > k, row k + 1 first, whose owner then goes on to y_k+1 before its other rows.  The
-// backward pass is the same on reversed indices with L_ki^T and D_k^-T.  Only the mbarrier it counts on tells that an
-// asynchronous store has arrived (a cluster barrier orders its issue), so after a pass every CTA waits for all nt
-// pieces, the ones that none of its rows needs too: x overwrites y only once every y has arrived everywhere, and no
-// CTA leaves while a store to it is under way.  A step's chain is two 64 x 64 products by
+// backward pass is the same on reversed indices with L_ki^T and D_k^-T.  A step's chain is two 64 x 64 products by
 // 256 threads and one remote store: 0.8 us (12 clusters of 83 cameras) to 1.4 us (one of 400, whose later steps also
 // have 7 rows per CTA to update), against 2.4 us with a cluster barrier, a gather of the partial products from all
-// CTAs and five block barriers per step.  Nothing depends on a tile's address on the vector, so
-// each thread keeps its elements of the next NB tiles in registers (loads in flight while it waits for y_k).
+// CTAs and five block barriers per step.
+// Only the mbarrier that it counts on tells that an asynchronous store has arrived (a cluster barrier orders its
+// issue).  A piece goes to no CTA that does not wait for it, so
+//   - no CTA leaves while a store to it is under way;
+//   - x_k never meets y_k on its way to the same place in a CTA: a CTA that gets y_k owns a row i > k, sends x_i only
+//     after its forward pass, in which it has waited for y_k, and x_k is formed from x_i.
+// Nothing depends on a tile's address on the vector, so each thread keeps its elements of the next NB tiles in registers (loads in flight while it waits for y_k).
 // NB = 4 tiles of the FP32 factor (64 registers; 3 and 4 alike at 15 tile rows, 4 better beyond, 5 spills).
 // Solve stage with one refinement step, before (k_tri_solve, one residual CTA per tile row) -> now: 12 clusters of 83
-// cameras 180 -> 73 us, 10 of 100 194 -> 77, 13 uneven of up to 297 753 -> 290, one of 400 1053 -> 317, 67 of 90
-// 350 -> 202; FP64, 4 clusters of 94 387 -> 220.
+// cameras 180 -> 66 us, 13 uneven of up to 297 753 -> 285, one of 400 1053 -> 310, 67 of 90 350 -> 197; FP64, 4 clusters
+// of 75 387 -> 201.  With every piece sent to all CTAs, and each waiting for all of a pass before the next and before it
+// leaves: 69, 295, 324 and 202.
 template <typename F, int T> struct PushLayout {
   static constexpr int V = 16 / (int)sizeof(F);          // elements per 16-byte load
   static constexpr int PARTS = 256 / T;                  // row products: threads per row
@@ -1771,22 +1774,29 @@ __global__ void __launch_bounds__(256, T == 64 ? 2 : 3) k_tri_push(DevProblem P,
   const int row = tid / PARTS, part = tid - row * PARTS;   // row products
   const int cgp = tid % CG, rp = tid / CG;                 // column products: rows rp NL ..
   bool dead = false;
-  uint32_t rvec[(CS + PARTS - 1) / PARTS], rbar[(CS + PARTS - 1) / PARTS];   // the peers this thread sends to
+  constexpr int PEERS = (CS + PARTS - 1) / PARTS;
+  uint32_t rvec[PEERS], rbar[PEERS];   // the peers this thread sends to
 #pragma unroll
-  for (int u = 0; u < (CS + PARTS - 1) / PARTS; ++u) {
+  for (int u = 0; u < PEERS; ++u) {
     const uint32_t peer = (uint32_t)min(part + PARTS * u, CS - 1);
     rvec[u] = tc::map_rank(tc::smem_u32(vec), peer);
     rbar[u] = tc::map_rank(tc::smem_u32(mbar), peer);
   }
-  // one pass; indices i of the pass run upwards: the tile row i (forward) or nt - 1 - i (backward)
+  // Indices i of a pass run upwards: the tile row i (forward) or nt - 1 - i (backward).  The largest of CTA r's, which
+  // are equal mod CS; it takes the pieces of the indices before it (-1: it has no row).
+  auto last_of = [&](int r, bool fwd) {
+    const int first = fwd ? r : ((nt - 1 - r) % CS + CS) % CS;
+    return r < CS && r < nt ? first + CS * ((nt - 1 - first) / CS) : -1;
+  };
+  // one pass
   auto pass = [&](auto fwd_c) {
     constexpr bool FWD = decltype(fwd_c)::value;
     const int me = FWD ? rank : ((nt - 1 - rank) % CS + CS) % CS;   // this CTA's pass indices are me mod CS
-    if (nown == 0) {
-      if constexpr (!FWD) cluster.barrier_wait();
-      return;
-    }
-    const int last = me + CS * ((nt - 1 - me) / CS);
+    if (nown == 0) return;
+    const int last = last_of(rank, FWD);
+    int rlast[PEERS];
+#pragma unroll
+    for (int u = 0; u < PEERS; ++u) rlast[u] = last_of(part + PARTS * u, FWD);
     // tasks: update of index i by the vector piece of index kk (i > kk), or the diagonal product of index i (diag)
     struct Task {
       int i, kk;
@@ -1843,7 +1853,6 @@ __global__ void __launch_bounds__(256, T == 64 ? 2 : 3) k_tri_push(DevProblem P,
       fetch(tk[b], buf[b]);
     }
     Task tn = next(tk[NB - 1]);
-    if constexpr (!FWD) cluster.barrier_wait();   // every y has arrived in every CTA
     int have = -1;   // the last step whose piece has arrived
     auto work = [&](const Task& t0, const F (&cur)[NL * V]) {
       const int slot = (at(t0.i) - rank) / CS;
@@ -1876,8 +1885,8 @@ __global__ void __launch_bounds__(256, T == 64 ? 2 : 3) k_tri_push(DevProblem P,
         const F y = row_sum(row_dot(cur, tv));
         const int g = at(t0.i) * T + row;
 #pragma unroll
-        for (int u = 0; u < (CS + PARTS - 1) / PARTS; ++u)
-          if (part + PARTS * u < CS)
+        for (int u = 0; u < PEERS; ++u)
+          if (rlast[u] > t0.i)
             tc::st_async(rvec[u] + (uint32_t)(g * sizeof(F)), y, rbar[u] + (uint32_t)(8 * ((FWD ? 0 : max_nt) + at(t0.i))));
         if (part == 0) {
           if constexpr (FWD) {
@@ -1925,21 +1934,16 @@ __global__ void __launch_bounds__(256, T == 64 ? 2 : 3) k_tri_push(DevProblem P,
       }
     }
   };
-  // all pieces of a pass (barriers first .. first + nt - 1) have arrived in this CTA (a CTA that gave up a wait sends
-  // its pieces all the same)
-  auto arrived = [&](int first) {
-    for (int i = tid; i < nt; i += 256)
-      if (!tc::mbar_wait_bounded(mbar + first + i, 0, tc::WAIT_NS)) dead = true;
-  };
   pass(std::true_type{});
-  arrived(0);
-  cluster.barrier_arrive();   // waited for once the backward pass's first tiles are in flight
   __syncthreads();   // y of this CTA's rows, before the backward pass reads it
   for (int e = tid; e < nown * 256 * V; e += 256) acc[e] = F(0);   // thread-private up to the reductions, but indexed by
   __syncthreads();                                                 // another layout here
   pass(std::false_type{});
-  arrived(max_nt);
-  if (dead) atomicOr(fail_flags + k, FAIL_WAIT);   // a piece never came: the step is rejected
+  if (dead) {   // a wait gave up: the step is rejected.  What is on its way to this CTA still has to arrive
+    atomicOr(fail_flags + k, FAIL_WAIT);
+    for (int i = 0; i < last_of(rank, true); ++i) tc::mbar_wait_bounded(mbar + i, 0, tc::WAIT_NS);
+    for (int i = 0; i < last_of(rank, false); ++i) tc::mbar_wait_bounded(mbar + max_nt + nt - 1 - i, 0, tc::WAIT_NS);
+  }
   cluster.sync();
 }
 

@@ -866,9 +866,9 @@ int pcg_iterate(const DevProblem& P, Scratch<real> W, CamSlots CS, const PcgBuff
   int it = 0;
   const double tol2 = tol * tol;
   // The GPU idles about 25 us at each reading of the residual (copy, synchronisation, the next launches); a solve
-  // runs on average half an interval past its tolerance.  An interval of 8 took 4404 us instead of 4186 for a step
-  // of 1000 cameras (full system), 2423 instead of 2472 for one of 500 cameras (split), and twice the products
-  // wherever four are enough.
+  // runs on average half an interval past its tolerance.  An interval of 8 took 4400 us (48 products) instead of 4180
+  // (44) for a step of 1000 cameras (full system), 2240 instead of 2330 (48 both) for one of 500 cameras (split), and
+  // twice the products wherever four are enough.
   constexpr int CHECK_EVERY = 4;
   while (it < max_iter) {
     const int upto = std::min(it + CHECK_EVERY, max_iter);
