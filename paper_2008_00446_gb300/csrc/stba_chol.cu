@@ -1259,8 +1259,8 @@ __device__ __forceinline__ void panel_tc(uint32_t* psm, StepShared& hs, float* L
 // of step kt; both read column kt, finished by the launch before.  kt = -1: panel 0 alone; FIRST: kt = 0.  The next
 // step's CTAs start under programmatic dependent launch: they read their task while this step's last CTAs finish.
 // Factorisation stage, before (panel and update launches on two streams, scaled copy, inverses of the diagonal
-// tiles) -> now: 12 clusters of 83 cameras 357 -> 209 us, 10 of 100 404 -> 229, 13 uneven of up to 297 2186 -> 922,
-// one of 400 1560 -> 707, 67 of 90 1057 -> 681.  Of it: the panel 98 us of 357 (12 clusters), update epilogue and no
+// tiles) -> now: 12 clusters of 83 cameras 357 -> 207 us, 10 of 100 404 -> 235, 13 uneven of up to 297 2186 -> 924,
+// one of 400 1560 -> 702, 67 of 90 1057 -> 680.  Of it: the panel 98 us of 357 (12 clusters), update epilogue and no
 // scaled copy 2 (13 uneven: 190 of 2186), one launch per step 28, dependent launch 16, split operands 4 (13 uneven:
 // 272).  Panels stacked with the
 // tiles below them also where they outnumber the SMs: a separate launch for the diagonal tiles (the split panel)
